@@ -27,16 +27,16 @@
 //    One exp2 per (row, key) on that unit alone costs 8 clocks per warp and logit against 4.6 for the
 //    contraction: the pass is bound by the exp rate.  Of each 8 columns, NPOLY take a polynomial on the
 //    FMA pipe instead (ten dispatch slots each, against three slots and eight clocks of the unit); the
-//    two kinds overlap only partly, and NPOLY = 1 measured best (0: 9.06 ms, 1: 8.63, 2: 8.90, 3: 9.32 at
-//    the bench shape).
-//  * To keep the slot count low there is no running maximum: the reference m of a row is the maximum of
-//    the first logits the thread saw, later logits may exceed it (2^x is evaluated for x up to 126), and
-//    only if a partial sum grows past 2^40 is the reference moved (a rare, slower path that also serves
-//    tiles cut by the end of the request or by the causal diagonal).
-// Polynomial: y = sat(x/252 + 1/2) clamps x to [-126, 126] inside the multiply-add that forms it;
-// j = round(x) by the magic-number addition, f = x - j in [-0.5, 0.5], 2^x = 2^j p(f) with p a cubic
-// fitted to 2^f (max relative error 7.5e-5, far inside the 2e-3 score tolerance), 2^j applied by adding
-// j to the exponent field.
+//    two kinds overlap only partly, and NPOLY = 1 measured best (16 layers of 8 x 35000 keys, 512 rows:
+//    0: 2.83 ms, 1: 2.75, 2: 2.84).
+//  * To keep the slot count low there is no running maximum: the reference e of a row is the maximum of
+//    the first logits the thread saw, in log2 units and rounded to an integer; later logits may exceed it
+//    (2^x is evaluated for x up to 126), and only if a partial sum grows past 2^40 is the reference moved (a
+//    rare, slower path that also serves tiles cut by the end of the request or by the causal diagonal).
+// Polynomial: textbook range reduction (Cody and Waite, Software Manual for the Elementary Functions, 1980):
+// x = v c = j + f with j the nearest integer (adding and subtracting 1.5 2^23) and f in [-0.5, 0.5], 2^f by a cubic
+// fitted here (max relative error 7.5e-5, far inside the 2e-3 score tolerance), 2^(j - e) by an integer addition to
+// the exponent field, j - e clamped to [-126, 126].  The reference being an integer, it enters in that addition only.
 #pragma once
 
 #include "tc_common.cuh"
@@ -45,55 +45,49 @@ namespace actkv {
 namespace tc {
 
 constexpr int LSE_NPOLY = 1;                     // columns of every 8 whose exp2 is the polynomial
+constexpr float EXP2_ROUND = 12582912.f;         // 1.5 * 2^23: adding it rounds to the nearest integer
 
-__device__ __forceinline__ float ffma_sat(float a, float b, float c) {
-  float d;
-  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-
-// 2^x for x = 252 y - 126, y in [0, 1]
-__device__ __forceinline__ float exp2_poly_y(float y) {
-  constexpr float MAGIC = 12582912.f;            // 1.5 * 2^23: adding it rounds to the nearest integer
-  const float t = fmaf(y, 252.f, MAGIC - 126.f); // MAGIC + j, j = round(x), in the low mantissa bits
-  const float j = t - MAGIC;
-  const float f = fmaf(y, 252.f, -126.f - j);    // x - j
+// 2^(v c - e) for an integer e, neg_e = -e
+__device__ __forceinline__ float exp2_poly(float v, float c, float neg_e) {
+  const float t = fmaf(v, c, EXP2_ROUND + neg_e);                  // j - e = round(v c - e) in the low mantissa bits
+  const float f = fmaf(v, c, neg_e - (t - EXP2_ROUND));            // v c - j
   float p = fmaf(0.0551716648042202f, f, 0.2426111251115799f);
   p = fmaf(p, f, 0.6932609677314758f);
   p = fmaf(p, f, 0.9999280571937561f);
-  return __int_as_float(__float_as_int(p) + (__float_as_int(t) << 23));
+  const float k = fminf(fmaxf(t, EXP2_ROUND - 126.f), EXP2_ROUND + 126.f);
+  return __int_as_float(__float_as_int(p) + (__float_as_int(k) << 23));
 }
 
-// 32 logits of one row, all visible, against the row's reference m (finite): returns
-// sum_i exp2((v_i - m) c).  nmc = -m c; c1 = c / 252, c0 = 1/2 - m c / 252.
+// 32 logits of one row, all visible, against the row's reference e (finite, below LSE_REF_MAX): returns
+// sum_i 2^(v_i c - e).  Two partial sums: the registers that more of them take cost more than the shorter chains give
+// (2.75 ms with two, 2.86 with four, for 16 layers of 8 x 35000 keys and 512 rows).
 template <int NPOLY>
-__device__ __forceinline__ float lse_fast32(const float* v, float c, float nmc, float c1, float c0) {
-  float s[4] = {0.f, 0.f, 0.f, 0.f};
+__device__ __forceinline__ float lse_fast32(const float* v, float c, float neg_e) {
+  float s[2] = {0.f, 0.f};
 #pragma unroll
   for (int g8 = 0; g8 < 4; ++g8) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const float x = v[g8 * 8 + i];
       // the polynomial columns are spread over the group so that the two kinds interleave in program order
-      const bool poly = (NPOLY >= 1 && i == 1) || (NPOLY >= 2 && i == 4) || (NPOLY >= 3 && i == 6) || (NPOLY >= 4 && i == 3);
-      const float e = poly ? exp2_poly_y(ffma_sat(x, c1, c0)) : exp2f(fmaf(x, c, nmc));
-      s[i & 3] += e;
+      const bool poly = (NPOLY >= 1 && i == 4) || (NPOLY >= 2 && i == 1) || (NPOLY >= 3 && i == 6) || (NPOLY >= 4 && i == 3);
+      s[i & 1] += poly ? exp2_poly(x, c, neg_e) : exp2f(fmaf(x, c, neg_e));
     }
   }
-  return (s[0] + s[1]) + (s[2] + s[3]);
+  return s[0] + s[1];
 }
 
 // The general form: logits n_lo <= i < nv (any integers) are visible; moves the reference to the maximum seen
-// so far.  Also the entry for a row's first logits (m = -inf, sum = 0).
-__device__ __forceinline__ void lse_slow32(const float* v, int n_lo, int nv, float c, float& m, float& sum) {
+// so far.  Also the entry for a row's first logits (e = -inf, sum = 0).
+__device__ __forceinline__ void lse_slow32(const float* v, int n_lo, int nv, float c, float& e, float& sum) {
   if (nv <= 0 || n_lo >= 32 || n_lo >= nv) return;
   float gm = -INFINITY;
 #pragma unroll
   for (int i = 0; i < 32; ++i) gm = fmaxf(gm, (i >= n_lo && i < nv) ? v[i] : -INFINITY);
-  if (gm > m) { sum = (m == -INFINITY) ? 0.f : sum * exp2f((m - gm) * c); m = gm; }
-  const float mc = m * c;
+  const float ge = rintf(gm * c);
+  if (ge > e) { sum = (e == -INFINITY) ? 0.f : sum * exp2f(e - ge); e = ge; }
 #pragma unroll
-  for (int i = 0; i < 32; ++i) sum += (i >= n_lo && i < nv) ? exp2f(fmaf(v[i], c, -mc)) : 0.f;
+  for (int i = 0; i < 32; ++i) sum += (i >= n_lo && i < nv) ? exp2f(fmaf(v[i], c, -e)) : 0.f;
 }
 
 constexpr int LSE_EPI_WARPS = 16;                // (TMEM lane quarter, accumulator, column half)
@@ -107,6 +101,7 @@ constexpr int LSE_THREADS = (LSE_EPI_WARP0 + LSE_EPI_WARPS) * 32;
 constexpr int LSE_SLOTS = 2;                     // accumulators
 constexpr int LSE_A_COLS = 256;                  // TMEM columns holding the four Q blocks
 constexpr float LSE_BIG = 1099511627776.f;       // 2^40: a partial sum beyond it moves the reference
+constexpr float LSE_REF_MAX = 1048576.f;         // references beyond 2^20 (rounding to integers needs |v c| < 2^22) take the general form
 
 struct LseBarriers {
   uint64_t k_full[8];
@@ -117,7 +112,7 @@ struct LseBarriers {
   uint64_t drained[2];
   uint32_t tmem_base;
   int abort_flag;
-  float2 state[2][4][2][128];  // (reference, sum) per (group, row block, column half, row in block)
+  float2 state[2][4][2][128];  // (reference e, sum of 2^(v c - e)) per (group, row block, column half, row in block)
 };
 
 // After tcgen05.wait::ld: ties the loaded registers to the wait, so that no use of them is scheduled
@@ -143,7 +138,7 @@ __device__ __forceinline__ int sel4(const int (&x)[4], int i) { return i == 0 ? 
 template <int NPOLY, bool WIN>
 __device__ __forceinline__ bool lse_job(LseBarriers* bars, volatile int* abort_flag, uint32_t tq, int grp, int job,
                                         int mb, float2* st, int nv_min, int nlo_max, const int (&jm)[4], const int (&jl)[4],
-                                        int key0, float c, float c1, int lane, long long wait_cycles) {
+                                        int key0, float c, int lane, long long wait_cycles) {
   float v[64];
   float* va = v;
   float* vb = v + 32;
@@ -156,11 +151,11 @@ __device__ __forceinline__ bool lse_job(LseBarriers* bars, volatile int* abort_f
   tc_fence_before();
   __syncwarp();
   if (lane == 0) mbar_arrive(smem_u32(&bars->tmem_empty[grp]));
-  bool slow = __any_sync(0xffffffffu, nv_min < 64 || (WIN && nlo_max > 0) || ms.x == -INFINITY);
+  // (a reference of -inf, before the row's first logits, fails the second test)
+  bool slow = __any_sync(0xffffffffu, nv_min < 64 || (WIN && nlo_max > 0) || !(fabsf(ms.x) < LSE_REF_MAX));
   if (!slow) {
-    const float nmc = -ms.x * c, c0 = fmaf(nmc, 1.f / 252.f, 0.5f);
-    const float ps = lse_fast32<NPOLY>(va, c, nmc, c1, c0) + lse_fast32<NPOLY>(vb, c, nmc, c1, c0);
-    slow = __any_sync(0xffffffffu, !(ps < LSE_BIG));
+    const float ps = lse_fast32<NPOLY>(va, c, -ms.x) + lse_fast32<NPOLY>(vb, c, -ms.x);
+    slow = __any_sync(0xffffffffu, !(fabsf(ps) < LSE_BIG));
     if (!slow) ms.y += ps;
   }
   if (slow) {
@@ -352,14 +347,14 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
     }
     const int jfast = min(min(jm[0], jm[1]), min(jm[2], jm[3]));
     const int jlmax = max(max(jl[0], jl[1]), max(jl[2], jl[3]));
-    const float c = a.scale_log2, c1 = c * (1.f / 252.f);
+    const float c = a.scale_log2;
     const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16) + LSE_A_COLS + grp * 128 + half * 64;
     // (key tile, row block) of this group's jobs, carried along without divisions: job = tile * n_mb + mb
     int mb = grp % n_mb, key0 = (t_begin + grp / n_mb) * TK + half * 64;
     const int mb_step = 2 % n_mb, tile_step = 2 / n_mb;
     for (int job = grp; job < n_jobs; job += 2) {
       epi_ok = lse_job<NPOLY, WIN>(bars, abort_flag, tq, grp, job, mb, &bars->state[grp][mb][half][rib], jfast - key0 + 1,
-                              jlmax - key0, jm, jl, key0, c, c1, lane, ta.wait_cycles);
+                              jlmax - key0, jm, jl, key0, c, lane, ta.wait_cycles);
       if (!epi_ok) break;
       mb += mb_step;
       key0 += tile_step * TK;
@@ -372,7 +367,6 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
   if (warp >= LSE_EPI_WARP0 && k == 0 && !*abort_flag) {
     // merge the four shares (group, column half) of each row, store (reference in log2 units, sum); (-inf, 0) when the
     // row saw no key of this chunk
-    const float c = a.scale_log2;
 #pragma unroll
     for (int mb = 0; mb < 4; ++mb) {
       const int n = mb * 128 + rib;
@@ -384,10 +378,9 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
         float ss = 0.f;
         if (mm > -INFINITY) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) ss += o[i].x > -INFINITY ? o[i].y * exp2f((o[i].x - mm) * c) : 0.f;
+          for (int i = 0; i < 4; ++i) ss += o[i].x > -INFINITY ? o[i].y * exp2f(o[i].x - mm) : 0.f;
         }
-        a.partials[((int64_t)u * a.n_chunks + chunk) * a.rows_max + row0 + n] =
-            make_float2(mm == -INFINITY ? mm : mm * a.scale_log2, ss);
+        a.partials[((int64_t)u * a.n_chunks + chunk) * a.rows_max + row0 + n] = make_float2(mm, ss);
       }
     }
   }
