@@ -60,7 +60,7 @@ typedef struct CUstream_st* actkv_stream_t;
  * Any strides with contiguous head dimensions describe a pool (slot-major [page][slot][head][dim]
  * pages as well as head-major [page][head][slot][dim] ones).  The tensor-core score path needs
  * page_size 16, 32, 64 or 128, head_dim 64 or 128, strides that are multiples of 8 elements and a
- * 128-byte aligned base; other shapes take the (much slower) FMA path.
+ * 128-byte aligned base; other shapes take warp-level matrix instructions.
  */
 typedef struct {
   void*   base;                 /* device, bf16 */
@@ -192,7 +192,7 @@ int actkv_score_sliding(const actkv_pool_t* pool /* host */, const actkv_tables_
 /* ---------------------------------------------------------------------------------------
  * actkv_score_path — which kernels actkv_score (streaming == 0) or actkv_score_accumulate
  * (streaming != 0) would run for this pool, group size, window bound, scale and query pointer:
- * 1 = the tensor-core kernels (tcgen05), 0 = the FMA kernels, negative = bad argument.
+ * 1 = the tensor-core kernels (tcgen05), 0 = the warp-level (mma.sync) kernels, negative = bad argument.
  * Launches nothing.  (Section 7.1 / Algorithm 3 are the same arithmetic on both paths.)
  */
 int actkv_score_path(const actkv_pool_t* pool /* host */, int32_t n_q_heads, int32_t max_win,
@@ -371,7 +371,7 @@ int actkv_compact(const actkv_pool_t* pool /* host */, const actkv_tables_t* tab
  *   result of the score does not depend on it.  On the tensor-core path four spare warps per CTA of the
  *   pooled-score kernel take items (32 (slot, head) pairs of one destination page of one request and
  *   layer) of the pending job from a queue for as long as their CTA is scoring; the LSE kernel (whose
- *   epilogue needs every register of the SM) and the FMA path take none.
+ *   epilogue needs every register of the SM) and the mma.sync path take none.
  * actkv_compact_end: the same arguments as the actkv_compact_begin it closes.  Copies every item
  *   not yet taken, then, when layer_end == pool->n_layers, updates the tables as actkv_compact does.
  * begin + end without a score call in between equals actkv_compact.  Pools the item copy does not

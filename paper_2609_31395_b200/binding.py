@@ -333,7 +333,7 @@ def actkv_score_sliding(pool: PoolDesc, tables: TablesDesc, layer_begin, layer_e
 
 
 def actkv_score_path(pool: PoolDesc, n_q_heads, max_win, sm_scale, q, streaming=False) -> int:
-    """1: the tensor-core kernels would run, 0: the FMA kernels."""
+    """1: the tensor-core kernels would run, 0: the warp-level (mma.sync) kernels."""
     rc = load().actkv_score_path(C.byref(pool), n_q_heads, max_win, float(sm_scale), _ptr(q, torch.bfloat16, "q"),
                                  int(bool(streaming)))
     if rc < 0:

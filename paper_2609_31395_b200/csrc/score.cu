@@ -1,12 +1,11 @@
 // actkv_score: host entry point and path selection.
 //   tensor-core path (score_tc.cuh): window x group rows >= 64 (any row count for the streaming update),
 //   page 16, head_dim 128, packed pool;
-//   FMA path (score_fma.cuh): everything else.
+//   warp-level mma path (score_mma.cuh): everything else.
 // actkv_score_accumulate (streaming, Algorithm 3 per decode step) runs the pooled-score pass alone against
 // the supplied LSE and folds its result into the running mean held in the score array.
 // Both write per-chunk (max, sum) partials of the LSE pass into the caller's workspace, merge them
 // with lse_combine_kernel, then run the pooled-score pass against the merged (or supplied) LSE.
-#include "score_fma.cuh"
 #include "score_tc.cuh"
 
 namespace actkv {
@@ -70,7 +69,7 @@ static int score_impl(int mode, const actkv_pool_t* pool, const actkv_tables_t* 
   if (D <= 0 || D % 8 != 0 || D > 256 || Hkv <= 0 || pool->page_size <= 0) return ACTKV_E_INVALID;
   if (n_q_heads <= 0 || n_q_heads % Hkv != 0) return ACTKV_E_INVALID;
   const int G = n_q_heads / Hkv;
-  if (G > FMA_RQ) return ACTKV_E_INVALID;
+  if (G > MAX_GROUP) return ACTKV_E_INVALID;
   if (R < 0 || sum_win < 0 || max_win < 0 || sum_tok < 0 || max_tok < 0 || window_left < 0) return ACTKV_E_INVALID;
   if (((uintptr_t)pool->base & 15) || pool->stride_layer % 8 || pool->stride_page % 8 || pool->stride_slot % 8 ||
       pool->stride_head % 8 || ((uintptr_t)q & 15))
@@ -121,8 +120,8 @@ static int score_impl(int mode, const actkv_pool_t* pool, const actkv_tables_t* 
     a.lse_chunk = chunk;
     a.n_chunks = (max_tok + chunk - 1) / chunk;    // <= lay.n_chunks
   }
-  a.n_tiles = (max_tok + FMA_TK - 1) / FMA_TK;
   a.scale_log2 = sm_scale * kLog2e;
+  a.page_shift = (pool->page_size & (pool->page_size - 1)) == 0 ? __builtin_ctz((unsigned)pool->page_size) : -1;
   a.causal = causal;
   a.win_left = window_left;
   a.acc_steps = acc_steps;
@@ -134,14 +133,8 @@ static int score_impl(int mode, const actkv_pool_t* pool, const actkv_tables_t* 
       int rc = score_tc_launch_lse(a, pool, max_tok, max_win, s);
       if (rc != ACTKV_OK) return rc;
     } else {
-      const int64_t grid1 = units * a.n_chunks;
-      if (grid1 > 0x7fffffffLL) return ACTKV_E_INVALID;
-      const size_t sm1 = score_fma_smem_bytes(D, lay.rows_max, 1);
-      if (sm1 > 200 * 1024) return ACTKV_E_INVALID;
-      if (ensure_dyn_smem(score_fma_kernel<1>, sm1) != cudaSuccess)
-        return ACTKV_E_CUDA;
-      score_fma_kernel<1><<<(unsigned)grid1, FMA_NT, sm1, s>>>(a);
-      ACTKV_CHECK_LAUNCH();
+      const int rc = wm::launch_lse(a, units, s);
+      if (rc != ACTKV_OK) return rc;
     }
     const int64_t n_rows_all = units * lay.rows_max;
     lse_combine_kernel<<<(unsigned)((n_rows_all + 255) / 256), 256, 0, s>>>(a, lse_buf, nullptr);
@@ -155,14 +148,7 @@ static int score_impl(int mode, const actkv_pool_t* pool, const actkv_tables_t* 
   if (!lse) return ACTKV_E_INVALID;
   a.lse = lse;
   if (use_tc) return score_tc_launch_score(a, pool, max_tok, max_win, s, (CompactWs*)copy_ws);
-  const int64_t grid2 = units * a.n_tiles;
-  if (grid2 > 0x7fffffffLL) return ACTKV_E_INVALID;
-  const size_t sm2 = score_fma_smem_bytes(D, lay.rows_max, 2);
-  if (ensure_dyn_smem(score_fma_kernel<2>, sm2) != cudaSuccess)
-    return ACTKV_E_CUDA;
-  score_fma_kernel<2><<<(unsigned)grid2, FMA_NT, sm2, s>>>(a);
-  ACTKV_CHECK_LAUNCH();
-  return ACTKV_OK;
+  return wm::launch_pool(a, units, max_tok, s);
 }
 
 int actkv_score(const actkv_pool_t* pool, const actkv_tables_t* tables, int32_t layer_begin,

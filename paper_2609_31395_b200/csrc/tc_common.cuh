@@ -4,7 +4,7 @@
 #include <cuda.h>
 
 #include "compact_job.cuh"
-#include "score_fma.cuh"
+#include "score_mma.cuh"
 
 namespace actkv {
 namespace tc {
