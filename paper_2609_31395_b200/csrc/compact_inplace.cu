@@ -206,7 +206,7 @@ __global__ void compact_inplace_plan_kernel(TablesView tab, PoolView pool, const
   ws->src_tab = src_tab;
   ws->dst_tab = dst_tab;
   ws->items_per_slab = (int32_t)max((int64_t)1, min(per_slab, (int64_t)0x7fffffff));
-  ws->pad2 = 0;
+  ws->free_count = 0;
 }
 
 // One warp per item: the 32 region slots [32 chunk, 32 chunk + 32) of one (layer, head, request), classified as

@@ -34,14 +34,15 @@ struct CompactWs {
   uint32_t* dst_tab;     // deferred in-place copy: resolved destinations, [n_items][32]; nullptr for the fresh-page form,
                          // whose destinations follow from the item number
   int32_t items_per_slab;  // items of one layer (>= 1): the layer of an item is item / items_per_slab
-  int32_t pad2;
-  // followed by int32 new_off[R], push_off[R], item_off[R + 1], new_pages[R * max_pages]
+  int32_t free_count;    // of the tables, when the plan was made
+  // followed by int32 old_len[R] (length of a request that is compacted, -1 of one that is not), push_off[R],
+  // item_off[R + 1] (first new page of a request in the run of new pages; in-place form: first item), new_pages[R * max_pages]
 };
 
-__host__ __device__ __forceinline__ int32_t* ws_new_off(CompactWs* w) { return reinterpret_cast<int32_t*>(w + 1); }
-__host__ __device__ __forceinline__ int32_t* ws_push_off(CompactWs* w, int R) { return ws_new_off(w) + R; }
-__host__ __device__ __forceinline__ int32_t* ws_item_off(CompactWs* w, int R) { return ws_new_off(w) + 2 * R; }
-__host__ __device__ __forceinline__ int32_t* ws_new_pages(CompactWs* w, int R) { return ws_new_off(w) + 3 * R + 1; }
+__host__ __device__ __forceinline__ int32_t* ws_old_len(CompactWs* w) { return reinterpret_cast<int32_t*>(w + 1); }
+__host__ __device__ __forceinline__ int32_t* ws_push_off(CompactWs* w, int R) { return ws_old_len(w) + R; }
+__host__ __device__ __forceinline__ int32_t* ws_item_off(CompactWs* w, int R) { return ws_old_len(w) + 2 * R; }
+__host__ __device__ __forceinline__ int32_t* ws_new_pages(CompactWs* w, int R) { return ws_old_len(w) + 3 * R + 1; }
 
 constexpr uint32_t CJ_NONE = 0xffffffffu;
 constexpr int32_t CJ_PLAN_MARK = 0x414b5650;      // a fresh-page plan
