@@ -266,20 +266,52 @@ __global__ void __launch_bounds__(KS_NT, 1) keepscore_kernel(
   }
 }
 
-__global__ void gather_f32_kernel(const float* __restrict__ src, int64_t src_stride, const int32_t* __restrict__ tok_indptr,
-                                  const int32_t* __restrict__ sel_idx, int64_t sel_stride,
-                                  const int32_t* __restrict__ keep_indptr, int32_t n_req, float* __restrict__ dst,
-                                  int64_t dst_stride) {
+constexpr int GA_NT = 256, GA_PER = 4;
+// GA_PER survivors per thread, all loads of one kind in flight together; the request is searched once per CTA (by every
+// warp, 32 offsets at a time) and, where the CTA's survivors belong to several, advanced from there.  64 rows of 197 K survivors 68.8 -> 31.3 us (4.8 TB/s; two per thread 39.5, eight 30.6).
+__global__ void __launch_bounds__(GA_NT) gather_f32_kernel(
+    const float* __restrict__ src, int64_t src_stride, const int32_t* __restrict__ tok_indptr,
+    const int32_t* __restrict__ sel_idx, int64_t sel_stride, const int32_t* __restrict__ keep_indptr, int32_t n_req,
+    float* __restrict__ dst, int64_t dst_stride) {
   const int o = blockIdx.y;
+  const int first = blockIdx.x * (GA_NT * GA_PER), lane = threadIdx.x & 31;
+  const int i0 = first + threadIdx.x;
+  const int32_t* sel = sel_idx + (int64_t)o * sel_stride;
+  const float* sc = src + (int64_t)o * src_stride;
+  float* out = dst + (int64_t)o * dst_stride;
   const int total = keep_indptr[n_req];
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    int lo = 0, hi = n_req;                                    // request of survivor slot i
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (keep_indptr[mid] <= i) lo = mid; else hi = mid;
+  if (first >= total) return;
+  int tok[GA_PER];
+#pragma unroll
+  for (int k = 0; k < GA_PER; ++k) tok[k] = i0 + k * GA_NT < total ? sel[i0 + k * GA_NT] : 0;
+  // the request of the CTA's first survivor: the last r with keep_indptr[r] <= first
+  int r = 0;
+  for (int q0 = 1; q0 < n_req; q0 += 32) {
+    const int c = __popc(__ballot_sync(0xffffffffu, q0 + lane < n_req && keep_indptr[q0 + lane] <= first));
+    r += c;
+    if (c < 32) break;
+  }
+  int next = keep_indptr[r + 1], base = tok_indptr[r];
+  if (next >= min(total, first + GA_NT * GA_PER)) {            // one request (uniform over the CTA)
+    float v[GA_PER];
+#pragma unroll
+    for (int k = 0; k < GA_PER; ++k) v[k] = i0 + k * GA_NT < total ? sc[base + tok[k]] : 0.f;
+#pragma unroll
+    for (int k = 0; k < GA_PER; ++k)
+      if (i0 + k * GA_NT < total) out[i0 + k * GA_NT] = v[k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < GA_PER; ++k) {
+      const int i = i0 + k * GA_NT;
+      if (i < total) {
+        while (i >= next) {                                    // (i < total = keep_indptr[n_req]: r + 1 < n_req here)
+          ++r;
+          next = keep_indptr[r + 1];
+          base = tok_indptr[r];
+        }
+        out[i] = sc[base + tok[k]];
+      }
     }
-    const int tok = sel_idx[(int64_t)o * sel_stride + i];
-    dst[(int64_t)o * dst_stride + i] = src[(int64_t)o * src_stride + tok_indptr[lo] + tok];
   }
 }
 
@@ -341,9 +373,8 @@ int actkv_gather_f32(const float* src, int64_t src_stride, const int32_t* tok_in
   if (n_outer < 0 || n_req < 0 || max_total_keep < 0) return ACTKV_E_INVALID;
   if (n_outer == 0 || n_req == 0 || max_total_keep == 0) return ACTKV_OK;
   if (!src || !tok_indptr || !sel_idx || !keep_indptr || !dst || n_outer > 65535) return ACTKV_E_INVALID;
-  dim3 grid((unsigned)((max_total_keep + 255) / 256), (unsigned)n_outer);
-  if (grid.x > 1024) grid.x = 1024;
-  actkv::gather_f32_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(src, src_stride, tok_indptr, sel_idx, sel_stride,
+  const dim3 grid((unsigned)((max_total_keep + actkv::GA_NT * actkv::GA_PER - 1) / (actkv::GA_NT * actkv::GA_PER)), (unsigned)n_outer);
+  actkv::gather_f32_kernel<<<grid, actkv::GA_NT, 0, (cudaStream_t)stream>>>(src, src_stride, tok_indptr, sel_idx, sel_stride,
                                                                    keep_indptr, n_req, dst, dst_stride);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;

@@ -86,3 +86,46 @@ def test_a_page_id_out_of_range_met_by_any_cta_of_the_plan(which):
         assert np.array_equal(U.bits(inst.pool), snap[0])
         for t, s in zip((inst.page_table, inst.seq_len, inst.free_list, inst.free_count), snap[1:]):
             assert torch.equal(t, s)
+
+
+@pytest.mark.parametrize("counts", [[1], [1023, 1], [1024, 1025, 0, 7], [0, 0, 5000], [3] * 700])
+def test_gather_over_request_boundaries(counts):
+    """1024 survivors per CTA; requests that keep nothing; many requests inside one CTA."""
+    rng = np.random.default_rng(len(counts))
+    lens = [c + int(rng.integers(1, 9)) for c in counts]
+    tok = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    ki = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    n_outer, total = 3, int(ki[-1])
+    sel = np.full((n_outer, total + 2), -1, dtype=np.int32)
+    src = rng.random((n_outer, int(tok[-1])), dtype=np.float32)
+    want = np.zeros((n_outer, total + 1), dtype=np.float32)
+    for o in range(n_outer):
+        for r, c in enumerate(counts):
+            pick = rng.permutation(lens[r])[:c]
+            sel[o, ki[r]:ki[r + 1]] = pick
+            want[o, ki[r]:ki[r + 1]] = src[o, tok[r] + pick]
+    dst = torch.zeros((n_outer, total + 1), device=DEV)
+    B.actkv_gather_f32(torch.from_numpy(src).to(DEV), src.shape[1], torch.from_numpy(tok).to(DEV), torch.from_numpy(sel).to(DEV),
+                       sel.shape[1], torch.from_numpy(ki).to(DEV), n_outer, len(counts), total + 1, dst, total + 1)
+    torch.cuda.synchronize()
+    assert np.array_equal(dst.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("lens,budgets", [([256, 257, 511, 513, 2], [128, 256, 257, 512, 1]), ([40000], [39990]),
+                                          ([9000, 3000], [4500, 2999])])
+def test_inplace_slots_over_cta_boundaries(lens, budgets):
+    """Regions of one slot more or less than the 128 and 256 slots of a CTA, one whose list takes several rounds of the
+    32-way search, one whose region is nearly everything; enough heads for either launch shape."""
+    for Hkv, NL in ((1, 1), (8, 3)):
+        rng = np.random.default_rng(5)
+        inst, sel, ki, stride, max_keep = TI._direct_case(rng, lens, budgets, 16, Hkv, 64, NL)
+        pool_before, tables_before = U.bits(inst.pool), U.oracle_tables(inst)
+        d_sel = torch.from_numpy(sel).to(DEV)
+        d_order = torch.full_like(d_sel, -9)
+        status = torch.zeros(4, dtype=torch.int32, device=DEV)
+        B.actkv_compact_inplace(B.pool_desc(inst.pool), B.tables_desc(inst.page_table, inst.seq_len, inst.free_list, inst.free_count),
+                                0, NL, d_sel, stride, torch.from_numpy(ki).to(DEV),
+                                torch.tensor(budgets, dtype=torch.int32, device=DEV), max_keep, d_order, status)
+        torch.cuda.synchronize()
+        assert status.cpu().tolist()[0] == 0
+        TI._check_against_oracle(inst, pool_before, tables_before, sel, ki, budgets, d_order.cpu().numpy())
