@@ -13,7 +13,7 @@
 // back.
 #include <mutex>
 
-#include "common.cuh"
+#include "select_core.cuh"
 
 #define ACTKV_TRY(expr)            \
   do {                             \
@@ -96,9 +96,9 @@ static int step_groups(const actkv_pool_t* pool, const actkv_tables_t* tab, cons
       if (budget_ready != nullptr) ACTKV_TRY(wait(s, budget_ready));
       ACTKV_TRY(actkv_keep_indptr(tab->seq_len, io->budget_dev, R, io->keep_indptr_dev, stream));
     }
-    ACTKV_TRY(actkv_select(io->score_dev, io->tok_indptr_dev, io->sum_tok, io->budget_dev, (l1 - l0) * Hkv, R,
-                           io->keep_indptr_dev, io->sel_idx_dev, io->sel_stride, nullptr, nullptr, nullptr, 0,
-                           io->status_dev, stream));
+    ACTKV_TRY(actkv::select_launch(io->score_dev, io->tok_indptr_dev, io->sum_tok, io->max_tok, io->budget_dev, (l1 - l0) * Hkv,
+                                   R, io->keep_indptr_dev, io->sel_idx_dev, io->sel_stride, nullptr, nullptr, io->status_dev,
+                                   s));
     if (g == n_groups - 1) {
       // nothing follows the last group that could carry its copies: the one-launch copy
       ACTKV_TRY(actkv_compact(pool, tab, l0, l1, io->sel_idx_dev, io->sel_stride, io->keep_indptr_dev, io->budget_dev,

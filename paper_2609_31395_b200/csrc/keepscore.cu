@@ -2,27 +2,21 @@
 // actkv_gather_f32 (the keep-scores of the survivors move with them, Algorithm 1 step 5 returns KS').
 //
 // Per (layer x KV head, request) unit, one CTA:
-//   1. mass m_i = floor(clip(score_i, 0, 256) * 2^32) as 64-bit integers; total = sum m_i (exact,
-//      read off the first histogram);
-//   2. mark = ceil(p_q * total / 10000); a radix search (digits of 12, 12 and 8 bits) over the
-//      order-preserving image of the scores, kept in shared memory, with 64-bit integer mass histograms
-//      finds the threshold score T with mass(score > T) < mark <= mass(score >= T) — exact, independent of
-//      summation order;
+//   1. mass m_i = floor(clip(score_i, 0, 256) * 2^32) as 64-bit integers; total = sum m_i (exact);
+//   2. mark = ceil(p_q * total / 10000); histograms of the integer mass over ever smaller key ranges (even bins, as
+//      in select_core.cuh) and a ranking of the last few entries find the threshold score T with
+//      mass(score > T) < mark <= mass(score >= T) — exact, independent of summation order;
 //   3. entries above T are hits; of the entries equal to T the first ceil((mark - mass_above)/m_T)
-//      by index are hits (ordered sweep with a block scan, as in select);
+//      by index are hits (the index of the last one is looked up only when not all of them are);
 //   4. KS = lambda*KS + score*[hit], one float32 rounding per operation; the score buffer is
 //      overwritten with the ranking key: KS, or +inf for the protected prefix.
 #include "select_core.cuh"
 
 namespace actkv {
 
-constexpr int KS_NT = 1024;
-constexpr int KS_ITEMS = 4;
+constexpr int KS_BINS = 2048;
+constexpr int KS_LIST = 256;             // entries that are ranked against one another
 
-__device__ __forceinline__ uint32_t ks_order_key(float x) {
-  uint32_t b = __float_as_uint(x);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
 __device__ __forceinline__ unsigned long long ks_mass(float x) {
   const float c = fminf(fmaxf(x, 0.f), 256.f);
   return __float2ull_rz(c * 4294967296.f);               // exact: a power-of-two scaling, then truncation
@@ -41,15 +35,7 @@ __device__ __forceinline__ float add_ieee(float a, float b) {
   return d;
 }
 
-__device__ __forceinline__ float ks_key_to_float(uint32_t k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
-
-constexpr int KS_BINS = 4096;
-constexpr size_t KS_SMEM = 232448 - 1024;                              // (nearly) all of an SM's shared memory
-constexpr int KS_CAP = (int)((KS_SMEM - KS_BINS * 12) / 4);            // keys that fit beside the histogram
 // (chunk sums stay below 2^32 for units of up to 2^17 entries; the total mass needs 2^16 or fewer, see below)
-
 // What the fused form needs of actkv_select's arguments.
 struct FusedSelectArgs {
   const int32_t* budget;
@@ -61,31 +47,43 @@ struct FusedSelectArgs {
   int32_t* status;
 };
 
-// FUSED: the ranking keys go straight into TopK (the second half of select_kernel, on the keys in shared memory)
-// instead of back to the score array: one read of the scores, one launch.  Every unit must fit in shared memory.
-template <bool FUSED>
-__global__ void __launch_bounds__(KS_NT, 1) keepscore_kernel(
+template <int NT>
+struct KeepShared {
+  SelectShared<NT> sel;
+  unsigned long long warp_tot[NT / 32];
+  unsigned long long mass[KS_LIST];      // of the entries in sel.list
+  unsigned long long above;
+  uint32_t bin, thr, eq_total;
+  int32_t last_tie;
+};
+
+// FUSED: the ranking keys go straight into TopK (select_core.cuh, on the keys in shared memory) instead of back to the
+// score array: one read of the scores, one launch.  Every unit must fit in shared memory.
+// What bounds it: latency, as in select.cu.  64 units x 16 requests of 8K-24K tokens 318 -> 146 us, 512 units of 35000
+// 328 -> 202 us (fixed digits of 12, 12 and 8 bits and two ordered sweeps with block scans before).
+template <bool FUSED, int NT>
+__global__ void __launch_bounds__(NT) keepscore_kernel(
     float* __restrict__ score, const int32_t* __restrict__ tok_indptr, int32_t sum_tok, int32_t n_req,
     int32_t p_q, float lambda, const int32_t* __restrict__ n_protect, float* __restrict__ keep_score,
-    uint32_t* __restrict__ hit_mask, FusedSelectArgs fs) {
-  static_assert(KS_NT == SEL_NT && KS_BINS == SEL_BINS, "the fused form runs select's second half in this CTA");
+    uint32_t* __restrict__ hit_mask, int32_t cap, FusedSelectArgs fs) {
+  constexpr int WARPS = NT / 32, PER = KS_BINS / NT;
   // A mass is below 2^41; its three 14-bit chunks are summed in three 32-bit histograms (native shared
-  // atomics; a 64-bit shared atomic is a compare-and-swap loop) and put together when the bins are scanned.
+  // atomics; a 64-bit shared atomic is a compare-and-swap loop) and put together when the bins are scanned.  A chunk
+  // of zeros, as most masses have, is not added.
   extern __shared__ __align__(16) uint32_t ks_smem[];
-  uint32_t* hist = ks_smem;                                            // [3][KS_BINS] mass chunks per digit
-  uint32_t* skeys = ks_smem + 3 * KS_BINS;                             // [KS_CAP] order keys of the unit
+  __shared__ KeepShared<NT> sh;
+  uint32_t* hist = ks_smem;                                            // [3][KS_BINS] mass chunks per bin
+  uint32_t* skeys = ks_smem + 3 * KS_BINS;                             // [cap] order keys of the unit
   auto hist_add = [&](uint32_t bin, unsigned long long m) {
-    atomicAdd(&hist[bin], (uint32_t)(m & 0x3fffull));
-    atomicAdd(&hist[KS_BINS + bin], (uint32_t)((m >> 14) & 0x3fffull));
-    atomicAdd(&hist[2 * KS_BINS + bin], (uint32_t)(m >> 28));
+    const uint32_t c0 = (uint32_t)m & 0x3fffu, c1 = (uint32_t)(m >> 14) & 0x3fffu, c2 = (uint32_t)(m >> 28);
+    if (c0) atomicAdd(&hist[bin], c0);
+    if (c1) atomicAdd(&hist[KS_BINS + bin], c1);
+    if (c2) atomicAdd(&hist[2 * KS_BINS + bin], c2);
   };
   auto hist_get = [&](int bin) -> unsigned long long {
     return (unsigned long long)hist[bin] + ((unsigned long long)hist[KS_BINS + bin] << 14) +
            ((unsigned long long)hist[2 * KS_BINS + bin] << 28);
   };
-  __shared__ unsigned long long warp_tot[KS_NT / 32];
-  __shared__ unsigned long long s_above, s_carry;
-  __shared__ uint32_t s_bin;
 
   const int u = blockIdx.x;
   const int r = u % n_req, o = u / n_req;
@@ -96,8 +94,8 @@ __global__ void __launch_bounds__(KS_NT, 1) keepscore_kernel(
     n_keep = min(max(fs.budget[r], 0), L);
     // as actkv_select: nothing after an earlier error of the step, and no store past the index buffer
     if (status_set(fs.status)) return;
-    if ((int64_t)fs.keep_indptr[r] + n_keep > fs.sel_stride) {
-      if (threadIdx.x == 0) report(fs.status, ACTKV_E_INVALID, r, n_keep);
+    if ((int64_t)fs.keep_indptr[r] + n_keep > fs.sel_stride || L > cap) {
+      if (threadIdx.x == 0) report(fs.status, ACTKV_E_INVALID, r, L > cap ? L : n_keep);
       return;
     }
     if (n_keep == 0 && fs.tie != nullptr && threadIdx.x == 0) fs.tie[u] = actkv_tie_t{0.f, 0, 0, 0};
@@ -106,164 +104,223 @@ __global__ void __launch_bounds__(KS_NT, 1) keepscore_kernel(
   float* sc = score + (int64_t)o * sum_tok + base;
   float* ks = keep_score + (int64_t)o * sum_tok + base;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool resident = L <= KS_CAP;                     // uniform over the CTA
-  auto key_at = [&](int i) -> uint32_t { return resident ? skeys[i] : ks_order_key(sc[i]); };
+  const bool resident = FUSED || L <= cap;               // uniform over the CTA
+  auto key_at = [&](int i) -> uint32_t { return resident ? skeys[i] : order_key(sc[i]); };
 
-  // ---- radix search: largest key T with mass(key >= T) >= mark; digits of 12, 12 and 8 bits ----
-  // The scores are read once (kept in shared memory as order keys; longer units re-read them from L2) and
-  // that read also fills the histogram of the first digit, whose bins add up to the total mass, from
-  // which  mark = ceil(p_q * total / 10000)  (total < 2^57 for up to 2^16 entries, p_q <= 10000 < 2^14: the
-  // product is taken in two halves to stay inside 64 bits).
-  for (int i = tid; i < 3 * KS_BINS; i += KS_NT) hist[i] = 0u;
-  __syncthreads();
-  for (int i = tid; i < L; i += KS_NT) {
-    const float x = sc[i];
-    const uint32_t k = ks_order_key(x);
-    if (resident) skeys[i] = k;
-    const unsigned long long m = ks_mass(x);
-    if (m != 0ull) hist_add(k >> 20, m);
-  }
-  uint32_t prefix = 0, mask = 0;
-  unsigned long long above = 0;        // mass of keys strictly above the current prefix range
-  unsigned long long mark = 0;
-#pragma unroll 1
-  for (int pass = 0; pass < 3; ++pass) {
-    const int shift = pass == 0 ? 20 : pass == 1 ? 8 : 0;
-    const uint32_t dmask = pass == 2 ? 255u : 4095u;
-    const int n_bins = (int)dmask + 1;
-    if (pass > 0) {
-      for (int i = tid; i < 3 * KS_BINS; i += KS_NT) hist[i] = 0u;
-      __syncthreads();
-      for (int i = tid; i < L; i += KS_NT) {
-        const uint32_t k = key_at(i);
-        if ((k & mask) == prefix) {
-          const unsigned long long m = ks_mass(ks_key_to_float(k));
-          if (m != 0ull) hist_add((k >> shift) & dmask, m);
-        }
-      }
-    }
-    __syncthreads();
-    // suffix sums over the bins, descending: thread t owns bins n_bins-1-4t .. n_bins-4-4t
-    const int per = n_bins / KS_NT;                      // 4, or 0 for the 256-bin pass (then one bin for tid < 256)
-    unsigned long long h[4] = {0ull, 0ull, 0ull, 0ull}, mine = 0ull;
-    if (per == 4) {
+  // ---- one read of the scores: order keys into shared memory, their range, the total mass ----
+  uint32_t lo = 0xffffffffu, hi = 0u;
+  unsigned long long total = 0ull;
+  for (int i0 = tid; i0 < L; i0 += 4 * NT) {             // four loads in flight per thread
+    float x[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) { h[j] = hist_get(n_bins - 1 - 4 * tid - j); mine += h[j]; }
-    } else if (tid < n_bins) {
-      h[0] = hist_get(n_bins - 1 - tid);
-      mine = h[0];
-    }
-    unsigned long long incl = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += t;
-    }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    unsigned long long acc = above + incl - mine;        // mass above this thread's first bin
-    unsigned long long total = 0ull;
-    for (int w = 0; w < KS_NT / 32; ++w) {
-      const unsigned long long t = warp_tot[w];
-      if (w < warp) acc += t;
-      total += t;
-    }
-    if (pass == 0) {
-      const unsigned long long q = total / 10000ull, rem = total % 10000ull;
-      mark = q * (unsigned long long)p_q + (rem * (unsigned long long)p_q + 9999ull) / 10000ull;
-    }
-    if (mark == 0ull) break;                             // nothing to cover: no hits (uniform over the CTA)
-    const int first_bin = per == 4 ? n_bins - 1 - 4 * tid : n_bins - 1 - tid;
+    for (int j = 0; j < 4; ++j) x[j] = i0 + j * NT < L ? sc[i0 + j * NT] : 0.f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      if (acc < mark && acc + h[j] >= mark) {            // exactly one bin over all threads crosses the mark
-        s_bin = (uint32_t)(first_bin - j);
-        s_above = acc;
+      if (i0 + j * NT < L) {
+        const uint32_t k = order_key(x[j]);
+        if (resident) skeys[i0 + j * NT] = k;
+        lo = min(lo, k);
+        hi = max(hi, k);
+        total += ks_mass(x[j]);
       }
-      acc += h[j];
+    }
+  }
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) total += __shfl_xor_sync(0xffffffffu, total, d);
+  if (lane == 0) sh.warp_tot[warp] = total;
+  block_range<NT>(sh.sel, lo, hi);                       // (its barrier also covers the keys and warp_tot)
+  total = lane < WARPS ? sh.warp_tot[lane] : 0ull;
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) total += __shfl_xor_sync(0xffffffffu, total, d);
+  // mark = ceil(p_q * total / 10000); total < 2^57 for up to 2^16 entries and p_q <= 10000 < 2^14: the product is
+  // taken in two halves to stay inside 64 bits
+  const unsigned long long mark = total / 10000ull * (unsigned long long)p_q +
+                                  (total % 10000ull * (unsigned long long)p_q + 9999ull) / 10000ull;
+
+  // ---- the largest key T with mass(key >= T) >= mark ----
+  uint32_t thr = 0u;                   // key of the last hit
+  int32_t last_tie = -1;               // entries equal to it are hits up to this index
+  if (mark > 0ull) {                   // (uniform over the CTA)
+    unsigned long long above = 0ull;   // mass of keys above the range in question
+    uint32_t span = hi - lo;
+    for (;;) {
+      const int shift = bin_shift(span, KS_BINS);
+      for (int i = tid; i < 3 * KS_BINS; i += NT) hist[i] = 0u;
+      if (tid == 0) sh.sel.n_list = 0u;
+      __syncthreads();
+      for (int i = tid; i < L; i += NT) {
+        const uint32_t k = key_at(i);
+        if (k - lo <= span) hist_add((k - lo) >> shift, ks_mass(key_to_float(k)));
+      }
+      __syncthreads();
+      // sums over the bins, descending
+      const int b0 = KS_BINS - PER * (tid + 1);
+      unsigned long long h[PER], mine = 0ull;
+#pragma unroll
+      for (int j = 0; j < PER; ++j) { h[j] = hist_get(b0 + j); mine += h[j]; }
+      unsigned long long acc = above + block_exclusive<NT, unsigned long long>(mine, sh.warp_tot);
+      if (acc < mark && acc + mine >= mark) {            // exactly one thread
+#pragma unroll
+        for (int j = PER - 1; j >= 0; --j) {
+          if (acc < mark && acc + h[j] >= mark) {
+            sh.bin = (uint32_t)(b0 + j);
+            sh.above = acc;
+          }
+          acc += h[j];
+        }
+      }
+      __syncthreads();
+      above = sh.above;
+      lo += sh.bin << shift;
+      span = (1u << shift) - 1u;
+      for (int i = tid; i < L; i += NT) {
+        const uint32_t k = key_at(i);
+        if (k - lo <= span) {
+          const uint32_t p = atomicAdd(&sh.sel.n_list, 1u);
+          if (p < (uint32_t)KS_LIST) { sh.sel.list[p] = k; sh.mass[p] = ks_mass(key_to_float(k)); }
+        }
+      }
+      __syncthreads();
+      const uint32_t count = sh.sel.n_list;
+      if (shift == 0) {                                  // a bin is one key
+        if (tid == 0) { sh.thr = lo; sh.eq_total = count; }
+        break;
+      }
+      if (count <= (uint32_t)KS_LIST) {
+        for (uint32_t i = tid; i < count; i += NT) {
+          const uint32_t v = sh.sel.list[i];
+          const unsigned long long m = sh.mass[i];
+          unsigned long long gt = above;
+          uint32_t equal = 0u;
+          for (uint32_t j = 0; j < count; ++j) {
+            const uint32_t w = sh.sel.list[j];
+            gt += w > v ? sh.mass[j] : 0ull;
+            equal += w == v;
+          }
+          if (gt < mark && gt + m * equal >= mark) {     // (every entry of that value: the same words)
+            sh.thr = v;
+            sh.above = gt;
+            sh.eq_total = equal;
+          }
+        }
+        break;
+      }
+      __syncthreads();
     }
     __syncthreads();
-    prefix |= s_bin << shift;
-    mask |= dmask << shift;
-    above = s_above;
-    __syncthreads();
-  }
-  uint32_t thr = 0;                    // key of the last hit
-  uint32_t ties_hit = 0;               // how many of the entries equal to thr are hits (lowest indices)
-  if (mark > 0) {
-    thr = prefix;
+    thr = sh.thr;
     // all entries with key == thr share one score, hence one mass (> 0: the bin crossed the mark)
-    const float tv = __uint_as_float((thr & 0x80000000u) ? (thr & 0x7fffffffu) : ~thr);
-    const unsigned long long thr_mass = ks_mass(tv);
-    const unsigned long long need_at_thr = mark - above;   // > 0 by construction
-    ties_hit = thr_mass > 0 ? (uint32_t)((need_at_thr + thr_mass - 1) / thr_mass) : 0u;
+    const unsigned long long thr_mass = ks_mass(key_to_float(thr));
+    const unsigned long long need = mark - sh.above;     // > 0 by construction
+    const unsigned long long ties_hit = thr_mass > 0ull ? (need + thr_mass - 1ull) / thr_mass : 0ull;
+    last_tie = L;
+    if (ties_hit < sh.eq_total) {
+      // the index of the ties_hit-th entry equal to thr: a contiguous segment per warp
+      const int seg = ((L + WARPS - 1) / WARPS + 31) & ~31;
+      const int i_begin = warp * seg, i_end = min(L, i_begin + seg);
+      uint32_t n_eq = 0u;
+      for (int i = i_begin + lane; i < i_end; i += 32) n_eq += key_at(i) == thr;
+      n_eq = __reduce_add_sync(0xffffffffu, n_eq);
+      if (lane == 0) sh.sel.warp_eq[warp] = n_eq;
+      if (tid == 0) sh.last_tie = -1;
+      __syncthreads();
+      uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp && lane < WARPS ? sh.sel.warp_eq[lane] : 0u);
+      if (ties_hit > before && ties_hit <= before + n_eq) {
+        for (int i0 = i_begin; i0 < i_end; i0 += 32) {
+          const int i = i0 + lane;
+          const bool eq = i < i_end && key_at(i) == thr;
+          const uint32_t bal = __ballot_sync(0xffffffffu, eq);
+          if (eq && before + __popc(bal & ((2u << lane) - 1u)) == ties_hit) sh.last_tie = i;
+          before += __popc(bal);
+        }
+      }
+      __syncthreads();
+      last_tie = sh.last_tie;
+    }
   }
 
-  // ---- ordered sweep: hits, keep-score update, ranking keys ----
-  if (FUSED) {                                           // the mass histograms are done with: first-digit counts of the ranking keys
-    __syncthreads();
-    for (int i = tid; i < KS_BINS; i += KS_NT) hist[i] = 0u;
-  }
-  if (tid == 0) s_carry = 0ull;
-  __syncthreads();
+  // ---- hits, keep-score update, ranking keys: every entry on its own ----
   const int np = n_protect ? n_protect[r] : 0;
   uint32_t* mrow = hit_mask ? hit_mask + (int64_t)o * ((sum_tok + 31) / 32) : nullptr;
-  for (int c0 = 0; c0 < L; c0 += KS_NT * KS_ITEMS) {
-    const int i0 = c0 + tid * KS_ITEMS;
-    float x[KS_ITEMS];
-    uint32_t eq[KS_ITEMS], gt[KS_ITEMS];
-    uint32_t n_eq = 0;
+  // (the protected entries, which rank as +inf, are counted apart: the range that TopK divides is that of the others)
+  constexpr uint32_t INF_KEY = 0xff800000u;
+  uint32_t n_inf = 0u;
+  lo = 0xffffffffu;
+  hi = 0u;
+  for (int i0 = tid; i0 < L; i0 += 4 * NT) {
+    float old[4];
 #pragma unroll
-    for (int k = 0; k < KS_ITEMS; ++k) {
-      const int i = i0 + k;
-      x[k] = (i < L) ? sc[i] : 0.f;
-      const uint32_t key = ks_order_key(x[k]);
-      gt[k] = (i < L) && mark > 0 && key > thr;
-      eq[k] = (i < L) && mark > 0 && key == thr;
-      n_eq += eq[k];
-    }
-    // exclusive scan of the tie counts in index order
-    uint32_t incl = n_eq;
+    for (int j = 0; j < 4; ++j) old[j] = i0 + j * NT < L ? ks[i0 + j * NT] : 0.f;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += t;
-    }
-    __shared__ uint32_t wsum[KS_NT / 32];
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    uint32_t before = (uint32_t)s_carry;
-    for (int w = 0; w < warp; ++w) before += wsum[w];
-    before += incl - n_eq;
-#pragma unroll
-    for (int k = 0; k < KS_ITEMS; ++k) {
-      const int i = i0 + k;
-      if (i < L) {
-        const bool hit = gt[k] || (eq[k] && before < ties_hit);
-        const float decayed = mul_ieee(lambda, ks[i]);
-        const float nk = hit ? add_ieee(decayed, x[k]) : decayed;
-        ks[i] = nk;
-        const float rank = (i < np) ? INFINITY : nk;          // what TopK ranks
-        if (FUSED) {
-          const uint32_t rk = ks_order_key(rank);
-          skeys[i] = rk;
-          atomicAdd(&hist[rk >> 20], 1u);
+    for (int j = 0; j < 4; ++j) {
+      const int i = i0 + j * NT;
+      if (i >= L) break;
+      const uint32_t k = key_at(i);
+      const bool hit = mark > 0ull && (k > thr || (k == thr && i <= last_tie));
+      const float decayed = mul_ieee(lambda, old[j]);
+      const float nk = hit ? add_ieee(decayed, key_to_float(k)) : decayed;
+      ks[i] = nk;
+      const float rank = (i < np) ? INFINITY : nk;            // what TopK ranks
+      if (FUSED) {
+        const uint32_t rk = order_key(rank);
+        skeys[i] = rk;
+        if (rk == INF_KEY) {
+          ++n_inf;
         } else {
-          sc[i] = rank;
+          lo = min(lo, rk);
+          hi = max(hi, rk);
         }
-        if (hit && mrow) atomicOr(&mrow[(base + i) >> 5], 1u << ((base + i) & 31));
+      } else {
+        sc[i] = rank;
       }
-      before += eq[k];
+      if (hit && mrow) atomicOr(&mrow[(base + i) >> 5], 1u << ((base + i) & 31));
     }
-    __syncthreads();
-    if (tid == KS_NT - 1) s_carry = before;
-    __syncthreads();
   }
   if (FUSED && n_keep > 0) {                             // uniform over the CTA
-    auto rank_key_at = [&](int i) -> uint32_t { return skeys[i]; };
-    select_threshold_and_emit(rank_key_at, hist, L, n_keep, fs.sel_idx + (int64_t)o * fs.sel_stride + fs.keep_indptr[r],
-                              fs.keep_mask ? fs.keep_mask + (int64_t)o * ((sum_tok + 31) / 32) : nullptr, base, fs.tie, u);
+    n_inf = __reduce_add_sync(0xffffffffu, n_inf);
+    __syncthreads();                                     // (the ranges of the first block_range have been read)
+    if (lane == 0) sh.sel.warp_eq[warp] = n_inf;
+    block_range<NT>(sh.sel, lo, hi);
+    n_inf = __reduce_add_sync(0xffffffffu, lane < WARPS ? sh.sel.warp_eq[lane] : 0u);
+    if (hi > INF_KEY) {                                  // (keys beyond +inf: NaN scores)
+      lo = min(lo, INF_KEY);
+      n_inf = 0u;
+    } else if (n_inf >= (uint32_t)n_keep) {
+      lo = hi = INF_KEY;
+      n_inf = 0u;
+    }
+    select_and_emit<NT, KS_BINS>([&](int i) { return skeys[i]; }, hist, sh.sel, lo, hi, L, n_keep,
+                                 fs.sel_idx + (int64_t)o * fs.sel_stride + fs.keep_indptr[r],
+                                 fs.keep_mask ? fs.keep_mask + (int64_t)o * ((sum_tok + 31) / 32) : nullptr, base, fs.tie, u, (int)n_inf);
   }
+}
+
+// max_tok: a bound on the unit lengths.
+template <bool FUSED, int NT>
+static int keepscore_launch_n(float* score, const int32_t* tok_indptr, int32_t sum_tok, int32_t max_tok, int64_t units,
+                              int32_t n_req, int32_t p_q, float lambda, const int32_t* n_protect, float* keep_score,
+                              uint32_t* hit_mask, const FusedSelectArgs& fs, cudaStream_t s) {
+  constexpr size_t fixed = 3 * KS_BINS * 4;
+  const size_t smem = resident_smem(fixed, max_tok);
+  if (ensure_dyn_smem(keepscore_kernel<FUSED, NT>, smem) != cudaSuccess) return ACTKV_E_CUDA;
+  keepscore_kernel<FUSED, NT><<<(unsigned)units, NT, smem, s>>>(score, tok_indptr, sum_tok, n_req, p_q, lambda, n_protect,
+                                                                keep_score, hit_mask, (int32_t)((smem - fixed) / 4), fs);
+  ACTKV_CHECK_LAUNCH();
+  return ACTKV_OK;
+}
+template <bool FUSED>
+static int keepscore_launch(float* score, const int32_t* tok_indptr, int32_t sum_tok, int32_t max_tok, int64_t units, int32_t n_req,
+                            int32_t p_q, float lambda, const int32_t* n_protect, float* keep_score, uint32_t* hit_mask,
+                            const FusedSelectArgs& fs, cudaStream_t s) {
+  const int nt = select_threads(units, max_tok);
+  if (nt == 256)
+    return keepscore_launch_n<FUSED, 256>(score, tok_indptr, sum_tok, max_tok, units, n_req, p_q, lambda, n_protect, keep_score,
+                                          hit_mask, fs, s);
+  if (nt == 512)
+    return keepscore_launch_n<FUSED, 512>(score, tok_indptr, sum_tok, max_tok, units, n_req, p_q, lambda, n_protect, keep_score,
+                                          hit_mask, fs, s);
+  return keepscore_launch_n<FUSED, 1024>(score, tok_indptr, sum_tok, max_tok, units, n_req, p_q, lambda, n_protect, keep_score,
+                                         hit_mask, fs, s);
 }
 
 constexpr int GA_NT = 256, GA_PER = 4;
@@ -317,6 +374,10 @@ __global__ void __launch_bounds__(GA_NT) gather_f32_kernel(
 
 }  // namespace actkv
 
+// longest unit of the one-launch form (the header names the figure)
+constexpr int32_t KS_FUSED_MAX = 45568;
+static_assert(3 * actkv::KS_BINS * 4 + (size_t)KS_FUSED_MAX * 4 <= actkv::SEL_SMEM_MAX, "fits in shared memory");
+
 extern "C" {
 
 int actkv_keepscore(float* score, const int32_t* tok_indptr, int32_t sum_tok, int32_t n_outer, int32_t n_req,
@@ -330,12 +391,9 @@ int actkv_keepscore(float* score, const int32_t* tok_indptr, int32_t sum_tok, in
   const int64_t units = (int64_t)n_outer * n_req;
   if (units > 0x7fffffffLL) return ACTKV_E_INVALID;
   const int32_t p_q = (int32_t)lrintf(top_p * 10000.f);
-  if (actkv::ensure_dyn_smem(actkv::keepscore_kernel<false>, actkv::KS_SMEM) != cudaSuccess)
-    return ACTKV_E_CUDA;
-  actkv::keepscore_kernel<false><<<(unsigned)units, actkv::KS_NT, actkv::KS_SMEM, (cudaStream_t)stream>>>(
-      score, tok_indptr, sum_tok, n_req, p_q, lambda, n_protect, keep_score, hit_mask, actkv::FusedSelectArgs{});
-  ACTKV_CHECK_LAUNCH();
-  return ACTKV_OK;
+  // (no unit is longer than all of them together)
+  return actkv::keepscore_launch<false>(score, tok_indptr, sum_tok, sum_tok, units, n_req, p_q, lambda, n_protect, keep_score,
+                                        hit_mask, actkv::FusedSelectArgs{}, (cudaStream_t)stream);
 }
 
 int actkv_keepscore_select(float* score, const int32_t* tok_indptr, int32_t sum_tok, int32_t max_tok, int32_t n_outer,
@@ -347,7 +405,7 @@ int actkv_keepscore_select(float* score, const int32_t* tok_indptr, int32_t sum_
   if (!(top_p >= 0.f && top_p <= 1.f) || !(lambda >= 0.f && lambda <= 1.f)) return ACTKV_E_INVALID;
   if (n_outer == 0 || n_req == 0 || sum_tok == 0) return ACTKV_OK;
   if (!score || !tok_indptr || !keep_score || !budget || !keep_indptr || !sel_idx) return ACTKV_E_INVALID;
-  if (max_tok > actkv::KS_CAP) {
+  if (max_tok > KS_FUSED_MAX) {
     // a unit that does not fit in shared memory: the two stages as two kernels (the ranking keys go through `score`)
     int rc = actkv_keepscore(score, tok_indptr, sum_tok, n_outer, n_req, top_p, lambda, n_protect, keep_score, hit_mask,
                              status, stream);
@@ -358,13 +416,9 @@ int actkv_keepscore_select(float* score, const int32_t* tok_indptr, int32_t sum_
   const int64_t units = (int64_t)n_outer * n_req;
   if (units > 0x7fffffffLL) return ACTKV_E_INVALID;
   const int32_t p_q = (int32_t)lrintf(top_p * 10000.f);
-  if (actkv::ensure_dyn_smem(actkv::keepscore_kernel<true>, actkv::KS_SMEM) != cudaSuccess)
-    return ACTKV_E_CUDA;
   actkv::FusedSelectArgs fs{budget, keep_indptr, sel_idx, sel_stride, keep_mask, tie_report, status};
-  actkv::keepscore_kernel<true><<<(unsigned)units, actkv::KS_NT, actkv::KS_SMEM, (cudaStream_t)stream>>>(
-      score, tok_indptr, sum_tok, n_req, p_q, lambda, n_protect, keep_score, hit_mask, fs);
-  ACTKV_CHECK_LAUNCH();
-  return ACTKV_OK;
+  return actkv::keepscore_launch<true>(score, tok_indptr, sum_tok, max_tok, units, n_req, p_q, lambda, n_protect, keep_score,
+                                       hit_mask, fs, (cudaStream_t)stream);
 }
 
 int actkv_gather_f32(const float* src, int64_t src_stride, const int32_t* tok_indptr, const int32_t* sel_idx,

@@ -1,46 +1,39 @@
 // actkv_select: TopK(score, k = B) per (layer x KV head, request) unit — Algorithm 1, step 5,
 // applied to the pooled action-region score.  One CTA per unit.  The unit's scores are read once and
-// kept in shared memory as order-preserving 32-bit keys (up to 53 K tokens; longer units re-read them
-// from L2); a most-significant-digit radix select with digits of 12, 12 and 8 bits (shared-memory
-// histograms, plain atomics: a warp's keys spread over many bins once the digit reaches into the
-// mantissa, and over the few dozen bins of the populated binades before) finds the n-th largest key
-// exactly; one ordered sweep with a block scan then emits the kept token indices in ascending order,
-// entries equal to the threshold being kept lowest index first.
+// kept in shared memory as order-preserving 32-bit keys (up to 52 K tokens; longer units re-read them
+// from L2); select_core.cuh finds the n-th largest key exactly and emits the kept indices.
+//
+// What bounds it: latency.  A unit is four sweeps over shared memory between a dozen barriers, so short units run with
+// small CTAs and only the shared memory that the host's bound on the lengths asks for, several per SM.
+// 512 units of 35000 keys 104 -> 83 us, 1024 of 16000 115 -> 82, 2048 of 1500 90 -> 34, 8 of 4096 9.7 -> 8.7 (fixed
+// digits of 12, 12 and 8 bits and an emitting sweep with block scans before).
 #include "select_core.cuh"
 
 namespace actkv {
 
-constexpr size_t SEL_SMEM = 232448 - 1024;                            // (nearly) all of an SM's shared memory: one CTA per SM
-constexpr int SEL_CAP = (int)((SEL_SMEM - SEL_BINS * 4) / 4);          // keys that fit beside the histogram
-
-__device__ __forceinline__ uint32_t order_key(float x) {
-  uint32_t b = __float_as_uint(x);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);     // larger float -> larger key
-}
-
-__global__ void __launch_bounds__(SEL_NT, 1) select_kernel(
+template <int NT, int BINS>
+__global__ void __launch_bounds__(NT) select_kernel(
     const float* __restrict__ score, const int32_t* __restrict__ tok_indptr, int32_t sum_tok,
     const int32_t* __restrict__ budget, int32_t n_req, const int32_t* __restrict__ keep_indptr,
     int32_t* __restrict__ sel_idx, int64_t sel_stride, uint32_t* __restrict__ keep_mask,
-    actkv_tie_t* __restrict__ tie, int32_t* status) {
+    actkv_tie_t* __restrict__ tie, int32_t cap, int32_t* status) {
   extern __shared__ __align__(16) uint32_t sel_smem[];
-  uint32_t* hist = sel_smem;                             // [SEL_BINS]
-  uint32_t* skeys = sel_smem + SEL_BINS;                 // [SEL_CAP]
+  __shared__ SelectShared<NT> sh;
+  uint32_t* hist = sel_smem;                             // [BINS]
+  uint32_t* skeys = sel_smem + BINS;                     // [cap]
   const int u = blockIdx.x;
   const int r = u % n_req, o = u / n_req;
-  const int base = tok_indptr[r];
-  const int L = tok_indptr[r + 1] - base;
-  int B = budget[r];
-  if (B < 0) B = 0;
-  const int n = min(B, L);
+  const int base = tok_indptr[r], end = tok_indptr[r + 1], b_raw = budget[r], kept = keep_indptr[r];
+  const int L = end - base;
+  const int n = min(b_raw < 0 ? 0 : b_raw, L);
   const float* sc = score + (int64_t)o * sum_tok + base;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
 
   // An earlier stage of the step failed (a score kernel that gave up, a bad table): its scores are not
   // consumed.  A budget the host did not size the index buffer for (the budgets are device data, e.g.
   // straight from actkv_budget) is reported before anything is stored.
   if (status_set(status)) return;
-  if ((int64_t)keep_indptr[r] + n > sel_stride) {
+  if ((int64_t)kept + n > sel_stride) {
     if (tid == 0) report(status, ACTKV_E_INVALID, r, n);
     return;
   }
@@ -48,33 +41,31 @@ __global__ void __launch_bounds__(SEL_NT, 1) select_kernel(
     if (tie != nullptr && tid == 0) tie[u] = actkv_tie_t{0.f, 0, 0, 0};
     return;
   }
-  const bool resident = L <= SEL_CAP;                    // uniform over the CTA
-  auto key_at = [&](int i) -> uint32_t { return resident ? skeys[i] : order_key(sc[i]); };
-  // The one read of the scores (16-byte vectors between an unaligned head and tail) also fills the
-  // histogram of the first digit.
-  for (int i = tid; i < SEL_BINS; i += SEL_NT) hist[i] = 0;
-  __syncthreads();
+  const bool resident = L <= cap;                        // uniform over the CTA
+  uint32_t lo = 0xffffffffu, hi = 0u;
+  // The one read of the scores (16-byte vectors between an unaligned head and tail) also takes their range.
   {
     auto take = [&](int i, float x) {
       const uint32_t k = order_key(x);
       if (resident) skeys[i] = k;
-      atomicAdd(&hist[k >> 20], 1u);
+      lo = min(lo, k);
+      hi = max(hi, k);
     };
     const int head = min(L, (int)((16u - ((uint32_t)(uintptr_t)sc & 15u)) & 15u) >> 2);
     const int n_vec = (L - head) >> 2;
     if (tid < head) take(tid, sc[tid]);
     const float4* sc4 = reinterpret_cast<const float4*>(sc + head);
     // (four loads in flight per thread: the read is bound by latency, not by bandwidth)
-    for (int v0 = tid; v0 < n_vec; v0 += 4 * SEL_NT) {
+    for (int v0 = tid; v0 < n_vec; v0 += 4 * NT) {
       float4 x[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int v = v0 + j * SEL_NT;
+        const int v = v0 + j * NT;
         x[j] = v < n_vec ? __ldg(sc4 + v) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int v = v0 + j * SEL_NT;
+        const int v = v0 + j * NT;
         if (v < n_vec) {
           const int i = head + 4 * v;
           take(i, x[j].x); take(i + 1, x[j].y); take(i + 2, x[j].z); take(i + 3, x[j].w);
@@ -84,21 +75,59 @@ __global__ void __launch_bounds__(SEL_NT, 1) select_kernel(
     const int tail0 = head + 4 * n_vec;
     if (tail0 + tid < L) take(tail0 + tid, sc[tail0 + tid]);
   }
-
-  select_threshold_and_emit(key_at, hist, L, n, sel_idx + (int64_t)o * sel_stride + keep_indptr[r],
-                            keep_mask ? keep_mask + (int64_t)o * ((sum_tok + 31) / 32) : nullptr, base, tie, u);
+  block_range<NT>(sh, lo, hi);
+  int32_t* out = sel_idx + (int64_t)o * sel_stride + kept;
+  uint32_t* mask_row = keep_mask ? keep_mask + (int64_t)o * ((sum_tok + 31) / 32) : nullptr;
+  if (resident)
+    select_and_emit<NT, BINS>([&](int i) { return skeys[i]; }, hist, sh, lo, hi, L, n, out, mask_row, base, tie, u);
+  else
+    select_and_emit<NT, BINS>([&](int i) { return order_key(sc[i]); }, hist, sh, lo, hi, L, n, out, mask_row, base, tie, u);
 }
 
-__global__ void keep_indptr_kernel(const int32_t* seq_len, const int32_t* budget, int32_t n_req,
-                                   int32_t* keep_indptr) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    int32_t acc = 0;
-    keep_indptr[0] = 0;
-    for (int r = 0; r < n_req; ++r) {
-      int32_t b = budget[r] < 0 ? 0 : budget[r];
-      acc += min(b, seq_len[r]);
-      keep_indptr[r + 1] = acc;
+template <int NT, int BINS>
+static int select_launch_n(const float* score, const int32_t* tok_indptr, int32_t sum_tok, int32_t max_tok, const int32_t* budget,
+                           int64_t units, int32_t n_req, const int32_t* keep_indptr, int32_t* sel_idx, int64_t sel_stride,
+                           uint32_t* keep_mask, actkv_tie_t* tie_report, int32_t* status, cudaStream_t s) {
+  const size_t smem = resident_smem(BINS * 4, max_tok);
+  if (ensure_dyn_smem(select_kernel<NT, BINS>, smem) != cudaSuccess) return ACTKV_E_CUDA;
+  select_kernel<NT, BINS><<<(unsigned)units, NT, smem, s>>>(score, tok_indptr, sum_tok, budget, n_req, keep_indptr, sel_idx,
+                                                            sel_stride, keep_mask, tie_report,
+                                                            (int32_t)((smem - BINS * 4) / 4), status);
+  ACTKV_CHECK_LAUNCH();
+  return ACTKV_OK;
+}
+
+int select_launch(const float* score, const int32_t* tok_indptr, int32_t sum_tok, int32_t max_tok, const int32_t* budget,
+                  int32_t n_outer, int32_t n_req, const int32_t* keep_indptr, int32_t* sel_idx, int64_t sel_stride,
+                  uint32_t* keep_mask, actkv_tie_t* tie_report, int32_t* status, cudaStream_t stream) {
+  const int64_t units = (int64_t)n_outer * n_req;
+  if (units > 0x7fffffffLL) return ACTKV_E_INVALID;
+  const int nt = select_threads(units, max_tok);
+  if (nt == 256)
+    return select_launch_n<256, 2048>(score, tok_indptr, sum_tok, max_tok, budget, units, n_req, keep_indptr, sel_idx,
+                                      sel_stride, keep_mask, tie_report, status, stream);
+  if (nt == 512)
+    return select_launch_n<512, 4096>(score, tok_indptr, sum_tok, max_tok, budget, units, n_req, keep_indptr, sel_idx,
+                                      sel_stride, keep_mask, tie_report, status, stream);
+  return select_launch_n<1024, 4096>(score, tok_indptr, sum_tok, max_tok, budget, units, n_req, keep_indptr, sel_idx,
+                                     sel_stride, keep_mask, tie_report, status, stream);
+}
+
+// One warp: inclusive scans of 32 requests at a time.
+__global__ void keep_indptr_kernel(const int32_t* seq_len, const int32_t* budget, int32_t n_req, int32_t* keep_indptr) {
+  const int lane = threadIdx.x;
+  int32_t acc = 0;
+  if (lane == 0) keep_indptr[0] = 0;
+  for (int r0 = 0; r0 < n_req; r0 += 32) {
+    const int r = r0 + lane;
+    int32_t v = r < n_req ? min(max(budget[r], 0), seq_len[r]) : 0;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int32_t t = __shfl_up_sync(0xffffffffu, v, d);
+      if (lane >= d) v += t;
     }
+    if (r < n_req) keep_indptr[r + 1] = acc + v;
+    acc += __shfl_sync(0xffffffffu, v, 31);
   }
 }
 
@@ -117,15 +146,9 @@ int actkv_select(const float* score, const int32_t* tok_indptr, int32_t sum_tok,
   if (n_outer < 0 || n_req < 0 || sum_tok < 0 || sel_stride < 0) return ACTKV_E_INVALID;
   if (n_outer == 0 || n_req == 0) return ACTKV_OK;
   if (!score || !tok_indptr || !budget || !keep_indptr || !sel_idx) return ACTKV_E_INVALID;
-  const int64_t units = (int64_t)n_outer * n_req;
-  if (units > 0x7fffffffLL) return ACTKV_E_INVALID;
-  if (actkv::ensure_dyn_smem(actkv::select_kernel, actkv::SEL_SMEM) != cudaSuccess)
-    return ACTKV_E_CUDA;
-  actkv::select_kernel<<<(unsigned)units, actkv::SEL_NT, actkv::SEL_SMEM, (cudaStream_t)stream>>>(
-      score, tok_indptr, sum_tok, budget, n_req, keep_indptr, sel_idx, sel_stride, keep_mask,
-      tie_report, status);
-  ACTKV_CHECK_LAUNCH();
-  return ACTKV_OK;
+  // (no unit is longer than all of them together)
+  return actkv::select_launch(score, tok_indptr, sum_tok, sum_tok, budget, n_outer, n_req, keep_indptr, sel_idx, sel_stride,
+                              keep_mask, tie_report, status, (cudaStream_t)stream);
 }
 
 int actkv_keep_indptr(const int32_t* seq_len, const int32_t* budget, int32_t n_req,

@@ -1,0 +1,99 @@
+"""TopK and the fused keep-score + TopK where their histograms, rankings and CTA shapes can go wrong: lengths around the
+limits of the CTA shapes and of the shared-memory copy, score sets that need one or many histogram levels, ties by the
+hundred at the threshold, protected prefixes around the budget."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import actkv_oracle as O
+from paper_2609_31395_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _scores(kind, shape, rng):
+    if kind == "equal":
+        return np.full(shape, 0.25, dtype=np.float32)
+    if kind == "zeros and ones":
+        return (rng.random(shape) < 0.3).astype(np.float32)
+    if kind == "few values":
+        return (rng.integers(0, 7, shape) / 7.0).astype(np.float32)
+    if kind == "one outlier":                              # the range is wide, nearly all keys share the lowest bin
+        x = (1e-6 + 1e-9 * rng.random(shape)).astype(np.float32)
+        x[..., shape[-1] // 2] = 200.0
+        return x
+    if kind == "subnormal":
+        return (rng.random(shape) * 1e-40).astype(np.float32)
+    return np.exp(2.0 * rng.standard_normal(shape)).astype(np.float32) / 4096.0
+
+
+def _case(kind, lens, budgets, n_outer, seed):
+    rng = np.random.default_rng(seed)
+    tok = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    keep = [min(b, L) for b, L in zip(budgets, lens)]
+    ki = np.concatenate([[0], np.cumsum(keep)]).astype(np.int32)
+    sc = np.concatenate([_scores(kind, (n_outer, L), rng) for L in lens], axis=1) if lens else None
+    return rng, tok, ki, np.ascontiguousarray(sc)
+
+
+KINDS = ["normal", "equal", "zeros and ones", "few values", "one outlier", "subnormal"]
+#        lengths, outer rows
+SHAPES = [([1, 2, 31, 33, 159, 160, 161], 3), ([1499, 1500, 1501, 2047], 2), ([8191, 8192, 100], 60), ([8193, 9000], 80),
+          ([24000, 23], 80), ([24001], 150), ([52735, 52736, 52737], 1), ([70001], 2)]
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("lens,n_outer", SHAPES)
+def test_topk(lens, n_outer, kind):
+    budgets = [max(1, L // 3) if i % 3 != 1 else L - 1 for i, L in enumerate(lens)]
+    _, tok, ki, sc = _case(kind, lens, budgets, n_outer, len(lens) + n_outer)
+    sel = torch.full((n_outer, int(ki[-1]) + 2), -1, dtype=torch.int32, device=DEV)
+    ties = torch.zeros((n_outer * len(lens), 4), dtype=torch.int32, device=DEV)
+    status = torch.zeros(4, dtype=torch.int32, device=DEV)
+    B.actkv_select(torch.from_numpy(sc).to(DEV), torch.from_numpy(tok).to(DEV), int(tok[-1]),
+                   torch.tensor(budgets, dtype=torch.int32, device=DEV), n_outer, len(lens), torch.from_numpy(ki).to(DEV), sel,
+                   sel.shape[1], None, ties, status, status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist()[0] == 0
+    got, tie = sel.cpu().numpy(), ties.cpu().numpy()
+    for o in sorted({0, n_outer // 2, n_outer - 1}):
+        for r, L in enumerate(lens):
+            x = sc[o, tok[r]:tok[r + 1]]
+            want = O.select_unit(x, budgets[r])
+            assert np.array_equal(got[o, ki[r]:ki[r + 1]], want), (o, r)
+            if len(want):
+                t = np.sort(x)[::-1][len(want) - 1]
+                u = o * len(lens) + r
+                assert tie[u, :1].view(np.float32)[0] == t and tie[u, 3] == len(want)
+                assert tie[u, 2] == (x == t).sum() and tie[u, 1] == len(want) - (x > t).sum()
+    assert (got[:, ki[-1]:] == -1).all()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("lens,n_outer", [([1, 40, 1500, 1501], 2), ([8192, 700], 80), ([9000, 24000], 76), ([45568], 1)])
+def test_keepscore_and_topk(lens, n_outer, kind):
+    for share, prot in ((3, 0.0), (2, 0.5), (4, 0.5), (1, 0.1)):       # budget = L / share, protected prefix = prot L
+        budgets = [max(1, L // share) for L in lens]
+        rng, tok, ki, sc = _case(kind, lens, budgets, n_outer, 7 * len(lens) + n_outer)
+        sc = np.minimum(sc, np.float32(1.0))
+        protect = [int(prot * L) for L in lens]
+        ks0 = (rng.random(sc.shape) ** 4).astype(np.float32)
+        ks0[:, ::3] = 0.0
+        d_ks = torch.from_numpy(ks0.copy()).to(DEV)
+        sel = torch.full((n_outer, int(ki[-1])), -1, dtype=torch.int32, device=DEV)
+        status = torch.zeros(4, dtype=torch.int32, device=DEV)
+        B.actkv_keepscore_select(torch.from_numpy(sc).to(DEV), torch.from_numpy(tok).to(DEV), int(tok[-1]), max(lens), n_outer,
+                                 len(lens), 0.9, 0.5, torch.tensor(protect, dtype=torch.int32, device=DEV), d_ks, None,
+                                 torch.tensor(budgets, dtype=torch.int32, device=DEV), torch.from_numpy(ki).to(DEV), sel,
+                                 sel.shape[1], None, None, status)
+        torch.cuda.synchronize()
+        assert status.cpu().tolist()[0] == 0
+        got_ks, got = d_ks.cpu().numpy(), sel.cpu().numpy()
+        for o in sorted({0, n_outer - 1}):
+            for r, L in enumerate(lens):
+                a, b = int(tok[r]), int(tok[r + 1])
+                hit = O.hit_mask_unit(sc[o, a:b], 0.9)
+                ks = O.keep_score_update(ks0[o, a:b], sc[o, a:b], hit, 0.5)
+                assert np.array_equal(got_ks[o, a:b].view(np.uint32), ks.view(np.uint32)), (o, r)
+                assert np.array_equal(got[o, ki[r]:ki[r + 1]], O.select_unit(O.rank_keys(ks, protect[r]), budgets[r])), (o, r)
