@@ -119,8 +119,6 @@ inline bool make_maps(const actkv_pool_t* pool, const void* q, int nls, int sum_
   return true;
 }
 
-constexpr size_t SMEM_LIMIT = 232448;        // 227 KB of dynamic shared memory per CTA
-
 // Fault-injection hook of the bounded waits (actkv_debug_inject_stall): while stall_tile >= 0 the K-tile
 // producers of every tensor-core score launch issue no tile from that one on, and every wait gives up after
 // `wait_cycles`.  Process-wide, read at launch.
@@ -181,7 +179,8 @@ inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_t
   ta.n_rg = (max_win * a.group + tc::MAX_ROWS - 1) / tc::MAX_ROWS;
   ta.row_begin = 0;
   ta.k5 = tc::pool_needs_5d(pool) ? 1 : 0;
-  ta.n_stages = 6;
+  const int nh = pool->head_dim / 64;
+  ta.n_stages = nh == 1 ? 8 : 6;
   ta.tiles_per_cta = 0;
   ta.n_kchunks = 0;
   ta.copy_ws = nullptr;              // (this kernel has no copy role)
@@ -189,14 +188,16 @@ inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_t
   const int64_t units = (int64_t)a.n_layers_sub * a.pool.n_kv_heads * a.tab.n_req;
   const int64_t grid = units * a.n_chunks * ta.n_rg;
   if (grid > 0x7fffffffLL) return ACTKV_E_INVALID;
-  const size_t smem = (size_t)ta.n_stages * tc::KTILE_BYTES + sizeof(tc::LseBarriers);
+  const size_t smem = (size_t)ta.n_stages * nh * tc::HALF_BYTES + sizeof(tc::LseBarriers);
   return score_tc_launch_lse_c(kmap, ta, (unsigned)grid, smem, s);
 }
 
 template <int G>
-inline int score_tc_launch_pool_g(const CUtensorMap& kmap, const CUtensorMap& qmap, const tc::TcArgs& ta, unsigned grid,
+inline int score_tc_launch_pool_g(const CUtensorMap& kmap, const CUtensorMap& qmap, const tc::TcArgs& ta, bool aug, unsigned grid,
                                   size_t smem, cudaStream_t s) {
-  auto kern = ta.a.pool.head_dim == 64 ? tc::score_tc_pool_kernel<G, 1> : tc::score_tc_pool_kernel<G, 2>;
+  const bool d64 = ta.a.pool.head_dim == 64;
+  auto kern = aug ? (d64 ? tc::score_tc_pool_kernel<G, 1, true> : tc::score_tc_pool_kernel<G, 2, true>)
+                  : (d64 ? tc::score_tc_pool_kernel<G, 1, false> : tc::score_tc_pool_kernel<G, 2, false>);
   // The warpgroups of this kernel re-divide the registers the launch allocates; the epilogue warpgroups would
   // wait for ever for registers that a smaller allocation does not have, so the allocation is checked first.
   if (kernel_num_regs(kern) < tc::POOL_REGS_ENTRY) return ACTKV_E_CUDA;
@@ -214,14 +215,18 @@ inline int score_tc_launch_score(ScoreArgs& a, const actkv_pool_t* pool, int max
   ta.a = a;
   const int Gp = tc::pow2_at_least(a.group);
   const int rows_all = max_win * Gp;
-  const int rows_pad = (std::min(rows_all, tc::MAX_ROWS) + 127) & ~127;      // per launch
+  const int nh = pool->head_dim / 64;
+  const int rows_pad = (std::min(rows_all, tc::MAX_ROWS) + 127) & ~127;      // of the largest unit, per launch
   const int n_rc = (rows_pad + 255) / 256;
-  const size_t q_bytes = (size_t)n_rc * 2 * tc::QBLK_BYTES;
-  const size_t fixed = q_bytes + tc::MAX_ROWS * 4 + sizeof(tc::PoolBarriers);
-  int stages = (int)((tc::SMEM_LIMIT - fixed) / tc::KTILE_BYTES);
-  if (stages > 6) stages = 6;
-  if (stages < 2) return ACTKV_E_INVALID;
-  ta.n_stages = stages;
+  // Every unit lays out its own shared memory: the widest one must have its queries and POOL_MIN_STAGES key tiles,
+  // everyone takes what is left for more of them.
+  // (the kernel without the LSE in the contraction when no unit would use it: few rows, or every window as long as the
+  // longest and that beyond the limit)
+  const bool aug = rows_all > 64 && !(rows_all > tc::aug_rows(nh) && (int64_t)a.sum_win == (int64_t)a.tab.n_req * max_win);
+  const size_t fixed = (size_t)n_rc * nh * tc::QBLK_BYTES + tc::POOL_FIXED;
+  const size_t tables = aug && rows_pad <= tc::aug_rows(nh) ? tc::AUG_K_BYTES + (size_t)n_rc * tc::AUG_CHUNK_BYTES : 0;
+  ta.n_stages = (int32_t)std::min<size_t>(tc::POOL_STAGES, (tc::SMEM_LIMIT - fixed) / (nh * tc::HALF_BYTES));
+  if (fixed + tables + tc::POOL_MIN_STAGES * nh * tc::HALF_BYTES > tc::SMEM_LIMIT) return ACTKV_E_INVALID;
   ta.n_rg = 0;
   ta.k5 = tc::pool_needs_5d(pool) ? 1 : 0;
   ta.copy_ws = copy_ws;
@@ -236,19 +241,19 @@ inline int score_tc_launch_score(ScoreArgs& a, const actkv_pool_t* pool, int max
   ta.n_kchunks = (max_tiles + ta.tiles_per_cta - 1) / ta.tiles_per_cta;
   const int64_t grid = units * ta.n_kchunks;
   if (grid > 0x7fffffffLL) return ACTKV_E_INVALID;
-  const size_t smem = fixed + (size_t)stages * tc::KTILE_BYTES;
+  const size_t smem = tc::SMEM_LIMIT;
   // a window of more than MAX_ROWS rows: one launch per group of MAX_ROWS rows (whole action tokens), in
   // stream order; the first writes the score, the others add their share of the mean
   for (int row_begin = 0; row_begin < rows_all; row_begin += tc::MAX_ROWS) {
     ta.row_begin = row_begin;
     int rc = ACTKV_E_INVALID;
     switch (Gp) {
-      case 1: rc = score_tc_launch_pool_g<1>(kmap, qmap, ta, (unsigned)grid, smem, s); break;
-      case 2: rc = score_tc_launch_pool_g<2>(kmap, qmap, ta, (unsigned)grid, smem, s); break;
-      case 4: rc = score_tc_launch_pool_g<4>(kmap, qmap, ta, (unsigned)grid, smem, s); break;
-      case 8: rc = score_tc_launch_pool_g<8>(kmap, qmap, ta, (unsigned)grid, smem, s); break;
-      case 16: rc = score_tc_launch_pool_g<16>(kmap, qmap, ta, (unsigned)grid, smem, s); break;
-      case 32: rc = score_tc_launch_pool_g<32>(kmap, qmap, ta, (unsigned)grid, smem, s); break;
+      case 1: rc = score_tc_launch_pool_g<1>(kmap, qmap, ta, aug, (unsigned)grid, smem, s); break;
+      case 2: rc = score_tc_launch_pool_g<2>(kmap, qmap, ta, aug, (unsigned)grid, smem, s); break;
+      case 4: rc = score_tc_launch_pool_g<4>(kmap, qmap, ta, aug, (unsigned)grid, smem, s); break;
+      case 8: rc = score_tc_launch_pool_g<8>(kmap, qmap, ta, aug, (unsigned)grid, smem, s); break;
+      case 16: rc = score_tc_launch_pool_g<16>(kmap, qmap, ta, aug, (unsigned)grid, smem, s); break;
+      case 32: rc = score_tc_launch_pool_g<32>(kmap, qmap, ta, aug, (unsigned)grid, smem, s); break;
       default: break;
     }
     if (rc != ACTKV_OK) return rc;

@@ -212,7 +212,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
 
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t k_smem = smem_base;                               // S x 32 KB
-  LseBarriers* bars = reinterpret_cast<LseBarriers*>(smem + (size_t)S * KTILE_BYTES);
+  LseBarriers* bars = reinterpret_cast<LseBarriers*>(smem + (size_t)S * (NH * HALF_BYTES));
   volatile int* abort_flag = &bars->abort_flag;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform
 
@@ -279,7 +279,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
       ok = mbar_wait_warp(smem_u32(&bars->k_full[s]), kpar, abort_flag, ta.wait_cycles);
       if (!ok) break;
       tc_fence_after();
-      const uint64_t desc_s = desc0 + (uint64_t)((s * KTILE_BYTES) >> 4);
+      const uint64_t desc_s = desc0 + (uint64_t)((s * (NH * HALF_BYTES)) >> 4);
       bool mine = false;
       for (int b = 0; b < n_mb; ++b, ++job) {
         if ((job & 1) != mw) continue;

@@ -41,52 +41,132 @@ struct PoolBarriers {
   float exch[TK];
 };
 
-// 64 columns of one accumulator lane: x = s for rows n .. n + 63 of this key, nlse = -lse*log2(e) of those rows
-// (-inf for padding rows).  Adds sum_w exp2(max_g(s*c + nlse)) over the action tokens w_first .. that lie
-// in [w_min, w_end) to `acc`.  Action tokens outside [w_min, w_end) do not count: below w_min the key is
-// not visible yet (causal rule), from w_end on the columns are padding (with a narrow MMA they were never
-// written and may hold anything).
-template <int G>
-__device__ __forceinline__ void pool_fold64(float* x, const float* nlse, int w_first, int w_min, int w_end, float c,
-                                            float& acc) {
-  const float4* l4 = reinterpret_cast<const float4*>(nlse);
-#pragma unroll
-  for (int q4 = 0; q4 < 16; ++q4) {
-    const float4 l = l4[q4];
-    ffma2(x[q4 * 4 + 0], x[q4 * 4 + 1], x[q4 * 4 + 0], x[q4 * 4 + 1], c, l.x, l.y);
-    ffma2(x[q4 * 4 + 2], x[q4 * 4 + 3], x[q4 * 4 + 2], x[q4 * 4 + 3], c, l.z, l.w);
+constexpr int POOL_STAGES = 8, POOL_MIN_STAGES = 2;          // key tiles in shared memory
+constexpr uint32_t POOL_FIXED = MAX_ROWS * 4 + sizeof(PoolBarriers);
+
+// The LSE in the contraction (AUG): 16 more columns of K, in which every key holds (1, 1, 1, 0, ...) and row n the
+// three bf16 parts of -lse_n / sm_scale, so that the accumulator is s - lse / sm_scale and the epilogue has neither a
+// multiply-add per column nor the shared-memory load that feeds it.  The three parts carry all 24 bits.
+// Both forms run into the power cap (32768 keys, 256 rows: 985-998 W at 1.04 GHz); this one saves issue slots and their
+// energy for one more MMA step in nine: head_dim 64, group 8, windows of 24-64 tokens, 24 layers 381 -> 326 us;
+// 32768 keys x 1, 16 layers 312 -> 302 us.
+// Rows up to which it is done: at head_dim 128 and more than 256 rows the queries leave room for three key tiles, of which
+// the tables would take one.
+__host__ __device__ constexpr int aug_rows(int nh) { return nh == 1 ? 512 : 256; }
+constexpr uint32_t AUG_ROW_BYTES = 32;
+constexpr uint32_t AUG_K_BYTES = TK * AUG_ROW_BYTES, AUG_CHUNK_BYTES = 256 * AUG_ROW_BYTES;
+__device__ __forceinline__ void aug_store(uint8_t* tile, int row, uint32_t lo, uint32_t hi) {
+  uint4* p = reinterpret_cast<uint4*>(tile + (row >> 3) * 256 + (row & 7) * 16);
+  p[0] = make_uint4(lo, hi, 0u, 0u);
+  p[8] = make_uint4(0u, 0u, 0u, 0u);
+}
+__device__ __forceinline__ void aug_row(uint8_t* tile, int row, float v) {
+  const uint32_t h = __bfloat16_as_ushort(__float2bfloat16(v));
+  uint32_t m = 0u, l = 0u;
+  if (fabsf(v) < 3.0e38f) {                   // (an infinite value is its own first part)
+    const float r1 = v - __uint_as_float(h << 16);
+    m = __bfloat16_as_ushort(__float2bfloat16(r1));
+    l = __bfloat16_as_ushort(__float2bfloat16(r1 - __uint_as_float(m << 16)));
   }
-  constexpr int WPG = 64 / G;                 // action tokens per 64-column group (G <= 32)
+  aug_store(tile, row, h | (m << 16), l);
+}
+
+// COLS columns of one accumulator lane: x = s for rows n .. n + COLS - 1 of this key (aug: s - lse / sm_scale), nlse =
+// -lse*log2(e) of those rows (-inf for padding rows).  Adds sum_w exp2(max_g(s*c + nlse)) over the action tokens w_first
+// .. to `acc`: all of them (full: every key of the tile sees every token and all columns are live), or those that lie
+// in [w_min, w_end).  Below w_min the key is
+// not visible yet (causal rule), from w_end on the columns are padding (with a narrow MMA they were never
+// written and may hold anything).  aug: the unit's LSE is part of the contraction (only in AUG launches).
+template <int G, bool AUG, int COLS>
+__device__ __forceinline__ void pool_fold(float* x, const float* nlse, bool aug, bool full, int w_first, int w_min, int w_end, float c,
+                                          float& acc) {
+  const float post = AUG ? (aug ? c : 1.f) : 1.f;
+  if (!AUG || !aug) {                         // (uniform over the CTA)
+    const float4* l4 = reinterpret_cast<const float4*>(nlse);
+#pragma unroll
+    for (int q4 = 0; q4 < COLS / 4; ++q4) {
+      const float4 l = l4[q4];
+      ffma2(x[q4 * 4 + 0], x[q4 * 4 + 1], x[q4 * 4 + 0], x[q4 * 4 + 1], c, l.x, l.y);
+      ffma2(x[q4 * 4 + 2], x[q4 * 4 + 3], x[q4 * 4 + 2], x[q4 * 4 + 3], c, l.z, l.w);
+    }
+  }
+  constexpr int WPG = COLS / G;               // action tokens of these columns (G <= COLS)
+  if (AUG && full) {                          // (uniform over the warp)
+    float s2[2] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < WPG; ++i) s2[i & 1] += exp2f(max_of<G>(x + i * G) * post);
+    acc += s2[0] + s2[1];
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < WPG; ++i) {
     const float mx = max_of<G>(x + i * G);
     const int w = w_first + i;
-    acc += (w >= w_min && w < w_end) ? exp2f(mx) : 0.f;
+    acc += (w >= w_min && w < w_end) ? exp2f(AUG ? mx * post : mx) : 0.f;
   }
 }
 
-template <int G>
-__device__ __forceinline__ void pool_job(uint32_t taddr, const float* nlse, int n_cg, int w_first, int w_min, int w_end,
-                                         float c, float& acc, uint32_t empty_bar, int lane) {
-  // At most 128 columns (n_cg <= 4 groups of 32): both 64-column loads are issued at once and the
-  // accumulator is handed back to the MMA warp as soon as they are in registers, before anything is folded.
-  const int n_c2 = (n_cg + 1) >> 1;
+// A job of at most 128 columns: the loads are issued at once and the
+// accumulator is handed back to the MMA warp as soon as they are in registers, before anything is folded.
+template <int G, bool AUG>
+__device__ __forceinline__ void pool_job(uint32_t taddr, const float* nlse, bool aug, int rows, bool whole, int w_first, int w_min,
+                                         int w_end, float c, float& acc, uint32_t empty_bar, int lane) {
+  auto hand_back = [&]() {
+    tmem_ld_wait();
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(empty_bar);
+  };
+  if constexpr (G <= 16 && !AUG) {
+    if (rows <= 16) {                         // (a decode-step update: G rows)
+      float v[16];
+      tmem_ld16(taddr, v);
+      hand_back();
+      pool_fold<G, AUG, 16>(v, nlse, false, false, w_first, w_min, w_end, c, acc);
+      return;
+    }
+  }
   float v[2][64];
   tmem_ld64(taddr, v[0]);
-  if (n_c2 > 1) tmem_ld64(taddr + 64, v[1]);
+  if (rows > 64) tmem_ld64(taddr + 64, v[1]);
+  hand_back();
+  pool_fold<G, AUG, 64>(v[0], nlse, aug, whole && rows >= 64, w_first, w_min, w_end, c, acc);
+  if (rows > 64) pool_fold<G, AUG, 64>(v[1], nlse + 64, aug, whole && rows >= 128, w_first + 64 / G, w_min, w_end, c, acc);
+}
+
+// A job of up to 256 columns, in two steps of 128; the accumulator goes back when the second one is in registers.
+// live: its columns that hold rows of the window.
+template <int G, bool AUG>
+__device__ __forceinline__ void pool_job256(uint32_t tq, const float* nl, bool aug, int live, bool full, int wf, int w_min, int w_end,
+                                            float c, float& acc, uint32_t empty_bar, int lane) {
+  float v[2][64];
+  auto hand_back = [&]() {
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(empty_bar);
+  };
+  tmem_ld64(tq, v[0]);
+  if (live > 64) tmem_ld64(tq + 64, v[1]);
   tmem_ld_wait();
-  tc_fence_before();
-  __syncwarp();
-  if (lane == 0) mbar_arrive(empty_bar);
-  pool_fold64<G>(v[0], nlse, w_first, w_min, w_end, c, acc);
-  if (n_c2 > 1) pool_fold64<G>(v[1], nlse + 64, w_first + 64 / G, w_min, w_end, c, acc);
+  if (live <= 128) hand_back();
+  pool_fold<G, AUG, 64>(v[0], nl, aug, full && live >= 64, wf, w_min, w_end, c, acc);
+  if (live > 64) pool_fold<G, AUG, 64>(v[1], nl + 64, aug, full && live >= 128, wf + 64 / G, w_min, w_end, c, acc);
+  if (live > 128) {
+    tmem_ld64(tq + 128, v[0]);
+    if (live > 192) tmem_ld64(tq + 192, v[1]);
+    tmem_ld_wait();
+    hand_back();
+    pool_fold<G, AUG, 64>(v[0], nl + 128, aug, full && live >= 192, wf + 128 / G, w_min, w_end, c, acc);
+    if (live > 192) pool_fold<G, AUG, 64>(v[1], nl + 192, aug, full && live >= 256, wf + 192 / G, w_min, w_end, c, acc);
+  }
 }
 
 // G: the group size rounded up to a power of two.  A group of a.group < G query heads is padded with
 // rows that drop out of the max (-lse = -inf); their queries are whatever the TMA box picks up behind
 // the group (the next group's heads, or zeros past the last head).
 // NH: 64-dim halves of the head dimension (head_dim = 64 NH).
-template <int G, int NH>
+// AUG: the LSE may be part of the contraction (units of 65 .. aug_rows rows).
+template <int G, int NH, bool AUG>
 __global__ void __launch_bounds__(POOL_THREADS, 1)
 score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap qmap, const TcArgs ta) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -136,13 +216,20 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
   const int n_rc = (rows_pad + 255) / 256;                // 256-row chunks per key tile: 1 or 2
   const int n_qblk = rows_pad / 128;
   const int n_jobs = n_tiles * n_rc;
-  const int S = ta.n_stages;
+  const bool aug_on = AUG && rows > 64 && rows <= aug_rows(NH);
 
   const uint32_t smem_base = smem_u32(smem);
-  const uint32_t q_bytes = (uint32_t)n_rc * 2 * QBLK_BYTES;     // per chunk: [2 halves][256 rows x 128 B]
+  // Shared memory is laid out for this unit, not for the largest one of the launch: what its queries leave free are
+  // key tiles in flight.  (With windows of 32 to 96 tokens in one launch, the short ones ran on the three stages that the
+  // longest leaves: 16 requests of 12K-20K tokens, group 4, 8 layers x 8 heads 1371 -> 1280 us.)
+  const uint32_t q_bytes = (uint32_t)n_rc * NH * QBLK_BYTES;    // per chunk: [NH halves][256 rows x 128 B]
+  const uint32_t aug_bytes = aug_on ? AUG_K_BYTES + (uint32_t)n_rc * AUG_CHUNK_BYTES : 0u;
+  // (The host's count where all units have the same layout: the very same number computed here cost the 512-row kernel 3 %.)
+  const int S = !AUG ? ta.n_stages : min(POOL_STAGES, (int)((SMEM_LIMIT - q_bytes - aug_bytes - POOL_FIXED) / (NH * HALF_BYTES)));
   const uint32_t q_smem = smem_base;
   const uint32_t k_smem = smem_base + q_bytes;
-  float* nlse = reinterpret_cast<float*>(smem + q_bytes + (size_t)S * KTILE_BYTES);       // [rows_pad]
+  uint8_t* aug = smem + q_bytes + (size_t)S * (NH * HALF_BYTES);                          // the K tile, then a tile per row chunk
+  float* nlse = reinterpret_cast<float*>(aug + aug_bytes);                                // [MAX_ROWS]
   PoolBarriers* bars = reinterpret_cast<PoolBarriers*>(reinterpret_cast<uint8_t*>(nlse) + MAX_ROWS * 4);
   volatile int* abort_flag = &bars->abort_flag;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform
@@ -170,8 +257,15 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
     // -lse of every row in log2 units; padding rows get -inf so that s*c + nlse drops out of the max
     const int g_real = a.group;
     const float* lse_base = a.lse + ((int64_t)slab * a.sum_win + w0 + w_begin) * a.n_q_heads + h * g_real;
-    for (int n = threadIdx.x; n < rows_pad; n += blockDim.x)
-      nlse[n] = (n < rows && (n % G) < g_real) ? -lse_base[(int64_t)(n / G) * a.n_q_heads + (n % G)] * kLog2e : -INFINITY;
+    for (int n = threadIdx.x; n < (aug_on ? n_rc * 256 : rows_pad); n += blockDim.x) {
+      const float l = (n < rows && (n % G) < g_real) ? -lse_base[(int64_t)(n / G) * a.n_q_heads + (n % G)] : -INFINITY;
+      if (AUG && aug_on) aug_row(aug + AUG_K_BYTES, n, l * (kLog2e / a.scale_log2));
+      else nlse[n] = l * kLog2e;
+    }
+    if (AUG && aug_on) {
+      for (int k = threadIdx.x; k < TK; k += blockDim.x) aug_store(aug, k, 0x3f803f80u, 0x3f80u);      // bf16 (1, 1, 1, 0, ...)
+      fence_proxy_async();
+    }
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(&bars->tmem_base), 512);
@@ -205,7 +299,7 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
       const int wrow = slab * a.sum_win + w0 + w_begin;
       for (int qb = 0; qb < n_qblk; ++qb)
         for (int hf = 0; hf < NH; ++hf)
-          tma_load_3d(q_smem + (qb >> 1) * 2 * QBLK_BYTES + hf * QBLK_BYTES + (qb & 1) * HALF_BYTES, &qmap,
+          tma_load_3d(q_smem + (qb >> 1) * NH * QBLK_BYTES + hf * QBLK_BYTES + (qb & 1) * HALF_BYTES, &qmap,
                       smem_u32(&bars->q_full), hf * 64, h * a.group, wrow + qb * (128 / G));
     }
     if (ta.k5) k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 0, 2, ta.wait_cycles, ta.stall_tile);
@@ -226,6 +320,7 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
     const int mw = warp - 1;
     const uint64_t kdesc0 = smem_desc_sw128(k_smem);
     const uint64_t qdesc0 = smem_desc_sw128(q_smem);
+    const uint64_t aug_a = smem_desc_k16(smem_u32(aug)), aug_b = smem_desc_k16(smem_u32(aug) + AUG_K_BYTES);
     // MMA width of each row chunk: its live rows rounded up to 16 (a decode-step update has only G)
     const int n0 = rows <= 256 ? max(16, (rows + 15) & ~15) : 256;
     const int n1 = max(16, (rows - 256 + 15) & ~15);
@@ -239,7 +334,7 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
       ok = mbar_wait_warp(smem_u32(&bars->k_full[s]), kpar, abort_flag, ta.wait_cycles);
       if (!ok) break;
       tc_fence_after();
-      const uint64_t adesc_s = kdesc0 + (uint64_t)((s * KTILE_BYTES) >> 4);
+      const uint64_t adesc_s = kdesc0 + (uint64_t)((s * (NH * HALF_BYTES)) >> 4);
       bool mine = false;
       for (int rc = 0; rc < n_rc; ++rc, ++job) {
         if ((job & 1) != mw) continue;
@@ -248,11 +343,14 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
         epar ^= 1u;
         tc_fence_after();
         if (leader) {
-          const uint64_t bdesc_c = qdesc0 + (uint64_t)((rc * 2 * QBLK_BYTES) >> 4);
+          const uint64_t bdesc_c = qdesc0 + (uint64_t)((rc * NH * QBLK_BYTES) >> 4);
 #pragma unroll
           for (int kk = 0; kk < 4 * NH; ++kk)
             umma_bf16(tmem_base + mw * 256, adesc_s + (uint64_t)(((kk >> 2) * HALF_BYTES + (kk & 3) * 32) >> 4),
                       bdesc_c + (uint64_t)(((kk >> 2) * QBLK_BYTES + (kk & 3) * 32) >> 4), idesc_c[rc], kk > 0 ? 1u : 0u);
+          // (last, so that the sum is rounded once at the magnitude of the LSE)
+          if (AUG && aug_on)
+            umma_bf16(tmem_base + mw * 256, aug_a, aug_b + (uint64_t)((rc * AUG_CHUNK_BYTES) >> 4), idesc_c[rc], 1u);
           umma_commit(full_bar);
         }
         mine = true;
@@ -301,7 +399,7 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
       const int b = wg;
       const int rc = (n_rc == 2) ? wg : 0;
       const uint32_t tq = taddr + b * 256;
-      const int n_cg_job = (min(rows, rc * 256 + 256) - rc * 256 + 31) / 32;       // 32-column groups with live rows: 1..8
+      const int live = min(rows, rc * 256 + 256) - rc * 256;                       // live columns: 1..256
       const float* nl = nlse + rc * 256;
       const int wf = w_begin + (rc * 256) / G;
       const uint32_t full_bar = smem_u32(&bars->tmem_full[b]), empty_bar = smem_u32(&bars->tmem_empty[b]);
@@ -312,33 +410,11 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
       for (int job = wg; job < n_jobs; job += 2, it += it_step, key += it_step * TK, fpar ^= 1u) {
         const int w_min = a.causal ? max(0, key - lw) : 0;
         const int w_end = win > 0 ? (a.causal ? min(W, key - lw + win) : (key >= L - win ? W : 0)) : W;
+        // every key of the tile sees every token
+        const bool full = win == 0 && (!a.causal || (t_begin + it) * TK + TK - 1 <= lw);
         if (!mbar_wait_warp(full_bar, fpar, abort_flag, ta.wait_cycles)) { ok = false; break; }
         tc_fence_after();
-        {
-          float v[2][64];
-          // columns [0, 128)
-          tmem_ld64(tq, v[0]);
-          if (n_cg_job > 2) tmem_ld64(tq + 64, v[1]);
-          tmem_ld_wait();
-          if (n_cg_job <= 4) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(empty_bar);
-          }
-          pool_fold64<G>(v[0], nl, wf, w_min, w_end, c, acc);
-          if (n_cg_job > 2) pool_fold64<G>(v[1], nl + 64, wf + 64 / G, w_min, w_end, c, acc);
-          if (n_cg_job > 4) {
-            // columns [128, 256)
-            tmem_ld64(tq + 128, v[0]);
-            if (n_cg_job > 6) tmem_ld64(tq + 192, v[1]);
-            tmem_ld_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(empty_bar);
-            pool_fold64<G>(v[0], nl + 128, wf + 128 / G, w_min, w_end, c, acc);
-            if (n_cg_job > 6) pool_fold64<G>(v[1], nl + 192, wf + 192 / G, w_min, w_end, c, acc);
-          }
-        }
+        pool_job256<G, AUG>(tq, nl, aug_on, live, full, wf, w_min, w_end, c, acc, empty_bar, lane);
         if (n_rc == 1) {
           if (key < L) { if (row_begin > 0) out[key] += acc * inv_w; else store_pooled(a, r, out + key, acc, acc * inv_w, W); }
           acc = 0.f;
@@ -383,8 +459,9 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
         const int w_end = win > 0 ? (a.causal ? min(W, key - lw + win) : (key >= L - win ? W : 0)) : W;
         if (!mbar_wait_warp(smem_u32(&bars->tmem_full[b]), (uint32_t)(job >> 1) & 1u, abort_flag, ta.wait_cycles)) break;
         tc_fence_after();
-        const int n_cg = (rows + 31) / 32;
-        pool_job<G>(taddr + b * 256, nlse, n_cg, w_begin, w_min, w_end, c, acc, smem_u32(&bars->tmem_empty[b]), lane);
+        const bool full = win == 0 && (!a.causal || (t_begin + job) * TK + TK - 1 <= lw);
+        pool_job<G, AUG>(taddr + b * 256, nlse, aug_on, rows, full, w_begin, w_min, w_end, c, acc, smem_u32(&bars->tmem_empty[b]),
+                         lane);
         if (key < L) { if (row_begin > 0) out[key] += acc * inv_w; else store_pooled(a, r, out + key, acc, acc * inv_w, W); }
         acc = 0.f;
       }

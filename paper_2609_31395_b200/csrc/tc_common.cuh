@@ -14,6 +14,7 @@ constexpr int HD = 128;                      // head dim
 constexpr uint32_t KTILE_BYTES = TK * HD * 2;        // 32 KB: [2 halves][128 keys][64 bf16]
 constexpr uint32_t HALF_BYTES = TK * 64 * 2;         // 16 KB
 constexpr uint32_t QBLK_BYTES = 128 * HD * 2;        // 32 KB per 128 rows
+constexpr size_t SMEM_LIMIT = 232448;        // 227 KB of dynamic shared memory per CTA
 constexpr int MAX_ROWS = 512;                // window x group rows (padded to 128) one CTA handles
 constexpr int MAX_ROWS_TOTAL = 4096;         // ... per unit: more than MAX_ROWS are taken in groups of MAX_ROWS
 // Bounded waits are counted on the SM cycle counter (cheap to read, unlike the global nanosecond timer).  The
@@ -276,6 +277,11 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
   d |= (uint64_t)2 << 61;                            // SWIZZLE_128B
   return d;
 }
+// K-major tile of 16 bf16 per row without swizzle: 8 rows x 16 bytes are contiguous (128 B), the two halves of K 128 B
+// apart, eight-row groups 256 B apart.
+__device__ __forceinline__ uint64_t smem_desc_k16(uint32_t addr) {
+  return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) | ((uint64_t)1 << 46);
+}
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
@@ -286,7 +292,7 @@ struct TcArgs {
   int32_t n_kchunks;         // pooled-score pass: CTAs per unit
   int32_t n_rg;              // LSE pass: groups of MAX_ROWS rows per unit (a grid dimension)
   int32_t row_begin;         // pooled-score pass: first row of this launch's row group (multiple of MAX_ROWS)
-  int32_t n_stages;          // K stages in shared memory
+  int32_t n_stages;          // K stages in shared memory (at most 8)
   int32_t k5;                // K tensor map has five dimensions (pages that are not slot-major), else four
   CompactWs* copy_ws;        // pending compaction of another layer group whose copies this launch's spare warps
                              // take on (nullptr: none)
@@ -356,7 +362,7 @@ __device__ __forceinline__ void k_tile_producer(const CUtensorMap* kmap, const S
     const int32_t my_pid = __shfl_sync(0xffffffffu, pid, ((i & 3) << lp_shift) | (lane & (ppt - 1)));
     if (lane < ppt * NH) {
       const int half = lane >> lp_shift;
-      const uint32_t dst = k_smem + s * KTILE_BYTES + half * HALF_BYTES + (lane & (ppt - 1)) * box_bytes;
+      const uint32_t dst = k_smem + s * (NH * HALF_BYTES) + half * HALF_BYTES + (lane & (ppt - 1)) * box_bytes;
       const uint32_t bar = smem_u32(&bars->k_full[s]);
       if constexpr (K5) tma_load_5d(dst, kmap, bar, half * 64, 0, h, my_pid, layer);
       else tma_load_4d(dst, kmap, bar, half * 64, h, my_pid * ps, layer);
