@@ -265,6 +265,7 @@ __device__ __forceinline__ void smem_kth_largest(const float* vals, int n, uint3
 
 __global__ void __launch_bounds__(SW_NT, 2) token_conf_sweep_kernel(
     const float* __restrict__ logits, int32_t vocab, int32_t k_top, const ConfOut out) {
+  pdl_begin(logits);
   extern __shared__ __align__(16) uint8_t sweep_raw[];
   SweepSmem* sm = reinterpret_cast<SweepSmem*>(sweep_raw);
   const int row = blockIdx.x, tid = threadIdx.x;
@@ -432,6 +433,7 @@ template <int NV>
 __global__ void __launch_bounds__(TC_NT) token_conf_cluster_kernel(const float* __restrict__ logits, int32_t vocab,
                                                                    int32_t k_top, int32_t n_parts, int32_t vecs_per_part,
                                                                    const ConfOut out) {
+  pdl_begin(logits);
   __shared__ ClusterSmem sm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int row = blockIdx.x / n_parts;
@@ -571,6 +573,7 @@ __global__ void __launch_bounds__(TR_NT) trend_kernel(
     int32_t hist_cap, BudgetParamsDev p, const int32_t* __restrict__ seq_len,
     const int32_t* __restrict__ budget_in, int32_t* __restrict__ budget_out, double* slope_out,
     float* pooled_ws, int32_t max_m) {
+  pdl_begin(tok_indptr, conf_hist, seq_len, budget_in);
   static_assert(TR_NT == 256, "one thread per bin of a digit");
   __shared__ float s_pool[TR_CAP], s_block[TR_CAP];
   __shared__ uint32_t s_hist[256];
@@ -698,12 +701,14 @@ static int launch_cluster(const float* logits, int32_t vocab, int32_t n_rows, in
   cfg.gridDim = dim3((unsigned)(n_rows * parts));
   cfg.blockDim = dim3(TC_NT);
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)parts;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   if (cudaLaunchKernelEx(&cfg, token_conf_cluster_kernel<NV>, logits, vocab, k, (int32_t)parts, (int32_t)vecs, out) != cudaSuccess) {
     (void)cudaGetLastError();
     return ACTKV_E_CUDA;
@@ -727,7 +732,8 @@ static int launch_token_conf(const float* logits, int32_t vocab, int32_t n_rows,
   }
   const size_t sm = sizeof(SweepSmem);
   if (ensure_dyn_smem(token_conf_sweep_kernel, sm) != cudaSuccess) return ACTKV_E_CUDA;
-  token_conf_sweep_kernel<<<(unsigned)n_rows, SW_NT, sm, s>>>(logits, vocab, k, out);
+  launch_pdl(token_conf_sweep_kernel, (unsigned)n_rows, SW_NT, sm, s,
+      logits, vocab, k, out);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -764,7 +770,7 @@ int actkv_budget(const float* logits, const int32_t* tok_indptr, int32_t n_rows,
   actkv::BudgetParamsDev p{params->w, params->s, params->b_percent, params->scale_up,
                            params->B_upper, params->clamp_lo_ppm, params->clamp_hi_ppm};
   const int32_t max_m = hist_cap;
-  actkv::trend_kernel<<<(unsigned)n_req, actkv::TR_NT, 0, s>>>(
+  actkv::launch_pdl(actkv::trend_kernel, (unsigned)n_req, actkv::TR_NT, 0, s,
       n_rows > 0 ? tok_indptr : nullptr, conf_hist, hist_len, hist_cap, p, seq_len, budget_in,
       budget_out, slope_out, pooled, max_m);
   ACTKV_CHECK_LAUNCH();

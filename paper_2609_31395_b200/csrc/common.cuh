@@ -5,7 +5,10 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <initializer_list>
 #include <mutex>
+#include <type_traits>
+#include <utility>
 
 #include "../../include/actkv.h"
 
@@ -32,6 +35,38 @@ __device__ __forceinline__ void report(int32_t* status, int32_t code, int32_t wh
 
 __device__ __forceinline__ bool status_set(const int32_t* status) {
   return status != nullptr && *((const volatile int32_t*)status) != 0;
+}
+
+// Programmatic dependent launch.  A step is a chain of kernels of which many take a few microseconds; every one of them is
+// launched while its predecessor on the stream still runs and begins here: it waits until that one has finished and its
+// writes are visible (and has, by the same rule, all kernels before it behind it), then allows the next launch.  What
+// overlaps is the launch itself, 1 to 2.5 us a kernel: a step of one 4K request (9 kernels) 50.9 -> 37.9 us, of 16 requests of
+// 2K 84.3 -> 71.7, the monitor's two kernels 24.5 -> 20.5, a region pass over 16 requests 677 -> 671.
+// Pointers whose loads the compiler may take for invariant (const __restrict__, __ldg) are handed through: what is loaded
+// from them then depends on the wait.
+template <class... Ptr>
+__device__ __forceinline__ void pdl_begin(Ptr&... ptr) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  (void)std::initializer_list<int>{([](auto& p) {
+    size_t g = __cvta_generic_to_global(p);              // (as a global address, so that the compiler still knows the space)
+    asm volatile("" : "+l"(g));
+    if (p != nullptr) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(__cvta_global_to_generic(g));
+  }(ptr), 0)...};
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);      // (ACTKV_CHECK_LAUNCH looks at the error)
 }
 
 // Plain-value copy of actkv_pool_t for kernel parameters.

@@ -40,6 +40,7 @@ constexpr int PLAN_PAGES = 4 * PLAN_NT;    // table entries of a request that a 
 __global__ void __launch_bounds__(PLAN_NT) compact_plan_kernel(TablesView tab, int32_t page_size, int32_t n_pages,
                                                                const int32_t* __restrict__ budget, int32_t max_keep,
                                                                CompactWs* ws, int32_t* status, CompactJobArgs job) {
+  pdl_begin(budget);
   const int R = tab.n_req, tid = threadIdx.x;
   __shared__ int32_t s_sum[4][PLAN_NT / 32];
   __shared__ int s_bad;
@@ -147,6 +148,7 @@ __global__ void __launch_bounds__(PLAN_NT) compact_plan_kernel(TablesView tab, i
 }
 
 __global__ void compact_stats_kernel(const CompactWs* ws, int32_t* out) {
+  pdl_begin();
   out[0] = ws->n_items;
   out[1] = ws->role_items;
 }
@@ -154,6 +156,7 @@ __global__ void compact_stats_kernel(const CompactWs* ws, int32_t* out) {
 // A further layer range of a step whose plan is already in the workspace (the plan depends on the tables and
 // the budgets only, not on the layers): only the job is recorded anew.
 __global__ void compact_rejob_kernel(CompactWs* ws, CompactJobArgs job, int32_t* status) {
+  pdl_begin();
   // the workspace must hold a plan of these very tables and this pool (a caller's mistake otherwise: reported,
   // and nothing is copied or finalized from what happens to be in the workspace)
   const bool mine = ws->pad == CJ_PLAN_MARK && ws->pool.base == job.pool.base && ws->tab.page_table == job.tab_page_table &&
@@ -191,6 +194,7 @@ __global__ void compact_rejob_kernel(CompactWs* ws, CompactJobArgs job, int32_t*
 
 // Resolves the sources of every item of a deferred copy (one warp per item).
 __global__ void __launch_bounds__(128) compact_resolve_kernel(CompactWs* ws) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   // A page id that some CTA of the plan kernel refused: nothing is copied.  (An error found by this very kernel may do
   // the same: an empty queue is right for any of them.  The status pointer is looked at only behind plan_ok: a workspace
@@ -214,6 +218,7 @@ __global__ void __launch_bounds__(CP_NT) compact_copy_kernel(
     PoolView pool, TablesView tab, int32_t layer_begin, const int32_t* __restrict__ sel_idx,
     int64_t sel_stride, const int32_t* __restrict__ keep_indptr, const int32_t* __restrict__ budget,
     CompactWs* ws, int32_t rows, int32_t parts, int32_t* status) {
+  pdl_begin(sel_idx, keep_indptr, budget);
   extern __shared__ __align__(16) int64_t cp_smem[];     // [2][rows]: source offsets, destination offsets
   const int R = tab.n_req;
   const int P = pool.page_size, H = pool.n_kv_heads, D = pool.head_dim;
@@ -284,6 +289,7 @@ __global__ void __launch_bounds__(CP_NT) compact_copy_kernel(
 __global__ void __launch_bounds__(PLAN_NT) compact_finalize_kernel(TablesView tab, int32_t page_size,
                                                                    const int32_t* __restrict__ budget, CompactWs* ws,
                                                                    const int32_t* status) {
+  pdl_begin(budget);
   const int R = tab.n_req, r = blockIdx.y, tid = threadIdx.x;
   const int32_t plan_ok = ws->plan_ok, failed = status_set(status) ? 1 : 0;
   const int32_t fc_new = ws->free_count - ws->total_new;
@@ -392,10 +398,11 @@ static int compact_plan(const actkv_pool_t* pool, const actkv_tables_t* tables, 
   job.vpr_shift = deferrable_shift(pool);
   job.deferred = deferred ? 1 : 0;
   if (reuse_plan)
-    compact_rejob_kernel<<<1, 1, 0, s>>>((CompactWs*)ws, job, status);
+    launch_pdl(compact_rejob_kernel, 1, 1, 0, s,
+      (CompactWs*)ws, job, status);
   else
-    compact_plan_kernel<<<status != nullptr ? table_grid(tables) : dim3(1, 1), PLAN_NT, 0, s>>>(
-        make_view(tables), pool->page_size, pool->n_pages, budget, max_keep, (CompactWs*)ws, status, job);
+    launch_pdl(compact_plan_kernel, status != nullptr ? table_grid(tables) : dim3(1, 1), PLAN_NT, 0, s,
+      make_view(tables), pool->page_size, pool->n_pages, budget, max_keep, (CompactWs*)ws, status, job);
   ACTKV_CHECK_LAUNCH();
   if (deferred && job.vpr_shift >= 0 && job.src_tab_items > 0) {
     // one warp per item of the largest job these arguments allow (short, independent chains of lookups)
@@ -404,7 +411,8 @@ static int compact_plan(const actkv_pool_t* pool, const actkv_tables_t* tables, 
     const int64_t jp = ((int64_t)pool->page_size * pool->n_kv_heads + 31) / 32;
     const int64_t items_max = std::min<int64_t>(max_x * tables->n_req * job.n_layers * jp, job.src_tab_items);
     const int64_t ctas = std::min<int64_t>(std::max<int64_t>(1, (items_max + 3) / 4), 1 << 20);
-    compact_resolve_kernel<<<(unsigned)ctas, 128, 0, s>>>((CompactWs*)ws);
+    launch_pdl(compact_resolve_kernel, (unsigned)ctas, 128, 0, s,
+      (CompactWs*)ws);
     ACTKV_CHECK_LAUNCH();
   }
   return ACTKV_OK;
@@ -433,13 +441,17 @@ static int compact_copy_all(const actkv_pool_t* pool, const actkv_tables_t* tabl
   const size_t sm = (size_t)2 * rows * sizeof(int64_t);
   const int vpr = pool->head_dim / 8;
   if (vpr == 16)
-    compact_copy_kernel<4><<<grid, CP_NT, sm, s>>>(pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
+    launch_pdl(compact_copy_kernel<4>, grid, CP_NT, sm, s,
+      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
   else if (vpr == 8)
-    compact_copy_kernel<3><<<grid, CP_NT, sm, s>>>(pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
+    launch_pdl(compact_copy_kernel<3>, grid, CP_NT, sm, s,
+      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
   else if (vpr == 32)
-    compact_copy_kernel<5><<<grid, CP_NT, sm, s>>>(pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
+    launch_pdl(compact_copy_kernel<5>, grid, CP_NT, sm, s,
+      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
   else
-    compact_copy_kernel<-1><<<grid, CP_NT, sm, s>>>(pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
+    launch_pdl(compact_copy_kernel<-1>, grid, CP_NT, sm, s,
+      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -447,7 +459,8 @@ static int compact_copy_all(const actkv_pool_t* pool, const actkv_tables_t* tabl
 static int compact_finalize(const actkv_pool_t* pool, const actkv_tables_t* tables, int32_t layer_end, const int32_t* budget,
                             void* ws, int32_t* status, cudaStream_t s) {
   if (layer_end != pool->n_layers) return ACTKV_OK;
-  compact_finalize_kernel<<<table_grid(tables), PLAN_NT, 0, s>>>(make_view(tables), pool->page_size, budget, (CompactWs*)ws, status);
+  launch_pdl(compact_finalize_kernel, table_grid(tables), PLAN_NT, 0, s,
+      make_view(tables), pool->page_size, budget, (CompactWs*)ws, status);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -487,7 +500,8 @@ int actkv_compact_begin(const actkv_pool_t* pool, const actkv_tables_t* tables, 
 
 int actkv_compact_stats(const void* ws, int32_t* stats, actkv_stream_t stream) {
   if (!ws || !stats) return ACTKV_E_INVALID;
-  actkv::compact_stats_kernel<<<1, 1, 0, (cudaStream_t)stream>>>((const actkv::CompactWs*)ws, stats);
+  actkv::launch_pdl(actkv::compact_stats_kernel, 1, 1, 0, (cudaStream_t)stream,
+      (const actkv::CompactWs*)ws, stats);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }

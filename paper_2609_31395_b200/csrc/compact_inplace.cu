@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(NT) compact_inplace_copy_kernel(
     PoolView pool, TablesView tab, int32_t layer_begin, const int32_t* __restrict__ sel_idx, int64_t sel_stride,
     const int32_t* __restrict__ keep_indptr, const int32_t* __restrict__ budget, int32_t max_keep,
     int32_t* __restrict__ new_order, int32_t* status) {
+  pdl_begin(sel_idx, keep_indptr, budget);
   constexpr int SLOTS = NT * PER, WORDS = SLOTS / 32;
   __shared__ uint32_t s_kept[WORDS];                         // bitmap of the kept slots
   __shared__ int32_t s_before[WORDS];                        // kept slots in earlier words
@@ -211,6 +212,7 @@ __global__ void compact_inplace_plan_kernel(TablesView tab, PoolView pool, const
                                             int32_t max_keep, int32_t want_order, int32_t layer_begin, int32_t n_layers,
                                             int32_t vpr_shift, uint32_t* src_tab, uint32_t* dst_tab, int64_t tab_items,
                                             CompactWs* ws, int32_t* status) {
+  pdl_begin(budget);
   if (threadIdx.x != 0) return;
   const int R = tab.n_req, P = pool.page_size;
   int32_t* item_off = ws_item_off(ws, R);
@@ -265,6 +267,7 @@ __global__ void compact_inplace_plan_kernel(TablesView tab, PoolView pool, const
 __global__ void __launch_bounds__(128) compact_inplace_resolve_kernel(
     CompactWs* ws, const int32_t* __restrict__ sel_idx, int64_t sel_stride, const int32_t* __restrict__ keep_indptr,
     int32_t* __restrict__ new_order) {
+  pdl_begin(sel_idx, keep_indptr);
   const int lane = threadIdx.x & 31;
   const int64_t n = cj_count(ws);
   const PoolView& pool = ws->pool;
@@ -353,6 +356,7 @@ constexpr int FIN_CTAS = 8, FIN_NT = 256;
 __global__ void __cluster_dims__(FIN_CTAS, 1, 1) __launch_bounds__(FIN_NT)
     compact_inplace_finalize_kernel(TablesView tab, int32_t page_size, int32_t n_pages, const int32_t* __restrict__ budget,
                                     int32_t* status) {
+  pdl_begin(budget);
   const int R = tab.n_req, tid = threadIdx.x, lane = tid & 31;
   __shared__ int64_t s_sum[FIN_NT / 32];
   const bool failed = status_set(status);
@@ -449,7 +453,10 @@ static int inplace_copy_launch(const actkv_pool_t* pool, const actkv_tables_t* t
               : vpr == 8 ? compact_inplace_copy_kernel<3, NT, PER>
               : vpr == 32 ? compact_inplace_copy_kernel<5, NT, PER>
                           : compact_inplace_copy_kernel<-1, NT, PER>;
-  kern<<<grid, NT, 0, s>>>(pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, max_keep, new_order, status);
+  // (launched plainly: with its CTAs placed while the selection kernel drains, the 16-request copy takes 571 us, not 455;
+  //  they then seem to keep that kernel's division of the SM between shared memory and L1)
+  kern<<<grid, NT, 0, s>>>(
+      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, max_keep, new_order, status);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -472,7 +479,8 @@ static int inplace_copy_all(const actkv_pool_t* pool, const actkv_tables_t* tabl
 static int inplace_finalize(const actkv_pool_t* pool, const actkv_tables_t* tables, int32_t layer_end, const int32_t* budget,
                             int32_t* status, cudaStream_t s) {
   if (layer_end == pool->n_layers) {
-    compact_inplace_finalize_kernel<<<FIN_CTAS, FIN_NT, 0, s>>>(make_view(tables), pool->page_size, pool->n_pages, budget, status);
+    launch_pdl(compact_inplace_finalize_kernel, FIN_CTAS, FIN_NT, 0, s,
+      make_view(tables), pool->page_size, pool->n_pages, budget, status);
     ACTKV_CHECK_LAUNCH();
   }
   return ACTKV_OK;
@@ -531,14 +539,16 @@ int actkv_compact_inplace_begin(const actkv_pool_t* pool, const actkv_tables_t* 
   uint32_t* dst_tab = (uint32_t*)((char*)ws + base + tab_bytes);
   // (not deferred: an empty job, so that a score call given this workspace finds nothing to do; actkv_compact_inplace_end
   //  then copies everything itself)
-  compact_inplace_plan_kernel<<<1, 32, 0, s>>>(make_view(tables), make_view(pool), budget, max_keep,
+  launch_pdl(compact_inplace_plan_kernel, 1, 32, 0, s,
+      make_view(tables), make_view(pool), budget, max_keep,
                                                new_order != nullptr ? 1 : 0, layer_begin, deferred ? nl : 0,
                                                deferred ? shift : -1, src_tab, dst_tab, deferred ? items_max : 0,
                                                (CompactWs*)ws, status);
   ACTKV_CHECK_LAUNCH();
   if (deferred && items_max > 0) {
     const int64_t ctas = std::min<int64_t>(std::max<int64_t>(1, (items_max + 3) / 4), 1 << 20);
-    compact_inplace_resolve_kernel<<<(unsigned)ctas, 128, 0, s>>>((CompactWs*)ws, sel_idx, sel_stride, keep_indptr, new_order);
+    launch_pdl(compact_inplace_resolve_kernel, (unsigned)ctas, 128, 0, s,
+      (CompactWs*)ws, sel_idx, sel_stride, keep_indptr, new_order);
     ACTKV_CHECK_LAUNCH();
   }
   return ACTKV_OK;

@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(NT) keepscore_kernel(
     float* __restrict__ score, const int32_t* __restrict__ tok_indptr, int32_t sum_tok, int32_t n_req,
     int32_t p_q, float lambda, const int32_t* __restrict__ n_protect, float* __restrict__ keep_score,
     uint32_t* __restrict__ hit_mask, int32_t cap, FusedSelectArgs fs) {
+  pdl_begin(tok_indptr, n_protect);
   constexpr int WARPS = NT / 32, PER = KS_BINS / NT;
   // A mass is below 2^41; its three 14-bit chunks are summed in three 32-bit histograms (native shared
   // atomics; a 64-bit shared atomic is a compare-and-swap loop) and put together when the bins are scanned.  A chunk
@@ -303,7 +304,8 @@ static int keepscore_launch_n(float* score, const int32_t* tok_indptr, int32_t s
   constexpr size_t fixed = 3 * KS_BINS * 4;
   const size_t smem = resident_smem(fixed, max_tok);
   if (ensure_dyn_smem(keepscore_kernel<FUSED, NT>, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  keepscore_kernel<FUSED, NT><<<(unsigned)units, NT, smem, s>>>(score, tok_indptr, sum_tok, n_req, p_q, lambda, n_protect,
+  launch_pdl(keepscore_kernel<FUSED, NT>, (unsigned)units, NT, smem, s,
+      score, tok_indptr, sum_tok, n_req, p_q, lambda, n_protect,
                                                                 keep_score, hit_mask, (int32_t)((smem - fixed) / 4), fs);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
@@ -330,6 +332,7 @@ __global__ void __launch_bounds__(GA_NT) gather_f32_kernel(
     const float* __restrict__ src, int64_t src_stride, const int32_t* __restrict__ tok_indptr,
     const int32_t* __restrict__ sel_idx, int64_t sel_stride, const int32_t* __restrict__ keep_indptr, int32_t n_req,
     float* __restrict__ dst, int64_t dst_stride) {
+  pdl_begin(src, tok_indptr, sel_idx, keep_indptr);
   const int o = blockIdx.y;
   const int first = blockIdx.x * (GA_NT * GA_PER), lane = threadIdx.x & 31;
   const int i0 = first + threadIdx.x;
@@ -428,7 +431,8 @@ int actkv_gather_f32(const float* src, int64_t src_stride, const int32_t* tok_in
   if (n_outer == 0 || n_req == 0 || max_total_keep == 0) return ACTKV_OK;
   if (!src || !tok_indptr || !sel_idx || !keep_indptr || !dst || n_outer > 65535) return ACTKV_E_INVALID;
   const dim3 grid((unsigned)((max_total_keep + actkv::GA_NT * actkv::GA_PER - 1) / (actkv::GA_NT * actkv::GA_PER)), (unsigned)n_outer);
-  actkv::gather_f32_kernel<<<grid, actkv::GA_NT, 0, (cudaStream_t)stream>>>(src, src_stride, tok_indptr, sel_idx, sel_stride,
+  actkv::launch_pdl(actkv::gather_f32_kernel, grid, actkv::GA_NT, 0, (cudaStream_t)stream,
+      src, src_stride, tok_indptr, sel_idx, sel_stride,
                                                                    keep_indptr, n_req, dst, dst_stride);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;

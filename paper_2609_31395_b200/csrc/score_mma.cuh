@@ -233,6 +233,7 @@ __device__ __forceinline__ Unit unit_of(const ScoreArgs& a, int u) {
 // LSE pass: partial (reference, sum of exp2) of every window row over one chunk of lse_chunk keys.
 template <int DB>
 __global__ void __launch_bounds__(NT, 4) score_mma_lse_kernel(const ScoreArgs a) {
+  pdl_begin();
   constexpr int KN = Keys<DB>::N, NK = KN / 8, MTILES = RCH / 16;
   extern __shared__ __align__(16) uint8_t wm_smem[];
   Smem<DB>& sm = *reinterpret_cast<Smem<DB>*>(wm_smem);
@@ -353,6 +354,7 @@ __global__ void __launch_bounds__(NT, 4) score_mma_lse_kernel(const ScoreArgs a)
 // heads drop out of the max (-lse = -inf).
 template <int DB, int GP>
 __global__ void __launch_bounds__(NT, 4) score_mma_pool_kernel(const ScoreArgs a, int keys_per_cta, int n_parts) {
+  pdl_begin();
   constexpr int MT = Keys<DB>::MT, KN = Keys<DB>::N, NG = GP == 32 ? 4 : 2;
   extern __shared__ __align__(16) uint8_t wm_smem[];
   Smem<DB>& sm = *reinterpret_cast<Smem<DB>*>(wm_smem);
@@ -475,7 +477,8 @@ __global__ void __launch_bounds__(NT, 4) score_mma_pool_kernel(const ScoreArgs a
 template <int DB>
 inline int launch_lse_d(const ScoreArgs& a, unsigned grid, cudaStream_t s) {
   if (ensure_dyn_smem(score_mma_lse_kernel<DB>, sizeof(Smem<DB>)) != cudaSuccess) return ACTKV_E_CUDA;
-  score_mma_lse_kernel<DB><<<grid, NT, sizeof(Smem<DB>), s>>>(a);
+  launch_pdl(score_mma_lse_kernel<DB>, grid, NT, sizeof(Smem<DB>), s,
+      a);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -491,7 +494,8 @@ inline int launch_lse(const ScoreArgs& a, int64_t units, cudaStream_t s) {
 template <int DB, int GP>
 inline int launch_pool_g(const ScoreArgs& a, unsigned grid, int keys, int parts, cudaStream_t s) {
   if (ensure_dyn_smem(score_mma_pool_kernel<DB, GP>, sizeof(Smem<DB>)) != cudaSuccess) return ACTKV_E_CUDA;
-  score_mma_pool_kernel<DB, GP><<<grid, NT, sizeof(Smem<DB>), s>>>(a, keys, parts);
+  launch_pdl(score_mma_pool_kernel<DB, GP>, grid, NT, sizeof(Smem<DB>), s,
+      a, keys, parts);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -523,6 +527,7 @@ inline int launch_pool(const ScoreArgs& a, int64_t units, int max_tok, cudaStrea
 
 // Merges the per-chunk (max, sum) partials of one window row into its LSE (natural log units).
 __global__ void lse_combine_kernel(const ScoreArgs a, float* lse_out, float* lse_out2) {
+  pdl_begin();
   const int R = a.tab.n_req, Hkv = a.pool.n_kv_heads, G = a.group;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over units * rows_max
   const int64_t total = (int64_t)a.n_layers_sub * Hkv * R * a.rows_max;

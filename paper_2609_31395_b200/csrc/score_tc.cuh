@@ -165,7 +165,8 @@ inline int score_tc_launch_lse_c(const CUtensorMap& kmap, const tc::TcArgs& ta, 
                   : (rgs ? (d64 ? tc::score_tc_lse_kernel<NPOLY, true, 1, false> : tc::score_tc_lse_kernel<NPOLY, true, 2, false>)
                          : (d64 ? tc::score_tc_lse_kernel<NPOLY, false, 1, false> : tc::score_tc_lse_kernel<NPOLY, false, 2, false>));
   if (ensure_dyn_smem(kern, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  kern<<<grid, tc::LSE_THREADS, smem, s>>>(kmap, ta);
+  launch_pdl(kern, grid, tc::LSE_THREADS, smem, s,
+      kmap, ta);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -202,7 +203,8 @@ inline int score_tc_launch_pool_g(const CUtensorMap& kmap, const CUtensorMap& qm
   // wait for ever for registers that a smaller allocation does not have, so the allocation is checked first.
   if (kernel_num_regs(kern) < tc::POOL_REGS_ENTRY) return ACTKV_E_CUDA;
   if (ensure_dyn_smem(kern, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  kern<<<grid, tc::POOL_THREADS, smem, s>>>(kmap, qmap, ta);
+  launch_pdl(kern, grid, tc::POOL_THREADS, smem, s,
+      kmap, qmap, ta);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }

@@ -173,6 +173,7 @@ __device__ __forceinline__ bool lse_job(LseBarriers* bars, volatile int* abort_f
 template <int NPOLY, bool ROW_GROUPS, int NH, bool WIN>
 __global__ void __launch_bounds__(LSE_THREADS, 1)
 score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
+  pdl_begin();
   extern __shared__ __align__(1024) uint8_t smem[];
   const ScoreArgs& a = ta.a;
   const int R = a.tab.n_req, Hkv = a.pool.n_kv_heads, G = a.group;

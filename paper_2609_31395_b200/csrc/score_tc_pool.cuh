@@ -169,6 +169,7 @@ __device__ __forceinline__ void pool_job256(uint32_t tq, const float* nl, bool a
 template <int G, int NH, bool AUG>
 __global__ void __launch_bounds__(POOL_THREADS, 1)
 score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap qmap, const TcArgs ta) {
+  pdl_begin();
   extern __shared__ __align__(1024) uint8_t smem[];
   const ScoreArgs& a = ta.a;
   const int R = a.tab.n_req, Hkv = a.pool.n_kv_heads;

@@ -17,6 +17,7 @@ __global__ void __launch_bounds__(NT) select_kernel(
     const int32_t* __restrict__ budget, int32_t n_req, const int32_t* __restrict__ keep_indptr,
     int32_t* __restrict__ sel_idx, int64_t sel_stride, uint32_t* __restrict__ keep_mask,
     actkv_tie_t* __restrict__ tie, int32_t cap, int32_t* status) {
+  pdl_begin(score, tok_indptr, budget, keep_indptr);
   extern __shared__ __align__(16) uint32_t sel_smem[];
   __shared__ SelectShared<NT> sh;
   uint32_t* hist = sel_smem;                             // [BINS]
@@ -90,7 +91,8 @@ static int select_launch_n(const float* score, const int32_t* tok_indptr, int32_
                            uint32_t* keep_mask, actkv_tie_t* tie_report, int32_t* status, cudaStream_t s) {
   const size_t smem = resident_smem(BINS * 4, max_tok);
   if (ensure_dyn_smem(select_kernel<NT, BINS>, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  select_kernel<NT, BINS><<<(unsigned)units, NT, smem, s>>>(score, tok_indptr, sum_tok, budget, n_req, keep_indptr, sel_idx,
+  launch_pdl(select_kernel<NT, BINS>, (unsigned)units, NT, smem, s,
+      score, tok_indptr, sum_tok, budget, n_req, keep_indptr, sel_idx,
                                                             sel_stride, keep_mask, tie_report,
                                                             (int32_t)((smem - BINS * 4) / 4), status);
   ACTKV_CHECK_LAUNCH();
@@ -115,6 +117,7 @@ int select_launch(const float* score, const int32_t* tok_indptr, int32_t sum_tok
 
 // One warp: inclusive scans of 32 requests at a time.
 __global__ void keep_indptr_kernel(const int32_t* seq_len, const int32_t* budget, int32_t n_req, int32_t* keep_indptr) {
+  pdl_begin();
   const int lane = threadIdx.x;
   int32_t acc = 0;
   if (lane == 0) keep_indptr[0] = 0;
@@ -154,7 +157,8 @@ int actkv_select(const float* score, const int32_t* tok_indptr, int32_t sum_tok,
 int actkv_keep_indptr(const int32_t* seq_len, const int32_t* budget, int32_t n_req,
                       int32_t* keep_indptr, actkv_stream_t stream) {
   if (n_req < 0 || !keep_indptr || (n_req > 0 && (!seq_len || !budget))) return ACTKV_E_INVALID;
-  actkv::keep_indptr_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(seq_len, budget, n_req, keep_indptr);
+  actkv::launch_pdl(actkv::keep_indptr_kernel, 1, 32, 0, (cudaStream_t)stream,
+      seq_len, budget, n_req, keep_indptr);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
