@@ -112,6 +112,7 @@ struct LseBarriers {
   uint64_t drained[2];
   uint32_t tmem_base;
   int abort_flag;
+  int last_key[4][128];        // last key the row of (row block, TMEM lane) sees
   float2 state[2][4][2][128];  // (reference e, sum of 2^(v c - e)) per (group, row block, column half, row in block)
 };
 
@@ -123,8 +124,6 @@ __device__ __forceinline__ void tmem_ld_fence(float* v) {
   for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
 }
 
-__device__ __forceinline__ int sel4(const int (&x)[4], int i) { return i == 0 ? x[0] : i == 1 ? x[1] : i == 2 ? x[2] : x[3]; }
-
 // One job as one epilogue warp sees it: the warp takes 64 columns (two register buffers of 32) of the
 // accumulator of its group, hands the accumulator back as soon as they are in registers, and folds them
 // into the row's (reference, sum) in `st`.  The two groups work on alternate jobs, so while one waits
@@ -132,13 +131,16 @@ __device__ __forceinline__ int sel4(const int (&x)[4], int i) { return i == 0 ? 
 //   tq      tensor-memory address of the group's accumulator, this warp's lane quarter and first column
 //   nv_min  visible columns (from the warp's first column) of the most restricted row of this thread
 //   nlo_max columns (from the warp's first column) below the first visible key of the most restricted row
-//   jm, jl  last / first visible key of this thread's row in each row block; key0 = key of the warp's first column
+//   last_key  last visible key of this thread's row; in shared memory, since only the slow path needs it and the loop is short
+//           of registers (with the keys of the four row blocks in them 910 us where this takes 895: 24 layers of 4 x 11000
+//           keys, head_dim 64, 192-512 rows; 36 layers of 32768 keys, 256 rows, 1 % less)
+//   key0    key of the warp's first column
 // WIN: the layer has a sliding window (a first visible key per row); kept out of the common instantiation, whose
 // epilogue should not carry the second bound.
 template <int NPOLY, bool WIN>
 __device__ __forceinline__ bool lse_job(LseBarriers* bars, volatile int* abort_flag, uint32_t tq, int grp, int job,
-                                        int mb, float2* st, int nv_min, int nlo_max, const int (&jm)[4], const int (&jl)[4],
-                                        int key0, float c, int lane, long long wait_cycles) {
+                                        const int* last_key, float2* st, int nv_min, int nlo_max, int win_left, int key0, float c,
+                                        long long wait_cycles) {
   float v[64];
   float* va = v;
   float* vb = v + 32;
@@ -150,7 +152,7 @@ __device__ __forceinline__ bool lse_job(LseBarriers* bars, volatile int* abort_f
   tmem_ld_fence<64>(v);
   tc_fence_before();
   __syncwarp();
-  if (lane == 0) mbar_arrive(smem_u32(&bars->tmem_empty[grp]));
+  if ((threadIdx.x & 31) == 0) mbar_arrive(smem_u32(&bars->tmem_empty[grp]));
   // (a reference of -inf, before the row's first logits, fails the second test)
   bool slow = __any_sync(0xffffffffu, nv_min < 64 || (WIN && nlo_max > 0) || !(fabsf(ms.x) < LSE_REF_MAX));
   if (!slow) {
@@ -159,7 +161,8 @@ __device__ __forceinline__ bool lse_job(LseBarriers* bars, volatile int* abort_f
     if (!slow) ms.y += ps;
   }
   if (slow) {
-    const int nv = sel4(jm, mb) - key0 + 1, nlo = WIN ? sel4(jl, mb) - key0 : 0;
+    const int nv = *last_key - key0 + 1;
+    const int nlo = WIN && win_left > 0 ? nv - win_left : 0;
     lse_slow32(va, nlo, nv, c, ms.x, ms.y);
     lse_slow32(vb, nlo - 32, nv - 32, c, ms.x, ms.y);
   }
@@ -336,26 +339,26 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars->q_ready));
     }
-    // last key each of this thread's rows sees (padding rows: every key, their sums are dropped)
-    // ... and the first one (0 unless the layer has a sliding window)
-    int jm[4], jl[4];
+    // last key each of this thread's rows sees (padding rows: every key, their sums are dropped); the most restricted row's,
+    // and the largest first key (0 unless the layer has a sliding window)
+    int jfast = L - 1, jlmax = 0;
 #pragma unroll
     for (int mb = 0; mb < 4; ++mb) {
       const int n = mb * 128 + rib;
-      jm[mb] = (a.causal && n < rows) ? (L - W + (row0 + n) / G) : (L - 1);
-      jl[mb] = (WIN && a.win_left > 0 && n < rows) ? max(0, jm[mb] - a.win_left + 1) : 0;
+      const int jm = (a.causal && n < rows) ? (L - W + (row0 + n) / G) : (L - 1);
+      bars->last_key[mb][rib] = jm;                              // (by the four warps of the quarter alike)
+      jfast = min(jfast, jm);
+      if (WIN && a.win_left > 0 && n < rows) jlmax = max(jlmax, jm - a.win_left + 1);
       bars->state[grp][mb][half][rib] = make_float2(-INFINITY, 0.f);
     }
-    const int jfast = min(min(jm[0], jm[1]), min(jm[2], jm[3]));
-    const int jlmax = max(max(jl[0], jl[1]), max(jl[2], jl[3]));
     const float c = a.scale_log2;
     const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16) + LSE_A_COLS + grp * 128 + half * 64;
     // (key tile, row block) of this group's jobs, carried along without divisions: job = tile * n_mb + mb
     int mb = grp % n_mb, key0 = (t_begin + grp / n_mb) * TK + half * 64;
     const int mb_step = 2 % n_mb, tile_step = 2 / n_mb;
     for (int job = grp; job < n_jobs; job += 2) {
-      epi_ok = lse_job<NPOLY, WIN>(bars, abort_flag, tq, grp, job, mb, &bars->state[grp][mb][half][rib], jfast - key0 + 1,
-                              jlmax - key0, jm, jl, key0, c, lane, ta.wait_cycles);
+      epi_ok = lse_job<NPOLY, WIN>(bars, abort_flag, tq, grp, job, &bars->last_key[mb][rib], &bars->state[grp][mb][half][rib],
+                                   jfast - key0 + 1, jlmax - key0, a.win_left, key0, c, ta.wait_cycles);
       if (!epi_ok) break;
       mb += mb_step;
       key0 += tile_step * TK;
