@@ -11,7 +11,6 @@ namespace tc {
 
 constexpr int TK = 128;                      // keys per tile
 constexpr int HD = 128;                      // head dim
-constexpr uint32_t KTILE_BYTES = TK * HD * 2;        // 32 KB: [2 halves][128 keys][64 bf16]
 constexpr uint32_t HALF_BYTES = TK * 64 * 2;         // 16 KB
 constexpr uint32_t QBLK_BYTES = 128 * HD * 2;        // 32 KB per 128 rows
 constexpr size_t SMEM_LIMIT = 232448;        // 227 KB of dynamic shared memory per CTA
@@ -298,18 +297,6 @@ struct TcArgs {
                              // take on (nullptr: none)
   int32_t stall_tile;        // fault-injection hook: the K-tile producers issue no tile from this one on (< 0: off)
   long long wait_cycles;     // limit of every bounded wait, in SM cycles
-};
-
-// Barrier block at the tail of dynamic shared memory.
-struct Barriers {
-  uint64_t k_full[8];
-  uint64_t k_empty[8];
-  uint64_t q_full;
-  uint64_t tmem_full[2];
-  uint64_t tmem_empty[2];
-  uint64_t drained;
-  uint32_t tmem_base;
-  int abort_flag;
 };
 
 __device__ __forceinline__ int32_t page_for_tile(const TablesView& tab, int32_t n_pages, int r, int lp, int n_lp,
