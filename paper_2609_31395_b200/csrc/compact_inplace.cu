@@ -22,6 +22,7 @@
 // queue of compact_job.cuh, so that the spare warps of the pooled-score kernel of the NEXT layer group execute
 // them (sources and destinations lie in layers that kernel does not touch) and a drain kernel what is left.
 #include "compact_job.cuh"
+#include "warp_search.cuh"
 
 namespace actkv {
 
@@ -39,15 +40,12 @@ __device__ __forceinline__ int lower_bound_i32(const int32_t* __restrict__ a, in
 // The same by one converged warp, 32 probes at a time: four round trips to memory for 64 K entries instead of sixteen.
 __device__ __forceinline__ int warp_lower_bound_i32(const int32_t* __restrict__ a, int n, int32_t key) {
   const int lane = threadIdx.x & 31;
-  int lo = 0, hi = n;                                        // the answer lies in [lo, hi]
-  while (hi - lo > 32) {
-    const int step = (hi - lo + 32) / 33;
-    const int probe = lo + (lane + 1) * step - 1;
-    const int c = __popc(__ballot_sync(0xffffffffu, probe < hi && a[probe] < key));
-    hi = min(hi, lo + (c + 1) * step - 1);
-    lo += c * step;
+  SearchSpan s{0, n};
+  while (s.hi - s.lo > 32) {
+    const int probe = search_probe(s, lane);
+    s = search_narrow(s, __popc(__ballot_sync(0xffffffffu, probe < s.hi && a[probe] < key)));
   }
-  return lo + __popc(__ballot_sync(0xffffffffu, lo + lane < hi && a[lo + lane] < key));
+  return s.lo + __popc(__ballot_sync(0xffffffffu, s.lo + lane < s.hi && a[s.lo + lane] < key));
 }
 
 // A CTA of NT threads takes PER * NT slots of the region.  The kept slots among them are marked in a bitmap (they are
