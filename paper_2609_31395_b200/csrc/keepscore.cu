@@ -51,7 +51,8 @@ template <int NT>
 struct KeepShared {
   SelectShared<NT> sel;
   unsigned long long warp_tot[NT / 32];
-  unsigned long long mass[KS_LIST];      // of the entries in sel.list
+  unsigned long long mass[KS_LIST];      // of the entries in `list`
+  uint32_t list[KS_LIST];                // (sel.list, of SEL_LIST entries, is too short)
   unsigned long long above;
   uint32_t bin, thr, eq_total;
   int32_t last_tie;
@@ -178,7 +179,7 @@ __global__ void __launch_bounds__(NT) keepscore_kernel(
         const uint32_t k = key_at(i);
         if (k - lo <= span) {
           const uint32_t p = atomicAdd(&sh.sel.n_list, 1u);
-          if (p < (uint32_t)KS_LIST) { sh.sel.list[p] = k; sh.mass[p] = ks_mass(key_to_float(k)); }
+          if (p < (uint32_t)KS_LIST) { sh.list[p] = k; sh.mass[p] = ks_mass(key_to_float(k)); }
         }
       }
       __syncthreads();
@@ -189,12 +190,12 @@ __global__ void __launch_bounds__(NT) keepscore_kernel(
       }
       if (count <= (uint32_t)KS_LIST) {
         for (uint32_t i = tid; i < count; i += NT) {
-          const uint32_t v = sh.sel.list[i];
+          const uint32_t v = sh.list[i];
           const unsigned long long m = sh.mass[i];
           unsigned long long gt = above;
           uint32_t equal = 0u;
           for (uint32_t j = 0; j < count; ++j) {
-            const uint32_t w = sh.sel.list[j];
+            const uint32_t w = sh.list[j];
             gt += w > v ? sh.mass[j] : 0ull;
             equal += w == v;
           }

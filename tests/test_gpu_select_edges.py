@@ -97,3 +97,43 @@ def test_keepscore_and_topk(lens, n_outer, kind):
                 ks = O.keep_score_update(ks0[o, a:b], sc[o, a:b], hit, 0.5)
                 assert np.array_equal(got_ks[o, a:b].view(np.uint32), ks.view(np.uint32)), (o, r)
                 assert np.array_equal(got[o, ki[r]:ki[r + 1]], O.select_unit(O.rank_keys(ks, protect[r]), budgets[r])), (o, r)
+
+
+@pytest.mark.parametrize("fused", [False, True])
+@pytest.mark.parametrize("n", [159, 160, 161, 200, 255, 256, 257, 400])
+@pytest.mark.parametrize("kind", ["distinct", "equal"])
+def test_keepscore_threshold_among_many_entries(kind, n, fused):
+    """n entries beside one another at the threshold: n neighbouring floats in one bin, around the length of the list that is
+    ranked; n equal ones, of which not all are hits."""
+    rng = np.random.default_rng(n)
+    L, n_outer = 700, 3
+    sc = np.zeros((n_outer, L), dtype=np.float32)
+    for o in range(n_outer):
+        at = rng.permutation(L)
+        steps = rng.permutation(n).astype(np.uint32) * (kind == "distinct")
+        sc[o, at[:n]] = (np.float32(0.001).view(np.uint32) + steps).astype(np.uint32).view(np.float32)
+        sc[o, at[n]] = 0.05                                # well below 90 % of the mass, and far above the others
+        sc[o, at[n + 1:n + 60]] = 1e-7
+    tok = torch.tensor([0, L], dtype=torch.int32, device=DEV)
+    d_ks = torch.zeros((n_outer, L), device=DEV)
+    mask = torch.zeros((n_outer, (L + 31) // 32), dtype=torch.int32, device=DEV)
+    status = torch.zeros(4, dtype=torch.int32, device=DEV)
+    d_sc = torch.from_numpy(sc.copy()).to(DEV)
+    if fused:
+        ki = torch.tensor([0, 300], dtype=torch.int32, device=DEV)
+        sel = torch.full((n_outer, 300), -1, dtype=torch.int32, device=DEV)
+        B.actkv_keepscore_select(d_sc, tok, L, L, n_outer, 1, 0.9, 0.5, None, d_ks, mask,
+                                 torch.tensor([300], dtype=torch.int32, device=DEV), ki, sel, 300, None, None, status)
+    else:
+        B.actkv_keepscore(d_sc, tok, L, n_outer, 1, 0.9, 0.5, None, d_ks, mask, status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist()[0] == 0
+    for o in range(n_outer):
+        hit = O.hit_mask_unit(sc[o], 0.9)
+        assert 0 < hit.sum() < n + 1                       # the threshold lies among the n
+        ks = O.keep_score_update(np.zeros(L, np.float32), sc[o], hit, 0.5)
+        assert np.array_equal(d_ks.cpu().numpy()[o].view(np.uint32), ks.view(np.uint32))
+        bits = np.unpackbits(mask.cpu().numpy()[o].view(np.uint8), bitorder="little")[:L].astype(bool)
+        assert np.array_equal(bits, hit)
+        if fused:
+            assert np.array_equal(sel.cpu().numpy()[o], O.select_unit(ks, 300))
