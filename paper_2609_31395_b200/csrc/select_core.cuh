@@ -106,7 +106,7 @@ __device__ __forceinline__ void select_and_emit(KeyAt key_at, uint32_t* hist, Se
     __syncthreads();
     remaining = sh.remaining;
     lo += sh.bin << shift;
-    span = (1u << shift) - 1u;
+    span = min((1u << shift) - 1u, hi - lo);              // (the last bin may reach past hi, where the n_above keys lie)
     const uint32_t count = sh.count;
     if (shift == 0) {                                     // a bin is one key
       if (tid == 0) { sh.thr = lo; sh.need_eq = remaining; sh.eq_total = count; }

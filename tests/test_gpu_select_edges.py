@@ -137,3 +137,23 @@ def test_keepscore_threshold_among_many_entries(kind, n, fused):
         assert np.array_equal(bits, hit)
         if fused:
             assert np.array_equal(sel.cpu().numpy()[o], O.select_unit(ks, 300))
+
+
+@pytest.mark.parametrize("prot", [50, 300])
+@pytest.mark.parametrize("n_big", [40, 150, 400])
+def test_topk_of_keep_scores_beside_the_protected_prefix(prot, n_big):
+    """Keep-scores close to the largest float: the last bin of their range reaches up to +inf, as which the prefix ranks."""
+    rng = np.random.default_rng(prot + n_big)
+    L, budget = 2000, prot + n_big // 2
+    ks0 = (1e-7 + 1e-6 * rng.random(L)).astype(np.float32)
+    ks0[prot:prot + n_big] = (3.3e38 + 9e36 * rng.random(n_big)).astype(np.float32)
+    d_ks = torch.from_numpy(ks0.copy()).to(DEV)
+    sel = torch.full((budget,), -1, dtype=torch.int32, device=DEV)
+    status = torch.zeros(4, dtype=torch.int32, device=DEV)
+    i32 = lambda *v: torch.tensor(v, dtype=torch.int32, device=DEV)  # noqa: E731
+    B.actkv_keepscore_select(torch.full((L,), 0.25, device=DEV), i32(0, L), L, L, 1, 1, 0.0, 1.0, i32(prot), d_ks, None, i32(budget),
+                             i32(0, budget), sel, budget, None, None, status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist()[0] == 0
+    assert np.array_equal(d_ks.cpu().numpy(), ks0)         # no hits, no decay
+    assert np.array_equal(sel.cpu().numpy(), O.select_unit(O.rank_keys(ks0, prot), budget))
