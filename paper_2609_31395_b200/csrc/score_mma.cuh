@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(NT, 4) score_mma_lse_kernel(const ScoreArgs a)
 #pragma unroll
       for (int w = 0; w < WARPS; ++w) ss += red[w * RCH + n].y * exp2f(red[w * RCH + n].x - mm);
       a.partials[((int64_t)u * a.n_chunks + chunk) * a.rows_max + row0 + n] =
-          ss > 0.f ? make_float2(mm, ss) : make_float2(-INFINITY, 0.f);
+          ss == 0.f ? make_float2(-INFINITY, 0.f) : make_float2(mm, ss);      // (a NaN is handed on)
     }
   }
 }
