@@ -72,6 +72,7 @@ namespace wm {
 constexpr int NT = 128;           // threads per CTA: four warps
 constexpr int WARPS = NT / 32;
 constexpr int RCH = 64;           // rows per chunk (the keys are read again for every further chunk)
+constexpr float NO_REF = -3.402823466e38f;     // LSE pass: the reference before the first visible logit (finite: its sum is 0)
 constexpr int POOL_KEYS = 2048;   // keys per CTA of the pooled-score pass (at most; 1024 and 4096 measured 1-3 % slower)
 
 __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
@@ -274,7 +275,7 @@ __global__ void __launch_bounds__(NT, 4) score_mma_lse_kernel(const ScoreArgs a)
 #pragma unroll
     for (int p = 0; p < MTILES; ++p)
 #pragma unroll
-      for (int i = 0; i < 2; ++i) { m[p][i] = -1e30f; s[p][i] = 0.f; }
+      for (int i = 0; i < 2; ++i) { m[p][i] = NO_REF; s[p][i] = 0.f; }
     for (int key0 = key_first; key0 < key_end; key0 += WARPS * KN) {
       Keys<DB> k;
       ks.take(k);
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(NT, 4) score_mma_lse_kernel(const ScoreArgs a)
           float mx = fmaxf(acc[0][2 * i], acc[0][2 * i + 1]);
 #pragma unroll
           for (int j = 1; j < NK; ++j) mx = fmaxf(mx, fmaxf(acc[j][2 * i], acc[j][2 * i + 1]));
-          mx *= c;
+          mx = __fmul_ru(mx, c);   // (rounded up: of a huge maximum the exponent below is then at most 0)
           // the reference follows the maximum only when it has fallen behind by 2^16: the sum stays far below overflow
           if (mx > m[p][i] + 16.f) { s[p][i] *= exp2f(m[p][i] - mx); m[p][i] = mx; }
           float e = 0.f;
@@ -344,8 +345,10 @@ __global__ void __launch_bounds__(NT, 4) score_mma_lse_kernel(const ScoreArgs a)
       float ss = 0.f;
 #pragma unroll
       for (int w = 0; w < WARPS; ++w) ss += red[w * RCH + n].y * exp2f(red[w * RCH + n].x - mm);
+      // a row that sees none of these keys has no reference; a sum of 0 beside one is that of logits whose rounding alone is
+      // beyond the range of exp2 (the largest counts 1); a NaN is handed on
       a.partials[((int64_t)u * a.n_chunks + chunk) * a.rows_max + row0 + n] =
-          ss == 0.f ? make_float2(-INFINITY, 0.f) : make_float2(mm, ss);      // (a NaN is handed on)
+          mm == NO_REF && ss == 0.f ? make_float2(-INFINITY, 0.f) : make_float2(mm, ss == 0.f ? 1.f : ss);
     }
   }
 }

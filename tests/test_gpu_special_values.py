@@ -41,7 +41,7 @@ def _logits(wl, inst):
     return s
 
 
-@pytest.mark.parametrize("value", VALUES)
+@pytest.mark.parametrize("value", VALUES + [1e30])
 @pytest.mark.parametrize("head_dim,group,window,causal,path", [(128, 4, 5, True, 0), (96, 3, 30, False, 0)])
 def test_lse(head_dim, group, window, causal, path, value):
     for position in POSITIONS:
