@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(NT, 4) score_mma_pool_kernel(const ScoreArgs a
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
                 auto add = [&](float y, int n) {
-                  float e = exp2f(y);
+                  float e = fmaxf(exp2f(y), 0.f);    // (NaN, as padding rows give with an infinite key, counts as nothing)
                   if constexpr (!decltype(all)::value) {
                     const int key = key0 + mt * 16 + h * 8 + (lane >> 2), w = n / GP;
                     const int w_min = a.causal ? max(0, key - lw) : 0;

@@ -1,5 +1,5 @@
 """Keys that hold infinities, NaN or huge numbers in the score kernels: the log-sum-exp of a row is NaN where one of its logits is
-NaN or +inf, and otherwise what the visible logits give, wherever in a tile such a key lies."""
+NaN or +inf, and otherwise what the visible logits give, wherever in a tile such a key lies; the other keys keep their scores."""
 import numpy as np
 import pytest
 import torch
@@ -59,3 +59,24 @@ def test_lse(head_dim, group, window, causal, path, value):
         m = ~np.isnan(want)
         # a fp32 dot product (2^-20 of a huge one) and, where an exponential is a polynomial, 7.5e-5 of it
         assert (np.abs(got[m] - want[m]) <= 1e-4 + 2e-6 * np.abs(want[m])).all(), position
+
+
+@pytest.mark.parametrize("value", VALUES)
+@pytest.mark.parametrize("head_dim,group,window,causal,path", [(128, 4, 5, True, 0), (96, 3, 30, False, 0), (64, 1, 3, False, 0)])
+def test_pooled_score(head_dim, group, window, causal, path, value):
+    """The other keys' scores do not depend on such a key; its own: +inf logits count as inf, NaN and -inf ones as nothing."""
+    for position in POSITIONS:
+        wl, inst, comp = _instance(head_dim, group, window, causal, value, position)
+        assert B.actkv_score_path(comp.pd, wl.n_q_heads, window, wl.sm_scale, inst.q) == path
+        s = _logits(wl, inst)
+        lse = np.full((1, window, wl.n_q_heads), 8.0, dtype=np.float32)
+        comp.run_score(inst.q, inst.win_indptr, inst.tok_indptr, wl.sm_scale, causal, lse_in=torch.from_numpy(lse).to(DEV))
+        torch.cuda.synchronize()
+        comp.check_status()
+        with np.errstate(over="ignore"):
+            a = np.nan_to_num(np.exp(np.where(s > -np.inf, s, -np.inf) - 8.0), nan=0.0, posinf=np.inf)
+        want = a.reshape(wl.n_kv_heads, window, group, -1).max(axis=2).sum(axis=1) / window
+        got = comp.score.cpu().numpy()[0]
+        big = want > 3e38
+        assert np.array_equal(np.isinf(got), big) and not np.isnan(got).any(), position
+        assert (np.abs(got[~big] - want[~big]) <= U.SCORE_RTOL * want[~big] + 1e-30).all(), position
