@@ -35,8 +35,8 @@
 //    rare, slower path that also serves tiles cut by the end of the request or by the causal diagonal).
 // Polynomial: textbook range reduction (Cody and Waite, Software Manual for the Elementary Functions, 1980):
 // x = v c = j + f with j the nearest integer (adding and subtracting 1.5 2^23) and f in [-0.5, 0.5], 2^f by a cubic
-// fitted here (max relative error 7.5e-5, far inside the 2e-3 score tolerance), 2^(j - e) by an integer addition to
-// the exponent field, j - e clamped to [-126, 126].  The reference being an integer, it enters in that addition only.
+// fitted here (max relative error 7.5e-5, far inside the 2e-3 score tolerance), 2^(j - e) from an exponent field,
+// j - e clamped to [-126, 126].  The reference being an integer, it enters in that factor only.
 #pragma once
 
 #include "tc_common.cuh"
@@ -47,15 +47,17 @@ namespace tc {
 constexpr int LSE_NPOLY = 1;                     // columns of every 8 whose exp2 is the polynomial
 constexpr float EXP2_ROUND = 12582912.f;         // 1.5 * 2^23: adding it rounds to the nearest integer
 
-// 2^(v c - e) for an integer e, neg_e = -e
-__device__ __forceinline__ float exp2_poly(float v, float c, float neg_e) {
-  const float t = fmaf(v, c, EXP2_ROUND + neg_e);                  // j - e = round(v c - e) in the low mantissa bits
-  const float f = fmaf(v, c, neg_e - (t - EXP2_ROUND));            // v c - j
+// 2^(v c - e) for an integer e; base = EXP2_ROUND - e.  2^(j - e) is multiplied in, not added to the exponent field of p:
+// beyond |v c| = 2^22, where f leaves its interval, and for infinite and NaN logits the product is then as small as it has to be,
+// or larger than LSE_BIG, or NaN, and the caller takes the general form.
+__device__ __forceinline__ float exp2_poly(float v, float c, float base) {
+  const float t = fmaf(v, c, base);                                // j - e = round(v c - e) in the low mantissa bits
+  const float f = fmaf(v, c, base - t);                            // v c - j
   float p = fmaf(0.0551716648042202f, f, 0.2426111251115799f);
   p = fmaf(p, f, 0.6932609677314758f);
   p = fmaf(p, f, 0.9999280571937561f);
   const float k = fminf(fmaxf(t, EXP2_ROUND - 126.f), EXP2_ROUND + 126.f);
-  return __int_as_float(__float_as_int(p) + (__float_as_int(k) << 23));
+  return p * __int_as_float((__float_as_int(k) << 23) + 0x3f800000);
 }
 
 // 32 logits of one row, all visible, against the row's reference e (finite, below LSE_REF_MAX): returns
@@ -64,6 +66,7 @@ __device__ __forceinline__ float exp2_poly(float v, float c, float neg_e) {
 template <int NPOLY>
 __device__ __forceinline__ float lse_fast32(const float* v, float c, float neg_e) {
   float s[2] = {0.f, 0.f};
+  const float base = EXP2_ROUND + neg_e;
 #pragma unroll
   for (int g8 = 0; g8 < 4; ++g8) {
 #pragma unroll
@@ -71,7 +74,7 @@ __device__ __forceinline__ float lse_fast32(const float* v, float c, float neg_e
       const float x = v[g8 * 8 + i];
       // the polynomial columns are spread over the group so that the two kinds interleave in program order
       const bool poly = (NPOLY >= 1 && i == 4) || (NPOLY >= 2 && i == 1) || (NPOLY >= 3 && i == 6) || (NPOLY >= 4 && i == 3);
-      s[i & 1] += poly ? exp2_poly(x, c, neg_e) : exp2f(fmaf(x, c, neg_e));
+      s[i & 1] += poly ? exp2_poly(x, c, base) : exp2f(fmaf(x, c, neg_e));
     }
   }
   return s[0] + s[1];
