@@ -197,8 +197,9 @@ template <int G>
 inline int score_tc_launch_pool_g(const CUtensorMap& kmap, const CUtensorMap& qmap, const tc::TcArgs& ta, bool aug, unsigned grid,
                                   size_t smem, cudaStream_t s) {
   const bool d64 = ta.a.pool.head_dim == 64;
-  auto kern = aug ? (d64 ? tc::score_tc_pool_kernel<G, 1, true> : tc::score_tc_pool_kernel<G, 2, true>)
-                  : (d64 ? tc::score_tc_pool_kernel<G, 1, false> : tc::score_tc_pool_kernel<G, 2, false>);
+  auto kern = d64 ? tc::score_tc_pool_kernel<G, 1, false> : tc::score_tc_pool_kernel<G, 2, false>;
+  if constexpr (tc::aug_group(G))
+    if (aug) kern = d64 ? tc::score_tc_pool_kernel<G, 1, true> : tc::score_tc_pool_kernel<G, 2, true>;
   // The warpgroups of this kernel re-divide the registers the launch allocates; the epilogue warpgroups would
   // wait for ever for registers that a smaller allocation does not have, so the allocation is checked first.
   if (kernel_num_regs(kern) < tc::POOL_REGS_ENTRY) return ACTKV_E_CUDA;
@@ -222,9 +223,9 @@ inline int score_tc_launch_score(ScoreArgs& a, const actkv_pool_t* pool, int max
   const int n_rc = (rows_pad + 255) / 256;
   // Every unit lays out its own shared memory: the widest one must have its queries and POOL_MIN_STAGES key tiles,
   // everyone takes what is left for more of them.
-  // (the kernel without the LSE in the contraction when no unit would use it: few rows, or every window as long as the
-  // longest and that beyond the limit)
-  const bool aug = rows_all > 64 && !(rows_all > tc::aug_rows(nh) && (int64_t)a.sum_win == (int64_t)a.tab.n_req * max_win);
+  // (the kernel without the LSE in the contraction when no unit would use it: few rows, a group it is not done for, or every
+  // window as long as the longest and that beyond the limit)
+  const bool aug = rows_all > 64 && tc::aug_group(Gp) && !(rows_all > tc::aug_rows(nh) && (int64_t)a.sum_win == (int64_t)a.tab.n_req * max_win);
   const size_t fixed = (size_t)n_rc * nh * tc::QBLK_BYTES + tc::POOL_FIXED;
   const size_t tables = aug && rows_pad <= tc::aug_rows(nh) ? tc::AUG_K_BYTES + (size_t)n_rc * tc::AUG_CHUNK_BYTES : 0;
   ta.n_stages = (int32_t)std::min<size_t>(tc::POOL_STAGES, (tc::SMEM_LIMIT - fixed) / (nh * tc::HALF_BYTES));

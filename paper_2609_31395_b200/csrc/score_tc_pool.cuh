@@ -45,13 +45,22 @@ constexpr int POOL_STAGES = 8, POOL_MIN_STAGES = 2;          // key tiles in sha
 constexpr uint32_t POOL_FIXED = MAX_ROWS * 4 + sizeof(PoolBarriers);
 
 // The LSE in the contraction (AUG): 16 more columns of K, in which every key holds (1, 1, 1, 0, ...) and row n the
-// three bf16 parts of -lse_n / sm_scale, so that the accumulator is s - lse / sm_scale and the epilogue has neither a
-// multiply-add per column nor the shared-memory load that feeds it.  The three parts carry all 24 bits.
+// three bf16 parts of -(lse_n - ref) / sm_scale, ref being the least finite LSE of the row's group.  The maximum over a group is
+// then one over bare accumulators, and the epilogue has a multiply-add (with -ref) per action token where it had one per column,
+// and fewer shared-memory loads.  The three parts carry all 24 bits.
+// Only differences within a group go through the tensor core, and before the queries do: it rounds its sums towards zero.
+// With the whole LSE in it the scores were 2e-7 to 3e-7 too large on average (40 random shapes against float64; without the
+// contraction and as it is now 2e-8 to 4e-8; 2-norm error at head_dim 64 1.9e-7, 1.5e-7 without, 1.2e-7 now).
 // Both forms run into the power cap (32768 keys, 256 rows: 985-998 W at 1.04 GHz); this one saves issue slots and their
-// energy for one more MMA step in nine: head_dim 64, group 8, windows of 24-64 tokens, 24 layers 381 -> 326 us;
-// 32768 keys x 1, 16 layers 312 -> 302 us.
+// energy for one more MMA step in nine: head_dim 64, group 8, windows of 24-64 tokens, 8 layers of 4 x 11000 keys 226 -> 174 us;
+// as a whole step, 36 layers of 32768 keys 1865 us without it and 1877 with it at 256 rows, host buffers at head_dim 64 2322 and
+// 2202.
+// Groups for which it is done (padded to a power of two): with one or two heads there is a multiply-add per column or two all the
+// same, and the values of ref would take the registers of the columns (2 heads: 536 us where the plain form takes 275, 8 layers of
+// 4 x 16000 keys, 8 heads); with 32 the plain form is the faster one (120 and 109 us).
 // Rows up to which it is done: at head_dim 128 and more than 256 rows the queries leave room for three key tiles, of which
 // the tables would take one.
+__host__ __device__ constexpr bool aug_group(int gp) { return gp >= 4 && gp <= 16; }
 __host__ __device__ constexpr int aug_rows(int nh) { return nh == 1 ? 512 : 256; }
 constexpr uint32_t AUG_ROW_BYTES = 32;
 constexpr uint32_t AUG_K_BYTES = TK * AUG_ROW_BYTES, AUG_CHUNK_BYTES = 256 * AUG_ROW_BYTES;
@@ -71,30 +80,25 @@ __device__ __forceinline__ void aug_row(uint8_t* tile, int row, float v) {
   aug_store(tile, row, h | (m << 16), l);
 }
 
-// COLS columns of one accumulator lane: x = s for rows n .. n + COLS - 1 of this key (aug: s - lse / sm_scale), nlse =
-// -lse*log2(e) of those rows (-inf for padding rows).  Adds sum_w exp2(max_g(s*c + nlse)) over the action tokens w_first
-// .. to `acc`: all of them (full: every key of the tile sees every token and all columns are live), or those that lie
-// in [w_min, w_end).  Below w_min the key is
-// not visible yet (causal rule), from w_end on the columns are padding (with a narrow MMA they were never
-// written and may hold anything).  aug: the unit's LSE is part of the contraction (only in AUG launches).
-template <int G, bool AUG, int COLS>
-__device__ __forceinline__ void pool_fold(float* x, const float* nlse, bool aug, bool full, int w_first, int w_min, int w_end, float c,
-                                          float& acc) {
-  const float post = AUG ? (aug ? c : 1.f) : 1.f;
-  if (!AUG || !aug) {                         // (uniform over the CTA)
-    const float4* l4 = reinterpret_cast<const float4*>(nlse);
+// COLS columns of one accumulator lane: x = s for rows n .. n + COLS - 1 of this key, nlse = -lse*log2(e) of those rows (-inf for
+// padding rows).  Adds sum_w exp2(max_g(s*c + nlse)) over the action tokens w_first .. that lie in [w_min, w_end) to `acc`.  Below
+// w_min the key is not visible yet (causal rule), from w_end on the columns are padding (with a narrow MMA they were never
+// written and may hold anything).  full: every key of the tile sees every token and all columns are live (uniform over the warp);
+// worth a branch where every column is a token (one head: 192 rows, 8 layers of 4 x 16000 keys 301 -> 279 us; two 275 -> 279).
+template <int G, int COLS>
+__device__ __forceinline__ void pool_fold(float* x, const float* nlse, bool full, int w_first, int w_min, int w_end, float c, float& acc) {
+  const float4* l4 = reinterpret_cast<const float4*>(nlse);
 #pragma unroll
-    for (int q4 = 0; q4 < COLS / 4; ++q4) {
-      const float4 l = l4[q4];
-      ffma2(x[q4 * 4 + 0], x[q4 * 4 + 1], x[q4 * 4 + 0], x[q4 * 4 + 1], c, l.x, l.y);
-      ffma2(x[q4 * 4 + 2], x[q4 * 4 + 3], x[q4 * 4 + 2], x[q4 * 4 + 3], c, l.z, l.w);
-    }
+  for (int q4 = 0; q4 < COLS / 4; ++q4) {
+    const float4 l = l4[q4];
+    ffma2(x[q4 * 4 + 0], x[q4 * 4 + 1], x[q4 * 4 + 0], x[q4 * 4 + 1], c, l.x, l.y);
+    ffma2(x[q4 * 4 + 2], x[q4 * 4 + 3], x[q4 * 4 + 2], x[q4 * 4 + 3], c, l.z, l.w);
   }
   constexpr int WPG = COLS / G;               // action tokens of these columns (G <= COLS)
-  if (AUG && full) {                          // (uniform over the warp)
+  if (G == 1 && full) {
     float s2[2] = {0.f, 0.f};
 #pragma unroll
-    for (int i = 0; i < WPG; ++i) s2[i & 1] += exp2f(max_of<G>(x + i * G) * post);
+    for (int i = 0; i < WPG; ++i) s2[i & 1] += exp2f(max_of<G>(x + i * G));
     acc += s2[0] + s2[1];
     return;
   }
@@ -102,14 +106,46 @@ __device__ __forceinline__ void pool_fold(float* x, const float* nlse, bool aug,
   for (int i = 0; i < WPG; ++i) {
     const float mx = max_of<G>(x + i * G);
     const int w = w_first + i;
-    acc += (w >= w_min && w < w_end) ? exp2f(AUG ? mx * post : mx) : 0.f;
+    acc += (w >= w_min && w < w_end) ? exp2f(mx) : 0.f;
+  }
+}
+
+// The same for 64 columns of a unit whose LSE is in the contraction: x = s - (lse - ref) / sm_scale, ref = -ref*log2(e) per action
+// token.
+template <int G>
+__device__ __forceinline__ void load_refs(float (&ref)[64 / G], const float* tab) {
+  if constexpr ((64 / G) % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q < 64 / G / 4; ++q) *reinterpret_cast<float4*>(ref + 4 * q) = reinterpret_cast<const float4*>(tab)[q];
+  } else {
+#pragma unroll
+    for (int i = 0; i < 64 / G; ++i) ref[i] = tab[i];
+  }
+}
+template <int G>
+__device__ __forceinline__ void pool_fold_aug(const float* x, const float (&ref)[64 / G], bool full, int w_first, int w_min, int w_end,
+                                              float c, float& acc) {
+  if (full) {
+    float s2[2] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 64 / G; ++i) s2[i & 1] += exp2f(fmaf(max_of<G>(x + i * G), c, ref[i]));
+    acc += s2[0] + s2[1];
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 64 / G; ++i) {
+    const float y = fmaf(max_of<G>(x + i * G), c, ref[i]);
+    const int w = w_first + i;
+    acc += (w >= w_min && w < w_end) ? exp2f(y) : 0.f;
   }
 }
 
 // A job of at most 128 columns: the loads are issued at once and the
 // accumulator is handed back to the MMA warp as soon as they are in registers, before anything is folded.
+// tab: -lse of every row or, aug, -ref of every action token.  (The two forms are kept apart from the loads on: with the fold
+// common to both, units with the LSE in the contraction took 210 us where they take 174: 8 layers of 4 x 11000 keys, head_dim 64.)
 template <int G, bool AUG>
-__device__ __forceinline__ void pool_job(uint32_t taddr, const float* nlse, bool aug, int rows, bool whole, int w_first, int w_min,
+__device__ __forceinline__ void pool_job(uint32_t taddr, const float* tab, bool aug, int rows, bool full, int w_first, int w_min,
                                          int w_end, float c, float& acc, uint32_t empty_bar, int lane) {
   auto hand_back = [&]() {
     tmem_ld_wait();
@@ -122,22 +158,33 @@ __device__ __forceinline__ void pool_job(uint32_t taddr, const float* nlse, bool
       float v[16];
       tmem_ld16(taddr, v);
       hand_back();
-      pool_fold<G, AUG, 16>(v, nlse, false, false, w_first, w_min, w_end, c, acc);
+      pool_fold<G, 16>(v, tab, false, w_first, w_min, w_end, c, acc);
       return;
     }
   }
   float v[2][64];
   tmem_ld64(taddr, v[0]);
   if (rows > 64) tmem_ld64(taddr + 64, v[1]);
+  if constexpr (AUG) {
+    if (aug) {                                // (more than 64 rows)
+      float ref[2][64 / G];
+      load_refs<G>(ref[0], tab);
+      load_refs<G>(ref[1], tab + 64 / G);
+      hand_back();
+      pool_fold_aug<G>(v[0], ref[0], full, w_first, w_min, w_end, c, acc);
+      pool_fold_aug<G>(v[1], ref[1], full && rows >= 128, w_first + 64 / G, w_min, w_end, c, acc);
+      return;
+    }
+  }
   hand_back();
-  pool_fold<G, AUG, 64>(v[0], nlse, aug, whole && rows >= 64, w_first, w_min, w_end, c, acc);
-  if (rows > 64) pool_fold<G, AUG, 64>(v[1], nlse + 64, aug, whole && rows >= 128, w_first + 64 / G, w_min, w_end, c, acc);
+  pool_fold<G, 64>(v[0], tab, full && rows >= 64, w_first, w_min, w_end, c, acc);
+  if (rows > 64) pool_fold<G, 64>(v[1], tab + 64, full && rows >= 128, w_first + 64 / G, w_min, w_end, c, acc);
 }
 
 // A job of up to 256 columns, in two steps of 128; the accumulator goes back when the second one is in registers.
 // live: its columns that hold rows of the window.
 template <int G, bool AUG>
-__device__ __forceinline__ void pool_job256(uint32_t tq, const float* nl, bool aug, int live, bool full, int wf, int w_min, int w_end,
+__device__ __forceinline__ void pool_job256(uint32_t tq, const float* tab, bool aug, int live, bool full, int wf, int w_min, int w_end,
                                             float c, float& acc, uint32_t empty_bar, int lane) {
   float v[2][64];
   auto hand_back = [&]() {
@@ -147,17 +194,39 @@ __device__ __forceinline__ void pool_job256(uint32_t tq, const float* nl, bool a
   };
   tmem_ld64(tq, v[0]);
   if (live > 64) tmem_ld64(tq + 64, v[1]);
+  if constexpr (AUG) {
+    if (aug) {
+      float ref[2][64 / G];
+      load_refs<G>(ref[0], tab);
+      load_refs<G>(ref[1], tab + 64 / G);
+      tmem_ld_wait();
+      if (live <= 128) hand_back();
+      pool_fold_aug<G>(v[0], ref[0], full && live >= 64, wf, w_min, w_end, c, acc);
+      if (live > 64) pool_fold_aug<G>(v[1], ref[1], full && live >= 128, wf + 64 / G, w_min, w_end, c, acc);
+      if (live > 128) {
+        tmem_ld64(tq + 128, v[0]);
+        if (live > 192) tmem_ld64(tq + 192, v[1]);
+        load_refs<G>(ref[0], tab + 128 / G);
+        load_refs<G>(ref[1], tab + 192 / G);
+        tmem_ld_wait();
+        hand_back();
+        pool_fold_aug<G>(v[0], ref[0], full && live >= 192, wf + 128 / G, w_min, w_end, c, acc);
+        if (live > 192) pool_fold_aug<G>(v[1], ref[1], full && live >= 256, wf + 192 / G, w_min, w_end, c, acc);
+      }
+      return;
+    }
+  }
   tmem_ld_wait();
   if (live <= 128) hand_back();
-  pool_fold<G, AUG, 64>(v[0], nl, aug, full && live >= 64, wf, w_min, w_end, c, acc);
-  if (live > 64) pool_fold<G, AUG, 64>(v[1], nl + 64, aug, full && live >= 128, wf + 64 / G, w_min, w_end, c, acc);
+  pool_fold<G, 64>(v[0], tab, full && live >= 64, wf, w_min, w_end, c, acc);
+  if (live > 64) pool_fold<G, 64>(v[1], tab + 64, full && live >= 128, wf + 64 / G, w_min, w_end, c, acc);
   if (live > 128) {
     tmem_ld64(tq + 128, v[0]);
     if (live > 192) tmem_ld64(tq + 192, v[1]);
     tmem_ld_wait();
     hand_back();
-    pool_fold<G, AUG, 64>(v[0], nl + 128, aug, full && live >= 192, wf + 128 / G, w_min, w_end, c, acc);
-    if (live > 192) pool_fold<G, AUG, 64>(v[1], nl + 192, aug, full && live >= 256, wf + 192 / G, w_min, w_end, c, acc);
+    pool_fold<G, 64>(v[0], tab + 128, full && live >= 192, wf + 128 / G, w_min, w_end, c, acc);
+    if (live > 192) pool_fold<G, 64>(v[1], tab + 192, full && live >= 256, wf + 192 / G, w_min, w_end, c, acc);
   }
 }
 
@@ -258,10 +327,18 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
     // -lse of every row in log2 units; padding rows get -inf so that s*c + nlse drops out of the max
     const int g_real = a.group;
     const float* lse_base = a.lse + ((int64_t)slab * a.sum_win + w0 + w_begin) * a.n_q_heads + h * g_real;
-    for (int n = threadIdx.x; n < (aug_on ? n_rc * 256 : rows_pad); n += blockDim.x) {
+    for (int n = threadIdx.x; n < (aug_on ? n_rc * 256 : rows_pad); n += blockDim.x) {      // (uniform over the warp)
       const float l = (n < rows && (n % G) < g_real) ? -lse_base[(int64_t)(n / G) * a.n_q_heads + (n % G)] : -INFINITY;
-      if (AUG && aug_on) aug_row(aug + AUG_K_BYTES, n, l * (kLog2e / a.scale_log2));
-      else nlse[n] = l * kLog2e;
+      if (AUG && aug_on) {
+        float ref = fabsf(l) < INFINITY ? l : -INFINITY;      // the largest finite -lse of the group, 0 when it has none
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) ref = fmaxf(ref, __shfl_xor_sync(0xffffffffu, ref, o));
+        if (ref == -INFINITY) ref = 0.f;
+        aug_row(aug + AUG_K_BYTES, n, (l - ref) * (kLog2e / a.scale_log2));
+        if (n % G == 0) nlse[n / G] = ref * kLog2e;
+      } else {
+        nlse[n] = l * kLog2e;
+      }
     }
     if (AUG && aug_on) {
       for (int k = threadIdx.x; k < TK; k += blockDim.x) aug_store(aug, k, 0x3f803f80u, 0x3f80u);      // bf16 (1, 1, 1, 0, ...)
@@ -345,13 +422,13 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
         tc_fence_after();
         if (leader) {
           const uint64_t bdesc_c = qdesc0 + (uint64_t)((rc * NH * QBLK_BYTES) >> 4);
+          const uint32_t begun = AUG && aug_on ? 1u : 0u;
+          if (AUG && aug_on)
+            umma_bf16(tmem_base + mw * 256, aug_a, aug_b + (uint64_t)((rc * AUG_CHUNK_BYTES) >> 4), idesc_c[rc], 0u);
 #pragma unroll
           for (int kk = 0; kk < 4 * NH; ++kk)
             umma_bf16(tmem_base + mw * 256, adesc_s + (uint64_t)(((kk >> 2) * HALF_BYTES + (kk & 3) * 32) >> 4),
-                      bdesc_c + (uint64_t)(((kk >> 2) * QBLK_BYTES + (kk & 3) * 32) >> 4), idesc_c[rc], kk > 0 ? 1u : 0u);
-          // (last, so that the sum is rounded once at the magnitude of the LSE)
-          if (AUG && aug_on)
-            umma_bf16(tmem_base + mw * 256, aug_a, aug_b + (uint64_t)((rc * AUG_CHUNK_BYTES) >> 4), idesc_c[rc], 1u);
+                      bdesc_c + (uint64_t)(((kk >> 2) * QBLK_BYTES + (kk & 3) * 32) >> 4), idesc_c[rc], kk > 0 ? 1u : begun);
           umma_commit(full_bar);
         }
         mine = true;
@@ -401,7 +478,7 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
       const int rc = (n_rc == 2) ? wg : 0;
       const uint32_t tq = taddr + b * 256;
       const int live = min(rows, rc * 256 + 256) - rc * 256;                       // live columns: 1..256
-      const float* nl = nlse + rc * 256;
+      const float* tab = nlse + rc * (AUG && aug_on ? 256 / G : 256);
       const int wf = w_begin + (rc * 256) / G;
       const uint32_t full_bar = smem_u32(&bars->tmem_full[b]), empty_bar = smem_u32(&bars->tmem_empty[b]);
       int it = (n_rc == 2) ? 0 : wg;
@@ -415,7 +492,7 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
         const bool full = win == 0 && (!a.causal || (t_begin + it) * TK + TK - 1 <= lw);
         if (!mbar_wait_warp(full_bar, fpar, abort_flag, ta.wait_cycles)) { ok = false; break; }
         tc_fence_after();
-        pool_job256<G, AUG>(tq, nl, aug_on, live, full, wf, w_min, w_end, c, acc, empty_bar, lane);
+        pool_job256<G, AUG>(tq, tab, aug_on, live, full, wf, w_min, w_end, c, acc, empty_bar, lane);
         if (n_rc == 1) {
           if (key < L) { if (row_begin > 0) out[key] += acc * inv_w; else store_pooled(a, r, out + key, acc, acc * inv_w, W); }
           acc = 0.f;

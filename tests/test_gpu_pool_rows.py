@@ -48,3 +48,24 @@ def test_rows(group, windows, head_dim, causal):
 def test_rows_with_an_infinite_lse(head_dim, windows):
     _check(synth.Workload("inf", 1, 2, 8, [500, 300], windows, [100, 50], head_dim=head_dim, table_style="fragmented", seed=3),
            spoil=True)
+
+
+@pytest.mark.parametrize("head_dim,group,windows", [(64, 8, [64, 20]), (64, 4, [128, 90]), (128, 4, [64, 40]), (128, 8, [32, 9]),
+                                                    (128, 1, [200, 70]), (64, 16, [32, 5])])
+def test_scores_are_not_rounded_to_one_side(head_dim, group, windows):
+    """The mean relative error against float64.  Sums rounded to nearest have next to none; sums of magnitude 8 to 16 (in log2
+    units) rounded towards zero make a score up to 2^-20 ln 2 = 6.6e-7 too large, half of that on average."""
+    lens = [3000, 1700]
+    wl = synth.Workload("bias", 2, 4, group, lens, windows, [L // 3 for L in lens], head_dim=head_dim, table_style="fragmented",
+                        seed=head_dim)
+    inst = synth.generate(wl, DEV)
+    comp = H.Compressor(inst.pool, inst.page_table, inst.seq_len, inst.free_list, inst.free_count, wl.n_q_heads, H.sizes_of(inst))
+    args = (U.bits(inst.pool), inst.page_table.cpu().numpy(), inst.seq_len.cpu().numpy(), U.bits(inst.q),
+            inst.win_indptr.cpu().numpy(), wl.n_q_heads, wl.sm_scale, False)
+    lse = O.score(*args)[1].astype(np.float32)
+    want = O.score(*args, lse_in=lse)[0]
+    comp.run_score(inst.q, inst.win_indptr, inst.tok_indptr, wl.sm_scale, False, lse_in=torch.from_numpy(lse).to(DEV))
+    torch.cuda.synchronize()
+    comp.check_status()
+    rel = comp.score.cpu().numpy().astype(np.float64) / want - 1.0
+    assert abs(rel.mean()) < 1e-7 and np.abs(rel).max() < 3e-6
