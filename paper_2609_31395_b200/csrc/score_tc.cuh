@@ -224,8 +224,8 @@ inline int score_tc_launch_score(ScoreArgs& a, const actkv_pool_t* pool, int max
   // Every unit lays out its own shared memory: the widest one must have its queries and POOL_MIN_STAGES key tiles,
   // everyone takes what is left for more of them.
   // (the kernel without the LSE in the contraction when no unit would use it: few rows, a group it is not done for, or every
-  // window as long as the longest and that beyond the limit)
-  const bool aug = rows_all > 64 && tc::aug_group(Gp) && !(rows_all > tc::aug_rows(nh) && (int64_t)a.sum_win == (int64_t)a.tab.n_req * max_win);
+  // window as long as the longest and that beyond the limit; or when dividing by the scale could overflow)
+  const bool aug = rows_all > 64 && tc::aug_group(Gp) && a.scale_log2 >= 1e-30f && !(rows_all > tc::aug_rows(nh) && (int64_t)a.sum_win == (int64_t)a.tab.n_req * max_win);
   const size_t fixed = (size_t)n_rc * nh * tc::QBLK_BYTES + tc::POOL_FIXED;
   const size_t tables = aug && rows_pad <= tc::aug_rows(nh) ? tc::AUG_K_BYTES + (size_t)n_rc * tc::AUG_CHUNK_BYTES : 0;
   ta.n_stages = (int32_t)std::min<size_t>(tc::POOL_STAGES, (tc::SMEM_LIMIT - fixed) / (nh * tc::HALF_BYTES));

@@ -69,3 +69,19 @@ def test_scores_are_not_rounded_to_one_side(head_dim, group, windows):
     comp.check_status()
     rel = comp.score.cpu().numpy().astype(np.float64) / want - 1.0
     assert abs(rel.mean()) < 1e-7 and np.abs(rel).max() < 3e-6
+
+
+def test_a_softmax_scale_whose_inverse_overflows():
+    """Every logit is next to 0 then, and a score is what the supplied LSEs say."""
+    wl = synth.Workload("scale", 1, 2, 4, [300, 200], [40, 30], [100, 50], table_style="fragmented", seed=1)
+    inst = synth.generate(wl, DEV)
+    comp = H.Compressor(inst.pool, inst.page_table, inst.seq_len, inst.free_list, inst.free_count, wl.n_q_heads, H.sizes_of(inst))
+    lse = np.random.default_rng(0).uniform(-20.0, 20.0, (1, 70, 8)).astype(np.float32)
+    comp.run_score(inst.q, inst.win_indptr, inst.tok_indptr, 2e-38, False, lse_in=torch.from_numpy(lse).to(DEV))
+    torch.cuda.synchronize()
+    comp.check_status()
+    got = comp.score.cpu().numpy()[0]
+    a = np.exp(-lse[0].astype(np.float64)).reshape(70, 2, 4).max(axis=2)
+    for r, (w0, w1, t0, t1) in enumerate([(0, 40, 0, 300), (40, 70, 300, 500)]):
+        want = a[w0:w1].mean(axis=0)
+        assert (np.abs(got[:, t0:t1] / want[:, None] - 1.0) < U.SCORE_RTOL).all(), r
