@@ -334,43 +334,44 @@ __global__ void __launch_bounds__(GA_NT) gather_f32_kernel(
     const int32_t* __restrict__ sel_idx, int64_t sel_stride, const int32_t* __restrict__ keep_indptr, int32_t n_req,
     float* __restrict__ dst, int64_t dst_stride) {
   pdl_begin(src, tok_indptr, sel_idx, keep_indptr);
-  const int o = blockIdx.y;
-  const int first = blockIdx.x * (GA_NT * GA_PER), lane = threadIdx.x & 31;
-  const int i0 = first + threadIdx.x;
+  const int o = blockIdx.y, lane = threadIdx.x & 31;
   const int32_t* sel = sel_idx + (int64_t)o * sel_stride;
   const float* sc = src + (int64_t)o * src_stride;
   float* out = dst + (int64_t)o * dst_stride;
   const int total = keep_indptr[n_req];
-  if (first >= total) return;
-  int tok[GA_PER];
+  // (one round when the host's bound holds)
+  for (int64_t first64 = (int64_t)blockIdx.x * (GA_NT * GA_PER); first64 < total; first64 += (int64_t)gridDim.x * (GA_NT * GA_PER)) {
+    const int first = (int)first64, i0 = first + threadIdx.x;
+    int tok[GA_PER];
 #pragma unroll
-  for (int k = 0; k < GA_PER; ++k) tok[k] = i0 + k * GA_NT < total ? sel[i0 + k * GA_NT] : 0;
-  // the request of the CTA's first survivor: the last r with keep_indptr[r] <= first
-  int r = 0;
-  for (int q0 = 1; q0 < n_req; q0 += 32) {
-    const int c = __popc(__ballot_sync(0xffffffffu, q0 + lane < n_req && keep_indptr[q0 + lane] <= first));
-    r += c;
-    if (c < 32) break;
-  }
-  int next = keep_indptr[r + 1], base = tok_indptr[r];
-  if (next >= min(total, first + GA_NT * GA_PER)) {            // one request (uniform over the CTA)
-    float v[GA_PER];
+    for (int k = 0; k < GA_PER; ++k) tok[k] = i0 + k * GA_NT < total ? sel[i0 + k * GA_NT] : 0;
+    // the request of the CTA's first survivor: the last r with keep_indptr[r] <= first
+    int r = 0;
+    for (int q0 = 1; q0 < n_req; q0 += 32) {
+      const int c = __popc(__ballot_sync(0xffffffffu, q0 + lane < n_req && keep_indptr[q0 + lane] <= first));
+      r += c;
+      if (c < 32) break;
+    }
+    int next = keep_indptr[r + 1], base = tok_indptr[r];
+    if (next >= min(total, first + GA_NT * GA_PER)) {          // one request (uniform over the CTA)
+      float v[GA_PER];
 #pragma unroll
-    for (int k = 0; k < GA_PER; ++k) v[k] = i0 + k * GA_NT < total ? sc[base + tok[k]] : 0.f;
+      for (int k = 0; k < GA_PER; ++k) v[k] = i0 + k * GA_NT < total ? sc[base + tok[k]] : 0.f;
 #pragma unroll
-    for (int k = 0; k < GA_PER; ++k)
-      if (i0 + k * GA_NT < total) out[i0 + k * GA_NT] = v[k];
-  } else {
+      for (int k = 0; k < GA_PER; ++k)
+        if (i0 + k * GA_NT < total) out[i0 + k * GA_NT] = v[k];
+    } else {
 #pragma unroll
-    for (int k = 0; k < GA_PER; ++k) {
-      const int i = i0 + k * GA_NT;
-      if (i < total) {
-        while (i >= next) {                                    // (i < total = keep_indptr[n_req]: r + 1 < n_req here)
-          ++r;
-          next = keep_indptr[r + 1];
-          base = tok_indptr[r];
+      for (int k = 0; k < GA_PER; ++k) {
+        const int i = i0 + k * GA_NT;
+        if (i < total) {
+          while (i >= next) {                                  // (i < total = keep_indptr[n_req]: r + 1 < n_req here)
+            ++r;
+            next = keep_indptr[r + 1];
+            base = tok_indptr[r];
+          }
+          out[i] = sc[base + tok[k]];
         }
-        out[i] = sc[base + tok[k]];
       }
     }
   }

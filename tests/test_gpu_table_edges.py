@@ -111,6 +111,17 @@ def test_gather_over_request_boundaries(counts):
     assert np.array_equal(dst.cpu().numpy(), want)
 
 
+def test_gather_takes_all_survivors_whatever_the_bound():
+    n, L = 5000, 6000
+    sel = np.sort(np.random.default_rng(3).permutation(L)[:n]).astype(np.int32)
+    src = np.random.default_rng(4).random((1, L), dtype=np.float32)
+    dst = torch.zeros((1, n), device=DEV)
+    i32 = lambda *v: torch.tensor(v, dtype=torch.int32, device=DEV)  # noqa: E731
+    B.actkv_gather_f32(torch.from_numpy(src).to(DEV), L, i32(0, L), torch.from_numpy(sel[None]).to(DEV), n, i32(0, n), 1, 1, 100, dst, n)
+    torch.cuda.synchronize()
+    assert np.array_equal(dst.cpu().numpy()[0], src[0, sel])
+
+
 @pytest.mark.parametrize("lens,budgets", [([256, 257, 511, 513, 2], [128, 256, 257, 512, 1]), ([40000], [39990]),
                                           ([9000, 3000], [4500, 2999])])
 def test_inplace_slots_over_cta_boundaries(lens, budgets):
