@@ -59,7 +59,8 @@ struct KeepShared {
 };
 
 // FUSED: the ranking keys go straight into TopK (select_core.cuh, on the keys in shared memory) instead of back to the
-// score array: one read of the scores, one launch.  Every unit must fit in shared memory.
+// score array: one read of the scores, one launch.  A unit longer than the host's bound does not fit in shared memory: its scores
+// and keep-scores are read again for every sweep.
 // What bounds it: latency, as in select.cu.  64 units x 16 requests of 8K-24K tokens 318 -> 146 us, 512 units of 35000
 // 328 -> 202 us (fixed digits of 12, 12 and 8 bits and two ordered sweeps with block scans before).
 template <bool FUSED, int NT>
@@ -96,8 +97,8 @@ __global__ void __launch_bounds__(NT) keepscore_kernel(
     n_keep = min(max(fs.budget[r], 0), L);
     // as actkv_select: nothing after an earlier error of the step, and no store past the index buffer
     if (status_set(fs.status)) return;
-    if ((int64_t)fs.keep_indptr[r] + n_keep > fs.sel_stride || L > cap) {
-      if (threadIdx.x == 0) report(fs.status, ACTKV_E_INVALID, r, L > cap ? L : n_keep);
+    if ((int64_t)fs.keep_indptr[r] + n_keep > fs.sel_stride) {
+      if (threadIdx.x == 0) report(fs.status, ACTKV_E_INVALID, r, n_keep);
       return;
     }
     if (n_keep == 0 && fs.tie != nullptr && threadIdx.x == 0) fs.tie[u] = actkv_tie_t{0.f, 0, 0, 0};
@@ -106,195 +107,204 @@ __global__ void __launch_bounds__(NT) keepscore_kernel(
   float* sc = score + (int64_t)o * sum_tok + base;
   float* ks = keep_score + (int64_t)o * sum_tok + base;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool resident = FUSED || L <= cap;               // uniform over the CTA
-  auto key_at = [&](int i) -> uint32_t { return resident ? skeys[i] : order_key(sc[i]); };
+  // (two bodies: as a branch inside one, the distinction cost 670 -> 680 us at the end of an action region)
+  auto unit = [&](auto is_resident) {
+    constexpr bool resident = decltype(is_resident)::value;
+    auto key_at = [&](int i) -> uint32_t { return resident ? skeys[i] : order_key(sc[i]); };
 
-  // ---- one read of the scores: order keys into shared memory, their range, the total mass ----
-  uint32_t lo = 0xffffffffu, hi = 0u;
-  unsigned long long total = 0ull;
-  for (int i0 = tid; i0 < L; i0 += 4 * NT) {             // four loads in flight per thread
-    float x[4];
+    // ---- one read of the scores: order keys into shared memory, their range, the total mass ----
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    unsigned long long total = 0ull;
+    for (int i0 = tid; i0 < L; i0 += 4 * NT) {             // four loads in flight per thread
+      float x[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) x[j] = i0 + j * NT < L ? sc[i0 + j * NT] : 0.f;
+      for (int j = 0; j < 4; ++j) x[j] = i0 + j * NT < L ? sc[i0 + j * NT] : 0.f;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (i0 + j * NT < L) {
-        const uint32_t k = order_key(x[j]);
-        if (resident) skeys[i0 + j * NT] = k;
-        lo = min(lo, k);
-        hi = max(hi, k);
-        total += ks_mass(x[j]);
+      for (int j = 0; j < 4; ++j) {
+        if (i0 + j * NT < L) {
+          const uint32_t k = order_key(x[j]);
+          if constexpr (resident) skeys[i0 + j * NT] = k;
+          lo = min(lo, k);
+          hi = max(hi, k);
+          total += ks_mass(x[j]);
+        }
       }
     }
-  }
 #pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) total += __shfl_xor_sync(0xffffffffu, total, d);
-  if (lane == 0) sh.warp_tot[warp] = total;
-  block_range<NT>(sh.sel, lo, hi);                       // (its barrier also covers the keys and warp_tot)
-  total = lane < WARPS ? sh.warp_tot[lane] : 0ull;
+    for (int d = 16; d >= 1; d >>= 1) total += __shfl_xor_sync(0xffffffffu, total, d);
+    if (lane == 0) sh.warp_tot[warp] = total;
+    block_range<NT>(sh.sel, lo, hi);                       // (its barrier also covers the keys and warp_tot)
+    total = lane < WARPS ? sh.warp_tot[lane] : 0ull;
 #pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) total += __shfl_xor_sync(0xffffffffu, total, d);
-  // mark = ceil(p_q * total / 10000); total < 2^57 for up to 2^16 entries and p_q <= 10000 < 2^14: the product is
-  // taken in two halves to stay inside 64 bits
-  const unsigned long long mark = total / 10000ull * (unsigned long long)p_q +
-                                  (total % 10000ull * (unsigned long long)p_q + 9999ull) / 10000ull;
+    for (int d = 16; d >= 1; d >>= 1) total += __shfl_xor_sync(0xffffffffu, total, d);
+    // mark = ceil(p_q * total / 10000); total < 2^57 for up to 2^16 entries and p_q <= 10000 < 2^14: the product is
+    // taken in two halves to stay inside 64 bits
+    const unsigned long long mark = total / 10000ull * (unsigned long long)p_q +
+                                    (total % 10000ull * (unsigned long long)p_q + 9999ull) / 10000ull;
 
-  // ---- the largest key T with mass(key >= T) >= mark ----
-  uint32_t thr = 0u;                   // key of the last hit
-  int32_t last_tie = -1;               // entries equal to it are hits up to this index
-  if (mark > 0ull) {                   // (uniform over the CTA)
-    unsigned long long above = 0ull;   // mass of keys above the range in question
-    uint32_t span = hi - lo;
-    for (;;) {
-      const int shift = bin_shift(span, KS_BINS);
-      for (int i = tid; i < 3 * KS_BINS; i += NT) hist[i] = 0u;
-      if (tid == 0) sh.sel.n_list = 0u;
+    // ---- the largest key T with mass(key >= T) >= mark ----
+    uint32_t thr = 0u;                   // key of the last hit
+    int32_t last_tie = -1;               // entries equal to it are hits up to this index
+    if (mark > 0ull) {                   // (uniform over the CTA)
+      unsigned long long above = 0ull;   // mass of keys above the range in question
+      uint32_t span = hi - lo;
+      for (;;) {
+        const int shift = bin_shift(span, KS_BINS);
+        for (int i = tid; i < 3 * KS_BINS; i += NT) hist[i] = 0u;
+        if (tid == 0) sh.sel.n_list = 0u;
+        __syncthreads();
+        for (int i = tid; i < L; i += NT) {
+          const uint32_t k = key_at(i);
+          if (k - lo <= span) hist_add((k - lo) >> shift, ks_mass(key_to_float(k)));
+        }
+        __syncthreads();
+        // sums over the bins, descending
+        const int b0 = KS_BINS - PER * (tid + 1);
+        unsigned long long h[PER], mine = 0ull;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) { h[j] = hist_get(b0 + j); mine += h[j]; }
+        unsigned long long acc = above + block_exclusive<NT, unsigned long long>(mine, sh.warp_tot);
+        if (acc < mark && acc + mine >= mark) {            // exactly one thread
+#pragma unroll
+          for (int j = PER - 1; j >= 0; --j) {
+            if (acc < mark && acc + h[j] >= mark) {
+              sh.bin = (uint32_t)(b0 + j);
+              sh.above = acc;
+            }
+            acc += h[j];
+          }
+        }
+        __syncthreads();
+        above = sh.above;
+        lo += sh.bin << shift;
+        span = (1u << shift) - 1u;
+        for (int i = tid; i < L; i += NT) {
+          const uint32_t k = key_at(i);
+          if (k - lo <= span) {
+            const uint32_t p = atomicAdd(&sh.sel.n_list, 1u);
+            if (p < (uint32_t)KS_LIST) { sh.list[p] = k; sh.mass[p] = ks_mass(key_to_float(k)); }
+          }
+        }
+        __syncthreads();
+        const uint32_t count = sh.sel.n_list;
+        if (shift == 0) {                                  // a bin is one key
+          if (tid == 0) { sh.thr = lo; sh.eq_total = count; }
+          break;
+        }
+        if (count <= (uint32_t)KS_LIST) {
+          for (uint32_t i = tid; i < count; i += NT) {
+            const uint32_t v = sh.list[i];
+            const unsigned long long m = sh.mass[i];
+            unsigned long long gt = above;
+            uint32_t equal = 0u;
+            for (uint32_t j = 0; j < count; ++j) {
+              const uint32_t w = sh.list[j];
+              gt += w > v ? sh.mass[j] : 0ull;
+              equal += w == v;
+            }
+            if (gt < mark && gt + m * equal >= mark) {     // (every entry of that value: the same words)
+              sh.thr = v;
+              sh.above = gt;
+              sh.eq_total = equal;
+            }
+          }
+          break;
+        }
+        __syncthreads();
+      }
       __syncthreads();
-      for (int i = tid; i < L; i += NT) {
+      thr = sh.thr;
+      // all entries with key == thr share one score, hence one mass (> 0: the bin crossed the mark)
+      const unsigned long long thr_mass = ks_mass(key_to_float(thr));
+      const unsigned long long need = mark - sh.above;     // > 0 by construction
+      const unsigned long long ties_hit = thr_mass > 0ull ? (need + thr_mass - 1ull) / thr_mass : 0ull;
+      last_tie = L;
+      if (ties_hit < sh.eq_total) {
+        // the index of the ties_hit-th entry equal to thr: a contiguous segment per warp
+        const int seg = ((L + WARPS - 1) / WARPS + 31) & ~31;
+        const int i_begin = warp * seg, i_end = min(L, i_begin + seg);
+        uint32_t n_eq = 0u;
+        for (int i = i_begin + lane; i < i_end; i += 32) n_eq += key_at(i) == thr;
+        n_eq = __reduce_add_sync(0xffffffffu, n_eq);
+        if (lane == 0) sh.sel.warp_eq[warp] = n_eq;
+        if (tid == 0) sh.last_tie = -1;
+        __syncthreads();
+        uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp && lane < WARPS ? sh.sel.warp_eq[lane] : 0u);
+        if (ties_hit > before && ties_hit <= before + n_eq) {
+          for (int i0 = i_begin; i0 < i_end; i0 += 32) {
+            const int i = i0 + lane;
+            const bool eq = i < i_end && key_at(i) == thr;
+            const uint32_t bal = __ballot_sync(0xffffffffu, eq);
+            if (eq && before + __popc(bal & ((2u << lane) - 1u)) == ties_hit) sh.last_tie = i;
+            before += __popc(bal);
+          }
+        }
+        __syncthreads();
+        last_tie = sh.last_tie;
+      }
+    }
+
+    // ---- hits, keep-score update, ranking keys: every entry on its own ----
+    const int np = n_protect ? n_protect[r] : 0;
+    uint32_t* mrow = hit_mask ? hit_mask + (int64_t)o * ((sum_tok + 31) / 32) : nullptr;
+    // (the protected entries, which rank as +inf, are counted apart: the range that TopK divides is that of the others)
+    constexpr uint32_t INF_KEY = 0xff800000u;
+    uint32_t n_inf = 0u;
+    lo = 0xffffffffu;
+    hi = 0u;
+    for (int i0 = tid; i0 < L; i0 += 4 * NT) {
+      float old[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) old[j] = i0 + j * NT < L ? ks[i0 + j * NT] : 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int i = i0 + j * NT;
+        if (i >= L) break;
         const uint32_t k = key_at(i);
-        if (k - lo <= span) hist_add((k - lo) >> shift, ks_mass(key_to_float(k)));
-      }
-      __syncthreads();
-      // sums over the bins, descending
-      const int b0 = KS_BINS - PER * (tid + 1);
-      unsigned long long h[PER], mine = 0ull;
-#pragma unroll
-      for (int j = 0; j < PER; ++j) { h[j] = hist_get(b0 + j); mine += h[j]; }
-      unsigned long long acc = above + block_exclusive<NT, unsigned long long>(mine, sh.warp_tot);
-      if (acc < mark && acc + mine >= mark) {            // exactly one thread
-#pragma unroll
-        for (int j = PER - 1; j >= 0; --j) {
-          if (acc < mark && acc + h[j] >= mark) {
-            sh.bin = (uint32_t)(b0 + j);
-            sh.above = acc;
+        const bool hit = mark > 0ull && (k > thr || (k == thr && i <= last_tie));
+        const float decayed = mul_ieee(lambda, old[j]);
+        const float nk = hit ? add_ieee(decayed, key_to_float(k)) : decayed;
+        ks[i] = nk;
+        const float rank = (i < np) ? INFINITY : nk;            // what TopK ranks
+        if (FUSED) {
+          const uint32_t rk = order_key(rank);
+          if constexpr (resident) skeys[i] = rk;
+          if (rk == INF_KEY) {
+            ++n_inf;
+          } else {
+            lo = min(lo, rk);
+            hi = max(hi, rk);
           }
-          acc += h[j];
-        }
-      }
-      __syncthreads();
-      above = sh.above;
-      lo += sh.bin << shift;
-      span = (1u << shift) - 1u;
-      for (int i = tid; i < L; i += NT) {
-        const uint32_t k = key_at(i);
-        if (k - lo <= span) {
-          const uint32_t p = atomicAdd(&sh.sel.n_list, 1u);
-          if (p < (uint32_t)KS_LIST) { sh.list[p] = k; sh.mass[p] = ks_mass(key_to_float(k)); }
-        }
-      }
-      __syncthreads();
-      const uint32_t count = sh.sel.n_list;
-      if (shift == 0) {                                  // a bin is one key
-        if (tid == 0) { sh.thr = lo; sh.eq_total = count; }
-        break;
-      }
-      if (count <= (uint32_t)KS_LIST) {
-        for (uint32_t i = tid; i < count; i += NT) {
-          const uint32_t v = sh.list[i];
-          const unsigned long long m = sh.mass[i];
-          unsigned long long gt = above;
-          uint32_t equal = 0u;
-          for (uint32_t j = 0; j < count; ++j) {
-            const uint32_t w = sh.list[j];
-            gt += w > v ? sh.mass[j] : 0ull;
-            equal += w == v;
-          }
-          if (gt < mark && gt + m * equal >= mark) {     // (every entry of that value: the same words)
-            sh.thr = v;
-            sh.above = gt;
-            sh.eq_total = equal;
-          }
-        }
-        break;
-      }
-      __syncthreads();
-    }
-    __syncthreads();
-    thr = sh.thr;
-    // all entries with key == thr share one score, hence one mass (> 0: the bin crossed the mark)
-    const unsigned long long thr_mass = ks_mass(key_to_float(thr));
-    const unsigned long long need = mark - sh.above;     // > 0 by construction
-    const unsigned long long ties_hit = thr_mass > 0ull ? (need + thr_mass - 1ull) / thr_mass : 0ull;
-    last_tie = L;
-    if (ties_hit < sh.eq_total) {
-      // the index of the ties_hit-th entry equal to thr: a contiguous segment per warp
-      const int seg = ((L + WARPS - 1) / WARPS + 31) & ~31;
-      const int i_begin = warp * seg, i_end = min(L, i_begin + seg);
-      uint32_t n_eq = 0u;
-      for (int i = i_begin + lane; i < i_end; i += 32) n_eq += key_at(i) == thr;
-      n_eq = __reduce_add_sync(0xffffffffu, n_eq);
-      if (lane == 0) sh.sel.warp_eq[warp] = n_eq;
-      if (tid == 0) sh.last_tie = -1;
-      __syncthreads();
-      uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp && lane < WARPS ? sh.sel.warp_eq[lane] : 0u);
-      if (ties_hit > before && ties_hit <= before + n_eq) {
-        for (int i0 = i_begin; i0 < i_end; i0 += 32) {
-          const int i = i0 + lane;
-          const bool eq = i < i_end && key_at(i) == thr;
-          const uint32_t bal = __ballot_sync(0xffffffffu, eq);
-          if (eq && before + __popc(bal & ((2u << lane) - 1u)) == ties_hit) sh.last_tie = i;
-          before += __popc(bal);
-        }
-      }
-      __syncthreads();
-      last_tie = sh.last_tie;
-    }
-  }
-
-  // ---- hits, keep-score update, ranking keys: every entry on its own ----
-  const int np = n_protect ? n_protect[r] : 0;
-  uint32_t* mrow = hit_mask ? hit_mask + (int64_t)o * ((sum_tok + 31) / 32) : nullptr;
-  // (the protected entries, which rank as +inf, are counted apart: the range that TopK divides is that of the others)
-  constexpr uint32_t INF_KEY = 0xff800000u;
-  uint32_t n_inf = 0u;
-  lo = 0xffffffffu;
-  hi = 0u;
-  for (int i0 = tid; i0 < L; i0 += 4 * NT) {
-    float old[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) old[j] = i0 + j * NT < L ? ks[i0 + j * NT] : 0.f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int i = i0 + j * NT;
-      if (i >= L) break;
-      const uint32_t k = key_at(i);
-      const bool hit = mark > 0ull && (k > thr || (k == thr && i <= last_tie));
-      const float decayed = mul_ieee(lambda, old[j]);
-      const float nk = hit ? add_ieee(decayed, key_to_float(k)) : decayed;
-      ks[i] = nk;
-      const float rank = (i < np) ? INFINITY : nk;            // what TopK ranks
-      if (FUSED) {
-        const uint32_t rk = order_key(rank);
-        skeys[i] = rk;
-        if (rk == INF_KEY) {
-          ++n_inf;
         } else {
-          lo = min(lo, rk);
-          hi = max(hi, rk);
+          sc[i] = rank;
         }
-      } else {
-        sc[i] = rank;
+        if (hit && mrow) atomicOr(&mrow[(base + i) >> 5], 1u << ((base + i) & 31));
       }
-      if (hit && mrow) atomicOr(&mrow[(base + i) >> 5], 1u << ((base + i) & 31));
     }
-  }
-  if (FUSED && n_keep > 0) {                             // uniform over the CTA
-    n_inf = __reduce_add_sync(0xffffffffu, n_inf);
-    __syncthreads();                                     // (the ranges of the first block_range have been read)
-    if (lane == 0) sh.sel.warp_eq[warp] = n_inf;
-    block_range<NT>(sh.sel, lo, hi);
-    n_inf = __reduce_add_sync(0xffffffffu, lane < WARPS ? sh.sel.warp_eq[lane] : 0u);
-    if (hi > INF_KEY) {                                  // (keys beyond +inf: NaN scores)
-      lo = min(lo, INF_KEY);
-      n_inf = 0u;
-    } else if (n_inf >= (uint32_t)n_keep) {
-      lo = hi = INF_KEY;
-      n_inf = 0u;
+    if (FUSED && n_keep > 0) {                             // uniform over the CTA
+      n_inf = __reduce_add_sync(0xffffffffu, n_inf);
+      __syncthreads();                                     // (the ranges of the first block_range have been read)
+      if (lane == 0) sh.sel.warp_eq[warp] = n_inf;
+      block_range<NT>(sh.sel, lo, hi);
+      n_inf = __reduce_add_sync(0xffffffffu, lane < WARPS ? sh.sel.warp_eq[lane] : 0u);
+      if (hi > INF_KEY) {                                  // (keys beyond +inf: NaN scores)
+        lo = min(lo, INF_KEY);
+        n_inf = 0u;
+      } else if (n_inf >= (uint32_t)n_keep) {
+        lo = hi = INF_KEY;
+        n_inf = 0u;
+      }
+      int32_t* out = fs.sel_idx + (int64_t)o * fs.sel_stride + fs.keep_indptr[r];
+      uint32_t* keep_row = fs.keep_mask ? fs.keep_mask + (int64_t)o * ((sum_tok + 31) / 32) : nullptr;
+      if constexpr (resident)
+        select_and_emit<NT, KS_BINS>([&](int i) { return skeys[i]; }, hist, sh.sel, lo, hi, L, n_keep, out, keep_row, base, fs.tie, u,
+                                     (int)n_inf);
+      else
+        select_and_emit<NT, KS_BINS>([&](int i) { return order_key(i < np ? INFINITY : ks[i]); }, hist, sh.sel, lo, hi, L, n_keep, out,
+                                     keep_row, base, fs.tie, u, (int)n_inf);
     }
-    select_and_emit<NT, KS_BINS>([&](int i) { return skeys[i]; }, hist, sh.sel, lo, hi, L, n_keep,
-                                 fs.sel_idx + (int64_t)o * fs.sel_stride + fs.keep_indptr[r],
-                                 fs.keep_mask ? fs.keep_mask + (int64_t)o * ((sum_tok + 31) / 32) : nullptr, base, fs.tie, u, (int)n_inf);
-  }
+  };
+  if (L <= cap) unit(std::true_type{}); else unit(std::false_type{});      // (uniform over the CTA)
 }
 
 // max_tok: a bound on the unit lengths.

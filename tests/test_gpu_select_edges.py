@@ -157,3 +157,26 @@ def test_topk_of_keep_scores_beside_the_protected_prefix(prot, n_big):
     assert status.cpu().tolist()[0] == 0
     assert np.array_equal(d_ks.cpu().numpy(), ks0)         # no hits, no decay
     assert np.array_equal(sel.cpu().numpy(), O.select_unit(O.rank_keys(ks0, prot), budget))
+
+
+@pytest.mark.parametrize("L,bound", [(3000, 100), (45568, 2000), (20000, 19999)])
+def test_keepscore_and_topk_of_a_unit_longer_than_the_bound(L, bound):
+    rng, tok, ki, sc = _case("normal", [L, 50], [L // 2, 20], 2, L)
+    sc = np.minimum(sc, np.float32(1.0))
+    ks0 = (rng.random(sc.shape) ** 4).astype(np.float32)
+    d_ks, d_sc = torch.from_numpy(ks0.copy()).to(DEV), torch.from_numpy(sc).to(DEV)
+    sel = torch.full((2, int(ki[-1])), -1, dtype=torch.int32, device=DEV)
+    status = torch.zeros(4, dtype=torch.int32, device=DEV)
+    i32 = lambda *v: torch.tensor(v, dtype=torch.int32, device=DEV)  # noqa: E731
+    B.actkv_keepscore_select(d_sc, torch.from_numpy(tok).to(DEV), int(tok[-1]), bound, 2, 2, 0.9, 0.5, i32(70, 0), d_ks, None,
+                             i32(L // 2, 20), torch.from_numpy(ki).to(DEV), sel, sel.shape[1], None, None, status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist()[0] == 0
+    assert np.array_equal(d_sc.cpu().numpy(), sc)          # left as they were
+    for o in range(2):
+        for r, (n, prot) in enumerate([(L // 2, 70), (20, 0)]):
+            a, b = int(tok[r]), int(tok[r + 1])
+            hit = O.hit_mask_unit(sc[o, a:b], 0.9)
+            ks = O.keep_score_update(ks0[o, a:b], sc[o, a:b], hit, 0.5)
+            assert np.array_equal(d_ks.cpu().numpy()[o, a:b].view(np.uint32), ks.view(np.uint32))
+            assert np.array_equal(sel.cpu().numpy()[o, ki[r]:ki[r + 1]], O.select_unit(O.rank_keys(ks, prot), n))
