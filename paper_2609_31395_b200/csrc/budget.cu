@@ -732,8 +732,7 @@ static int launch_token_conf(const float* logits, int32_t vocab, int32_t n_rows,
   }
   const size_t sm = sizeof(SweepSmem);
   if (ensure_dyn_smem(token_conf_sweep_kernel, sm) != cudaSuccess) return ACTKV_E_CUDA;
-  launch_pdl(token_conf_sweep_kernel, (unsigned)n_rows, SW_NT, sm, s,
-      logits, vocab, k, out);
+  launch_pdl(token_conf_sweep_kernel, (unsigned)n_rows, SW_NT, sm, s, logits, vocab, k, out);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -771,8 +770,7 @@ int actkv_budget(const float* logits, const int32_t* tok_indptr, int32_t n_rows,
                            params->B_upper, params->clamp_lo_ppm, params->clamp_hi_ppm};
   const int32_t max_m = hist_cap;
   actkv::launch_pdl(actkv::trend_kernel, (unsigned)n_req, actkv::TR_NT, 0, s,
-      n_rows > 0 ? tok_indptr : nullptr, conf_hist, hist_len, hist_cap, p, seq_len, budget_in,
-      budget_out, slope_out, pooled, max_m);
+                    n_rows > 0 ? tok_indptr : nullptr, conf_hist, hist_len, hist_cap, p, seq_len, budget_in, budget_out, slope_out, pooled, max_m);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }

@@ -398,11 +398,10 @@ static int compact_plan(const actkv_pool_t* pool, const actkv_tables_t* tables, 
   job.vpr_shift = deferrable_shift(pool);
   job.deferred = deferred ? 1 : 0;
   if (reuse_plan)
-    launch_pdl(compact_rejob_kernel, 1, 1, 0, s,
-      (CompactWs*)ws, job, status);
+    launch_pdl(compact_rejob_kernel, 1, 1, 0, s, (CompactWs*)ws, job, status);
   else
-    launch_pdl(compact_plan_kernel, status != nullptr ? table_grid(tables) : dim3(1, 1), PLAN_NT, 0, s,
-      make_view(tables), pool->page_size, pool->n_pages, budget, max_keep, (CompactWs*)ws, status, job);
+    launch_pdl(compact_plan_kernel, status != nullptr ? table_grid(tables) : dim3(1, 1), PLAN_NT, 0, s, make_view(tables),
+               pool->page_size, pool->n_pages, budget, max_keep, (CompactWs*)ws, status, job);
   ACTKV_CHECK_LAUNCH();
   if (deferred && job.vpr_shift >= 0 && job.src_tab_items > 0) {
     // one warp per item of the largest job these arguments allow (short, independent chains of lookups)
@@ -411,8 +410,7 @@ static int compact_plan(const actkv_pool_t* pool, const actkv_tables_t* tables, 
     const int64_t jp = ((int64_t)pool->page_size * pool->n_kv_heads + 31) / 32;
     const int64_t items_max = std::min<int64_t>(max_x * tables->n_req * job.n_layers * jp, job.src_tab_items);
     const int64_t ctas = std::min<int64_t>(std::max<int64_t>(1, (items_max + 3) / 4), 1 << 20);
-    launch_pdl(compact_resolve_kernel, (unsigned)ctas, 128, 0, s,
-      (CompactWs*)ws);
+    launch_pdl(compact_resolve_kernel, (unsigned)ctas, 128, 0, s, (CompactWs*)ws);
     ACTKV_CHECK_LAUNCH();
   }
   return ACTKV_OK;
@@ -441,17 +439,17 @@ static int compact_copy_all(const actkv_pool_t* pool, const actkv_tables_t* tabl
   const size_t sm = (size_t)2 * rows * sizeof(int64_t);
   const int vpr = pool->head_dim / 8;
   if (vpr == 16)
-    launch_pdl(compact_copy_kernel<4>, grid, CP_NT, sm, s,
-      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
+    launch_pdl(compact_copy_kernel<4>, grid, CP_NT, sm, s, pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w,
+               rows, parts, status);
   else if (vpr == 8)
-    launch_pdl(compact_copy_kernel<3>, grid, CP_NT, sm, s,
-      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
+    launch_pdl(compact_copy_kernel<3>, grid, CP_NT, sm, s, pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w,
+               rows, parts, status);
   else if (vpr == 32)
-    launch_pdl(compact_copy_kernel<5>, grid, CP_NT, sm, s,
-      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
+    launch_pdl(compact_copy_kernel<5>, grid, CP_NT, sm, s, pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w,
+               rows, parts, status);
   else
-    launch_pdl(compact_copy_kernel<-1>, grid, CP_NT, sm, s,
-      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w, rows, parts, status);
+    launch_pdl(compact_copy_kernel<-1>, grid, CP_NT, sm, s, pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, w,
+               rows, parts, status);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -459,8 +457,8 @@ static int compact_copy_all(const actkv_pool_t* pool, const actkv_tables_t* tabl
 static int compact_finalize(const actkv_pool_t* pool, const actkv_tables_t* tables, int32_t layer_end, const int32_t* budget,
                             void* ws, int32_t* status, cudaStream_t s) {
   if (layer_end != pool->n_layers) return ACTKV_OK;
-  launch_pdl(compact_finalize_kernel, table_grid(tables), PLAN_NT, 0, s,
-      make_view(tables), pool->page_size, budget, (CompactWs*)ws, status);
+  launch_pdl(compact_finalize_kernel, table_grid(tables), PLAN_NT, 0, s, make_view(tables),
+             pool->page_size, budget, (CompactWs*)ws, status);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -500,8 +498,7 @@ int actkv_compact_begin(const actkv_pool_t* pool, const actkv_tables_t* tables, 
 
 int actkv_compact_stats(const void* ws, int32_t* stats, actkv_stream_t stream) {
   if (!ws || !stats) return ACTKV_E_INVALID;
-  actkv::launch_pdl(actkv::compact_stats_kernel, 1, 1, 0, (cudaStream_t)stream,
-      (const actkv::CompactWs*)ws, stats);
+  actkv::launch_pdl(actkv::compact_stats_kernel, 1, 1, 0, (cudaStream_t)stream, (const actkv::CompactWs*)ws, stats);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }

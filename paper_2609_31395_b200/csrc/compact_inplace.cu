@@ -453,8 +453,7 @@ static int inplace_copy_launch(const actkv_pool_t* pool, const actkv_tables_t* t
                           : compact_inplace_copy_kernel<-1, NT, PER>;
   // (launched plainly: with its CTAs placed while the selection kernel drains, the 16-request copy takes 571 us, not 455;
   //  they then seem to keep that kernel's division of the SM between shared memory and L1)
-  kern<<<grid, NT, 0, s>>>(
-      pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, max_keep, new_order, status);
+  kern<<<grid, NT, 0, s>>>(pv, tv, layer_begin, sel_idx, sel_stride, keep_indptr, budget, max_keep, new_order, status);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -477,8 +476,8 @@ static int inplace_copy_all(const actkv_pool_t* pool, const actkv_tables_t* tabl
 static int inplace_finalize(const actkv_pool_t* pool, const actkv_tables_t* tables, int32_t layer_end, const int32_t* budget,
                             int32_t* status, cudaStream_t s) {
   if (layer_end == pool->n_layers) {
-    launch_pdl(compact_inplace_finalize_kernel, FIN_CTAS, FIN_NT, 0, s,
-      make_view(tables), pool->page_size, pool->n_pages, budget, status);
+    launch_pdl(compact_inplace_finalize_kernel, FIN_CTAS, FIN_NT, 0, s, make_view(tables),
+               pool->page_size, pool->n_pages, budget, status);
     ACTKV_CHECK_LAUNCH();
   }
   return ACTKV_OK;
@@ -537,16 +536,14 @@ int actkv_compact_inplace_begin(const actkv_pool_t* pool, const actkv_tables_t* 
   uint32_t* dst_tab = (uint32_t*)((char*)ws + base + tab_bytes);
   // (not deferred: an empty job, so that a score call given this workspace finds nothing to do; actkv_compact_inplace_end
   //  then copies everything itself)
-  launch_pdl(compact_inplace_plan_kernel, 1, 32, 0, s,
-      make_view(tables), make_view(pool), budget, max_keep,
-                                               new_order != nullptr ? 1 : 0, layer_begin, deferred ? nl : 0,
-                                               deferred ? shift : -1, src_tab, dst_tab, deferred ? items_max : 0,
-                                               (CompactWs*)ws, status);
+  launch_pdl(compact_inplace_plan_kernel, 1, 32, 0, s, make_view(tables), make_view(pool), budget, max_keep,
+             new_order != nullptr ? 1 : 0, layer_begin, deferred ? nl : 0, deferred ? shift : -1, src_tab, dst_tab,
+             deferred ? items_max : 0, (CompactWs*)ws, status);
   ACTKV_CHECK_LAUNCH();
   if (deferred && items_max > 0) {
     const int64_t ctas = std::min<int64_t>(std::max<int64_t>(1, (items_max + 3) / 4), 1 << 20);
-    launch_pdl(compact_inplace_resolve_kernel, (unsigned)ctas, 128, 0, s,
-      (CompactWs*)ws, sel_idx, sel_stride, keep_indptr, new_order);
+    launch_pdl(compact_inplace_resolve_kernel, (unsigned)ctas, 128, 0, s, (CompactWs*)ws, sel_idx, sel_stride, keep_indptr,
+               new_order);
     ACTKV_CHECK_LAUNCH();
   }
   return ACTKV_OK;

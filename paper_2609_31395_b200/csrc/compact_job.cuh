@@ -205,12 +205,9 @@ __global__ void __launch_bounds__(128) compact_drain_kernel(CompactWs* ws) {
 inline void launch_drain(CompactWs* w, int shift, int64_t items_max, cudaStream_t s) {
   const int64_t want = (items_max + 3) / 4;
   const unsigned grid = (unsigned)(want < 1 ? 1 : (want > 148 * 8 ? 148 * 8 : want));
-  if (shift == 3) launch_pdl(compact_drain_kernel<3>, grid, 128, 0, s,
-      w);
-  else if (shift == 4) launch_pdl(compact_drain_kernel<4>, grid, 128, 0, s,
-      w);
-  else launch_pdl(compact_drain_kernel<5>, grid, 128, 0, s,
-      w);
+  if (shift == 3) launch_pdl(compact_drain_kernel<3>, grid, 128, 0, s, w);
+  else if (shift == 4) launch_pdl(compact_drain_kernel<4>, grid, 128, 0, s, w);
+  else launch_pdl(compact_drain_kernel<5>, grid, 128, 0, s, w);
 }
 
 // log2 of the 16-byte vectors per row when the warp-level item copy takes this pool: head_dim 64, 128 or 256,

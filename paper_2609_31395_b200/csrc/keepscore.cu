@@ -315,9 +315,8 @@ static int keepscore_launch_n(float* score, const int32_t* tok_indptr, int32_t s
   constexpr size_t fixed = 3 * KS_BINS * 4;
   const size_t smem = resident_smem(fixed, max_tok);
   if (ensure_dyn_smem(keepscore_kernel<FUSED, NT>, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  launch_pdl(keepscore_kernel<FUSED, NT>, (unsigned)units, NT, smem, s,
-      score, tok_indptr, sum_tok, n_req, p_q, lambda, n_protect,
-                                                                keep_score, hit_mask, (int32_t)((smem - fixed) / 4), fs);
+  launch_pdl(keepscore_kernel<FUSED, NT>, (unsigned)units, NT, smem, s, score, tok_indptr, sum_tok, n_req, p_q, lambda,
+             n_protect, keep_score, hit_mask, (int32_t)((smem - fixed) / 4), fs);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -443,9 +442,8 @@ int actkv_gather_f32(const float* src, int64_t src_stride, const int32_t* tok_in
   if (n_outer == 0 || n_req == 0 || max_total_keep == 0) return ACTKV_OK;
   if (!src || !tok_indptr || !sel_idx || !keep_indptr || !dst || n_outer > 65535) return ACTKV_E_INVALID;
   const dim3 grid((unsigned)((max_total_keep + actkv::GA_NT * actkv::GA_PER - 1) / (actkv::GA_NT * actkv::GA_PER)), (unsigned)n_outer);
-  actkv::launch_pdl(actkv::gather_f32_kernel, grid, actkv::GA_NT, 0, (cudaStream_t)stream,
-      src, src_stride, tok_indptr, sel_idx, sel_stride,
-                                                                   keep_indptr, n_req, dst, dst_stride);
+  actkv::launch_pdl(actkv::gather_f32_kernel, grid, actkv::GA_NT, 0, (cudaStream_t)stream, src, src_stride, tok_indptr,
+                    sel_idx, sel_stride, keep_indptr, n_req, dst, dst_stride);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }

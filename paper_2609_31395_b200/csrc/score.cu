@@ -137,8 +137,7 @@ static int score_impl(int mode, const actkv_pool_t* pool, const actkv_tables_t* 
       if (rc != ACTKV_OK) return rc;
     }
     const int64_t n_rows_all = units * lay.rows_max;
-    launch_pdl(lse_combine_kernel, (unsigned)((n_rows_all + 255) / 256), 256, 0, s,
-      a, lse_buf, nullptr);
+    launch_pdl(lse_combine_kernel, (unsigned)((n_rows_all + 255) / 256), 256, 0, s, a, lse_buf);
     ACTKV_CHECK_LAUNCH();
     lse = lse_buf;
   } else if (lse_out != nullptr && lse_in != nullptr && lse_out != lse_in) {

@@ -480,8 +480,7 @@ __global__ void __launch_bounds__(NT, 4) score_mma_pool_kernel(const ScoreArgs a
 template <int DB>
 inline int launch_lse_d(const ScoreArgs& a, unsigned grid, cudaStream_t s) {
   if (ensure_dyn_smem(score_mma_lse_kernel<DB>, sizeof(Smem<DB>)) != cudaSuccess) return ACTKV_E_CUDA;
-  launch_pdl(score_mma_lse_kernel<DB>, grid, NT, sizeof(Smem<DB>), s,
-      a);
+  launch_pdl(score_mma_lse_kernel<DB>, grid, NT, sizeof(Smem<DB>), s, a);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -497,8 +496,7 @@ inline int launch_lse(const ScoreArgs& a, int64_t units, cudaStream_t s) {
 template <int DB, int GP>
 inline int launch_pool_g(const ScoreArgs& a, unsigned grid, int keys, int parts, cudaStream_t s) {
   if (ensure_dyn_smem(score_mma_pool_kernel<DB, GP>, sizeof(Smem<DB>)) != cudaSuccess) return ACTKV_E_CUDA;
-  launch_pdl(score_mma_pool_kernel<DB, GP>, grid, NT, sizeof(Smem<DB>), s,
-      a, keys, parts);
+  launch_pdl(score_mma_pool_kernel<DB, GP>, grid, NT, sizeof(Smem<DB>), s, a, keys, parts);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -529,7 +527,7 @@ inline int launch_pool(const ScoreArgs& a, int64_t units, int max_tok, cudaStrea
 }  // namespace wm
 
 // Merges the per-chunk (max, sum) partials of one window row into its LSE (natural log units).
-__global__ void lse_combine_kernel(const ScoreArgs a, float* lse_out, float* lse_out2) {
+__global__ void lse_combine_kernel(const ScoreArgs a, float* lse_out) {
   pdl_begin();
   const int R = a.tab.n_req, Hkv = a.pool.n_kv_heads, G = a.group;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over units * rows_max
@@ -554,7 +552,6 @@ __global__ void lse_combine_kernel(const ScoreArgs a, float* lse_out, float* lse
   const int w = row / G, g = row % G;
   const int64_t o = ((int64_t)slab * a.sum_win + w0 + w) * a.n_q_heads + h * G + g;
   lse_out[o] = lse;
-  if (lse_out2 != nullptr) lse_out2[o] = lse;
 }
 
 }  // namespace actkv

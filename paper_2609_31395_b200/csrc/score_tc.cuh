@@ -72,51 +72,49 @@ inline int best_split(int64_t units, int tiles, int ovh, int n_max) {
   return best;
 }
 
-inline bool make_maps(const actkv_pool_t* pool, const void* q, int nls, int sum_win, int n_q_heads, int G,
-                      CUtensorMap* kmap, CUtensorMap* qmap) {
+inline bool make_kmap(const actkv_pool_t* pool, CUtensorMap* kmap) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
-  {
-    // K half of the pool.  Slot-major pages whose slots continue across pages: [layer][slot (page*16 + s)]
-    // [head][dim], four dimensions (measured 13 % faster than five on the K stream).  Any other page layout
-    // (head-major pages): [layer][page][head][slot][dim] with the caller's strides.  A box is one page of
-    // one head, 64 dims: page_size rows of 128 B.
-    CUresult res;
-    if (!pool_needs_5d(pool)) {
-      cuuint64_t dims[4] = {(cuuint64_t)pool->head_dim, (cuuint64_t)pool->n_kv_heads, (cuuint64_t)pool->n_pages * pool->page_size,
-                            (cuuint64_t)pool->n_layers};
-      cuuint64_t strides[3] = {(cuuint64_t)pool->stride_head * 2, (cuuint64_t)pool->stride_slot * 2,
-                               (cuuint64_t)pool->stride_layer * 2};
-      cuuint32_t box[4] = {64, 1, (cuuint32_t)pool->page_size, 1};
-      cuuint32_t es[4] = {1, 1, 1, 1};
-      res = enc(kmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, pool->base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    } else {
-      cuuint64_t dims[5] = {(cuuint64_t)pool->head_dim, (cuuint64_t)pool->page_size, (cuuint64_t)pool->n_kv_heads,
-                            (cuuint64_t)pool->n_pages, (cuuint64_t)pool->n_layers};
-      cuuint64_t strides[4] = {(cuuint64_t)pool->stride_slot * 2, (cuuint64_t)pool->stride_head * 2,
-                               (cuuint64_t)pool->stride_page * 2, (cuuint64_t)pool->stride_layer * 2};
-      cuuint32_t box[5] = {64, (cuuint32_t)pool->page_size, 1, 1, 1};
-      cuuint32_t es[5] = {1, 1, 1, 1, 1};
-      res = enc(kmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, pool->base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    }
-    if (res != CUDA_SUCCESS) return false;
+  // K half of the pool.  Slot-major pages whose slots continue across pages: [layer][slot (page*16 + s)]
+  // [head][dim], four dimensions (measured 13 % faster than five on the K stream).  Any other page layout
+  // (head-major pages): [layer][page][head][slot][dim] with the caller's strides.  A box is one page of
+  // one head, 64 dims: page_size rows of 128 B.
+  CUresult res;
+  if (!pool_needs_5d(pool)) {
+    cuuint64_t dims[4] = {(cuuint64_t)pool->head_dim, (cuuint64_t)pool->n_kv_heads, (cuuint64_t)pool->n_pages * pool->page_size,
+                          (cuuint64_t)pool->n_layers};
+    cuuint64_t strides[3] = {(cuuint64_t)pool->stride_head * 2, (cuuint64_t)pool->stride_slot * 2,
+                             (cuuint64_t)pool->stride_layer * 2};
+    cuuint32_t box[4] = {64, 1, (cuuint32_t)pool->page_size, 1};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    res = enc(kmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, pool->base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  } else {
+    cuuint64_t dims[5] = {(cuuint64_t)pool->head_dim, (cuuint64_t)pool->page_size, (cuuint64_t)pool->n_kv_heads,
+                          (cuuint64_t)pool->n_pages, (cuuint64_t)pool->n_layers};
+    cuuint64_t strides[4] = {(cuuint64_t)pool->stride_slot * 2, (cuuint64_t)pool->stride_head * 2,
+                             (cuuint64_t)pool->stride_page * 2, (cuuint64_t)pool->stride_layer * 2};
+    cuuint32_t box[5] = {64, (cuuint32_t)pool->page_size, 1, 1, 1};
+    cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    res = enc(kmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, pool->base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   }
-  {
-    // q: [slab*sum_win + w][q head][128]; a box is (64 dims, the G heads of one group, 128/G window rows)
-    const cuuint64_t D = (cuuint64_t)pool->head_dim;
-    cuuint64_t dims[3] = {D, (cuuint64_t)n_q_heads, (cuuint64_t)nls * sum_win};
-    cuuint64_t strides[2] = {D * 2, (cuuint64_t)n_q_heads * D * 2};
-    const int Gp = pow2_at_least(G);                 // the pooled-score kernel pads a group to a power of two
-    cuuint32_t box[3] = {64, (cuuint32_t)Gp, (cuuint32_t)(128 / Gp)};
-    cuuint32_t es[3] = {1, 1, 1};
-    if (enc(qmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(q), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return false;
-  }
-  return true;
+  return res == CUDA_SUCCESS;
+}
+
+inline bool make_qmap(const actkv_pool_t* pool, const void* q, int nls, int sum_win, int n_q_heads, int G, CUtensorMap* qmap) {
+  EncodeTiledFn enc = encode_fn();
+  if (!enc) return false;
+  // q: [slab*sum_win + w][q head][128]; a box is (64 dims, the G heads of one group, 128/G window rows)
+  const cuuint64_t D = (cuuint64_t)pool->head_dim;
+  cuuint64_t dims[3] = {D, (cuuint64_t)n_q_heads, (cuuint64_t)nls * sum_win};
+  cuuint64_t strides[2] = {D * 2, (cuuint64_t)n_q_heads * D * 2};
+  const int Gp = pow2_at_least(G);                 // the pooled-score kernel pads a group to a power of two
+  cuuint32_t box[3] = {64, (cuuint32_t)Gp, (cuuint32_t)(128 / Gp)};
+  cuuint32_t es[3] = {1, 1, 1};
+  return enc(qmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(q), dims, strides, box, es,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Fault-injection hook of the bounded waits (actkv_debug_inject_stall): while stall_tile >= 0 the K-tile
@@ -165,16 +163,15 @@ inline int score_tc_launch_lse_c(const CUtensorMap& kmap, const tc::TcArgs& ta, 
                   : (rgs ? (d64 ? tc::score_tc_lse_kernel<NPOLY, true, 1, false> : tc::score_tc_lse_kernel<NPOLY, true, 2, false>)
                          : (d64 ? tc::score_tc_lse_kernel<NPOLY, false, 1, false> : tc::score_tc_lse_kernel<NPOLY, false, 2, false>));
   if (ensure_dyn_smem(kern, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  launch_pdl(kern, grid, tc::LSE_THREADS, smem, s,
-      kmap, ta);
+  launch_pdl(kern, grid, tc::LSE_THREADS, smem, s, kmap, ta);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
 
 inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_tok, int max_win, cudaStream_t s) {
   (void)max_tok;
-  CUtensorMap kmap, qmap;
-  if (!tc::make_maps(pool, a.q, a.n_layers_sub, a.sum_win, a.n_q_heads, a.group, &kmap, &qmap)) return ACTKV_E_CUDA;
+  CUtensorMap kmap;
+  if (!tc::make_kmap(pool, &kmap)) return ACTKV_E_CUDA;
   tc::TcArgs ta;
   ta.a = a;
   ta.n_rg = (max_win * a.group + tc::MAX_ROWS - 1) / tc::MAX_ROWS;
@@ -204,8 +201,7 @@ inline int score_tc_launch_pool_g(const CUtensorMap& kmap, const CUtensorMap& qm
   // wait for ever for registers that a smaller allocation does not have, so the allocation is checked first.
   if (kernel_num_regs(kern) < tc::POOL_REGS_ENTRY) return ACTKV_E_CUDA;
   if (ensure_dyn_smem(kern, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  launch_pdl(kern, grid, tc::POOL_THREADS, smem, s,
-      kmap, qmap, ta);
+  launch_pdl(kern, grid, tc::POOL_THREADS, smem, s, kmap, qmap, ta);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -213,7 +209,8 @@ inline int score_tc_launch_pool_g(const CUtensorMap& kmap, const CUtensorMap& qm
 inline int score_tc_launch_score(ScoreArgs& a, const actkv_pool_t* pool, int max_tok, int max_win, cudaStream_t s,
                                  CompactWs* copy_ws) {
   CUtensorMap kmap, qmap;
-  if (!tc::make_maps(pool, a.q, a.n_layers_sub, a.sum_win, a.n_q_heads, a.group, &kmap, &qmap)) return ACTKV_E_CUDA;
+  if (!tc::make_kmap(pool, &kmap) || !tc::make_qmap(pool, a.q, a.n_layers_sub, a.sum_win, a.n_q_heads, a.group, &qmap))
+    return ACTKV_E_CUDA;
   tc::TcArgs ta;
   ta.a = a;
   const int Gp = tc::pow2_at_least(a.group);

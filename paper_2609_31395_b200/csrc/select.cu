@@ -91,10 +91,8 @@ static int select_launch_n(const float* score, const int32_t* tok_indptr, int32_
                            uint32_t* keep_mask, actkv_tie_t* tie_report, int32_t* status, cudaStream_t s) {
   const size_t smem = resident_smem(BINS * 4, max_tok);
   if (ensure_dyn_smem(select_kernel<NT, BINS>, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  launch_pdl(select_kernel<NT, BINS>, (unsigned)units, NT, smem, s,
-      score, tok_indptr, sum_tok, budget, n_req, keep_indptr, sel_idx,
-                                                            sel_stride, keep_mask, tie_report,
-                                                            (int32_t)((smem - BINS * 4) / 4), status);
+  launch_pdl(select_kernel<NT, BINS>, (unsigned)units, NT, smem, s, score, tok_indptr, sum_tok, budget, n_req, keep_indptr,
+             sel_idx, sel_stride, keep_mask, tie_report, (int32_t)((smem - BINS * 4) / 4), status);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -157,8 +155,7 @@ int actkv_select(const float* score, const int32_t* tok_indptr, int32_t sum_tok,
 int actkv_keep_indptr(const int32_t* seq_len, const int32_t* budget, int32_t n_req,
                       int32_t* keep_indptr, actkv_stream_t stream) {
   if (n_req < 0 || !keep_indptr || (n_req > 0 && (!seq_len || !budget))) return ACTKV_E_INVALID;
-  actkv::launch_pdl(actkv::keep_indptr_kernel, 1, 32, 0, (cudaStream_t)stream,
-      seq_len, budget, n_req, keep_indptr);
+  actkv::launch_pdl(actkv::keep_indptr_kernel, 1, 32, 0, (cudaStream_t)stream, seq_len, budget, n_req, keep_indptr);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
