@@ -743,7 +743,8 @@ extern "C" {
 
 size_t actkv_budget_workspace_bytes(int32_t n_rows, int32_t n_req, int32_t hist_cap) {
   if (n_rows < 0 || n_req < 0 || hist_cap < 0) return 0;
-  // new confidences + one pooled sequence of at most hist_cap values per request
+  // one pooled sequence of at most hist_cap values per request, behind 4 bytes per row that no kernel uses (the confidences go
+  // straight into the history; callers have sized their workspaces by this figure)
   return actkv::align_up((size_t)n_rows * 4, 256) + actkv::align_up((size_t)n_req * hist_cap * 4, 256);
 }
 

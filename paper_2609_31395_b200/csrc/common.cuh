@@ -37,8 +37,8 @@ __device__ __forceinline__ bool status_set(const int32_t* status) {
   return status != nullptr && *((const volatile int32_t*)status) != 0;
 }
 
-// Programmatic dependent launch.  A step is a chain of kernels of which many take a few microseconds; every one of them is
-// launched while its predecessor on the stream still runs and begins here: it waits until that one has finished and its
+// Programmatic dependent launch.  A step is a chain of kernels of which many take a few microseconds; every one of them (but
+// the in-place copy, compact_inplace.cu) is launched while its predecessor on the stream still runs and begins here: it waits until that one has finished and its
 // writes are visible (and has, by the same rule, all kernels before it behind it), then allows the next launch.  What
 // overlaps is the launch itself, 1 to 2.5 us a kernel: a step of one 4K request (9 kernels) 50.9 -> 37.9 us, of 16 requests of
 // 2K 84.3 -> 71.7, the monitor's two kernels 24.5 -> 20.5, a region pass over 16 requests 677 -> 671.

@@ -1,6 +1,6 @@
 // actkv_score: host entry point and path selection.
-//   tensor-core path (score_tc.cuh): window x group rows >= 64 (any row count for the streaming update),
-//   page 16, head_dim 128, packed pool;
+//   tensor-core path (score_tc.cuh): window x group rows >= 64 (any row count for the streaming update), pages of 16 to 128
+//   tokens, head_dim 64 or 128, any strides TMA takes (score_tc_supported);
 //   warp-level mma path (score_mma.cuh): everything else.
 // actkv_score_accumulate (streaming, Algorithm 3 per decode step) runs the pooled-score pass alone against
 // the supplied LSE and folds its result into the running mean held in the score array.
@@ -21,8 +21,9 @@ static ScoreWsLayout score_ws_layout(int32_t n_kv_heads, int32_t n_req, int32_t 
   const int G = n_q_heads / (n_kv_heads > 0 ? n_kv_heads : 1);
   l.rows_max = max_win * G;
   // Chunks per unit of a launch over `units` units: enough for LSE_ITEMS work items of at least
-  // LSE_CHUNK_LONG keys, or for LSE_ITEMS_MIN items of at least LSE_CHUNK keys when that leaves SMs idle.  units x n_chunks <= LSE_ITEMS + 2 units, and that bound grows with the unit count,
-  // so a workspace sized for a layer range also serves every call on fewer layers.
+  // LSE_CHUNK_LONG keys, or for LSE_ITEMS_MIN items of at least LSE_CHUNK keys when that leaves SMs idle.
+  // units x n_chunks <= LSE_ITEMS + 2 units, and that bound grows with the unit count, so a workspace sized for a layer range
+  // also serves every call on fewer layers.
   const int64_t units = (int64_t)nls * n_kv_heads * n_req;
   const int64_t by_len = max_tok > 0 ? (max_tok + LSE_CHUNK - 1) / LSE_CHUNK : 1;
   const int64_t by_len_long = max_tok > 0 ? (max_tok + LSE_CHUNK_LONG - 1) / LSE_CHUNK_LONG : 1;

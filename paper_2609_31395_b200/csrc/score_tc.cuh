@@ -132,12 +132,18 @@ inline void apply_hook(TcArgs& ta) {
 
 }  // namespace tc
 
-// The tensor-core path takes: pages of 16, 32, 64 or 128 tokens, head_dim 128 or 64, slot-major or head-major pages (any strides that are
-// multiples of 16 bytes), 128-byte aligned
-// base, group size <= 32 (padded to a power of two in the pooled-score pass), min_rows <= window x group rows <= 4096 (a CTA handles up to 512;
-// more are taken in groups of 512 rows), positive softmax scale.
-// The full score (LSE + pooled pass) takes it from 64 rows up; the streaming update, which runs the
-// pooled pass alone and is bound by the K reads, from a single row.
+// The tensor-core path takes: pages of 16, 32, 64 or 128 tokens, head_dim 128 or 64, slot-major or head-major pages (any
+// strides that are multiples of 16 bytes), 128-byte aligned base, group size <= 32 (padded to a power of two in the
+// pooled-score pass), min_rows <= window x group rows <= 4096 (a CTA handles up to 512; more are taken in groups of 512
+// rows), positive softmax scale.
+// The full score (LSE + pooled pass) takes it from 64 rows up; the streaming update, which runs the pooled pass alone and is
+// bound by the K reads, from a single row.  The two families, us, 4 layers x 8 heads, 8 requests of 9000 keys, head_dim 128,
+// group 4 (mma.sync beyond 48 rows on a pool 16 bytes off the 128-byte boundary, which costs it up to a quarter):
+//   rows             16         32         48         64         96
+//   LSE, mma / tc    118 / -    135 / -    159 / -    206 / 163  356 / 164
+//   pooled, mma / tc 107 / 119  131 / 121  163 / 121  212 / 122  367 / 127
+// so the LSE passes meet around 48 rows, and one line for both passes is late for the pooled one.  head_dim 64, group 8, 8
+// layers: LSE 170 at 48 rows, 204 / 228 at 64, 337 / 230 at 96.
 inline bool score_tc_supported(const actkv_pool_t* p, int G, int max_win, float sm_scale, const void* q,
                                int min_rows = 64) {
   if (p->page_size != 16 && p->page_size != 32 && p->page_size != 64 && p->page_size != 128) return false;

@@ -50,11 +50,11 @@ constexpr uint32_t POOL_FIXED = MAX_ROWS * 4 + sizeof(PoolBarriers);
 // and fewer shared-memory loads.  The three parts carry all 24 bits.
 // Only differences within a group go through the tensor core, and before the queries do: it rounds its sums towards zero.
 // With the whole LSE in it the scores were 2e-7 to 3e-7 too large on average (40 random shapes against float64; without the
-// contraction and as it is now 2e-8 to 4e-8; 2-norm error at head_dim 64 1.9e-7, 1.5e-7 without, 1.2e-7 now).
+// contraction and as it is now 2e-8 to 4e-8; 2-norm error at head_dim 64 1.9e-7, 1.5e-7 without, 1.4e-7 now).
 // Both forms run into the power cap (32768 keys, 256 rows: 985-998 W at 1.04 GHz); this one saves issue slots and their
 // energy for one more MMA step in nine: head_dim 64, group 8, windows of 24-64 tokens, 8 layers of 4 x 11000 keys 226 -> 174 us;
-// as a whole step, 36 layers of 32768 keys 1865 us without it and 1877 with it at 256 rows, host buffers at head_dim 64 2322 and
-// 2202.
+// whole steps, 36 layers of 32768 keys, 256 rows 1907 -> 1869 us, host buffers at head_dim 64 2322 -> 2205.  (Short launches
+// at head_dim 128, which the cap does not reach, are 1-4 % slower with it: 8 layers of 4 x 16000 keys, 256 rows 123 -> 127 us.)
 // Groups for which it is done (padded to a power of two): with one or two heads there is a multiply-add per column or two all the
 // same, and the values of ref would take the registers of the columns (2 heads: 536 us where the plain form takes 275, 8 layers of
 // 4 x 16000 keys, 8 heads); with 32 the plain form is the faster one (120 and 109 us).

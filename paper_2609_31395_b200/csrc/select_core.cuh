@@ -181,8 +181,8 @@ inline size_t resident_smem(size_t fixed, int64_t max_tok) {
   return want < SEL_SMEM_MAX ? want : SEL_SMEM_MAX;
 }
 
-// Threads per unit for units of up to max_tok keys: all 1024 for few units, where the sweeps are the latency; 256 and 512
-// while several such CTAs fill an SM and there are enough units to do so.  Keep-score update + TopK, against 1024 threads
+// Threads per unit for units of up to max_tok keys: 1024 where the sweeps are the latency, that is for long units and for few
+// of them; 256 and 512 where several such CTAs fill an SM; 256 for units too short to occupy more, however few.  Keep-score update + TopK, against 1024 threads
 // throughout: 2048 units of 1500 keys 48 / 119 us, 1024 of 3000 40 / 75, 1024 of 6000 68 / 107, 1024 of 16000 154 / 183,
 // 200 of 20000 57 / 66; 64 units of 3000 keys 17 us with 256 threads, 13 with 1024.
 inline int select_threads(int64_t units, int64_t max_tok) {
