@@ -644,16 +644,16 @@ __global__ void __launch_bounds__(TR_NT) trend_kernel(
       __syncthreads();
     }
     const float qv = okey_inv(s_prefix);
-    // R = values <= q in time order; slope in float64 against their positions 0 .. n - 1, whose mean (n - 1) / 2 and sum
-    // of squared deviations n (n^2 - 1) / 12 are known
+    // R = values <= q in time order; least-squares slope in float64 against their positions 0 .. n - 1, whose mean (n - 1) / 2 and
+    // sum of squared deviations n (n^2 - 1) / 12 are known.  The deviations of the positions add up to nothing, so the values
+    // themselves are summed: a product of a half-integer and a float is exact, and so are the sums of some ten thousand of them.
+    // A slope that is zero comes out as zero, whatever the order (the budget follows its sign; with the values' deviations from their
+    // rounded mean it was noise of either sign).
     int n = 0;
-    double sy = 0.0;
-    for (int m = tid; m < M; m += TR_NT)
-      if (Rp[m] <= qv) { sy += (double)Rp[m]; ++n; }
-    sy = block_reduce_sum(sy, s_red);
+    for (int m = tid; m < M; m += TR_NT) n += Rp[m] <= qv ? 1 : 0;
     n = (int)block_reduce_sum((double)n, s_red);
     if (n >= 2) {
-      const double xm = (double)(n - 1) * 0.5, ym = sy / (double)n;
+      const double xm = (double)(n - 1) * 0.5;
       double sxy = 0.0;
       int before = 0;                                   // values of R in earlier rounds of TR_NT
       for (int m0 = 0; m0 < M; m0 += TR_NT) {
@@ -668,10 +668,11 @@ __global__ void __launch_bounds__(TR_NT) trend_kernel(
           if (w < warp) i += (int)s_warp[w];
           before += (int)s_warp[w];
         }
-        if (in) sxy += ((double)i - xm) * ((double)Rp[m] - ym);
+        if (in) sxy += ((double)i - xm) * (double)Rp[m];
       }
       sxy = block_reduce_sum(sxy, s_red);
-      alpha = sxy / ((double)n * ((double)n * (double)n - 1.0) / 12.0);
+      // (infinite values have no slope)
+      alpha = fabs(sxy) < (double)INFINITY ? sxy / ((double)n * ((double)n * (double)n - 1.0) / 12.0) : (double)NAN;
     }
   }
   if (tid == 0) {

@@ -62,3 +62,29 @@ def test_trend(w, s, length):
     tok = torch.zeros(3, dtype=torch.int32, device=DEV)
     _compare(torch.zeros((0, 16), device=DEV), tok, hist, torch.tensor([length, max(0, length - 5)], dtype=torch.int32),
              torch.tensor([512, 700], dtype=torch.int32), params)
+
+
+@pytest.mark.parametrize("n", [3, 5, 64, 255, 256, 257, 999, 4000])
+def test_a_slope_of_zero_is_zero(n):
+    """Histories that read the same backwards: the slope is 0 and the budgets stay.  One with an infinite confidence has none."""
+    R = 9
+    params = B.BudgetParams.paper_defaults()
+    params.w = params.s = 1
+    params.b_percent = 100.0
+    g = torch.Generator().manual_seed(n)
+    hist = 1.0 + 8.0 * torch.rand((R, n), generator=g)
+    hist[0] = 4.0
+    hist[0, n // 2] = 4.25                                 # (an even n: not symmetric, falls or rises)
+    hist[1] = (hist[1] * 4).round() / 4
+    hist[1:] = torch.where(torch.arange(n) < (n + 1) // 2, hist[1:], hist[1:].flip(1))
+    hist[8, 0] = float("inf")
+    i32 = lambda v: torch.full((R,), v, dtype=torch.int32, device=DEV)  # noqa: E731
+    out, slope, status = i32(0), torch.full((R,), 7.0, dtype=torch.float64, device=DEV), torch.zeros(4, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.actkv_budget_workspace_bytes(0, R, n), dtype=torch.uint8, device=DEV)
+    B.actkv_budget(None, None, 0, 16, hist.to(DEV), i32(n), n, params, None, i32(512), out, slope, R, ws, status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist()[0] == 0
+    slope, out = slope.cpu(), out.cpu()
+    zero = slice(0, 8) if n % 2 else slice(1, 8)
+    assert (slope[zero] == 0).all() and (out[zero] == 512).all()
+    assert torch.isnan(slope[8]) and out[8] == 512
