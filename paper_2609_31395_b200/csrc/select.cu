@@ -100,6 +100,9 @@ static int select_launch_n(const float* score, const int32_t* tok_indptr, int32_
 int select_launch(const float* score, const int32_t* tok_indptr, int32_t sum_tok, int32_t max_tok, const int32_t* budget,
                   int32_t n_outer, int32_t n_req, const int32_t* keep_indptr, int32_t* sel_idx, int64_t sel_stride,
                   uint32_t* keep_mask, actkv_tie_t* tie_report, int32_t* status, cudaStream_t stream) {
+  if (n_outer < 0 || n_req < 0 || sum_tok < 0 || sel_stride < 0) return ACTKV_E_INVALID;
+  if (n_outer == 0 || n_req == 0) return ACTKV_OK;
+  if (!score || !tok_indptr || !budget || !keep_indptr || !sel_idx) return ACTKV_E_INVALID;
   const int64_t units = (int64_t)n_outer * n_req;
   if (units > 0x7fffffffLL) return ACTKV_E_INVALID;
   const int nt = select_threads(units, max_tok);
@@ -144,9 +147,6 @@ int actkv_select(const float* score, const int32_t* tok_indptr, int32_t sum_tok,
                  uint32_t* keep_mask, actkv_tie_t* tie_report, void* ws, size_t ws_bytes,
                  int32_t* status, actkv_stream_t stream) {
   (void)ws; (void)ws_bytes;
-  if (n_outer < 0 || n_req < 0 || sum_tok < 0 || sel_stride < 0) return ACTKV_E_INVALID;
-  if (n_outer == 0 || n_req == 0) return ACTKV_OK;
-  if (!score || !tok_indptr || !budget || !keep_indptr || !sel_idx) return ACTKV_E_INVALID;
   // (no unit is longer than all of them together)
   return actkv::select_launch(score, tok_indptr, sum_tok, sum_tok, budget, n_outer, n_req, keep_indptr, sel_idx, sel_stride,
                               keep_mask, tie_report, status, (cudaStream_t)stream);

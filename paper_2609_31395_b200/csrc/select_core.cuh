@@ -191,7 +191,7 @@ inline int select_threads(int64_t units, int64_t max_tok) {
   return 1024;
 }
 
-// Launches actkv_select's kernel with a bound on the unit lengths (select.cu).
+// actkv_select with a bound on the unit lengths: checks the arguments and launches the kernel (select.cu).
 int select_launch(const float* score, const int32_t* tok_indptr, int32_t sum_tok, int32_t max_tok, const int32_t* budget,
                   int32_t n_outer, int32_t n_req, const int32_t* keep_indptr, int32_t* sel_idx, int64_t sel_stride,
                   uint32_t* keep_mask, actkv_tie_t* tie_report, int32_t* status, cudaStream_t stream);
