@@ -47,17 +47,17 @@ namespace tc {
 constexpr int LSE_NPOLY = 1;                     // columns of every 8 whose exp2 is the polynomial
 constexpr float EXP2_ROUND = 12582912.f;         // 1.5 * 2^23: adding it rounds to the nearest integer
 
-// 2^(v c - e) for an integer e; base = EXP2_ROUND - e.  2^(j - e) is multiplied in, not added to the exponent field of p:
+// 2^(v c - e) for an integer e; base = EXP2_ROUND + 127 - e.  2^(j - e) is multiplied in, not added to the exponent field of p:
 // beyond |v c| = 2^22, where f leaves its interval, and for infinite and NaN logits the product is then as small as it has to be,
 // or larger than LSE_BIG, or NaN, and the caller takes the general form.
 __device__ __forceinline__ float exp2_poly(float v, float c, float base) {
-  const float t = fmaf(v, c, base);                                // j - e = round(v c - e) in the low mantissa bits
+  const float t = fmaf(v, c, base);                                // j - e + 127, j = round(v c): the exponent field, in the low bits
   const float f = fmaf(v, c, base - t);                            // v c - j
   float p = fmaf(0.0551716648042202f, f, 0.2426111251115799f);
   p = fmaf(p, f, 0.6932609677314758f);
   p = fmaf(p, f, 0.9999280571937561f);
-  const float k = fminf(fmaxf(t, EXP2_ROUND - 126.f), EXP2_ROUND + 126.f);
-  return p * __int_as_float((__float_as_int(k) << 23) + 0x3f800000);
+  const float k = fminf(fmaxf(t, EXP2_ROUND + 1.f), EXP2_ROUND + 253.f);
+  return p * __int_as_float(__float_as_int(k) << 23);
 }
 
 // 32 logits of one row, all visible, against the row's reference e (finite, below LSE_REF_MAX): returns
@@ -66,7 +66,7 @@ __device__ __forceinline__ float exp2_poly(float v, float c, float base) {
 template <int NPOLY>
 __device__ __forceinline__ float lse_fast32(const float* v, float c, float neg_e) {
   float s[2] = {0.f, 0.f};
-  const float base = EXP2_ROUND + neg_e;
+  const float base = EXP2_ROUND + 127.f + neg_e;
 #pragma unroll
   for (int g8 = 0; g8 < 4; ++g8) {
 #pragma unroll
