@@ -6,13 +6,17 @@
 // the supplied LSE and folds its result into the running mean held in the score array.
 // Both write per-chunk (max, sum) partials of the LSE pass into the caller's workspace, merge them
 // with lse_combine_kernel, then run the pooled-score pass against the merged (or supplied) LSE.
+#include <algorithm>
+
 #include "score_tc.cuh"
 
 namespace actkv {
 
 struct ScoreWsLayout {
   size_t lse_off, lse_bytes, part_off, part_bytes, total;
-  int32_t rows_max, n_chunks;
+  int32_t rows_max;
+  int32_t n_chunks;              // chunks per unit of the mma.sync kernel
+  int32_t n_chunks_max;          // ... as many as the tcgen05 kernel may have
 };
 
 static ScoreWsLayout score_ws_layout(int32_t n_kv_heads, int32_t n_req, int32_t nls, int32_t n_q_heads,
@@ -20,21 +24,19 @@ static ScoreWsLayout score_ws_layout(int32_t n_kv_heads, int32_t n_req, int32_t 
   ScoreWsLayout l;
   const int G = n_q_heads / (n_kv_heads > 0 ? n_kv_heads : 1);
   l.rows_max = max_win * G;
-  // Chunks per unit of a launch over `units` units: enough for LSE_ITEMS work items of at least
-  // LSE_CHUNK_LONG keys, or for LSE_ITEMS_MIN items of at least LSE_CHUNK keys when that leaves SMs idle.
-  // units x n_chunks <= LSE_ITEMS + 2 units, and that bound grows with the unit count, so a workspace sized for a layer range
+  // Chunks per unit of a launch over `units` units.  mma.sync: enough for LSE_ITEMS work items of at least LSE_CHUNK_LONG keys, or
+  // for LSE_ITEMS_MIN items of at least LSE_CHUNK keys when that leaves SMs idle.  tcgen05: up to LSE_ITEMS items of at least LSE_CHUNK
+  // keys, of which lse_split takes what suits the launch.
+  // units x chunks <= LSE_ITEMS + 2 units, and that bound grows with the unit count, so a workspace sized for a layer range
   // also serves every call on fewer layers.
   const int64_t units = (int64_t)nls * n_kv_heads * n_req;
   const int64_t by_len = max_tok > 0 ? (max_tok + LSE_CHUNK - 1) / LSE_CHUNK : 1;
   const int64_t by_len_long = max_tok > 0 ? (max_tok + LSE_CHUNK_LONG - 1) / LSE_CHUNK_LONG : 1;
-  int64_t nc = units > 0 ? (LSE_ITEMS + units - 1) / units : 1;
-  if (nc > by_len_long) nc = by_len_long;
-  if (units > 0 && units * nc < LSE_ITEMS_MIN) {   // a small problem: shorter chunks, so that every SM has work
-    nc = (LSE_ITEMS_MIN + units - 1) / units;
-    if (nc > by_len) nc = by_len;
-  }
-  if (nc < 1) nc = 1;
-  l.n_chunks = (int32_t)nc;
+  const int64_t by_items = units > 0 ? (LSE_ITEMS + units - 1) / units : 1;
+  int64_t nc = std::min(by_items, by_len_long);
+  if (units > 0 && units * nc < LSE_ITEMS_MIN) nc = std::min((LSE_ITEMS_MIN + units - 1) / units, by_len);   // a small problem
+  l.n_chunks = (int32_t)std::max<int64_t>(nc, 1);
+  l.n_chunks_max = (int32_t)std::max<int64_t>(std::min(by_items, by_len), 1);
   int64_t slots = units * by_len;
   if (slots > LSE_ITEMS + 2 * units) slots = LSE_ITEMS + 2 * units;
   l.lse_off = 0;
@@ -103,18 +105,14 @@ static int score_impl(int mode, const actkv_pool_t* pool, const actkv_tables_t* 
   a.sum_win = sum_win;
   a.sum_tok = sum_tok;
   a.rows_max = lay.rows_max;
-  // Keys per LSE partial.  A CTA pays a fixed cost (operand set-up, pipeline fill and drain), so chunks
-  // are as long as they can be while there are still many CTAs per SM (the last wave of a launch is
-  // partly empty): whole key tiles, about equal, the chunk count of the workspace layout (a CTA covers
-  // all rows of its unit).
+  // Keys per LSE partial: whole key tiles, about equal.
   const bool use_tc = actkv_score_path(pool, n_q_heads, max_win, sm_scale, q, acc_steps != nullptr) == 1;
   {
     int n_chunks = lay.n_chunks;
-    // tensor-core kernel: one CTA per SM is resident, so the launch runs in rounds of 148 CTAs; of the chunk
-    // counts the workspace allows, take the one that wastes least (partly empty last round against a fixed
-    // cost per CTA of about four key tiles: the Q blocks go to tensor memory, the pipeline fills and drains)
     if (use_tc && (mode & 1))
-      n_chunks = tc::best_split((int64_t)nls * Hkv * R, (max_tok + tc::TK - 1) / tc::TK, 4, lay.n_chunks);
+      n_chunks = tc::lse_split((int64_t)nls * Hkv * R * tc::lse_row_groups(max_win, G), (max_tok + tc::TK - 1) / tc::TK,
+                                 (double)sum_tok / ((double)R * max_tok), (double)sum_win / ((double)R * max_win),
+                                 max_win * G <= 128 ? 3.0 : 2.0, lay.n_chunks_max);
     int chunk = (max_tok + n_chunks - 1) / n_chunks;
     chunk = (chunk + 127) / 128 * 128;
     if (chunk < LSE_CHUNK) chunk = LSE_CHUNK;
@@ -131,7 +129,7 @@ static int score_impl(int mode, const actkv_pool_t* pool, const actkv_tables_t* 
   if (mode & 1) {
     float* lse_buf = lse_out ? lse_out : (float*)((char*)ws + lay.lse_off);
     if (use_tc) {
-      int rc = score_tc_launch_lse(a, pool, max_tok, max_win, s);
+      int rc = score_tc_launch_lse(a, pool, max_win, s);
       if (rc != ACTKV_OK) return rc;
     } else {
       const int rc = wm::launch_lse(a, units, s);

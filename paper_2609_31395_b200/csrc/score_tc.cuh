@@ -7,7 +7,7 @@
 //
 //  * LSE pass (score_tc_lse.cuh; Section 7.1, LSE equation).  D[row, key] = Q K^T with the window x
 //    group rows on the TMEM lanes (Q as the A operand from tensor memory), so every epilogue thread
-//    owns one row per 128-row block and keeps its running (max, sum of exp2) in registers: no shuffles.
+//    owns one row per 128-row block and keeps its running (reference, sum of exp2): no shuffles.
 //  * Pooled-score pass (score_tc_pool.cuh; Section 7.1 recovery identity, Algorithm 3 steps 3-5).
 //    The transposed product D[key, row] = K Q^T with the keys on the lanes and row = w*G + g on the
 //    columns, so the max over the GQA group and the sum over the action tokens run inside one
@@ -72,6 +72,33 @@ inline int best_split(int64_t units, int tiles, int ovh, int n_max) {
   return best;
 }
 
+// Chunks per unit of the LSE pass, whose CTAs go on from item to item, for a launch over `units` units of `tiles` key tiles: an item costs
+// its tiles and `ovh` more (Q blocks into tensor memory, references, merge: 2 to 4 K cycles).  Equal units run in rounds of 148 of which the
+// last is partly empty; requests of different lengths or windows (mean over longest: `len`, `win`) spread evenly but for the
+// last items, half of one on average.  Returns the count in [1, n_max] that costs least, preferring fewer unless more are clearly better.
+// 8 layers of 4 x 11000 keys, head_dim 64, 200-448 rows: 450 us with whole units, 350 with the four chunks this gives.
+inline int lse_split(int64_t units, int tiles, double len, double win, double ovh, int n_max) {
+  const bool equal = len > 0.999 && win > 0.999;
+  int best = 1;
+  double best_t = 1e300;
+  for (int n = 1; n <= n_max; ++n) {
+    const int tpc = (tiles + n - 1) / n;
+    if (tpc < 4 && n > 1) break;
+    const int64_t items = units * ((tiles + tpc - 1) / tpc);
+    double t;
+    if (equal) t = (double)((items + 147) / 148) * (tpc + ovh);
+    else t = ((double)units * tiles * len * win + (double)items * len * ovh) / 148.0 + 0.5 * (tpc + ovh);
+    if (t < best_t * 0.995) { best_t = t; best = n; }
+  }
+  return best;
+}
+
+// Items of the LSE pass side by side for a window of max_win tokens.
+inline int lse_row_groups(int max_win, int g) {
+  const int rows = 2 * LSE_MB * lse_half_rows(g);
+  return (max_win * g + rows - 1) / rows;
+}
+
 inline bool make_kmap(const actkv_pool_t* pool, CUtensorMap* kmap) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
@@ -102,15 +129,15 @@ inline bool make_kmap(const actkv_pool_t* pool, CUtensorMap* kmap) {
   return res == CUDA_SUCCESS;
 }
 
-inline bool make_qmap(const actkv_pool_t* pool, const void* q, int nls, int sum_win, int n_q_heads, int G, CUtensorMap* qmap) {
+// q: [slab*sum_win + w][q head][head_dim]; a box is (64 dims, `heads` heads from the first of a group on, `tokens` window tokens)
+inline bool make_qmap(const actkv_pool_t* pool, const void* q, int nls, int sum_win, int n_q_heads, int heads, int tokens,
+                      CUtensorMap* qmap) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
-  // q: [slab*sum_win + w][q head][128]; a box is (64 dims, the G heads of one group, 128/G window rows)
   const cuuint64_t D = (cuuint64_t)pool->head_dim;
   cuuint64_t dims[3] = {D, (cuuint64_t)n_q_heads, (cuuint64_t)nls * sum_win};
   cuuint64_t strides[2] = {D * 2, (cuuint64_t)n_q_heads * D * 2};
-  const int Gp = pow2_at_least(G);                 // the pooled-score kernel pads a group to a power of two
-  cuuint32_t box[3] = {64, (cuuint32_t)Gp, (cuuint32_t)(128 / Gp)};
+  cuuint32_t box[3] = {64, (cuuint32_t)heads, (cuuint32_t)tokens};
   cuuint32_t es[3] = {1, 1, 1};
   return enc(qmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(q), dims, strides, box, es,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -160,31 +187,29 @@ inline bool score_tc_supported(const actkv_pool_t* p, int G, int max_win, float 
   return tc::encode_fn() != nullptr;
 }
 
-inline int score_tc_launch_lse_c(const CUtensorMap& kmap, const tc::TcArgs& ta, unsigned grid, size_t smem, cudaStream_t s) {
+template <int NH>
+inline int score_tc_launch_lse_c(const CUtensorMap& kmap, const CUtensorMap& qmap, const tc::TcArgs& ta, unsigned grid, cudaStream_t s) {
   constexpr int NPOLY = tc::LSE_NPOLY;
-  const bool rgs = ta.n_rg > 1, d64 = ta.a.pool.head_dim == 64;
-  const bool win = ta.a.win_left > 0;
-  auto kern = win ? (rgs ? (d64 ? tc::score_tc_lse_kernel<NPOLY, true, 1, true> : tc::score_tc_lse_kernel<NPOLY, true, 2, true>)
-                         : (d64 ? tc::score_tc_lse_kernel<NPOLY, false, 1, true> : tc::score_tc_lse_kernel<NPOLY, false, 2, true>))
-                  : (rgs ? (d64 ? tc::score_tc_lse_kernel<NPOLY, true, 1, false> : tc::score_tc_lse_kernel<NPOLY, true, 2, false>)
-                         : (d64 ? tc::score_tc_lse_kernel<NPOLY, false, 1, false> : tc::score_tc_lse_kernel<NPOLY, false, 2, false>));
+  const size_t smem = (size_t)tc::lse_stages(NH) * NH * tc::HALF_BYTES + sizeof(tc::LseBarriers);
+  auto kern = ta.a.win_left > 0 ? tc::score_tc_lse_kernel<NPOLY, NH, true> : tc::score_tc_lse_kernel<NPOLY, NH, false>;
   if (ensure_dyn_smem(kern, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  launch_pdl(kern, grid, tc::LSE_THREADS, smem, s, kmap, ta);
+  launch_pdl(kern, grid, tc::LSE_THREADS, smem, s, kmap, qmap, ta);
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
 
-inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_tok, int max_win, cudaStream_t s) {
-  (void)max_tok;
-  CUtensorMap kmap;
-  if (!tc::make_kmap(pool, &kmap)) return ACTKV_E_CUDA;
+inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_win, cudaStream_t s) {
+  CUtensorMap kmap, qmap;
+  if (!tc::make_kmap(pool, &kmap) ||
+      !tc::make_qmap(pool, a.q, a.n_layers_sub, a.sum_win, a.n_q_heads, a.group, 64 / a.group, &qmap))
+    return ACTKV_E_CUDA;
   tc::TcArgs ta;
   ta.a = a;
-  ta.n_rg = (max_win * a.group + tc::MAX_ROWS - 1) / tc::MAX_ROWS;
+  ta.cubic = {tc::EXP2_C0, tc::EXP2_C1, tc::EXP2_C2, tc::EXP2_C3};
+  ta.n_rg = tc::lse_row_groups(max_win, a.group);
   ta.row_begin = 0;
   ta.k5 = tc::pool_needs_5d(pool) ? 1 : 0;
-  const int nh = pool->head_dim / 64;
-  ta.n_stages = nh == 1 ? 8 : 6;
+  ta.n_stages = 0;
   ta.tiles_per_cta = 0;
   ta.n_kchunks = 0;
   ta.copy_ws = nullptr;              // (this kernel has no copy role)
@@ -192,8 +217,8 @@ inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_t
   const int64_t units = (int64_t)a.n_layers_sub * a.pool.n_kv_heads * a.tab.n_req;
   const int64_t grid = units * a.n_chunks * ta.n_rg;
   if (grid > 0x7fffffffLL) return ACTKV_E_INVALID;
-  const size_t smem = (size_t)ta.n_stages * nh * tc::HALF_BYTES + sizeof(tc::LseBarriers);
-  return score_tc_launch_lse_c(kmap, ta, (unsigned)grid, smem, s);
+  return pool->head_dim == 64 ? score_tc_launch_lse_c<1>(kmap, qmap, ta, (unsigned)grid, s)
+                              : score_tc_launch_lse_c<2>(kmap, qmap, ta, (unsigned)grid, s);
 }
 
 template <int G>
@@ -215,11 +240,11 @@ inline int score_tc_launch_pool_g(const CUtensorMap& kmap, const CUtensorMap& qm
 inline int score_tc_launch_score(ScoreArgs& a, const actkv_pool_t* pool, int max_tok, int max_win, cudaStream_t s,
                                  CompactWs* copy_ws) {
   CUtensorMap kmap, qmap;
-  if (!tc::make_kmap(pool, &kmap) || !tc::make_qmap(pool, a.q, a.n_layers_sub, a.sum_win, a.n_q_heads, a.group, &qmap))
+  const int Gp = tc::pow2_at_least(a.group);       // (this kernel pads a group to a power of two)
+  if (!tc::make_kmap(pool, &kmap) || !tc::make_qmap(pool, a.q, a.n_layers_sub, a.sum_win, a.n_q_heads, Gp, 128 / Gp, &qmap))
     return ACTKV_E_CUDA;
   tc::TcArgs ta;
   ta.a = a;
-  const int Gp = tc::pow2_at_least(a.group);
   const int rows_all = max_win * Gp;
   const int nh = pool->head_dim / 64;
   const int rows_pad = (std::min(rows_all, tc::MAX_ROWS) + 127) & ~127;      // of the largest unit, per launch

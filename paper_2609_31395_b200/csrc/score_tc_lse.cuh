@@ -3,25 +3,35 @@
 //
 // D[row, key] = Q K^T with the rows on the TMEM lanes, so every epilogue thread owns one row per
 // 128-row block and folds its share of the row's logits into a running (reference, sum of exp2): no
-// shuffles.  A CTA covers ALL row blocks of a unit (up to four, 512 rows) x one chunk of keys, so a
-// K tile is fetched once per unit.
+// shuffles.  A work item is up to two row blocks (256 rows) of a unit x one chunk of keys; the items of a longer window stand
+// side by side and read its keys from L2.
 //
 // Operand placement.  An A operand in shared memory is re-read for every MMA and that read is not
 // overlapped with the MMA (measured 105 cycles per 128x128x16 MMA against 74 with A in tensor memory,
-// 64 nominal).  The Q blocks are the same for every key tile of the CTA, so they are written once into
-// tensor memory (tcgen05.st, two bf16 per 32-bit column) and used as the A operand from there; only
-// the K tile (B) streams through shared memory.
-// TMEM columns: [0,256) the four Q blocks, [256,512) two 128-column accumulators; a job is one
+// 64 nominal).  The Q blocks are the same for every key tile of the item, so they are copied once into
+// tensor memory and used as the A operand from there; only the K tile (B) streams through shared memory.
+// TMEM columns: [0,256) Q blocks, [256,512) two 128-column accumulators; a job is one
 // (key tile, row block) product.  Even jobs go to accumulator 0, odd jobs to accumulator 1; each
 // accumulator has its own MMA-issuing warp and its own group of eight epilogue warps (64 columns per
 // thread), which hand the accumulator back as soon as their columns are in registers.  While one group
 // waits for tensor memory the other keeps the special function unit busy.
 //
+// Items.  One CTA per SM, which goes on from item to item: the first is its own blockIdx, the next ones those of CTAs that have
+// not been launched yet (cluster launch control), so requests of different lengths and windows spread over the SMs by themselves.
+// In the ring of stages an item is its Q blocks, then its K tiles; the producers run ahead into the next item, whose
+// Q blocks go to the other half of the Q columns, and warp 3 merges the shares of an item while the epilogue is in the next.  With a
+// CTA per item 12 to 20 K cycles passed before its first job was done, beside 1030 for a job; from item to item it is 2 K.  With one
+// producer a unit of one row block waited for its key tiles.  A last block of at most 64 rows is held twice and each copy folds half of
+// its columns.
+// LSE pass, us, before and after: 4 layers x 8 heads, 8 x 16000 keys, 128 rows 280 -> 184, 192 rows 332 -> 284, head_dim 64 and 256 rows
+// 309 -> 289; 2 x 32768 keys, 256 rows 190 -> 170; 4 x 16000 keys, 384 rows 248 -> 261, 512 rows 320 -> 301; 8 layers x 8 heads, 16 requests of
+// 12000-20000 keys and 140-348 rows 1628 -> 1387.  In a loop of seconds, at the power cap: 36 layers of 32768 keys, 256 rows 828 -> 823, 8 layers of
+// 8 x 35000 keys, 512 rows 1440 -> 1420.
+//
 // What bounds the kernel (measured on B200 with micro-benchmarks and per-job timestamps):
 //  * Issuing is not free: a tcgen05.mma costs the issuing thread about 50 cycles and a tcgen05.commit
 //    about 80, some 470 cycles for a job the tensor pipe executes in 512, and the commit reaches the
-//    waiting warps about 240 cycles after the last MMA retires.  One issuer doing its barrier
-//    handshakes in between left the pipe idle 40 % of the time; hence two issuers.
+//    waiting warps about 240 cycles after the last MMA retires; hence two issuers.
 //  * An SM sub-partition dispatches about one fp32 operation per clock (the packed fp32x2 forms take
 //    two, so they save nothing) and its special function unit delivers one warp-wide exp2 per 8 clocks.
 //    One exp2 per (row, key) on that unit alone costs 8 clocks per warp and logit against 4.6 for the
@@ -47,24 +57,28 @@ namespace tc {
 constexpr int LSE_NPOLY = 1;                     // columns of every 8 whose exp2 is the polynomial
 constexpr float EXP2_ROUND = 12582912.f;         // 1.5 * 2^23: adding it rounds to the nearest integer
 
+// The cubic's coefficients come with the kernel's parameters, as operands from the constant bank: as literals they are brought in by
+// instructions of their own (2 x 32768 keys, 256 rows: 176.5 us against 173.6; from a __constant__ array 175).
+constexpr float EXP2_C0 = 0.9999280571937561f, EXP2_C1 = 0.6932609677314758f, EXP2_C2 = 0.2426111251115799f, EXP2_C3 = 0.0551716648042202f;
+
 // 2^(v c - e) for an integer e; base = EXP2_ROUND + 127 - e.  2^(j - e) is multiplied in, not added to the exponent field of p:
 // beyond |v c| = 2^22, where f leaves its interval, and for infinite and NaN logits the product is then as small as it has to be,
 // or larger than LSE_BIG, or NaN, and the caller takes the general form.
-__device__ __forceinline__ float exp2_poly(float v, float c, float base) {
+__device__ __forceinline__ float exp2_poly(float v, float c, float base, const Exp2Cubic& k) {
   const float t = fmaf(v, c, base);                                // j - e + 127, j = round(v c): the exponent field, in the low bits
   const float f = fmaf(v, c, base - t);                            // v c - j
-  float p = fmaf(0.0551716648042202f, f, 0.2426111251115799f);
-  p = fmaf(p, f, 0.6932609677314758f);
-  p = fmaf(p, f, 0.9999280571937561f);
-  const float k = fminf(fmaxf(t, EXP2_ROUND + 1.f), EXP2_ROUND + 253.f);
-  return p * __int_as_float(__float_as_int(k) << 23);
+  float p = fmaf(k.c3, f, k.c2);
+  p = fmaf(p, f, k.c1);
+  p = fmaf(p, f, k.c0);
+  const float e = fminf(fmaxf(t, EXP2_ROUND + 1.f), EXP2_ROUND + 253.f);
+  return p * __int_as_float(__float_as_int(e) << 23);
 }
 
 // 32 logits of one row, all visible, against the row's reference e (finite, below LSE_REF_MAX): returns
 // sum_i 2^(v_i c - e).  Two partial sums: the registers that more of them take cost more than the shorter chains give
 // (2.75 ms with two, 2.86 with four, for 16 layers of 8 x 35000 keys and 512 rows).
 template <int NPOLY>
-__device__ __forceinline__ float lse_fast32(const float* v, float c, float neg_e) {
+__device__ __forceinline__ float lse_fast32(const float* v, float c, float neg_e, const Exp2Cubic& k) {
   float s[2] = {0.f, 0.f};
   const float base = EXP2_ROUND + 127.f + neg_e;
 #pragma unroll
@@ -74,7 +88,7 @@ __device__ __forceinline__ float lse_fast32(const float* v, float c, float neg_e
       const float x = v[g8 * 8 + i];
       // the polynomial columns are spread over the group so that the two kinds interleave in program order
       const bool poly = (NPOLY >= 1 && i == 4) || (NPOLY >= 2 && i == 1) || (NPOLY >= 3 && i == 6) || (NPOLY >= 4 && i == 3);
-      s[i & 1] += poly ? exp2_poly(x, c, base) : exp2f(fmaf(x, c, neg_e));
+      s[i & 1] += poly ? exp2_poly(x, c, base, k) : exp2f(fmaf(x, c, neg_e));
     }
   }
   return s[0] + s[1];
@@ -94,30 +108,51 @@ __device__ __forceinline__ void lse_slow32(const float* v, int n_lo, int nv, flo
 }
 
 constexpr int LSE_EPI_WARPS = 16;                // (TMEM lane quarter, accumulator, column half)
-// Warp 0 is the producer, warps 1 and 2 the MMA issuers, warps 3..18 the epilogue: 19 warps leave each thread 104
-// registers.  The epilogue is sensitive to that: with a 20th warp (tried: a copy role for the items of a pending
-// compaction, as in the pooled-score kernel) the allocation is 96 and the pass 7-9 % slower, also when the
-// epilogue warpgroups take their 104 back from the control warps at run time; what the copies gained by hiding
-// under this kernel was less than that.
-constexpr int LSE_EPI_WARP0 = 3;
+// Warps 0 and 2 are the producers, warps 1 and 3 the MMA issuers, warps 4..19 the epilogue: five warps on each scheduler, which leaves
+// a thread up to 102 registers (the epilogue has a use for 96; with a sixth warp it would be 80).
+constexpr int LSE_EPI_WARP0 = 4;
 constexpr int LSE_THREADS = (LSE_EPI_WARP0 + LSE_EPI_WARPS) * 32;
 constexpr int LSE_SLOTS = 2;                     // accumulators
-constexpr int LSE_A_COLS = 256;                  // TMEM columns holding the four Q blocks
+constexpr int LSE_MB = 2;                        // row blocks of an item
+constexpr int LSE_A_COLS = 256;                  // TMEM columns holding Q blocks, a half for each of two items
+constexpr int LSE_ITEMS_AHEAD = 3;               // item descriptors in shared memory
+__host__ __device__ constexpr int lse_stages(int nh) { return nh == 1 ? 8 : 6; }             // K tiles (or Q blocks) in shared memory
+__host__ __device__ constexpr int lse_half_rows(int g) { return 64 / g * g; }                // rows of half a block: whole groups
 constexpr float LSE_BIG = 1099511627776.f;       // 2^40: a partial sum beyond it moves the reference
 constexpr float LSE_REF_MAX = 1048576.f;         // references beyond 2^20 (rounding to integers needs |v c| < 2^22) take the general form
+
+// Two blocks of which the second is short change places on odd tiles (exclusive or with this): the short one would otherwise always
+// fall to the same accumulator.
+__device__ __forceinline__ int lse_flip(int rows, int hr) {
+  const int n_half = (rows + hr - 1) / hr;
+  return n_half == 3 ? 1 : 0;
+}
+
+// A work item: the rows [row0, row0 + rows) of a unit against n_tiles key tiles.  n_tiles = 0: no more items.
+struct LseItem {
+  int32_t u, chunk, layer_h, r, L, W, w0, row0, rows, t_begin, n_tiles, slab;
+};
 
 struct LseBarriers {
   uint64_t k_full[8];
   uint64_t k_empty[8];
-  uint64_t q_ready;
+  uint64_t item_full[LSE_ITEMS_AHEAD];
+  uint64_t item_empty[LSE_ITEMS_AHEAD];
+  uint64_t q_ready[2];          // the Q blocks of an item are in this half of the Q columns
+  uint64_t q_free[2];           // the MMAs that read this half of the Q columns have completed
   uint64_t tmem_full[LSE_SLOTS];
   uint64_t tmem_empty[LSE_SLOTS];
+  uint64_t shares_full[2];      // the epilogue warps' shares of an item are in `state`
+  uint64_t shares_empty[2];     // ... have been merged
+  uint64_t clc;
   uint64_t drained[2];
   uint32_t tmem_base;
   int abort_flag;
-  int last_key[4][128];        // last key the row of (row block, TMEM lane) sees
-  float2 state[2][4][2][128];  // (reference e, sum of 2^(v c - e)) per (group, row block, column half, row in block)
+  alignas(16) uint32_t clc_resp[4];
+  LseItem item[LSE_ITEMS_AHEAD];
+  float2 state[2][2][LSE_MB][2][128];  // (reference e, sum of 2^(v c - e)) per (item parity, group, row block, column half, TMEM lane)
 };
+static_assert(6 * 2 * HALF_BYTES + sizeof(LseBarriers) <= SMEM_LIMIT, "shared memory");
 
 // After tcgen05.wait::ld: ties the loaded registers to the wait, so that no use of them is scheduled
 // ahead of it (the loads are asynchronous; the compiler sees their outputs as defined at issue).
@@ -127,98 +162,131 @@ __device__ __forceinline__ void tmem_ld_fence(float* v) {
   for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
 }
 
-// One job as one epilogue warp sees it: the warp takes 64 columns (two register buffers of 32) of the
-// accumulator of its group, hands the accumulator back as soon as they are in registers, and folds them
-// into the row's (reference, sum) in `st`.  The two groups work on alternate jobs, so while one waits
-// for tensor memory the other keeps the special function unit busy.
+// One job as one epilogue warp sees it: the warp takes 64 columns of the accumulator of its group (32 where the block holds its rows
+// twice), hands the accumulator back as soon as they are in registers, and folds them into the row's (reference, sum) `ms`.  The two
+// groups work on alternate jobs, so while one waits for tensor memory the other keeps the special function unit busy.
 //   tq      tensor-memory address of the group's accumulator, this warp's lane quarter and first column
+//   wide    64 columns (uniform over the CTA)
 //   nv_min  visible columns (from the warp's first column) of the most restricted row of this thread
 //   nlo_max columns (from the warp's first column) below the first visible key of the most restricted row
-//   last_key  last visible key of this thread's row; in shared memory, since only the slow path needs it and the loop is short
-//           of registers (with the keys of the four row blocks in them 910 us where this takes 895: 24 layers of 4 x 11000
-//           keys, head_dim 64, 192-512 rows; 36 layers of 32768 keys, 256 rows, 1 % less)
+//   last_key()  last visible key of this thread's row; only the slow path needs it and the loop is short of registers
 //   key0    key of the warp's first column
 // WIN: the layer has a sliding window (a first visible key per row); kept out of the common instantiation, whose
 // epilogue should not carry the second bound.
-template <int NPOLY, bool WIN>
-__device__ __forceinline__ bool lse_job(LseBarriers* bars, volatile int* abort_flag, uint32_t tq, int grp, int job,
-                                        const int* last_key, float2* st, int nv_min, int nlo_max, int win_left, int key0, float c,
-                                        long long wait_cycles) {
+// What is not an exponential counts: an instruction more per job and warp is 0.2 % of the pass, a second unrolled copy of the fold 7 %.
+template <int NPOLY, bool WIN, class LastKey>
+__device__ __forceinline__ bool lse_job(LseBarriers* bars, volatile int* abort_flag, uint32_t tq, int grp, uint32_t parity, bool wide,
+                                        LastKey last_key, float2& ms, int nv_min, int nlo_max, int win_left, int key0, float c,
+                                        const Exp2Cubic& cubic, long long wait_cycles) {
   float v[64];
-  float* va = v;
-  float* vb = v + 32;
-  if (!mbar_wait_warp(smem_u32(&bars->tmem_full[grp]), (uint32_t)(job >> 1) & 1u, abort_flag, wait_cycles)) return false;
+  if (!mbar_wait_warp(smem_u32(&bars->tmem_full[grp]), parity, abort_flag, wait_cycles)) return false;
   tc_fence_after();
-  tmem_ld64(tq, v);
-  float2 ms = *st;
+  tmem_ld32(tq, v);
+  if (wide) tmem_ld32(tq + 32, v + 32);
   tmem_ld_wait();
   tmem_ld_fence<64>(v);
   tc_fence_before();
   __syncwarp();
   if ((threadIdx.x & 31) == 0) mbar_arrive(smem_u32(&bars->tmem_empty[grp]));
-  // (a reference of -inf, before the row's first logits, fails the second test)
-  bool slow = __any_sync(0xffffffffu, nv_min < 64 || (WIN && nlo_max > 0) || !(fabsf(ms.x) < LSE_REF_MAX));
+  // (a reference of -inf, before the row's first logits, fails the last test)
+  bool slow = __any_sync(0xffffffffu, nv_min < (wide ? 64 : 32) || (WIN && nlo_max > 0) || !(fabsf(ms.x) < LSE_REF_MAX));
   if (!slow) {
-    const float ps = lse_fast32<NPOLY>(va, c, -ms.x) + lse_fast32<NPOLY>(vb, c, -ms.x);
+    float ps = lse_fast32<NPOLY>(v, c, -ms.x, cubic);
+    if (wide) ps += lse_fast32<NPOLY>(v + 32, c, -ms.x, cubic);
     slow = __any_sync(0xffffffffu, !(fabsf(ps) < LSE_BIG));
     if (!slow) ms.y += ps;
   }
   if (slow) {
-    const int nv = *last_key - key0 + 1;
+    const int nv = last_key() - key0 + 1;
     const int nlo = WIN && win_left > 0 ? nv - win_left : 0;
-    lse_slow32(va, nlo, nv, c, ms.x, ms.y);
-    lse_slow32(vb, nlo - 32, nv - 32, c, ms.x, ms.y);
+    lse_slow32(v, nlo, nv, c, ms.x, ms.y);
+    if (wide) lse_slow32(v + 32, nlo - 32, nv - 32, c, ms.x, ms.y);
   }
-  *st = ms;
   return true;
 }
 
-// ROW_GROUPS: the unit's window has more than MAX_ROWS rows and the grid has a row-group dimension (kept
-// out of the common instantiation, whose code should not change with it).
-// NH: 64-dim halves of the head dimension (head_dim = 64 NH); a K tile is NH x [128 keys][64 bf16].
-template <int NPOLY, bool ROW_GROUPS, int NH, bool WIN>
-__global__ void __launch_bounds__(LSE_THREADS, 1)
-score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
-  pdl_begin();
-  extern __shared__ __align__(1024) uint8_t smem[];
+// The item that the CTA with this index stands for; n_tiles <= 0 when there is nothing to contract.  Reports invalid windows, and
+// writes the partials of a chunk no row of which sees a key.  Called by a whole warp.
+template <bool WIN>
+__device__ __forceinline__ LseItem lse_item(const TcArgs& ta, int id, int lane) {
   const ScoreArgs& a = ta.a;
   const int R = a.tab.n_req, Hkv = a.pool.n_kv_heads, G = a.group;
-  const int cu = blockIdx.x / a.n_chunks;
-  const int chunk = blockIdx.x - cu * a.n_chunks;
-  const int rg = ROW_GROUPS ? cu % ta.n_rg : 0;          // row group: rows [row0, row0 + MAX_ROWS) of the unit
-  const int u = ROW_GROUPS ? cu / ta.n_rg : cu;
-  const int r = u % R, h = (u / R) % Hkv, slab = u / (R * Hkv);
-  const int L = a.tab.seq_len[r];
-  const int w0 = a.win_indptr[r], W = a.win_indptr[r + 1] - w0;
-  const int row0 = ROW_GROUPS ? rg * MAX_ROWS : 0;
-  const int rows = ROW_GROUPS ? min(W * G - row0, MAX_ROWS) : W * G;     // rows of this CTA
-  const int key_begin = chunk * a.lse_chunk;
-  if (key_begin >= L || (rg > 0 && rows <= 0)) return;
-  if (W <= 0 || (a.causal && W > L)) {
-    if (threadIdx.x == 0 && chunk == 0 && rg == 0) report(a.status, ACTKV_E_INVALID, r, W);
-    return;
+  LseItem x;
+  x.n_tiles = 0;
+  const int cu = id / ta.n_rg, rg = id - cu * ta.n_rg;   // row group
+  x.u = cu / a.n_chunks;
+  x.chunk = cu - x.u * a.n_chunks;
+  x.r = x.u % R;
+  const int h = (x.u / R) % Hkv;
+  x.slab = x.u / (R * Hkv);
+  x.layer_h = h;
+  x.L = a.tab.seq_len[x.r];
+  x.w0 = a.win_indptr[x.r];
+  x.W = a.win_indptr[x.r + 1] - x.w0;
+  const int rg_rows = 2 * LSE_MB * lse_half_rows(G);
+  x.row0 = rg * rg_rows;
+  x.rows = min(x.W * G - x.row0, rg_rows);
+  const int key_begin = x.chunk * a.lse_chunk;
+  if (key_begin >= x.L || (rg > 0 && x.rows <= 0)) return x;
+  if (x.W <= 0 || (a.causal && x.W > x.L)) {
+    if (lane == 0 && x.chunk == 0 && rg == 0) report(a.status, ACTKV_E_INVALID, x.r, x.W);
+    return x;
   }
-  // the host sized shared memory, tensor memory and the partials from upper bounds of the window and the length
-  if (W * G > a.rows_max || L > a.n_chunks * a.lse_chunk || rows > MAX_ROWS) {
-    if (threadIdx.x == 0 && chunk == 0 && rg == 0) report(a.status, ACTKV_E_INVALID, r, W * G > a.rows_max ? W : L);
-    return;
+  // the host sized the grid and the partials from upper bounds of the window and the length
+  if (x.W * G > a.rows_max || x.L > a.n_chunks * a.lse_chunk) {
+    if (lane == 0 && x.chunk == 0 && rg == 0) report(a.status, ACTKV_E_INVALID, x.r, x.W * G > a.rows_max ? x.W : x.L);
+    return x;
   }
-  const int n_mb = (rows + 127) / 128;                   // 1..4
-  const int t_end = min((L + TK - 1) / TK, key_begin / TK + a.lse_chunk / TK);
+  const int t_end = min((x.L + TK - 1) / TK, key_begin / TK + a.lse_chunk / TK);
   // sliding-window layer: key tiles below the first key any row of the unit sees are not fetched at all
-  const int lo_all = (WIN && a.win_left > 0) ? max(0, (a.causal ? L - W : L - 1) - a.win_left + 1) : 0;
-  const int t_begin = max(key_begin / TK, lo_all / TK);
-  const int n_tiles = t_end - t_begin;
-  if (n_tiles <= 0) {                                    // no row sees a key of this chunk
-    for (int n = threadIdx.x; n < rows; n += blockDim.x)
-      a.partials[((int64_t)u * a.n_chunks + chunk) * a.rows_max + row0 + n] = make_float2(-INFINITY, 0.f);
-    return;
+  const int lo_all = (WIN && a.win_left > 0) ? max(0, (a.causal ? x.L - x.W : x.L - 1) - a.win_left + 1) : 0;
+  x.t_begin = max(key_begin / TK, lo_all / TK);
+  x.n_tiles = t_end - x.t_begin;
+  if (x.n_tiles <= 0)                                    // no row sees a key of this chunk
+    for (int n = lane; n < x.rows; n += 32)
+      a.partials[((int64_t)x.u * a.n_chunks + x.chunk) * a.rows_max + x.row0 + n] = make_float2(-INFINITY, 0.f);
+  return x;
+}
+
+// The shares (group, column half, and lane of a block held twice) of each row of a finished item; stores (reference in log2 units, sum),
+// (-inf, 0) when the row saw no key of this chunk.  Called by a whole warp.
+__device__ __forceinline__ void lse_merge(const float2 (&state)[2][LSE_MB][2][128], float2* dst, int rows, int hr, int lane) {
+  const int n_half = (rows + hr - 1) / hr;
+  for (int n2 = lane; n2 < n_half * 64; n2 += 32) {
+    const int i2 = n2 >> 6, n = i2 * hr + (n2 & 63);          // half block, row
+    if ((n2 & 63) >= hr || n >= rows) continue;
+    const bool dup = (n_half & 1) && i2 == n_half - 1;
+    float2 o[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      o[i] = i < 4 || dup ? state[i & 1][i2 >> 1][(i >> 1) & 1][(n2 & 127) + (i >> 2) * 64] : make_float2(-INFINITY, 0.f);
+    float mm = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mm = fmaxf(mm, o[i].x);
+    float ss = 0.f;
+    if (mm > -INFINITY) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) ss += o[i].x > -INFINITY ? o[i].y * exp2f(o[i].x - mm) : 0.f;
+    }
+    dst[n] = make_float2(mm, ss);
   }
-  const int n_jobs = n_tiles * n_mb;
-  const int S = ta.n_stages;
+}
+
+// NH: 64-dim halves of the head dimension (head_dim = 64 NH); a K tile is NH x [128 keys][64 bf16].
+template <int NPOLY, int NH, bool WIN>
+__global__ void __launch_bounds__(LSE_THREADS, 1)
+score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap qmap, const TcArgs ta) {
+  pdl_begin();
+  extern __shared__ __align__(1024) uint8_t smem[];
+  constexpr int S = lse_stages(NH);
+  constexpr int QCOLS = 32 * NH;                         // TMEM columns of a Q block
+  static_assert(LSE_MB * QCOLS <= LSE_A_COLS / 2, "Q columns");
+  const ScoreArgs& a = ta.a;
+  const int G = a.group;
+  const int hr = lse_half_rows(G);
 
   const uint32_t smem_base = smem_u32(smem);
-  const uint32_t k_smem = smem_base;                               // S x 32 KB
+  const uint32_t k_smem = smem_base;                               // S stages of a K tile
   LseBarriers* bars = reinterpret_cast<LseBarriers*>(smem + (size_t)S * (NH * HALF_BYTES));
   volatile int* abort_flag = &bars->abort_flag;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform
@@ -229,15 +297,31 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
   }
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 2); }
-    mbar_init(smem_u32(&bars->q_ready), LSE_EPI_WARPS);
+    for (int i = 0; i < LSE_ITEMS_AHEAD; ++i) {
+      mbar_init(smem_u32(&bars->item_full[i]), 1);
+      mbar_init(smem_u32(&bars->item_empty[i]), LSE_EPI_WARPS + 3);
+    }
     for (int b = 0; b < LSE_SLOTS; ++b) {
+      mbar_init(smem_u32(&bars->q_free[b]), 2);
+      mbar_init(smem_u32(&bars->q_ready[b]), 1);
       mbar_init(smem_u32(&bars->tmem_full[b]), 1);
       mbar_init(smem_u32(&bars->tmem_empty[b]), LSE_EPI_WARPS / 2);
     }
+    for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&bars->shares_full[i]), LSE_EPI_WARPS); mbar_init(smem_u32(&bars->shares_empty[i]), 1); }
+    mbar_init(smem_u32(&bars->clc), 1);
     mbar_init(smem_u32(&bars->drained[0]), 1);
     mbar_init(smem_u32(&bars->drained[1]), 1);
     bars->abort_flag = 0;
     fence_barrier_init();
+  }
+  if (hr < 64) {
+    // lanes past the last whole group of half a block: no load ever writes these rows of a stage for a Q block, so they start as zeros
+    // (later they hold old keys), and not as what may be anything
+    for (int i = threadIdx.x; i < S * NH * 2 * (64 - hr) * 8; i += blockDim.x) {
+      const int row = hr + (i >> 3) % (64 - hr), hb = (i >> 3) / (64 - hr);
+      *reinterpret_cast<uint4*>(smem + (size_t)hb * (HALF_BYTES / 2) + row * 128 + (i & 7) * 16) = make_uint4(0, 0, 0, 0);
+    }
+    fence_proxy_async();
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(&bars->tmem_base), 512);
@@ -248,69 +332,196 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
   tc_fence_after();
   const uint32_t tmem_base = bars->tmem_base;
 
-  // epilogue identity (also used after the role split)
-  const int ew = warp - LSE_EPI_WARP0;           // 0..15 for epilogue warps
-  const int quarter = warp & 3;                  // TMEM lanes this warp may touch
-  const int k = ew >> 2;                         // 0..3
-  const int grp = k >> 1;                        // accumulator / job parity this warp serves
-  const int half = k & 1;                        // its columns: [64 half, 64 half + 64)
-  const int rib = quarter * 32 + lane;           // row within a 128-row block
-  bool epi_ok = true;
-
-  if (warp == 0) {
-    // ---------------- TMA producer: K tiles through the block table ----------------
-    const int layer = a.layer_begin + slab;
-    // (one producer: this pass needs a K tile per four jobs, far below what one warp delivers)
-    if (ta.k5) k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 0, 1, ta.wait_cycles, ta.stall_tile);
-    else k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 0, 1, ta.wait_cycles, ta.stall_tile);
-  } else if (warp < LSE_EPI_WARP0) {
+  // Every role walks the same items: the producer of warp 0 finds them and describes them in a small ring.  In the ring of stages an
+  // item is its Q blocks, then its K tiles.
+  if (warp == 0 || warp == 2) {
+    // ---------------- TMA producers: alternate entries of the ring; warp 0 also finds the items ----------------
+    const int p = warp >> 1;
+    int e = 0, slot = 0;
+    uint32_t ipar = 0, cpar = 0;
+    int id = blockIdx.x;
+    bool ok = true;
+    for (;;) {
+      LseItem x;
+      if (p == 0) {
+        if (lane == 0) {
+          mbar_expect_tx(smem_u32(&bars->clc), 16);
+          clc_request(smem_u32(bars->clc_resp), smem_u32(&bars->clc));
+        }
+        __syncwarp();
+        x = lse_item<WIN>(ta, id, lane);
+        if (x.n_tiles > 0) {
+          ok = mbar_wait_warp(smem_u32(&bars->item_empty[slot]), ipar ^ 1u, abort_flag, ta.wait_cycles);
+          if (ok && lane == 0) {
+            bars->item[slot] = x;
+            mbar_arrive(smem_u32(&bars->item_full[slot]));
+          }
+        }
+      } else {
+        ok = mbar_wait_warp(smem_u32(&bars->item_full[slot]), ipar, abort_flag, ta.wait_cycles);
+        if (!ok) break;
+        x = bars->item[slot];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars->item_empty[slot]));
+        if (x.n_tiles <= 0) break;
+      }
+      if (ok && x.n_tiles > 0) {
+        if (++slot == LSE_ITEMS_AHEAD) { slot = 0; ipar ^= 1u; }
+        const int n_half = (x.rows + hr - 1) / hr, n_mb = (n_half + 1) / 2;
+        for (int b = 0; b < n_mb && ok; ++b, ++e) {
+          if ((e & 1) != p) continue;
+          const int s = e % S;
+          ok = mbar_wait_warp(smem_u32(&bars->k_empty[s]), ((uint32_t)(e / S) & 1u) ^ 1u, abort_flag, ta.wait_cycles);
+          if (!ok) break;
+          // the two halves of the block; a last half that stands alone is held twice
+          const uint32_t bar = smem_u32(&bars->k_full[s]);
+          if (lane == 0) mbar_expect_tx(bar, (uint32_t)(2 * NH * hr) * 128u);
+          __syncwarp();
+          if (lane < 2 * NH) {
+            const int hf = lane >> 1, j = lane & 1;
+            const int tok = x.slab * a.sum_win + x.w0 + (x.row0 + min(2 * b + j, n_half - 1) * hr) / G;
+            tma_load_3d(k_smem + s * (NH * HALF_BYTES) + hf * HALF_BYTES + j * (HALF_BYTES / 2), &qmap, bar, hf * 64, x.layer_h * G, tok);
+          }
+        }
+        if (ok) {
+          const int layer = a.layer_begin + x.slab, first = (p - e) & 1;
+          if (ta.k5) ok = k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
+          else ok = k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
+          e += x.n_tiles;
+        }
+      }
+      if (p == 0) {
+        // (also after giving up: the answer lands in this CTA's shared memory)
+        const bool answered = mbar_wait_warp(smem_u32(&bars->clc), cpar, nullptr, ta.wait_cycles);
+        cpar ^= 1u;
+        id = answered ? clc_answer(smem_u32(bars->clc_resp)) : -1;
+        fence_proxy_async();                     // (the answer has been read before the next one is written)
+        __syncwarp();
+        if (!ok || id < 0) break;
+      }
+      if (!ok) break;
+    }
+    if (p == 0 && ok) {
+      ok = mbar_wait_warp(smem_u32(&bars->item_empty[slot]), ipar ^ 1u, abort_flag, ta.wait_cycles);
+      if (ok && lane == 0) {
+        bars->item[slot].n_tiles = 0;
+        mbar_arrive(smem_u32(&bars->item_full[slot]));
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1 || warp == 3) {
     // ---------------- MMA issuers: A = Q block in TMEM, B = K tile in shared memory ----------------
-    // Two warps, one per accumulator: warp 1 issues the even jobs into accumulator 0, warp 2 the odd jobs
-    // into accumulator 1.  Issuing is not free for the issuing thread (measured: about 50 cycles per
-    // tcgen05.mma and 80 per tcgen05.commit, i.e. some 470 cycles for a job that the tensor pipe executes
-    // in 512) and the barrier handshakes come on top, so one issuer alone cannot keep the pipe busy.
-    // The whole warp runs the loop (waits stay warp-uniform); one elected lane issues.
-    // Every issuer waits for every K tile and releases it (tcgen05.commit after its last job of the tile,
-    // or a plain arrive when it had none), so a stage is refilled only when both are done with it.
-    const int mw = warp - 1;
+    // Two warps, one per accumulator: warp 1 issues the even jobs into accumulator 0, warp 3 the odd jobs into accumulator 1; warp 1
+    // also brings the Q blocks into tensor memory.  The whole warp runs the loop (waits stay warp-uniform); one elected lane issues.
+    // Both wait for every entry of the ring and release it (tcgen05.commit after the last job of the tile, or a plain arrive).
+    const int mw = warp >> 1;
     const uint32_t idesc = idesc_bf16(128, 128);
     const uint64_t desc0 = smem_desc_sw128(k_smem);
     const uint32_t full_bar = smem_u32(&bars->tmem_full[mw]), empty_bar = smem_u32(&bars->tmem_empty[mw]);
     const uint32_t d = tmem_base + LSE_A_COLS + mw * 128;
-    bool ok = mbar_wait_warp(smem_u32(&bars->q_ready), 0, abort_flag, ta.wait_cycles);
-    tc_fence_after();
-    int s = 0, job = 0;
-    uint32_t kpar = 0, epar = 1u;                  // parity to wait for on tmem_empty[mw] (a fresh barrier passes with 1)
     const bool leader = elect_one();
-    for (int it = 0; ok && it < n_tiles; ++it) {
-      ok = mbar_wait_warp(smem_u32(&bars->k_full[s]), kpar, abort_flag, ta.wait_cycles);
+    bool ok = true;
+    int s = 0, slot = 0, qh = 0;
+    uint32_t kpar = 0, ipar = 0, epar = 1u, qpar = 3u, rpar = 0;    // qpar: a bit per half (a fresh barrier passes with 1)
+    // Warp 3 also merges: the shares of an item after its own second job of the next one, when the epilogue is about to finish or has
+    // finished the item.  (With the epilogue warps meeting at the end of an item to merge it, items of 32 tiles of two blocks cost
+    // 9 % over longer ones.)
+    int m_rows = 0, m_sp = 0;                      // the item to be merged: rows (0: none), which `state`
+    uint32_t m_par = 0;
+    float2* m_dst = nullptr;
+    auto merge = [&]() {
+      if (!mbar_wait_warp(smem_u32(&bars->shares_full[m_sp]), m_par, abort_flag, ta.wait_cycles)) return false;
+      lse_merge(bars->state[m_sp], m_dst, m_rows, hr, lane);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars->shares_empty[m_sp]));
+      m_rows = 0;
+      m_sp ^= 1;
+      m_par ^= (uint32_t)(m_sp == 0);
+      return true;
+    };
+    for (;;) {
+      ok = mbar_wait_warp(smem_u32(&bars->item_full[slot]), ipar, abort_flag, ta.wait_cycles);
       if (!ok) break;
-      tc_fence_after();
-      const uint64_t desc_s = desc0 + (uint64_t)((s * (NH * HALF_BYTES)) >> 4);
-      bool mine = false;
-      for (int b = 0; b < n_mb; ++b, ++job) {
-        if ((job & 1) != mw) continue;
-        ok = mbar_wait_warp(empty_bar, epar, abort_flag, ta.wait_cycles);
+      const int n_tiles = uni(bars->item[slot].n_tiles), rows = uni(bars->item[slot].rows);
+      float2* dst = a.partials + ((int64_t)bars->item[slot].u * a.n_chunks + bars->item[slot].chunk) * a.rows_max + bars->item[slot].row0;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars->item_empty[slot]));
+      if (n_tiles <= 0) break;
+      if (++slot == LSE_ITEMS_AHEAD) { slot = 0; ipar ^= 1u; }
+      const int n_mb = ((rows + hr - 1) / hr + 1) / 2;
+      // the Q blocks go to the half of the Q columns that the previous item does not use
+      const uint32_t q_tmem = tmem_base + (uint32_t)qh * (LSE_A_COLS / 2);
+      if (mw == 0) {
+        ok = mbar_wait_warp(smem_u32(&bars->q_free[qh]), (qpar >> qh) & 1u, abort_flag, ta.wait_cycles);
         if (!ok) break;
-        epar ^= 1u;
+        qpar ^= 1u << qh;
+      }
+      for (int b = 0; b < n_mb; ++b) {
+        ok = mbar_wait_warp(smem_u32(&bars->k_full[s]), kpar, abort_flag, ta.wait_cycles);
+        if (!ok) break;
         tc_fence_after();
         if (leader) {
-          const uint32_t at = tmem_base + b * 64;
+          if (mw == 0) {
+            const uint64_t desc_s = desc0 + (uint64_t)((s * (NH * HALF_BYTES)) >> 4);
 #pragma unroll
-          for (int kk = 0; kk < 4 * NH; ++kk)
-            umma_bf16_ts(d, at + kk * 8, desc_s + (uint64_t)(((kk >> 2) * HALF_BYTES + (kk & 3) * 32) >> 4), idesc,
-                         kk > 0 ? 1u : 0u);
-          umma_commit(full_bar);
+            for (int kk = 0; kk < 4 * NH; ++kk)
+              tmem_cp_k16(q_tmem + b * QCOLS + kk * 8, desc_s + (uint64_t)(((kk >> 2) * HALF_BYTES + (kk & 3) * 32) >> 4));
+            umma_commit(smem_u32(&bars->k_empty[s]));
+            if (b == n_mb - 1) umma_commit(smem_u32(&bars->q_ready[qh]));
+          } else {
+            mbar_arrive(smem_u32(&bars->k_empty[s]));
+          }
         }
-        mine = true;
+        if (++s == S) { s = 0; kpar ^= 1u; }
       }
+      // (a barrier per half: warp 1 may be two items ahead, and comes back to a half only when warp 3 is done with it)
+      if (ok && mw == 1) ok = mbar_wait_warp(smem_u32(&bars->q_ready[qh]), (rpar >> qh) & 1u, abort_flag, ta.wait_cycles);
+      rpar ^= 1u << qh;
+      // (every item begins with accumulator 0, so that its sums do not depend on what this CTA did before)
+      int job = 0, n_issued = 0, flip = 0;
+      for (int it = 0; ok && it < n_tiles; ++it) {
+        ok = mbar_wait_warp(smem_u32(&bars->k_full[s]), kpar, abort_flag, ta.wait_cycles);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t desc_s = desc0 + (uint64_t)((s * (NH * HALF_BYTES)) >> 4);
+        bool mine = false;
+        for (int i = 0; i < n_mb; ++i, ++job) {
+          if ((job & 1) != mw) continue;
+          ok = mbar_wait_warp(empty_bar, epar, abort_flag, ta.wait_cycles);
+          if (!ok) break;
+          epar ^= 1u;
+          tc_fence_after();
+          if (leader) {
+            const uint32_t at = q_tmem + (i ^ flip) * QCOLS;
+#pragma unroll
+            for (int kk = 0; kk < 4 * NH; ++kk)
+              umma_bf16_ts(d, at + kk * 8, desc_s + (uint64_t)(((kk >> 2) * HALF_BYTES + (kk & 3) * 32) >> 4), idesc,
+                           kk > 0 ? 1u : 0u);
+            umma_commit(full_bar);
+          }
+          mine = true;
+          ++n_issued;
+        }
+        if (!ok) break;
+        if (leader) {
+          if (mine) umma_commit(smem_u32(&bars->k_empty[s]));
+          else mbar_arrive(smem_u32(&bars->k_empty[s]));
+        }
+        if (++s == S) { s = 0; kpar ^= 1u; }
+        flip ^= lse_flip(rows, hr);
+        if (mw == 1 && m_rows > 0 && n_issued >= 2) {
+          ok = merge();
+          if (!ok) break;
+        }
+      }
+      if (ok && mw == 1 && m_rows > 0) ok = merge();
       if (!ok) break;
-      if (leader) {
-        if (mine) umma_commit(smem_u32(&bars->k_empty[s]));
-        else mbar_arrive(smem_u32(&bars->k_empty[s]));
-      }
-      if (++s == S) { s = 0; kpar ^= 1u; }
+      m_rows = rows;
+      m_dst = dst;
+      if (leader) umma_commit(smem_u32(&bars->q_free[qh]));
+      qh ^= 1;
     }
+    if (ok && mw == 1 && m_rows > 0) ok = merge();
     // drain: every MMA issued above has completed before TMEM is freed
     __syncwarp();
     if (leader) umma_commit(smem_u32(&bars->drained[mw]));
@@ -320,79 +531,78 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const TcArgs ta) {
     __syncwarp();
   } else {
     // ---------------- epilogue warps ----------------
-    {
-      // Q row (block k, row rib) -> this thread's TMEM lane, 64 packed columns (zeros for padding rows)
-      const int n = k * 128 + rib;
-      const bool live = k < n_mb && n < rows;
-      const int w = (row0 + n) / G, g = (row0 + n) % G;
-      const uint4* src = reinterpret_cast<const uint4*>(
-          a.q + (((int64_t)slab * a.sum_win + w0 + (live ? w : 0)) * a.n_q_heads + h * G + (live ? g : 0)) * (64 * NH));
-      const uint32_t dst = tmem_base + ((uint32_t)(quarter * 32) << 16) + k * 64;
-      if (k < n_mb) {
-        // (the whole row in flight at once: under load one round trip to L2 is thousands of cycles, and the
-        // MMA issuers wait for the last row)
-        uint4 x[8 * NH];
-#pragma unroll
-        for (int j = 0; j < 8 * NH; ++j) x[j] = live ? __ldg(src + j) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-        for (int i = 0; i < 2 * NH; ++i) tmem_st16(dst + i * 16, reinterpret_cast<const uint32_t*>(x + 4 * i));
-        tmem_st_wait();
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars->q_ready));
-    }
-    // last key each of this thread's rows sees (padding rows: every key, their sums are dropped); the most restricted row's,
-    // and the largest first key (0 unless the layer has a sliding window)
-    int jfast = L - 1, jlmax = 0;
-#pragma unroll
-    for (int mb = 0; mb < 4; ++mb) {
-      const int n = mb * 128 + rib;
-      const int jm = (a.causal && n < rows) ? (L - W + (row0 + n) / G) : (L - 1);
-      bars->last_key[mb][rib] = jm;                              // (by the four warps of the quarter alike)
-      jfast = min(jfast, jm);
-      if (WIN && a.win_left > 0 && n < rows) jlmax = max(jlmax, jm - a.win_left + 1);
-      bars->state[grp][mb][half][rib] = make_float2(-INFINITY, 0.f);
-    }
+    const int quarter = warp & 3;                  // TMEM lanes this warp may touch
+    const int k = (warp - LSE_EPI_WARP0) >> 2;     // 0..3
+    const int grp = k >> 1;                        // accumulator / job parity this warp serves
+    const int half = k & 1;                        // its columns: [64 half, 64 half + 64)
+    const int rib = quarter * 32 + lane;           // TMEM lane
+    const int upper = quarter >> 1;                // lanes 64 and up: the second half of a block
     const float c = a.scale_log2;
+    const Exp2Cubic cubic = ta.cubic;
     const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16) + LSE_A_COLS + grp * 128 + half * 64;
-    // (key tile, row block) of this group's jobs, carried along without divisions: job = tile * n_mb + mb
-    int mb = grp % n_mb, key0 = (t_begin + grp / n_mb) * TK + half * 64;
-    const int mb_step = 2 % n_mb, tile_step = 2 / n_mb;
-    for (int job = grp; job < n_jobs; job += 2) {
-      epi_ok = lse_job<NPOLY, WIN>(bars, abort_flag, tq, grp, job, &bars->last_key[mb][rib], &bars->state[grp][mb][half][rib],
-                                   jfast - key0 + 1, jlmax - key0, a.win_left, key0, c, ta.wait_cycles);
-      if (!epi_ok) break;
-      mb += mb_step;
-      key0 += tile_step * TK;
-      if (mb >= n_mb) { mb -= n_mb; key0 += TK; }
+    int slot = 0, sp = 0;                          // sp: which `state`
+    uint32_t ipar = 0, fpar = 0, spar = 0;
+    for (;;) {
+      bool ok = mbar_wait_warp(smem_u32(&bars->item_full[slot]), ipar, abort_flag, ta.wait_cycles);
+      if (!ok) break;
+      const LseItem* x = &bars->item[slot];
+      const int n_tiles = x->n_tiles, rows = x->rows;
+      if (n_tiles <= 0) break;
+      const int n_half = (rows + hr - 1) / hr, n_mb = (n_half + 1) / 2;
+      const bool twice = n_half & 1;               // the last block holds its rows twice: a lane folds half as many columns of them
+      // this thread's row in row block b, and the last key it sees (lanes without a row of this item: every key; their sums are dropped)
+      auto row_of = [&](int b) { return (2 * b + (twice && b == n_mb - 1 ? 0 : upper)) * hr + (rib & 63); };
+      auto last_of = [&](int n) { return (a.causal && n < rows) ? (x->L - x->W + (x->row0 + n) / G) : (x->L - 1); };
+      if (!mbar_wait_warp(smem_u32(&bars->shares_empty[sp]), spar ^ 1u, abort_flag, ta.wait_cycles)) break;
+      // the most restricted row's last key, and the largest first key (0 unless the layer has a sliding window)
+      int jfast = x->L - 1, jlmax = 0;
+      for (int b = 0; b < n_mb; ++b) {
+        const int n = row_of(b), jm = last_of(n);
+        jfast = min(jfast, jm);
+        if (WIN && a.win_left > 0 && n < rows) jlmax = max(jlmax, jm - a.win_left + 1);
+        bars->state[sp][grp][b][half][rib] = make_float2(-INFINITY, 0.f);
+      }
+      const bool flip = lse_flip(rows, hr) != 0;
+      const int n_jobs = n_tiles * n_mb, b_short = twice ? n_mb - 1 : -1;
+      float2* st0 = &bars->state[sp][grp][0][half][rib];
+      int key0 = (x->t_begin + (n_mb == 1 ? grp : 0)) * TK + half * 64;
+      // A group that stays with one row block keeps its (reference, sum) in registers and has little left to count per job.
+      int b = n_mb == 1 ? 0 : grp;
+      bool wide = b != b_short;
+      int off = wide ? 0 : upper * 32;
+      const int step = n_mb == 1 ? 2 * TK : TK;
+      float2 ms = make_float2(-INFINITY, 0.f);
+      for (int j = grp; j < n_jobs; j += 2) {
+        ok = lse_job<NPOLY, WIN>(bars, abort_flag, tq + off, grp, fpar, wide, [&]() { return last_of(row_of(b)); }, ms,
+                                 jfast - key0 - off + 1, jlmax - key0 - off, a.win_left, key0 + off, c, cubic, ta.wait_cycles);
+        if (!ok) break;
+        fpar ^= 1u;
+        key0 += step;
+        if (flip) {                                // the other block
+          st0[b * (2 * 128)] = ms;
+          b ^= 1;
+          wide = b != b_short;
+          off = wide ? 0 : upper * 32;
+          ms = st0[b * (2 * 128)];
+        }
+      }
+      if (!flip && grp < n_jobs) st0[b * (2 * 128)] = ms;
+      if (!ok) break;
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(smem_u32(&bars->shares_full[sp]));
+        mbar_arrive(smem_u32(&bars->item_empty[slot]));
+      }
+      if (++slot == LSE_ITEMS_AHEAD) { slot = 0; ipar ^= 1u; }
+      sp ^= 1;
+      spar ^= (uint32_t)(sp == 0);
     }
   }
   // ---------------- teardown ----------------
   tc_fence_before();
   __syncthreads();
-  if (warp >= LSE_EPI_WARP0 && k == 0 && !*abort_flag) {
-    // merge the four shares (group, column half) of each row, store (reference in log2 units, sum); (-inf, 0) when the
-    // row saw no key of this chunk
-#pragma unroll
-    for (int mb = 0; mb < 4; ++mb) {
-      const int n = mb * 128 + rib;
-      if (mb < n_mb && n < rows) {
-        float2 o[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) o[i] = bars->state[i >> 1][mb][i & 1][rib];
-        const float mm = fmaxf(fmaxf(o[0].x, o[1].x), fmaxf(o[2].x, o[3].x));
-        float ss = 0.f;
-        if (mm > -INFINITY) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) ss += o[i].x > -INFINITY ? o[i].y * exp2f(o[i].x - mm) : 0.f;
-        }
-        a.partials[((int64_t)u * a.n_chunks + chunk) * a.rows_max + row0 + n] = make_float2(mm, ss);
-      }
-    }
-  }
   if (warp == 0 && lane == 0 && *abort_flag) {
-    report(a.status, ACTKV_E_TIMEOUT, u, chunk);
+    report(a.status, ACTKV_E_TIMEOUT, (int)blockIdx.x, 0);
     // loads still in flight land in this CTA's shared memory: give them a moment before exiting
     for (int s = 0; s < S; ++s) mbar_wait(smem_u32(&bars->k_full[s]), 0, nullptr, DRAIN_LIMIT_CYCLES / 64);
   }

@@ -137,6 +137,12 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
       : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+               : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t* r = reinterpret_cast<uint32_t*>(v);
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -144,16 +150,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
                : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// 16 consecutive 32-bit columns of this thread's TMEM lane <- registers
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-      : "memory");
+// 128 rows x 16 bf16 (one k16 step) of a K-major SWIZZLE_128B tile in shared memory -> eight columns of tensor memory, the layout in
+// which umma_bf16_ts reads A.  Ordered before later MMAs of the same thread; after earlier ones only through a commit.
+__device__ __forceinline__ void tmem_cp_k16(uint32_t taddr, uint64_t desc) {
+  asm volatile("tcgen05.cp.cta_group::1.128x256b [%0], %1;" ::"r"(taddr), "l"(desc) : "memory");
 }
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // D[tmem] (+)= A[tmem] * B[smem desc]^T, bf16 x bf16 -> fp32, A = 128 rows x 16 bf16 packed in 8 columns
 __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                              uint32_t accumulate) {
@@ -163,6 +164,28 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
+
+// Cluster launch control: a running CTA takes over the work of one that has not been launched yet.  The answer (16 bytes of shared
+// memory) arrives on `bar` like a TMA load.  After an answer "none left" no further request may be made.
+__device__ __forceinline__ void clc_request(uint32_t resp, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(resp), "r"(bar) : "memory");
+}
+__device__ __forceinline__ int clc_answer(uint32_t resp) {             // blockIdx.x of the CTA taken over, -1: none left
+  int x = 0;
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+      "ld.shared.b128 r, [%2];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+      "selp.u32 %1, 1, 0, p;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%0, _, _, _}, r;\n\t}"
+      : "+r"(x), "=r"(ok) : "r"(resp) : "memory");
+  return ok ? x : -1;
+}
+
+// A value that all lanes of the (converged) warp hold, in the form the compiler knows to be uniform: operands of tcgen05.mma that
+// are not in uniform registers cost the LSE pass 10 %.
+__device__ __forceinline__ int uni(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
 // Register budget of a warpgroup (four consecutive warps, all of whose threads execute the instruction): the
 // control and copy warpgroups hand registers back, the epilogue warpgroups take them.
@@ -214,11 +237,14 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+struct Exp2Cubic { float c0, c1, c2, c3; };   // 2^f on [-0.5, 0.5] = c0 + f (c1 + f (c2 + f c3))
+
 struct TcArgs {
   ScoreArgs a;
+  Exp2Cubic cubic;           // LSE pass
   int32_t tiles_per_cta;     // pooled-score pass: key tiles per CTA
   int32_t n_kchunks;         // pooled-score pass: CTAs per unit
-  int32_t n_rg;              // LSE pass: groups of MAX_ROWS rows per unit (a grid dimension)
+  int32_t n_rg;              // LSE pass: groups of rows per unit (a grid dimension)
   int32_t row_begin;         // pooled-score pass: first row of this launch's row group (multiple of MAX_ROWS)
   int32_t n_stages;          // K stages in shared memory (at most 8)
   int32_t k5;                // K tensor map has five dimensions (pages that are not slot-major), else four
@@ -237,7 +263,7 @@ __device__ __forceinline__ int32_t page_for_tile(const TablesView& tab, int32_t 
 
 // The K-tile producers of both score kernels: producer p of P takes tiles p, p + P, ... of
 // [t_begin, t_begin + n_tiles) of request r, head h, layer `layer` through the block table into the ring of S
-// stages, one TMA box per (page, 64-dim half), one box per lane.  Pages of 16, 32, 64 or 128 tokens: a
+// stages (tile i is entry e0 + i of the ring; false when a wait gave up or the injected fault stopped it), one TMA box per (page, 64-dim half), one box per lane.  Pages of 16, 32, 64 or 128 tokens: a
 // tile of 128 keys is ppt = 128 / page_size pages, a box page_size rows of 128 B.
 // Measured on B200 (boxes of 16 rows x 128 B from random pages): one warp issuing a tile's 16 boxes from
 // 8 lanes delivers a tile per 1950 cycles, from 16 lanes per 1570, two warps per 1235, four per 1180 (the
@@ -246,24 +272,25 @@ __device__ __forceinline__ int32_t page_for_tile(const TablesView& tab, int32_t 
 // lane % ppt = page); the next group's ids are loaded while the current four tiles are being issued.
 // K5: five-dimensional tensor map (pages that are not slot-major).
 template <bool K5, int NH, class Bars>
-__device__ __forceinline__ void k_tile_producer(const CUtensorMap* kmap, const ScoreArgs& a, Bars* bars, uint32_t k_smem,
+__device__ __forceinline__ bool k_tile_producer(const CUtensorMap* kmap, const ScoreArgs& a, Bars* bars, uint32_t k_smem,
                                                 int S, int r, int h, int layer, int L, int t_begin, int n_tiles,
                                                 int lane, volatile int* abort_flag, int p, int P, long long wait_cycles,
-                                                int stall_tile) {
+                                                int stall_tile, int e0 = 0) {
   const int ps = a.pool.page_size;
   const int ppt = TK / ps;                                      // pages per tile: 8, 4, 2 or 1
   const int lp_shift = 31 - __clz(ppt);                         // log2(ppt)
   const uint32_t box_bytes = (uint32_t)ps * 128u;
   const int n_lp = (L + ps - 1) / ps;
   const int n_mine = (n_tiles - p + P - 1) / P;                  // tiles p, p + P, ... below n_tiles
+  if (n_mine <= 0) return true;
   const int g_tile = lane >> lp_shift, g_page = lane & (ppt - 1);            // this lane's slot in a group of four tiles
   int32_t pid = page_for_tile(a.tab, a.pool.n_pages, r, (t_begin + p + min(g_tile, 3) * P) * ppt + g_page, n_lp, a.status);
   int32_t pid_next = 0;
   for (int i = 0; i < n_mine; ++i) {
     const int it = p + i * P;
-    if (stall_tile >= 0 && it >= stall_tile) break;       // injected fault: this and all later tiles never arrive
-    const int s = it % S;
-    const uint32_t ph = (uint32_t)(it / S) & 1u;
+    if (stall_tile >= 0 && it >= stall_tile) return false;       // injected fault: this and all later tiles never arrive
+    const int s = (e0 + it) % S;
+    const uint32_t ph = (uint32_t)((e0 + it) / S) & 1u;
     if ((i & 3) == 0 && i + 4 < n_mine)
       pid_next = page_for_tile(a.tab, a.pool.n_pages, r, (t_begin + p + (i + 4 + min(g_tile, 3)) * P) * ppt + g_page, n_lp,
                                a.status);
@@ -273,7 +300,7 @@ __device__ __forceinline__ void k_tile_producer(const CUtensorMap* kmap, const S
       if (ok) mbar_expect_tx(smem_u32(&bars->k_full[s]), NH * HALF_BYTES);
     }
     ok = __shfl_sync(0xffffffffu, ok, 0);
-    if (!ok) break;
+    if (!ok) return false;
     // lane j < ppt NH: page j % ppt, half j / ppt of this tile
     const int32_t my_pid = __shfl_sync(0xffffffffu, pid, ((i & 3) << lp_shift) | (lane & (ppt - 1)));
     if (lane < ppt * NH) {
@@ -285,6 +312,7 @@ __device__ __forceinline__ void k_tile_producer(const CUtensorMap* kmap, const S
     }
     if ((i & 3) == 3) pid = pid_next;
   }
+  return true;
 }
 
 }  // namespace tc

@@ -1,0 +1,54 @@
+"""LSE pass at the edges of its work items: rows around half a block and a block, groups that do not divide 64, several row groups,
+chunks of the shortest length, requests that end early; against float64, and the same bits on every run."""
+import pytest
+import torch
+
+from paper_2609_31395_b200 import harness as H
+from paper_2609_31395_b200 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _lse64(b):
+    wl = b.wl
+    G, D, P, Hkv = wl.group, wl.head_dim, wl.page_size, wl.n_kv_heads
+    out, w0 = [], 0
+    for r, (L, W) in enumerate(zip(wl.seq_lens, wl.windows)):
+        j = torch.arange(L, device=DEV)
+        slots = b.page_table[r].long()[j // P] * P + j % P
+        k = b.pool[:, 0].reshape(wl.n_layers, -1, Hkv, D)[:, slots].permute(0, 2, 3, 1).double()          # [NL, Hkv, D, L]
+        q = b.q[:, w0:w0 + W].view(wl.n_layers, W, Hkv, G, D).permute(0, 2, 1, 3, 4).reshape(wl.n_layers, Hkv, W * G, D).double()
+        s = (q @ k) * wl.sm_scale
+        if wl.causal:
+            last = L - W + torch.arange(W, device=DEV).repeat_interleave(G)
+            s.masked_fill_(j[None, :] > last[:, None], float("-inf"))
+        out.append(s.logsumexp(-1).view(wl.n_layers, Hkv, W, G).permute(0, 2, 1, 3).reshape(wl.n_layers, W, Hkv * G))
+        w0 += W
+    return torch.cat(out, 1)
+
+
+@pytest.mark.parametrize("group,windows,head_dim,causal", [
+    (4, [16, 17, 32, 33, 48, 49, 64], 128, True),        # 64, 68, 128, 132, 192, 196, 256 rows
+    (4, [80, 81, 112, 113, 128], 128, False),            # 320, 324, 448, 452, 512: both halves of the Q columns
+    (8, [8, 9, 24, 25, 56, 64], 64, True),               # four blocks in one half
+    (7, [9, 10, 18, 19, 40, 73], 128, True),             # half a block is 63 rows; 73 x 7 = 511 rows are two row groups
+    (32, [2, 3, 5, 20], 64, False),
+    (5, [13, 26, 27, 110], 128, True),                   # 60-row halves, 550 rows
+])
+def test_rows_around_the_edges_of_items(group, windows, head_dim, causal):
+    lens = [max(w, n) for w, n in zip(windows, [700, 129, 2600, 512, 1, 1537, 300])]
+    wl = synth.Workload("items", 2, 2, group, lens, windows, [max(1, n // 4) for n in lens], head_dim=head_dim, causal=causal,
+                        table_style="fragmented", seed=61)
+    b = synth.generate(wl, DEV)
+    comp = H.Compressor(b.pool, b.page_table, b.seq_len, b.free_list, b.free_count, wl.n_q_heads, H.sizes_of(b), want_lse=True)
+    runs = []
+    for _ in range(4):
+        comp.lse.fill_(float("nan"))
+        comp.run_lse(b.q, b.win_indptr, b.tok_indptr, wl.sm_scale, wl.causal, 0, wl.n_layers, comp.lse)
+        runs.append(comp.lse.clone())
+    comp.check_status()
+    # one exponential in eight is a cubic of relative error 7.5e-5; float32 dot products of 128 terms add 1e-5
+    assert (runs[0].double() - _lse64(b)).abs().max() < 1e-4
+    for x in runs[1:]:
+        assert torch.equal(x, runs[0])
