@@ -223,9 +223,8 @@ __device__ __forceinline__ LseItem lse_item(const TcArgs& ta, int id, int lane) 
   x.L = a.tab.seq_len[x.r];
   x.w0 = a.win_indptr[x.r];
   x.W = a.win_indptr[x.r + 1] - x.w0;
-  const int rg_rows = 2 * LSE_MB * lse_half_rows(G);
-  x.row0 = rg * rg_rows;
-  x.rows = min(x.W * G - x.row0, rg_rows);
+  x.row0 = rg * ta.rg_rows;
+  x.rows = min(x.W * G - x.row0, ta.rg_rows);
   const int key_begin = x.chunk * a.lse_chunk;
   if (key_begin >= x.L || (rg > 0 && x.rows <= 0)) return x;
   if (x.W <= 0 || (a.causal && x.W > x.L)) {
@@ -295,7 +294,9 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
     if (threadIdx.x == 0) report(a.status, ACTKV_E_CUDA, -2, (int32_t)smem_base);
     return;
   }
-  if (threadIdx.x == 0) {
+  LseItem x_next;
+  if (warp == 0) x_next = lse_item<WIN>(ta, blockIdx.x, lane);     // (its loads are under way while the others set up)
+  if (threadIdx.x == 96) {
     for (int s = 0; s < S; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 2); }
     for (int i = 0; i < LSE_ITEMS_AHEAD; ++i) {
       mbar_init(smem_u32(&bars->item_full[i]), 1);
@@ -339,7 +340,6 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
     const int p = warp >> 1;
     int e = 0, slot = 0;
     uint32_t ipar = 0, cpar = 0;
-    int id = blockIdx.x;
     bool ok = true;
     for (;;) {
       LseItem x;
@@ -349,7 +349,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
           clc_request(smem_u32(bars->clc_resp), smem_u32(&bars->clc));
         }
         __syncwarp();
-        x = lse_item<WIN>(ta, id, lane);
+        x = x_next;
         if (x.n_tiles > 0) {
           ok = mbar_wait_warp(smem_u32(&bars->item_empty[slot]), ipar ^ 1u, abort_flag, ta.wait_cycles);
           if (ok && lane == 0) {
@@ -394,10 +394,11 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
         // (also after giving up: the answer lands in this CTA's shared memory)
         const bool answered = mbar_wait_warp(smem_u32(&bars->clc), cpar, nullptr, ta.wait_cycles);
         cpar ^= 1u;
-        id = answered ? clc_answer(smem_u32(bars->clc_resp)) : -1;
+        const int id = answered ? clc_answer(smem_u32(bars->clc_resp)) : -1;
         fence_proxy_async();                     // (the answer has been read before the next one is written)
         __syncwarp();
         if (!ok || id < 0) break;
+        x_next = lse_item<WIN>(ta, id, lane);
       }
       if (!ok) break;
     }

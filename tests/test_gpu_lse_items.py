@@ -52,3 +52,33 @@ def test_rows_around_the_edges_of_items(group, windows, head_dim, causal):
     assert (runs[0].double() - _lse64(b)).abs().max() < 1e-4
     for x in runs[1:]:
         assert torch.equal(x, runs[0])
+
+
+@pytest.mark.parametrize("group,windows,lens,head_dim,causal", [
+    (4, [32], [4096], 128, False),                       # 128 rows as two items, eight chunks
+    (4, [64, 17], [1500, 129], 128, True),               # 256 and 68 rows as items of half a block
+    (8, [64], [300], 64, True),                          # 512 rows, one chunk
+    (7, [19, 9], [700, 513], 128, True),                 # 63-row halves: 133 and 63 rows
+    (16, [40], [2000], 64, False),                       # 640 rows: two launches of the pooled-score pass
+])
+def test_launches_that_leave_sms_idle(group, windows, lens, head_dim, causal):
+    wl = synth.Workload("few", 1, 2, group, lens, windows, [max(1, n // 4) for n in lens], head_dim=head_dim, causal=causal,
+                        table_style="fragmented", seed=67)
+    b = synth.generate(wl, DEV)
+    args = (b.q, b.win_indptr, b.tok_indptr, wl.sm_scale, wl.causal, 0, 1)
+    comp = H.Compressor(b.pool, b.page_table, b.seq_len, b.free_list, b.free_count, wl.n_q_heads, H.sizes_of(b), want_lse=True)
+    lse = torch.full_like(comp.lse, float("nan"))
+    comp.run_lse(*args, lse)
+    assert (lse.double() - _lse64(b)).abs().max() < 1e-4        # (the cubic and float32 dot products, as above)
+    comp.run_score(*args, lse_in=lse)
+    want = comp.score.clone()
+    # both passes in one call: the same bits as one after the other
+    comp.lse.fill_(float("nan"))
+    comp.score.fill_(float("nan"))
+    comp.run_score(*args)
+    comp.check_status()
+    assert torch.equal(comp.lse, lse) and torch.equal(comp.score, want)
+    comp.lse = None                                             # nobody asks for the LSE: it goes to the workspace
+    comp.score.fill_(float("nan"))
+    comp.run_score(*args)
+    assert torch.equal(comp.score, want)
