@@ -207,17 +207,6 @@ inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_w
   ta.a = a;
   ta.cubic = {tc::EXP2_C0, tc::EXP2_C1, tc::EXP2_C2, tc::EXP2_C3};
   ta.n_rg = tc::lse_row_groups(max_win, a.group);
-  ta.rg_rows = 2 * tc::LSE_MB * tc::lse_half_rows(a.group);
-  const int64_t units = (int64_t)a.n_layers_sub * a.pool.n_kv_heads * a.tab.n_req;
-  // SMs left without an item: items of half the rows, down to half a block (whose rows are then held twice), which read the same keys
-  // once more from L2.  With the pooled-score pass split down to two key tiles and the first item read ahead of the barriers, a step of one
-  // layer x 8 heads, 4096 keys, 128 rows 39.4 -> 37.6 us.
-  while (ta.rg_rows > tc::lse_half_rows(a.group)) {
-    const int n_rg = (max_win * a.group + ta.rg_rows / 2 - 1) / (ta.rg_rows / 2);
-    if (units * a.n_chunks * n_rg > 148) break;
-    ta.rg_rows /= 2;
-    ta.n_rg = n_rg;
-  }
   ta.row_begin = 0;
   ta.k5 = tc::pool_needs_5d(pool) ? 1 : 0;
   ta.n_stages = 0;
@@ -225,6 +214,7 @@ inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_w
   ta.n_kchunks = 0;
   ta.copy_ws = nullptr;              // (this kernel has no copy role)
   tc::apply_hook(ta);
+  const int64_t units = (int64_t)a.n_layers_sub * a.pool.n_kv_heads * a.tab.n_req;
   const int64_t grid = units * a.n_chunks * ta.n_rg;
   if (grid > 0x7fffffffLL) return ACTKV_E_INVALID;
   return pool->head_dim == 64 ? score_tc_launch_lse_c<1>(kmap, qmap, ta, (unsigned)grid, s)

@@ -223,8 +223,9 @@ __device__ __forceinline__ LseItem lse_item(const TcArgs& ta, int id, int lane) 
   x.L = a.tab.seq_len[x.r];
   x.w0 = a.win_indptr[x.r];
   x.W = a.win_indptr[x.r + 1] - x.w0;
-  x.row0 = rg * ta.rg_rows;
-  x.rows = min(x.W * G - x.row0, ta.rg_rows);
+  const int rg_rows = 2 * LSE_MB * lse_half_rows(G);
+  x.row0 = rg * rg_rows;
+  x.rows = min(x.W * G - x.row0, rg_rows);
   const int key_begin = x.chunk * a.lse_chunk;
   if (key_begin >= x.L || (rg > 0 && x.rows <= 0)) return x;
   if (x.W <= 0 || (a.causal && x.W > x.L)) {

@@ -245,7 +245,6 @@ struct TcArgs {
   int32_t tiles_per_cta;     // pooled-score pass: key tiles per CTA
   int32_t n_kchunks;         // pooled-score pass: CTAs per unit
   int32_t n_rg;              // LSE pass: groups of rows per unit (a grid dimension)
-  int32_t rg_rows;           // LSE pass: rows of a group, 1, 2 or 4 halves of a row block
   int32_t row_begin;         // pooled-score pass: first row of this launch's row group (multiple of MAX_ROWS)
   int32_t n_stages;          // K stages in shared memory (at most 8)
   int32_t k5;                // K tensor map has five dimensions (pages that are not slot-major), else four

@@ -55,9 +55,9 @@ def test_rows_around_the_edges_of_items(group, windows, head_dim, causal):
 
 
 @pytest.mark.parametrize("group,windows,lens,head_dim,causal", [
-    (4, [32], [4096], 128, False),                       # 128 rows as two items, eight chunks
-    (4, [64, 17], [1500, 129], 128, True),               # 256 and 68 rows as items of half a block
-    (8, [64], [300], 64, True),                          # 512 rows, one chunk
+    (4, [32], [4096], 128, False),                       # one item of rows, eight chunks
+    (4, [64, 17], [1500, 129], 128, True),               # a full item, and one of 68 rows
+    (8, [64], [300], 64, True),                          # 512 rows, one chunk: two items side by side
     (7, [19, 9], [700, 513], 128, True),                 # 63-row halves: 133 and 63 rows
     (16, [40], [2000], 64, False),                       # 640 rows: two launches of the pooled-score pass
 ])
