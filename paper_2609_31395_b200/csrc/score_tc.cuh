@@ -95,8 +95,7 @@ inline int lse_split(int64_t units, int tiles, double len, double win, double ov
 
 // Items of the LSE pass side by side for a window of max_win tokens.
 inline int lse_row_groups(int max_win, int g) {
-  const int rows = 2 * LSE_MB * lse_half_rows(g);
-  return (max_win * g + rows - 1) / rows;
+  return (max_win * g + LSE_MB * 128 - 1) / (LSE_MB * 128);
 }
 
 inline bool make_kmap(const actkv_pool_t* pool, CUtensorMap* kmap) {

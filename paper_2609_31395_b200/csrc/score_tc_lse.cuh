@@ -117,16 +117,12 @@ constexpr int LSE_MB = 2;                        // row blocks of an item
 constexpr int LSE_A_COLS = 256;                  // TMEM columns holding Q blocks, a half for each of two items
 constexpr int LSE_ITEMS_AHEAD = 3;               // item descriptors in shared memory
 __host__ __device__ constexpr int lse_stages(int nh) { return nh == 1 ? 8 : 6; }             // K tiles (or Q blocks) in shared memory
-__host__ __device__ constexpr int lse_half_rows(int g) { return 64 / g * g; }                // rows of half a block: whole groups
 constexpr float LSE_BIG = 1099511627776.f;       // 2^40: a partial sum beyond it moves the reference
 constexpr float LSE_REF_MAX = 1048576.f;         // references beyond 2^20 (rounding to integers needs |v c| < 2^22) take the general form
 
 // Two blocks of which the second is short change places on odd tiles (exclusive or with this): the short one would otherwise always
 // fall to the same accumulator.
-__device__ __forceinline__ int lse_flip(int rows, int hr) {
-  const int n_half = (rows + hr - 1) / hr;
-  return n_half == 3 ? 1 : 0;
-}
+__device__ __forceinline__ int lse_flip(int rows) { return (rows + 63) / 64 == 3 ? 1 : 0; }
 
 // A work item: the rows [row0, row0 + rows) of a unit against n_tiles key tiles.  n_tiles = 0: no more items.
 struct LseItem {
@@ -223,9 +219,8 @@ __device__ __forceinline__ LseItem lse_item(const TcArgs& ta, int id, int lane) 
   x.L = a.tab.seq_len[x.r];
   x.w0 = a.win_indptr[x.r];
   x.W = a.win_indptr[x.r + 1] - x.w0;
-  const int rg_rows = 2 * LSE_MB * lse_half_rows(G);
-  x.row0 = rg * rg_rows;
-  x.rows = min(x.W * G - x.row0, rg_rows);
+  x.row0 = rg * LSE_MB * 128;
+  x.rows = min(x.W * G - x.row0, LSE_MB * 128);
   const int key_begin = x.chunk * a.lse_chunk;
   if (key_begin >= x.L || (rg > 0 && x.rows <= 0)) return x;
   if (x.W <= 0 || (a.causal && x.W > x.L)) {
@@ -248,18 +243,44 @@ __device__ __forceinline__ LseItem lse_item(const TcArgs& ta, int id, int lane) 
   return x;
 }
 
+// 64 rows of the item from row n0 on into half a block of a stage, as the TMA unit would lay them out (128-byte swizzle); zeros where
+// the item has no row.  For what is no box of whole groups: the ragged end of a window, and groups that do not divide 64.  Asynchronous
+// copies without registers: the whole half block is in flight at once.  Called by a whole warp.
+// (Few instructions count: beside the epilogue the producer gets an issue slot every several cycles.)
+template <int NH>
+__device__ __forceinline__ void lse_q_rows(const ScoreArgs& a, const LseItem& x, uint32_t dst, int n0, int lane) {
+  constexpr int RPI = 32 / (8 * NH);                          // rows per step of the warp
+  const int G = a.group, live = min(x.rows - n0, 64);
+  int off[2];                                                 // where the rows lane and lane + 32 begin, from the window's first token on
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int n = x.row0 + n0 + min(lane + 32 * i, live - 1), w = n / G;
+    off[i] = (w * a.n_q_heads + (n - w * G)) * (64 * NH);
+  }
+  const int r = lane / (8 * NH), c = lane % (8 * NH);
+  const __nv_bfloat16* src = a.q + (((int64_t)x.slab * a.sum_win + x.w0) * a.n_q_heads + x.layer_h * G) * (64 * NH) + c * 8;
+  const uint32_t d = dst + (c >> 3) * HALF_BYTES + r * 128 + (((c & 7) ^ r) << 4);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+#pragma unroll 4
+    for (int k = 0; k < 32; k += RPI) {
+      const int o = __shfl_sync(0xffffffffu, off[i], k + r), row = 32 * i + k;
+      cp_async16((d ^ ((k & 7) << 4)) + row * 128, src + o, row + r < live ? 16u : 0u);
+    }
+  }
+}
+
 // The shares (group, column half, and lane of a block held twice) of each row of a finished item; stores (reference in log2 units, sum),
 // (-inf, 0) when the row saw no key of this chunk.  Called by a whole warp.
-__device__ __forceinline__ void lse_merge(const float2 (&state)[2][LSE_MB][2][128], float2* dst, int rows, int hr, int lane) {
-  const int n_half = (rows + hr - 1) / hr;
-  for (int n2 = lane; n2 < n_half * 64; n2 += 32) {
-    const int i2 = n2 >> 6, n = i2 * hr + (n2 & 63);          // half block, row
-    if ((n2 & 63) >= hr || n >= rows) continue;
+__device__ __forceinline__ void lse_merge(const float2 (&state)[2][LSE_MB][2][128], float2* dst, int rows, int lane) {
+  const int n_half = (rows + 63) / 64;
+  for (int n = lane; n < rows; n += 32) {
+    const int i2 = n >> 6;                                    // half block
     const bool dup = (n_half & 1) && i2 == n_half - 1;
     float2 o[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      o[i] = i < 4 || dup ? state[i & 1][i2 >> 1][(i >> 1) & 1][(n2 & 127) + (i >> 2) * 64] : make_float2(-INFINITY, 0.f);
+      o[i] = i < 4 || dup ? state[i & 1][i2 >> 1][(i >> 1) & 1][(n & 127) + (i >> 2) * 64] : make_float2(-INFINITY, 0.f);
     float mm = -INFINITY;
 #pragma unroll
     for (int i = 0; i < 8; ++i) mm = fmaxf(mm, o[i].x);
@@ -283,7 +304,6 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
   static_assert(LSE_MB * QCOLS <= LSE_A_COLS / 2, "Q columns");
   const ScoreArgs& a = ta.a;
   const int G = a.group;
-  const int hr = lse_half_rows(G);
 
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t k_smem = smem_base;                               // S stages of a K tile
@@ -315,15 +335,6 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
     mbar_init(smem_u32(&bars->drained[1]), 1);
     bars->abort_flag = 0;
     fence_barrier_init();
-  }
-  if (hr < 64) {
-    // lanes past the last whole group of half a block: no load ever writes these rows of a stage for a Q block, so they start as zeros
-    // (later they hold old keys), and not as what may be anything
-    for (int i = threadIdx.x; i < S * NH * 2 * (64 - hr) * 8; i += blockDim.x) {
-      const int row = hr + (i >> 3) % (64 - hr), hb = (i >> 3) / (64 - hr);
-      *reinterpret_cast<uint4*>(smem + (size_t)hb * (HALF_BYTES / 2) + row * 128 + (i & 7) * 16) = make_uint4(0, 0, 0, 0);
-    }
-    fence_proxy_async();
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(&bars->tmem_base), 512);
@@ -368,20 +379,32 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
       }
       if (ok && x.n_tiles > 0) {
         if (++slot == LSE_ITEMS_AHEAD) { slot = 0; ipar ^= 1u; }
-        const int n_half = (x.rows + hr - 1) / hr, n_mb = (n_half + 1) / 2;
+        const int n_half = (x.rows + 63) / 64, n_mb = (n_half + 1) / 2;
         for (int b = 0; b < n_mb && ok; ++b, ++e) {
           if ((e & 1) != p) continue;
           const int s = e % S;
           ok = mbar_wait_warp(smem_u32(&bars->k_empty[s]), ((uint32_t)(e / S) & 1u) ^ 1u, abort_flag, ta.wait_cycles);
           if (!ok) break;
-          // the two halves of the block; a last half that stands alone is held twice
-          const uint32_t bar = smem_u32(&bars->k_full[s]);
-          if (lane == 0) mbar_expect_tx(bar, (uint32_t)(2 * NH * hr) * 128u);
+          // The two halves of the block; a last half that stands alone is held twice.  Whole groups all of whose rows the item has
+          // come as TMA boxes.  Lanes without a row hold zeros: they take part in the votes of the epilogue, so what they hold must be the
+          // same in every run, and no other request's.
+          const uint32_t bar = smem_u32(&bars->k_full[s]), dst = k_smem + s * (NH * HALF_BYTES);
+          auto first_row = [&](int j) { return min(2 * b + j, n_half - 1) * 64; };
+          auto is_box = [&](int j) { return 64 % G == 0 && first_row(j) + 64 <= x.rows; };
+          const int n_box = (is_box(0) ? 1 : 0) + (is_box(1) ? 1 : 0);
+          if (n_box < 2) {
+            for (int j = 0; j < 2; ++j)
+              if (!is_box(j)) lse_q_rows<NH>(a, x, dst + j * (HALF_BYTES / 2), first_row(j), lane);
+            cp_async_wait_all();
+            fence_proxy_async();                 // (the copies are read by tcgen05.cp)
+            __syncwarp();
+          }
+          if (lane == 0) mbar_expect_tx(bar, (uint32_t)(n_box * NH) * (HALF_BYTES / 2));
           __syncwarp();
-          if (lane < 2 * NH) {
+          if (lane < 2 * NH && is_box(lane & 1)) {
             const int hf = lane >> 1, j = lane & 1;
-            const int tok = x.slab * a.sum_win + x.w0 + (x.row0 + min(2 * b + j, n_half - 1) * hr) / G;
-            tma_load_3d(k_smem + s * (NH * HALF_BYTES) + hf * HALF_BYTES + j * (HALF_BYTES / 2), &qmap, bar, hf * 64, x.layer_h * G, tok);
+            const int tok = x.slab * a.sum_win + x.w0 + (x.row0 + first_row(j)) / G;
+            tma_load_3d(dst + hf * HALF_BYTES + j * (HALF_BYTES / 2), &qmap, bar, hf * 64, x.layer_h * G, tok);
           }
         }
         if (ok) {
@@ -433,7 +456,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
     float2* m_dst = nullptr;
     auto merge = [&]() {
       if (!mbar_wait_warp(smem_u32(&bars->shares_full[m_sp]), m_par, abort_flag, ta.wait_cycles)) return false;
-      lse_merge(bars->state[m_sp], m_dst, m_rows, hr, lane);
+      lse_merge(bars->state[m_sp], m_dst, m_rows, lane);
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars->shares_empty[m_sp]));
       m_rows = 0;
@@ -450,7 +473,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
       if (lane == 0) mbar_arrive(smem_u32(&bars->item_empty[slot]));
       if (n_tiles <= 0) break;
       if (++slot == LSE_ITEMS_AHEAD) { slot = 0; ipar ^= 1u; }
-      const int n_mb = ((rows + hr - 1) / hr + 1) / 2;
+      const int n_mb = (rows + 127) / 128;
       // the Q blocks go to the half of the Q columns that the previous item does not use
       const uint32_t q_tmem = tmem_base + (uint32_t)qh * (LSE_A_COLS / 2);
       if (mw == 0) {
@@ -510,7 +533,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
           else mbar_arrive(smem_u32(&bars->k_empty[s]));
         }
         if (++s == S) { s = 0; kpar ^= 1u; }
-        flip ^= lse_flip(rows, hr);
+        flip ^= lse_flip(rows);
         if (mw == 1 && m_rows > 0 && n_issued >= 2) {
           ok = merge();
           if (!ok) break;
@@ -550,10 +573,10 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
       const LseItem* x = &bars->item[slot];
       const int n_tiles = x->n_tiles, rows = x->rows;
       if (n_tiles <= 0) break;
-      const int n_half = (rows + hr - 1) / hr, n_mb = (n_half + 1) / 2;
+      const int n_half = (rows + 63) / 64, n_mb = (n_half + 1) / 2;
       const bool twice = n_half & 1;               // the last block holds its rows twice: a lane folds half as many columns of them
       // this thread's row in row block b, and the last key it sees (lanes without a row of this item: every key; their sums are dropped)
-      auto row_of = [&](int b) { return (2 * b + (twice && b == n_mb - 1 ? 0 : upper)) * hr + (rib & 63); };
+      auto row_of = [&](int b) { return (2 * b + (twice && b == n_mb - 1 ? 0 : upper)) * 64 + (rib & 63); };
       auto last_of = [&](int n) { return (a.causal && n < rows) ? (x->L - x->W + (x->row0 + n) / G) : (x->L - 1); };
       if (!mbar_wait_warp(smem_u32(&bars->shares_empty[sp]), spar ^ 1u, abort_flag, ta.wait_cycles)) break;
       // the most restricted row's last key, and the largest first key (0 unless the layer has a sliding window)
@@ -564,7 +587,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
         if (WIN && a.win_left > 0 && n < rows) jlmax = max(jlmax, jm - a.win_left + 1);
         bars->state[sp][grp][b][half][rib] = make_float2(-INFINITY, 0.f);
       }
-      const bool flip = lse_flip(rows, hr) != 0;
+      const bool flip = lse_flip(rows) != 0;
       const int n_jobs = n_tiles * n_mb, b_short = twice ? n_mb - 1 : -1;
       float2* st0 = &bars->state[sp][grp][0][half][rib];
       int key0 = (x->t_begin + (n_mb == 1 ? grp : 0)) * TK + half * 64;
