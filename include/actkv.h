@@ -573,9 +573,11 @@ int actkv_compact_noalloc(const actkv_pool_t* pool /* host */, const actkv_table
  * real fault: while after_tile >= 0, the K-tile producers of every such launch of this process
  * issue no key tile with index >= after_tile of their CTA (nothing is left in flight: the loads are
  * simply not issued), and every wait gives up after about wait_limit_us microseconds instead of the
- * default two seconds.  after_tile < 0 restores normal operation.  Host-side, process-wide, takes
- * effect at the next launch; not for production use.
+ * default two seconds.  after_tile = ACTKV_STALL_ANSWER: every key tile arrives, but the CTAs of the
+ * LSE pass never learn which work item to go on to.  after_tile < 0 restores normal operation.
+ * Host-side, process-wide, takes effect at the next launch; not for production use.
  */
+#define ACTKV_STALL_ANSWER  0x7fffffff
 int actkv_debug_inject_stall(int32_t after_tile, int32_t wait_limit_us);
 
 /* Library version string (host pointer to static storage). */

@@ -16,6 +16,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libactkv.so")
 
 OK, E_INVALID, E_WORKSPACE, E_CUDA, E_BADPAGE, E_NOFREE, E_BADINDEX, E_TIMEOUT = 0, -1, -2, -3, -4, -5, -6, -7
+STALL_ANSWER = 0x7fffffff
 E_TOOBIG = -8
 ERROR_NAMES = {E_INVALID: "ACTKV_E_INVALID", E_WORKSPACE: "ACTKV_E_WORKSPACE", E_CUDA: "ACTKV_E_CUDA",
                E_BADPAGE: "ACTKV_E_BADPAGE", E_NOFREE: "ACTKV_E_NOFREE", E_BADINDEX: "ACTKV_E_BADINDEX",

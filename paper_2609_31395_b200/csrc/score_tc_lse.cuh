@@ -416,8 +416,15 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
       }
       if (p == 0) {
         // (also after giving up: the answer lands in this CTA's shared memory)
-        const bool answered = mbar_wait_warp(smem_u32(&bars->clc), cpar, nullptr, ta.wait_cycles);
+        bool answered = mbar_wait_warp(smem_u32(&bars->clc), cpar, nullptr, ta.wait_cycles);
         cpar ^= 1u;
+        // injected fault: the answer does not arrive (there is no second one to wait for; the roles that wait for the item do so longer)
+        if (ta.stall_tile == STALL_ANSWER) answered = mbar_wait_warp(smem_u32(&bars->clc), cpar, nullptr, ta.wait_cycles / 4);
+        if (!answered) {                         // the CTA it names may have been cancelled: nobody would do its item
+          if (lane == 0) *abort_flag = 1;
+          ok = false;
+          mbar_wait_warp(smem_u32(&bars->clc), cpar ^ 1u, nullptr, DRAIN_LIMIT_CYCLES);
+        }
         const int id = answered ? clc_answer(smem_u32(bars->clc_resp)) : -1;
         fence_proxy_async();                     // (the answer has been read before the next one is written)
         __syncwarp();

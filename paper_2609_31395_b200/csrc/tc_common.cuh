@@ -243,6 +243,8 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+constexpr int32_t STALL_ANSWER = ACTKV_STALL_ANSWER;       // TcArgs::stall_tile: see actkv_debug_inject_stall
+
 struct Exp2Cubic { float c0, c1, c2, c3; };   // 2^f on [-0.5, 0.5] = c0 + f (c1 + f (c2 + f c3))
 
 struct TcArgs {

@@ -80,6 +80,44 @@ def test_a_wait_that_runs_out_is_reported_and_the_step_does_nothing(which):
         assert torch.equal(a, b)
 
 
+def _many_items(seed):
+    # 512 window rows are two items per (unit, chunk): 640 and more, so that every CTA of the LSE pass goes on to others; request 13
+    # alone has more than three key tiles
+    lens = [200 + 2 * i for i in range(16)]
+    lens[13] = 900
+    return synth.Workload("items", 5, 4, 8, lens, [64] * 16, [n // 4 for n in lens], table_style="fragmented", seed=seed)
+
+
+def _lse_stalled(after_tile, seed):
+    """Status of an LSE pass under the injected fault; the same buffers then give the bits of a run without it."""
+    from paper_2609_31395_b200 import harness as H
+    wl = _many_items(seed)
+    b = synth.generate(wl, DEV)
+    comp = H.Compressor(b.pool, b.page_table, b.seq_len, b.free_list, b.free_count, wl.n_q_heads, H.sizes_of(b), want_lse=True)
+    args = (b.q, b.win_indptr, b.tok_indptr, wl.sm_scale, wl.causal, 0, wl.n_layers)
+    comp.run_lse(*args, comp.lse)
+    comp.check_status()
+    want = comp.lse.clone()
+    B.actkv_debug_inject_stall(after_tile, 5000)
+    try:
+        comp.run_lse(*args, comp.lse)
+        torch.cuda.synchronize()
+    finally:
+        B.actkv_debug_inject_stall(-1)
+    st = comp.status.cpu().tolist()
+    comp.status.zero_()
+    comp.lse.fill_(float("nan"))
+    comp.run_lse(*args, comp.lse)
+    comp.check_status()
+    assert torch.equal(comp.lse, want)
+    return wl, st
+
+
+def test_a_lost_answer_about_the_next_item_is_reported():
+    _, st = _lse_stalled(B.STALL_ANSWER, 43)
+    assert st[0] == B.E_TIMEOUT, st
+
+
 def test_hook_rejects_a_stall_without_a_limit():
     with pytest.raises(B.ActKVError):
         B.actkv_debug_inject_stall(0, 0)
