@@ -19,7 +19,7 @@
  *     workspace too small, launch failure).  What only the device can see (a page id out of
  *     range, a free list that is too short) is written to the caller's `status[4]` int32 words:
  *     status[0] = first error code (0 while clean), status[1..2] = where (request / unit,
- *     offending value).  Kernels never trap.  An out-of-range page id met by a score kernel is
+ *     offending value; unit and key chunk of a wait that gave up).  Kernels never trap.  An out-of-range page id met by a score kernel is
  *     replaced by page 0 for the read and reported; a copy whose source or destination page id is
  *     out of range is dropped and reported (nothing is read from or written to a page the request
  *     does not own).  Once status[0] is set, actkv_select and the compaction calls of the same

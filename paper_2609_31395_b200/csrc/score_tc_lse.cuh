@@ -144,6 +144,7 @@ struct LseBarriers {
   uint64_t drained[2];
   uint32_t tmem_base;
   int abort_flag;
+  int at[2];                    // unit and chunk of the item that is being contracted (the first one at first): where a wait gave up
   alignas(16) uint32_t clc_resp[4];
   LseItem item[LSE_ITEMS_AHEAD];
   float2 state[2][2][LSE_MB][2][128];  // (reference e, sum of 2^(v c - e)) per (item parity, group, row block, column half, TMEM lane)
@@ -334,6 +335,8 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
     mbar_init(smem_u32(&bars->drained[0]), 1);
     mbar_init(smem_u32(&bars->drained[1]), 1);
     bars->abort_flag = 0;
+    bars->at[0] = (int)blockIdx.x / ta.n_rg / a.n_chunks;
+    bars->at[1] = (int)blockIdx.x / ta.n_rg % a.n_chunks;
     fence_barrier_init();
   }
   if (warp == 1) {
@@ -476,6 +479,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
       if (!ok) break;
       const int n_tiles = uni(bars->item[slot].n_tiles), rows = uni(bars->item[slot].rows);
       float2* dst = a.partials + ((int64_t)bars->item[slot].u * a.n_chunks + bars->item[slot].chunk) * a.rows_max + bars->item[slot].row0;
+      if (mw == 0 && lane < 2 && n_tiles > 0) bars->at[lane] = lane == 0 ? bars->item[slot].u : bars->item[slot].chunk;
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars->item_empty[slot]));
       if (n_tiles <= 0) break;
@@ -634,7 +638,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
   tc_fence_before();
   __syncthreads();
   if (warp == 0 && lane == 0 && *abort_flag) {
-    report(a.status, ACTKV_E_TIMEOUT, (int)blockIdx.x, 0);
+    report(a.status, ACTKV_E_TIMEOUT, bars->at[0], bars->at[1]);
     // loads still in flight land in this CTA's shared memory: give them a moment before exiting
     for (int s = 0; s < S; ++s) mbar_wait(smem_u32(&bars->k_full[s]), 0, nullptr, DRAIN_LIMIT_CYCLES / 64);
   }

@@ -118,6 +118,14 @@ def test_a_lost_answer_about_the_next_item_is_reported():
     assert st[0] == B.E_TIMEOUT, st
 
 
+def test_the_place_of_a_stall_is_the_unit_and_the_chunk():
+    wl, st = _lse_stalled(3, 44)                   # only request 13 has tiles from the fourth on
+    assert st[0] == B.E_TIMEOUT, st
+    n_units = wl.n_layers * wl.n_kv_heads * wl.n_req
+    assert 0 <= st[1] < n_units and st[1] % wl.n_req == 13, st
+    assert st[2] in (0, 1), st                     # 900 keys are at most two chunks
+
+
 def test_hook_rejects_a_stall_without_a_limit():
     with pytest.raises(B.ActKVError):
         B.actkv_debug_inject_stall(0, 0)
