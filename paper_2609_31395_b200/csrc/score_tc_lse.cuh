@@ -144,6 +144,7 @@ struct LseBarriers {
   uint64_t drained[2];
   uint32_t tmem_base;
   int abort_flag;
+  int issued[2];                // entries of the ring below which a producer has issued its loads
   int at[2];                    // unit and chunk of the item that is being contracted (the first one at first): where a wait gave up
   alignas(16) uint32_t clc_resp[4];
   LseItem item[LSE_ITEMS_AHEAD];
@@ -385,8 +386,8 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
         const int n_half = (x.rows + 63) / 64, n_mb = (n_half + 1) / 2;
         for (int b = 0; b < n_mb && ok; ++b, ++e) {
           if ((e & 1) != p) continue;
-          const int s = e % S;
-          ok = mbar_wait_warp(smem_u32(&bars->k_empty[s]), ((uint32_t)(e / S) & 1u) ^ 1u, abort_flag, ta.wait_cycles);
+          const int s = ring_stage(e, S);
+          ok = mbar_wait_warp(smem_u32(&bars->k_empty[s]), ring_parity(e, S) ^ 1u, abort_flag, ta.wait_cycles);
           if (!ok) break;
           // The two halves of the block; a last half that stands alone is held twice.  Whole groups all of whose rows the item has
           // come as TMA boxes.  Lanes without a row hold zeros: they take part in the votes of the epilogue, so what they hold must be the
@@ -412,9 +413,11 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
         }
         if (ok) {
           const int layer = a.layer_begin + x.slab, first = (p - e) & 1;
-          if (ta.k5) ok = k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
-          else ok = k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
-          e += x.n_tiles;
+          int done;
+          if (ta.k5) done = k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
+          else done = k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
+          ok = done >= x.n_tiles;
+          e += done;
         }
       }
       if (p == 0) {
@@ -443,6 +446,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
         mbar_arrive(smem_u32(&bars->item_full[slot]));
       }
     }
+    if (lane == 0) bars->issued[p] = e;
     __syncwarp();
   } else if (warp == 1 || warp == 3) {
     // ---------------- MMA issuers: A = Q block in TMEM, B = K tile in shared memory ----------------
@@ -637,10 +641,9 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
   // ---------------- teardown ----------------
   tc_fence_before();
   __syncthreads();
-  if (warp == 0 && lane == 0 && *abort_flag) {
-    report(a.status, ACTKV_E_TIMEOUT, bars->at[0], bars->at[1]);
-    // loads still in flight land in this CTA's shared memory: give them a moment before exiting
-    for (int s = 0; s < S; ++s) mbar_wait(smem_u32(&bars->k_full[s]), 0, nullptr, DRAIN_LIMIT_CYCLES / 64);
+  if (warp == 0 && *abort_flag) {
+    if (lane == 0) report(a.status, ACTKV_E_TIMEOUT, bars->at[0], bars->at[1]);
+    drain_loads(bars, S);
   }
   __syncthreads();
   if (warp == 1) {
