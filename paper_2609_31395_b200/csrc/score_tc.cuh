@@ -192,7 +192,7 @@ inline int score_tc_launch_lse_c(const CUtensorMap& kmap, const CUtensorMap& qma
   const size_t smem = (size_t)tc::lse_stages(NH) * NH * tc::HALF_BYTES + sizeof(tc::LseBarriers);
   auto kern = ta.a.win_left > 0 ? tc::score_tc_lse_kernel<NPOLY, NH, true> : tc::score_tc_lse_kernel<NPOLY, NH, false>;
   if (ensure_dyn_smem(kern, smem) != cudaSuccess) return ACTKV_E_CUDA;
-  launch_pdl(kern, grid, tc::LSE_THREADS, smem, s, kmap, qmap, ta);
+  launch_pdl(kern, grid, tc::LSE_THREADS, smem, s, kmap, qmap, ta, tc::Exp2Cubic{tc::EXP2_C0, tc::EXP2_C1, tc::EXP2_C2, tc::EXP2_C3});
   ACTKV_CHECK_LAUNCH();
   return ACTKV_OK;
 }
@@ -204,7 +204,6 @@ inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_w
     return ACTKV_E_CUDA;
   tc::TcArgs ta;
   ta.a = a;
-  ta.cubic = {tc::EXP2_C0, tc::EXP2_C1, tc::EXP2_C2, tc::EXP2_C3};
   ta.n_rg = tc::lse_row_groups(max_win, a.group);
   ta.row_begin = 0;
   ta.k5 = tc::pool_needs_5d(pool) ? 1 : 0;

@@ -298,7 +298,8 @@ __device__ __forceinline__ void lse_merge(const float2 (&state)[2][LSE_MB][2][12
 // NH: 64-dim halves of the head dimension (head_dim = 64 NH); a K tile is NH x [128 keys][64 bf16].
 template <int NPOLY, int NH, bool WIN>
 __global__ void __launch_bounds__(LSE_THREADS, 1)
-score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap qmap, const TcArgs ta) {
+score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap qmap, const TcArgs ta,
+                    const Exp2Cubic cubic) {
   pdl_begin();
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int S = lse_stages(NH);
@@ -578,7 +579,6 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
     const int rib = quarter * 32 + lane;           // TMEM lane
     const int upper = quarter >> 1;                // lanes 64 and up: the second half of a block
     const float c = a.scale_log2;
-    const Exp2Cubic cubic = ta.cubic;
     const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16) + LSE_A_COLS + grp * 128 + half * 64;
     int slot = 0, sp = 0;                          // sp: which `state`
     uint32_t ipar = 0, fpar = 0, spar = 0;

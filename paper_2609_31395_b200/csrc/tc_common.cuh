@@ -250,7 +250,6 @@ struct Exp2Cubic { float c0, c1, c2, c3; };   // 2^f on [-0.5, 0.5] = c0 + f (c1
 
 struct TcArgs {
   ScoreArgs a;
-  Exp2Cubic cubic;           // LSE pass
   int32_t tiles_per_cta;     // pooled-score pass: key tiles per CTA
   int32_t n_kchunks;         // pooled-score pass: CTAs per unit
   int32_t n_rg;              // LSE pass: groups of rows per unit (a grid dimension)
