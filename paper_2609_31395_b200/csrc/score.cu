@@ -110,14 +110,14 @@ static int score_impl(int mode, const actkv_pool_t* pool, const actkv_tables_t* 
   {
     int n_chunks = lay.n_chunks;
     if (use_tc && (mode & 1))
-      n_chunks = tc::lse_split((int64_t)nls * Hkv * R * tc::lse_row_groups(max_win, G), (max_tok + tc::TK - 1) / tc::TK,
+      n_chunks = tc::lse_split((int64_t)nls * Hkv * R * tc::lse_row_groups(max_win * G), (max_tok + tc::TK - 1) / tc::TK,
                                  (double)sum_tok / ((double)R * max_tok), (double)sum_win / ((double)R * max_win),
-                                 max_win * G <= 128 ? 3.0 : 2.0, lay.n_chunks_max);
+                                 tc::lse_item_overhead(max_win * G, D), lay.n_chunks_max);
     int chunk = (max_tok + n_chunks - 1) / n_chunks;
     chunk = (chunk + 127) / 128 * 128;
     if (chunk < LSE_CHUNK) chunk = LSE_CHUNK;
     a.lse_chunk = chunk;
-    a.n_chunks = (max_tok + chunk - 1) / chunk;    // <= lay.n_chunks
+    a.n_chunks = (max_tok + chunk - 1) / chunk;    // <= lay.n_chunks or, tcgen05, lay.n_chunks_max: the partials' size rests on it
   }
   a.scale_log2 = sm_scale * kLog2e;
   a.page_shift = (pool->page_size & (pool->page_size - 1)) == 0 ? __builtin_ctz((unsigned)pool->page_size) : -1;

@@ -72,11 +72,20 @@ inline int best_split(int64_t units, int tiles, int ovh, int n_max) {
   return best;
 }
 
-// Chunks per unit of the LSE pass, whose CTAs go on from item to item, for a launch over `units` units of `tiles` key tiles: an item costs
-// its tiles and `ovh` more (Q blocks into tensor memory, references, merge: 2 to 4 K cycles).  Equal units run in rounds of 148 of which the
-// last is partly empty; requests of different lengths or windows (mean over longest: `len`, `win`) spread evenly but for the
-// last items, half of one on average.  Returns the count in [1, n_max] that costs least, preferring fewer unless more are clearly better.
-// 8 layers of 4 x 11000 keys, head_dim 64, 200-448 rows: 450 us with whole units, 350 with the four chunks this gives.
+// What a work item of the LSE pass costs beside its key tiles, in tiles (Q blocks into tensor memory, references, merge): 4 K cycles; 8 K
+// where its Q blocks wait for the columns of the item before (measured from job to job: 2157 cycles a tile of two blocks in whole units, 2423
+// on average in eight chunks; three blocks 2255 x 1.5, and 2615 x 1.5).
+inline double lse_item_overhead(int rows, int head_dim) {
+  return rows <= 128 ? 3.0 : rows > 256 && rows <= 384 && head_dim == 128 ? 2.8 : 2.0;
+}
+
+// Chunks per unit of the LSE pass, whose CTAs go on from item to item, for a launch over `units` units of `tiles` key tiles, an item costing
+// its tiles and `ovh` more.  Equal units run in rounds of 148 of which the last is partly empty; requests of different lengths or windows
+// (mean over longest: `len`, `win`) spread evenly but for the last items, half of one on average, once there are more items than SMs.
+// Returns the count in [1, n_max] that costs least, preferring fewer unless more are clearly better.
+// 8 layers x 8 heads, 4 requests of 6500-15000 keys, head_dim 64, 200-512 rows: 410 us with whole units, 341 with the three chunks this
+// gives (four 336, five 334, eight 344).  4 layers x 8 heads, 4 x 16000 keys, 192 rows: 148 us with whole units, 158 with eight chunks (a
+// difference of 0.5 % in the model decided for those before).
 inline int lse_split(int64_t units, int tiles, double len, double win, double ovh, int n_max) {
   const bool equal = len > 0.999 && win > 0.999;
   int best = 1;
@@ -87,15 +96,11 @@ inline int lse_split(int64_t units, int tiles, double len, double win, double ov
     const int64_t items = units * ((tiles + tpc - 1) / tpc);
     double t;
     if (equal) t = (double)((items + 147) / 148) * (tpc + ovh);
+    else if (items <= 148) t = tpc + ovh;
     else t = ((double)units * tiles * len * win + (double)items * len * ovh) / 148.0 + 0.5 * (tpc + ovh);
-    if (t < best_t * 0.995) { best_t = t; best = n; }
+    if (t < best_t * 0.99) { best_t = t; best = n; }
   }
   return best;
-}
-
-// Items of the LSE pass side by side for a window of max_win tokens.
-inline int lse_row_groups(int max_win, int g) {
-  return (max_win * g + LSE_MB * 128 - 1) / (LSE_MB * 128);
 }
 
 inline bool make_kmap(const actkv_pool_t* pool, CUtensorMap* kmap) {
@@ -204,7 +209,7 @@ inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_w
     return ACTKV_E_CUDA;
   tc::TcArgs ta;
   ta.a = a;
-  ta.n_rg = tc::lse_row_groups(max_win, a.group);
+  ta.n_rg = tc::lse_row_groups(max_win * a.group);
   ta.row_begin = 0;
   ta.k5 = tc::pool_needs_5d(pool) ? 1 : 0;
   ta.n_stages = 0;

@@ -3,8 +3,8 @@
 //
 // D[row, key] = Q K^T with the rows on the TMEM lanes, so every epilogue thread owns one row per
 // 128-row block and folds its share of the row's logits into a running (reference, sum of exp2): no
-// shuffles.  A work item is up to two row blocks (256 rows) of a unit x one chunk of keys; the items of a longer window stand
-// side by side and read its keys from L2.
+// shuffles.  A work item is up to three row blocks of a unit (two where a window is longer than 384 rows) x one chunk of keys; the items of
+// a longer window stand side by side and each fetches the keys.
 //
 // Operand placement.  An A operand in shared memory is re-read for every MMA and that read is not
 // overlapped with the MMA (measured 105 cycles per 128x128x16 MMA against 74 with A in tensor memory,
@@ -19,14 +19,15 @@
 // Items.  One CTA per SM, which goes on from item to item: the first is its own blockIdx, the next ones those of CTAs that have
 // not been launched yet (cluster launch control), so requests of different lengths and windows spread over the SMs by themselves.
 // In the ring of stages an item is its Q blocks, then its K tiles; the producers run ahead into the next item, whose
-// Q blocks go to the other half of the Q columns, and warp 3 merges the shares of an item while the epilogue is in the next.  With a
-// CTA per item 12 to 20 K cycles passed before its first job was done, beside 1030 for a job; from item to item it is 2 K.  With one
+// Q blocks go to the other half of the Q columns (three blocks at head_dim 128 wait for it), and warp 3 merges the shares of an item while
+// the epilogue is in the next.  With a CTA per item 12 to 20 K cycles passed before its first job was done, beside 1030 for a job; from item to item it is 2 K.  With one
 // producer a unit of one row block waited for its key tiles.  A last block of at most 64 rows is held twice and each copy folds half of
 // its columns.
 // LSE pass, us, before and after: 4 layers x 8 heads, 8 x 16000 keys, 128 rows 280 -> 184, 192 rows 332 -> 284, head_dim 64 and 256 rows
-// 309 -> 289; 2 x 32768 keys, 256 rows 190 -> 170; 4 x 16000 keys, 384 rows 248 -> 261, 512 rows 320 -> 301; 8 layers x 8 heads, 16 requests of
+// 309 -> 289; 2 x 32768 keys, 256 rows 190 -> 170; 4 x 16000 keys, 512 rows 320 -> 301; 8 layers x 8 heads, 16 requests of
 // 12000-20000 keys and 140-348 rows 1628 -> 1387.  In a loop of seconds, at the power cap: 36 layers of 32768 keys, 256 rows 828 -> 823, 8 layers of
-// 8 x 35000 keys, 512 rows 1440 -> 1420.
+// 8 x 35000 keys, 512 rows 1440 -> 1420.  Slower than a CTA per unit: 353 to 384 rows (4 x 16000 keys, 384 rows 240 -> 252; with two items a
+// unit 258).
 //
 // What bounds the kernel (measured on B200 with micro-benchmarks and per-job timestamps):
 //  * Issuing is not free: a tcgen05.mma costs the issuing thread about 50 cycles and a tcgen05.commit
@@ -113,12 +114,20 @@ constexpr int LSE_EPI_WARPS = 16;                // (TMEM lane quarter, accumula
 constexpr int LSE_EPI_WARP0 = 4;
 constexpr int LSE_THREADS = (LSE_EPI_WARP0 + LSE_EPI_WARPS) * 32;
 constexpr int LSE_SLOTS = 2;                     // accumulators
-constexpr int LSE_MB = 2;                        // row blocks of an item
+constexpr int LSE_MB = 3;                        // row blocks of an item, at most
 constexpr int LSE_A_COLS = 256;                  // TMEM columns holding Q blocks, a half for each of two items
 constexpr int LSE_ITEMS_AHEAD = 3;               // item descriptors in shared memory
 __host__ __device__ constexpr int lse_stages(int nh) { return nh == 1 ? 8 : 6; }             // K tiles (or Q blocks) in shared memory
 constexpr float LSE_BIG = 1099511627776.f;       // 2^40: a partial sum beyond it moves the reference
 constexpr float LSE_REF_MAX = 1048576.f;         // references beyond 2^20 (rounding to integers needs |v c| < 2^22) take the general form
+
+// Row groups per unit of a launch whose longest window has `rows` rows, and rows of a group: two blocks, or one group of three.  A third
+// block as an item of its own fetches all key tiles once more for half the products (4 layers x 8 heads, 4 x 16000 keys, us, two items / one:
+// 260 rows 250 / 219, 320 251 / 223, 384 258 / 252; head_dim 64, 8 layers, 4 x 11000 keys, group 8: 264 rows 300 / 279, 384 326 / 314).  Beyond
+// 384 rows groups of three were slower than of two, since fewer and larger items end less evenly: 640 rows, 2 layers x 4 heads, 4 x 8000 keys
+// 67.5 / 75.3.
+__host__ __device__ constexpr int lse_row_groups(int rows) { return rows <= 384 ? 1 : (rows + 255) / 256; }
+__host__ __device__ constexpr int lse_group_rows(int n_rg) { return n_rg == 1 ? 384 : 256; }
 
 // Two blocks of which the second is short change places on odd tiles (exclusive or with this): the short one would otherwise always
 // fall to the same accumulator.
@@ -221,8 +230,8 @@ __device__ __forceinline__ LseItem lse_item(const TcArgs& ta, int id, int lane) 
   x.L = a.tab.seq_len[x.r];
   x.w0 = a.win_indptr[x.r];
   x.W = a.win_indptr[x.r + 1] - x.w0;
-  x.row0 = rg * LSE_MB * 128;
-  x.rows = min(x.W * G - x.row0, LSE_MB * 128);
+  x.row0 = rg * lse_group_rows(ta.n_rg);
+  x.rows = min(x.W * G - x.row0, lse_group_rows(ta.n_rg));
   const int key_begin = x.chunk * a.lse_chunk;
   if (key_begin >= x.L || (rg > 0 && x.rows <= 0)) return x;
   if (x.W <= 0 || (a.causal && x.W > x.L)) {
@@ -304,7 +313,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int S = lse_stages(NH);
   constexpr int QCOLS = 32 * NH;                         // TMEM columns of a Q block
-  static_assert(LSE_MB * QCOLS <= LSE_A_COLS / 2, "Q columns");
+  static_assert(LSE_MB * QCOLS <= LSE_A_COLS, "Q columns");
   const ScoreArgs& a = ta.a;
   const int G = a.group;
 
@@ -490,12 +499,16 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
       if (n_tiles <= 0) break;
       if (++slot == LSE_ITEMS_AHEAD) { slot = 0; ipar ^= 1u; }
       const int n_mb = (rows + 127) / 128;
-      // the Q blocks go to the half of the Q columns that the previous item does not use
-      const uint32_t q_tmem = tmem_base + (uint32_t)qh * (LSE_A_COLS / 2);
+      // the Q blocks go to the half of the Q columns that the previous item does not use; three at head_dim 128 take the first part of the
+      // other half too, and wait until that item's products are done
+      const uint32_t q_col = (uint32_t)qh * (LSE_A_COLS / 2);
+      auto q_block = [&](int b) { return tmem_base + ((q_col + b * QCOLS) & (LSE_A_COLS - 1)); };
+      const bool both = n_mb * QCOLS > LSE_A_COLS / 2;
       if (mw == 0) {
         ok = mbar_wait_warp(smem_u32(&bars->q_free[qh]), (qpar >> qh) & 1u, abort_flag, ta.wait_cycles);
+        if (ok && both) ok = mbar_wait_warp(smem_u32(&bars->q_free[qh ^ 1]), (qpar >> (qh ^ 1)) & 1u, abort_flag, ta.wait_cycles);
         if (!ok) break;
-        qpar ^= 1u << qh;
+        qpar ^= both ? 3u : 1u << qh;
       }
       for (int b = 0; b < n_mb; ++b) {
         ok = mbar_wait_warp(smem_u32(&bars->k_full[s]), kpar, abort_flag, ta.wait_cycles);
@@ -506,7 +519,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
             const uint64_t desc_s = desc0 + (uint64_t)((s * (NH * HALF_BYTES)) >> 4);
 #pragma unroll
             for (int kk = 0; kk < 4 * NH; ++kk)
-              tmem_cp_k16(q_tmem + b * QCOLS + kk * 8, desc_s + (uint64_t)(((kk >> 2) * HALF_BYTES + (kk & 3) * 32) >> 4));
+              tmem_cp_k16(q_block(b) + kk * 8, desc_s + (uint64_t)(((kk >> 2) * HALF_BYTES + (kk & 3) * 32) >> 4));
             umma_commit(smem_u32(&bars->k_empty[s]));
             if (b == n_mb - 1) umma_commit(smem_u32(&bars->q_ready[qh]));
           } else {
@@ -533,7 +546,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
           epar ^= 1u;
           tc_fence_after();
           if (leader) {
-            const uint32_t at = q_tmem + (i ^ flip) * QCOLS;
+            const uint32_t at = q_block(i ^ flip);
 #pragma unroll
             for (int kk = 0; kk < 4 * NH; ++kk)
               umma_bf16_ts(d, at + kk * 8, desc_s + (uint64_t)(((kk >> 2) * HALF_BYTES + (kk & 3) * 32) >> 4), idesc,
@@ -559,7 +572,10 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
       if (!ok) break;
       m_rows = rows;
       m_dst = dst;
-      if (leader) umma_commit(smem_u32(&bars->q_free[qh]));
+      if (leader) {
+        umma_commit(smem_u32(&bars->q_free[qh]));
+        if (both) umma_commit(smem_u32(&bars->q_free[qh ^ 1]));
+      }
       qh ^= 1;
     }
     if (ok && mw == 1 && m_rows > 0) ok = merge();
@@ -602,31 +618,40 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
         if (WIN && a.win_left > 0 && n < rows) jlmax = max(jlmax, jm - a.win_left + 1);
         bars->state[sp][grp][b][half][rib] = make_float2(-INFINITY, 0.f);
       }
-      const bool flip = lse_flip(rows) != 0;
+      const bool moves = lse_flip(rows) != 0 || n_mb == 3;
       const int n_jobs = n_tiles * n_mb, b_short = twice ? n_mb - 1 : -1;
       float2* st0 = &bars->state[sp][grp][0][half][rib];
       int key0 = (x->t_begin + (n_mb == 1 ? grp : 0)) * TK + half * 64;
-      // A group that stays with one row block keeps its (reference, sum) in registers and has little left to count per job.
+      // Two blocks that change places, and three: the next job is of the block before this one, cyclically, and of the same tile only
+      // from the first of three to the last.  The (reference, sum) of all blocks stay in registers: ms is the next job's, m1 and m2 the
+      // ones after it (in shared memory 284 -> 276 us for 384 rows, 4 layers x 8 heads, 4 x 16000 keys, at the power cap; 192 rows 179 -> 174).
       int b = n_mb == 1 ? 0 : grp;
       bool wide = b != b_short;
       int off = wide ? 0 : upper * 32;
       const int step = n_mb == 1 ? 2 * TK : TK;
-      float2 ms = make_float2(-INFINITY, 0.f);
+      float2 ms = make_float2(-INFINITY, 0.f), m1 = ms, m2 = ms;
       for (int j = grp; j < n_jobs; j += 2) {
         ok = lse_job<NPOLY, WIN>(bars, abort_flag, tq + off, grp, fpar, wide, [&]() { return last_of(row_of(b)); }, ms,
                                  jfast - key0 - off + 1, jlmax - key0 - off, a.win_left, key0 + off, c, cubic, ta.wait_cycles);
         if (!ok) break;
         fpar ^= 1u;
         key0 += step;
-        if (flip) {                                // the other block
-          st0[b * (2 * 128)] = ms;
-          b ^= 1;
+        if (moves) {
+          if (b == 0 && n_mb == 3) key0 -= TK;
+          b = (b == 0 ? n_mb : b) - 1;
           wide = b != b_short;
           off = wide ? 0 : upper * 32;
-          ms = st0[b * (2 * 128)];
+          const float2 t = ms;
+          ms = m1;
+          if (n_mb == 3) { m1 = m2; m2 = t; } else m1 = t;
         }
       }
-      if (!flip && grp < n_jobs) st0[b * (2 * 128)] = ms;
+      if (moves || grp < n_jobs) st0[b * (2 * 128)] = ms;
+      if (moves) {
+        b = (b == 0 ? n_mb : b) - 1;
+        st0[b * (2 * 128)] = m1;
+        if (n_mb == 3) st0[(b == 0 ? 2 : b - 1) * (2 * 128)] = m2;
+      }
       if (!ok) break;
       __syncwarp();
       if (lane == 0) {

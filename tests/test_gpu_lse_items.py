@@ -58,6 +58,27 @@ def test_rows_around_the_edges_of_items(group, windows, head_dim, causal):
         assert torch.equal(x, runs[0])
 
 
+@pytest.mark.parametrize("head_dim", [128, 64])
+@pytest.mark.parametrize("max_rows", [384, 800])
+def test_items_of_one_to_three_blocks_in_turn(max_rows, head_dim):
+    # an item of three blocks takes Q columns of both halves at head_dim 128: every order of items of different widths in one CTA
+    rows = [n for n in (260, 384, 64, 320, 256, 324, 128, 192, 388, 512, 516, 640, 644, 768, 772, 800) if n <= max_rows]
+    windows = [n // 4 for n in rows + rows[::-1]]
+    lens = [max(w, 130 + 67 * i) for i, w in enumerate(windows)]
+    wl = synth.Workload("blocks", 8, 4, 4, lens, windows, [n // 4 for n in lens], head_dim=head_dim, causal=True,
+                        table_style="fragmented", seed=73)
+    b = synth.generate(wl, DEV)
+    comp = H.Compressor(b.pool, b.page_table, b.seq_len, b.free_list, b.free_count, wl.n_q_heads, H.sizes_of(b), want_lse=True)
+    runs = []
+    for _ in range(3):
+        comp.lse.fill_(float("nan"))
+        comp.run_lse(b.q, b.win_indptr, b.tok_indptr, wl.sm_scale, wl.causal, 0, wl.n_layers, comp.lse)
+        runs.append(comp.lse.clone())
+    comp.check_status()
+    assert (runs[0].double() - _lse64(b)).abs().max() < 1e-4        # (the cubic and float32 dot products, as above)
+    assert torch.equal(runs[1], runs[0]) and torch.equal(runs[2], runs[0])
+
+
 @pytest.mark.parametrize("group,windows,lens,head_dim,causal", [
     (4, [32], [4096], 128, False),                       # one item of rows, eight chunks
     (4, [64, 17], [1500, 129], 128, True),               # a full item, and one of 68 rows
