@@ -223,6 +223,6 @@ int actkv_debug_inject_stall(int32_t after_tile, int32_t wait_limit_us) {
   return ACTKV_OK;
 }
 
-const char* actkv_version(void) { return "actkv-b200 0.2 (sm_100a)"; }
+const char* actkv_version(void) { return "actkv-b200 0.3 (sm_100a)"; }
 
 }  // extern "C"
