@@ -165,8 +165,8 @@ inline void apply_hook(TcArgs& ta) {
 
 // The tensor-core path takes: pages of 16, 32, 64 or 128 tokens, head_dim 128 or 64, slot-major or head-major pages (any
 // strides that are multiples of 16 bytes), 128-byte aligned base, group size <= 32 (padded to a power of two in the
-// pooled-score pass), min_rows <= window x group rows <= 4096 (a CTA handles up to 512; more are taken in groups of 512
-// rows), positive softmax scale.
+// pooled-score pass), min_rows <= window x group rows <= 4096 (more than 512 are taken in groups: of 512 rows a launch in the
+// pooled-score pass, of 256 an item in the LSE pass), positive softmax scale.
 // The full score (LSE + pooled pass) takes it from 64 rows up; the streaming update, which runs the pooled pass alone and is
 // bound by the K reads, from a single row.  The two families, us, 4 layers x 8 heads, 8 requests of 9000 keys, head_dim 128,
 // group 4 (mma.sync beyond 48 rows on a pool 16 bytes off the 128-byte boundary, which costs it up to a quarter):

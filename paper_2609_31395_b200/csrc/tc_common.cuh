@@ -15,8 +15,8 @@ constexpr int HD = 128;                      // head dim
 constexpr uint32_t HALF_BYTES = TK * 64 * 2;         // 16 KB
 constexpr uint32_t QBLK_BYTES = 128 * HD * 2;        // 32 KB per 128 rows
 constexpr size_t SMEM_LIMIT = 232448;        // 227 KB of dynamic shared memory per CTA
-constexpr int MAX_ROWS = 512;                // window x group rows (padded to 128) one CTA handles
-constexpr int MAX_ROWS_TOTAL = 4096;         // ... per unit: more than MAX_ROWS are taken in groups of MAX_ROWS
+constexpr int MAX_ROWS = 512;                // window x group rows (padded to 128) a CTA of the pooled-score pass handles
+constexpr int MAX_ROWS_TOTAL = 4096;         // ... per unit: that pass takes more than MAX_ROWS in groups of MAX_ROWS
 // Bounded waits are counted on the SM cycle counter (cheap to read, unlike the global nanosecond timer).  The
 // counter runs at 2.1 GHz at most, so a limit of n cycles lasts at least n / 2.1 ns.
 constexpr long long WAIT_LIMIT_CYCLES = 4000000000ll;      // default limit of a wait: about two seconds
