@@ -84,8 +84,8 @@ inline double lse_item_overhead(int rows, int head_dim) {
 // (mean over longest: `len`, `win`) spread evenly but for the last items, half of one on average, once there are more items than SMs.
 // Returns the count in [1, n_max] that costs least, preferring fewer unless more are clearly better.
 // 8 layers x 8 heads, 4 requests of 6500-15000 keys, head_dim 64, 200-512 rows: 410 us with whole units, 341 with the three chunks this
-// gives (four 336, five 334, eight 344).  4 layers x 8 heads, 4 x 16000 keys, 192 rows: 148 us with whole units, 158 with eight chunks (a
-// difference of 0.5 % in the model decided for those before).
+// gives (four 336, five 334, eight 344).  4 layers x 8 heads, 4 x 16000 keys, 192 rows: 148 us with whole units, 158 with eight chunks (half
+// a percent in the model decided for those before).
 inline int lse_split(int64_t units, int tiles, double len, double win, double ovh, int n_max) {
   const bool equal = len > 0.999 && win > 0.999;
   int best = 1;
@@ -98,7 +98,7 @@ inline int lse_split(int64_t units, int tiles, double len, double win, double ov
     if (equal) t = (double)((items + 147) / 148) * (tpc + ovh);
     else if (items <= 148) t = tpc + ovh;
     else t = ((double)units * tiles * len * win + (double)items * len * ovh) / 148.0 + 0.5 * (tpc + ovh);
-    if (t < best_t * 0.99) { best_t = t; best = n; }
+    if (t < best_t * (equal ? 0.99 : 0.995)) { best_t = t; best = n; }
   }
   return best;
 }
