@@ -153,7 +153,7 @@ struct LseBarriers {
   uint64_t drained[2];
   uint32_t tmem_base;
   int abort_flag;
-  int issued[2];                // entries of the ring below which a producer has issued its loads
+  uint32_t k_last[8];           // parity of a stage's last load (RING_UNUSED: none yet)
   int at[2];                    // unit and chunk of the item that is being contracted (the first one at first): where a wait gave up
   alignas(16) uint32_t clc_resp[4];
   LseItem item[LSE_ITEMS_AHEAD];
@@ -330,7 +330,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
   LseItem x_next;
   if (warp == 0) x_next = lse_item<WIN>(ta, blockIdx.x, lane);     // (its loads are under way while the others set up)
   if (threadIdx.x == 96) {
-    for (int s = 0; s < S; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 2); }
+    for (int s = 0; s < S; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 2); bars->k_last[s] = RING_UNUSED; }
     for (int i = 0; i < LSE_ITEMS_AHEAD; ++i) {
       mbar_init(smem_u32(&bars->item_full[i]), 1);
       mbar_init(smem_u32(&bars->item_empty[i]), LSE_EPI_WARPS + 3);
@@ -413,7 +413,7 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
             fence_proxy_async();                 // (the copies are read by tcgen05.cp)
             __syncwarp();
           }
-          if (lane == 0) mbar_expect_tx(bar, (uint32_t)(n_box * NH) * (HALF_BYTES / 2));
+          if (lane == 0) { bars->k_last[s] = ring_parity(e, S); mbar_expect_tx(bar, (uint32_t)(n_box * NH) * (HALF_BYTES / 2)); }
           __syncwarp();
           if (lane < 2 * NH && is_box(lane & 1)) {
             const int hf = lane >> 1, j = lane & 1;
@@ -423,11 +423,9 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
         }
         if (ok) {
           const int layer = a.layer_begin + x.slab, first = (p - e) & 1;
-          int done;
-          if (ta.k5) done = k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
-          else done = k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
-          ok = done >= x.n_tiles;
-          e += done;
+          if (ta.k5) ok = k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
+          else ok = k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, x.r, x.layer_h, layer, x.L, x.t_begin, x.n_tiles, lane, abort_flag, first, 2, ta.wait_cycles, ta.stall_tile, e);
+          e += x.n_tiles;
         }
       }
       if (p == 0) {
@@ -456,7 +454,6 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
         mbar_arrive(smem_u32(&bars->item_full[slot]));
       }
     }
-    if (lane == 0) bars->issued[p] = e;
     __syncwarp();
   } else if (warp == 1 || warp == 3) {
     // ---------------- MMA issuers: A = Q block in TMEM, B = K tile in shared memory ----------------
@@ -666,8 +663,8 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
   // ---------------- teardown ----------------
   tc_fence_before();
   __syncthreads();
-  if (warp == 0 && *abort_flag) {
-    if (lane == 0) report(a.status, ACTKV_E_TIMEOUT, bars->at[0], bars->at[1]);
+  if (warp == 0 && lane == 0 && *abort_flag) {
+    report(a.status, ACTKV_E_TIMEOUT, bars->at[0], bars->at[1]);
     drain_loads(bars, S);
   }
   __syncthreads();

@@ -37,7 +37,7 @@ struct PoolBarriers {
   uint64_t drained[2];
   uint32_t tmem_base;
   int abort_flag;
-  int issued[2];              // key tiles below which a producer has issued its loads
+  uint32_t k_last[8];         // parity of a stage's last load (RING_UNUSED: none yet)
   int prod_done;              // the first producer has issued its last key tile: the copy role takes no more items
   float exch[TK];
 };
@@ -310,7 +310,7 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
     return;
   }
   if (threadIdx.x == 0) {
-    for (int s = 0; s < S; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 2); }
+    for (int s = 0; s < S; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 2); bars->k_last[s] = RING_UNUSED; }
     mbar_init(smem_u32(&bars->q_full), 1);
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&bars->tmem_full[b]), 1);
@@ -381,16 +381,13 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
           tma_load_3d(q_smem + (qb >> 1) * NH * QBLK_BYTES + hf * QBLK_BYTES + (qb & 1) * HALF_BYTES, &qmap,
                       smem_u32(&bars->q_full), hf * 64, h * a.group, wrow + qb * (128 / G));
     }
-    int done;
-    if (ta.k5) done = k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 0, 2, ta.wait_cycles, ta.stall_tile);
-    else done = k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 0, 2, ta.wait_cycles, ta.stall_tile);
-    if (lane == 0) { bars->prod_done = 1; bars->issued[0] = done; }
+    if (ta.k5) k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 0, 2, ta.wait_cycles, ta.stall_tile);
+    else k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 0, 2, ta.wait_cycles, ta.stall_tile);
+    if (lane == 0) bars->prod_done = 1;
   } else if (warp == POOL_PRODUCER2) {
     const int layer = a.layer_begin + slab;
-    int done;
-    if (ta.k5) done = k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 1, 2, ta.wait_cycles, ta.stall_tile);
-    else done = k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 1, 2, ta.wait_cycles, ta.stall_tile);
-    if (lane == 0) bars->issued[1] = done;
+    if (ta.k5) k_tile_producer<true, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 1, 2, ta.wait_cycles, ta.stall_tile);
+    else k_tile_producer<false, NH>(&kmap, a, bars, k_smem, S, r, h, layer, L, t_begin, n_tiles, lane, abort_flag, 1, 2, ta.wait_cycles, ta.stall_tile);
   } else {
     // ---------------- MMA issuers: D[key, row] = K Q^T ----------------
     // Two warps, one per accumulator: warp 1 issues the even jobs, warp 2 the odd ones.  Issuing costs the
@@ -552,9 +549,9 @@ score_tc_pool_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
   // ---------------- teardown ----------------
   tc_fence_before();
   __syncthreads();
-  if (warp == 0 && *abort_flag) {
-    if (lane == 0) report(a.status, ACTKV_E_TIMEOUT, u, kchunk);
-    mbar_wait_warp(smem_u32(&bars->q_full), 0, nullptr, DRAIN_LIMIT_CYCLES / 64);
+  if (warp == 0 && lane == 0 && *abort_flag) {
+    report(a.status, ACTKV_E_TIMEOUT, u, kchunk);
+    mbar_wait(smem_u32(&bars->q_full), 0, nullptr, DRAIN_LIMIT_CYCLES / 64);
     drain_loads(bars, S);
   }
   __syncthreads();

@@ -271,8 +271,8 @@ __device__ __forceinline__ int32_t page_for_tile(const TablesView& tab, int32_t 
 
 // The K-tile producers of both score kernels: producer p of P takes tiles p, p + P, ... of
 // [t_begin, t_begin + n_tiles) of request r, head h, layer `layer` through the block table into the ring of S
-// stages (tile i is entry e0 + i of the ring), one TMA box per (page, 64-dim half), one box per lane.  Returns n_tiles, or the first of
-// its tiles that it did not issue because a wait gave up or the injected fault stopped it.  Pages of 16, 32, 64 or 128 tokens: a
+// stages (tile i is entry e0 + i of the ring), one TMA box per (page, 64-dim half), one box per lane.  False when a wait gave up or the
+// injected fault stopped it.  Pages of 16, 32, 64 or 128 tokens: a
 // tile of 128 keys is ppt = 128 / page_size pages, a box page_size rows of 128 B.
 // Measured on B200 (boxes of 16 rows x 128 B from random pages): one warp issuing a tile's 16 boxes from
 // 8 lanes delivers a tile per 1950 cycles, from 16 lanes per 1570, two warps per 1235, four per 1180 (the
@@ -281,7 +281,7 @@ __device__ __forceinline__ int32_t page_for_tile(const TablesView& tab, int32_t 
 // lane % ppt = page); the next group's ids are loaded while the current four tiles are being issued.
 // K5: five-dimensional tensor map (pages that are not slot-major).
 template <bool K5, int NH, class Bars>
-__device__ __forceinline__ int k_tile_producer(const CUtensorMap* kmap, const ScoreArgs& a, Bars* bars, uint32_t k_smem,
+__device__ __forceinline__ bool k_tile_producer(const CUtensorMap* kmap, const ScoreArgs& a, Bars* bars, uint32_t k_smem,
                                                 int S, int r, int h, int layer, int L, int t_begin, int n_tiles,
                                                 int lane, volatile int* abort_flag, int p, int P, long long wait_cycles,
                                                 int stall_tile, int e0 = 0) {
@@ -291,13 +291,13 @@ __device__ __forceinline__ int k_tile_producer(const CUtensorMap* kmap, const Sc
   const uint32_t box_bytes = (uint32_t)ps * 128u;
   const int n_lp = (L + ps - 1) / ps;
   const int n_mine = (n_tiles - p + P - 1) / P;                  // tiles p, p + P, ... below n_tiles
-  if (n_mine <= 0) return n_tiles;
+  if (n_mine <= 0) return true;
   const int g_tile = lane >> lp_shift, g_page = lane & (ppt - 1);            // this lane's slot in a group of four tiles
   int32_t pid = page_for_tile(a.tab, a.pool.n_pages, r, (t_begin + p + min(g_tile, 3) * P) * ppt + g_page, n_lp, a.status);
   int32_t pid_next = 0;
   for (int i = 0; i < n_mine; ++i) {
     const int it = p + i * P;
-    if (stall_tile >= 0 && it >= stall_tile) return it;          // injected fault: this and all later tiles never arrive
+    if (stall_tile >= 0 && it >= stall_tile) return false;       // injected fault: this and all later tiles never arrive
     const int s = ring_stage(e0 + it, S);
     const uint32_t ph = ring_parity(e0 + it, S);
     if ((i & 3) == 0 && i + 4 < n_mine)
@@ -306,10 +306,10 @@ __device__ __forceinline__ int k_tile_producer(const CUtensorMap* kmap, const Sc
     int ok = 1;
     if (lane == 0) {
       ok = mbar_wait(smem_u32(&bars->k_empty[s]), ph ^ 1u, abort_flag, wait_cycles) ? 1 : 0;
-      if (ok) mbar_expect_tx(smem_u32(&bars->k_full[s]), NH * HALF_BYTES);
+      if (ok) { bars->k_last[s] = ph; mbar_expect_tx(smem_u32(&bars->k_full[s]), NH * HALF_BYTES); }
     }
     ok = __shfl_sync(0xffffffffu, ok, 0);
-    if (!ok) return it;
+    if (!ok) return false;
     // lane j < ppt NH: page j % ppt, half j / ppt of this tile
     const int32_t my_pid = __shfl_sync(0xffffffffu, pid, ((i & 3) << lp_shift) | (lane & (ppt - 1)));
     if (lane < ppt * NH) {
@@ -321,14 +321,15 @@ __device__ __forceinline__ int k_tile_producer(const CUtensorMap* kmap, const Sc
     }
     if ((i & 3) == 3) pid = pid_next;
   }
-  return n_tiles;
+  return true;
 }
 
-// Tear-down after a give-up: the key tiles (and Q blocks) still in flight land in this CTA's shared memory; they are waited for, with a
-// limit.  Called by a whole warp.
+// Tear-down after a give-up: the key tiles (and Q blocks) still in flight land in this CTA's shared memory; one thread waits for them, with
+// a limit.  (In this form, with the parities recorded as the loads are issued: with the last load of each stage worked out here the
+// pooled-score kernel was 2 % slower, 24 layers of 4 requests, head_dim 64: 471 -> 482 us, though nothing ever runs it.)
 template <class Bars>
 __device__ __forceinline__ void drain_loads(Bars* bars, int S) {
-  ring_drain(bars->issued, S, [&](int s, uint32_t parity) { mbar_wait_warp(smem_u32(&bars->k_full[s]), parity, nullptr, DRAIN_LIMIT_CYCLES / 64); });
+  for (int s = 0; s < S; ++s) mbar_wait(smem_u32(&bars->k_full[s]), bars->k_last[s], nullptr, DRAIN_LIMIT_CYCLES / 64);
 }
 
 }  // namespace tc

@@ -30,8 +30,12 @@ int main() {
           if (!possible) continue;
           std::vector<int> phases(S);                               // completed phases of the stage's barrier
           for (int s = 0; s < S; ++s) phases[s] = last[s] < 0 ? 0 : last[s] / S + ((flight >> s & 1) ? 0 : 1);
-          std::vector<bool> held(S, false);                         // a wait for parity x passes when the phase under way has the other parity
-          ring_drain(ends, S, [&](int s, unsigned par) { if ((unsigned)(phases[s] & 1) == par) held[s] = true; });
+          // what the producers recorded; a wait for parity x passes when the phase under way has the other parity
+          std::vector<unsigned> recorded(S, RING_UNUSED);
+          for (int e = 0; e < std::max(end0, end1); ++e)
+            if (e < ends[e % 2]) recorded[ring_stage(e, S)] = ring_parity(e, S);
+          std::vector<bool> held(S);
+          for (int s = 0; s < S; ++s) held[s] = (unsigned)(phases[s] & 1) == recorded[s];
           for (int s = 0; s < S; ++s) bad += held[s] != (last[s] >= 0 && (flight >> s & 1));
         }
       }
