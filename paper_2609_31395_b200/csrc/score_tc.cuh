@@ -191,11 +191,11 @@ inline bool score_tc_supported(const actkv_pool_t* p, int G, int max_win, float 
   return tc::encode_fn() != nullptr;
 }
 
-template <int NH>
+template <int NH, bool REGS>
 inline int score_tc_launch_lse_c(const CUtensorMap& kmap, const CUtensorMap& qmap, const tc::TcArgs& ta, unsigned grid, cudaStream_t s) {
   constexpr int NPOLY = tc::LSE_NPOLY;
   const size_t smem = (size_t)tc::lse_stages(NH) * NH * tc::HALF_BYTES + sizeof(tc::LseBarriers);
-  auto kern = ta.a.win_left > 0 ? tc::score_tc_lse_kernel<NPOLY, NH, true> : tc::score_tc_lse_kernel<NPOLY, NH, false>;
+  auto kern = ta.a.win_left > 0 ? tc::score_tc_lse_kernel<NPOLY, NH, true, REGS> : tc::score_tc_lse_kernel<NPOLY, NH, false, REGS>;
   if (ensure_dyn_smem(kern, smem) != cudaSuccess) return ACTKV_E_CUDA;
   launch_pdl(kern, grid, tc::LSE_THREADS, smem, s, kmap, qmap, ta, tc::Exp2Cubic{tc::EXP2_C0, tc::EXP2_C1, tc::EXP2_C2, tc::EXP2_C3});
   ACTKV_CHECK_LAUNCH();
@@ -220,8 +220,10 @@ inline int score_tc_launch_lse(ScoreArgs& a, const actkv_pool_t* pool, int max_w
   const int64_t units = (int64_t)a.n_layers_sub * a.pool.n_kv_heads * a.tab.n_req;
   const int64_t grid = units * a.n_chunks * ta.n_rg;
   if (grid > 0x7fffffffLL) return ACTKV_E_INVALID;
-  return pool->head_dim == 64 ? score_tc_launch_lse_c<1>(kmap, qmap, ta, (unsigned)grid, s)
-                              : score_tc_launch_lse_c<2>(kmap, qmap, ta, (unsigned)grid, s);
+  const bool regs = tc::lse_moves(max_win * a.group);
+  if (pool->head_dim == 64)
+    return regs ? score_tc_launch_lse_c<1, true>(kmap, qmap, ta, (unsigned)grid, s) : score_tc_launch_lse_c<1, false>(kmap, qmap, ta, (unsigned)grid, s);
+  return regs ? score_tc_launch_lse_c<2, true>(kmap, qmap, ta, (unsigned)grid, s) : score_tc_launch_lse_c<2, false>(kmap, qmap, ta, (unsigned)grid, s);
 }
 
 template <int G>

@@ -132,6 +132,10 @@ __host__ __device__ constexpr int lse_group_rows(int n_rg) { return n_rg == 1 ? 
 // Two blocks of which the second is short change places on odd tiles (exclusive or with this): the short one would otherwise always
 // fall to the same accumulator.
 __device__ __forceinline__ int lse_flip(int rows) { return (rows + 63) / 64 == 3 ? 1 : 0; }
+// Launches whose longest window is an item of blocks that change places with every job (these two, and three): the kernel that keeps
+// all (reference, sum) in registers, four more.  384 rows 265 -> 252 us, 192 rows 177 -> 174 (4 layers x 8 heads, 4 x 16000 keys), 16 requests of
+// 140-348 rows 1565 -> 1543; other launches are slower with it: 512 rows, 8 x 35000 keys, 1405 -> 1415, a step of one 4K request 38.04 -> 38.27.
+inline bool lse_moves(int rows) { return rows > 256 ? rows <= 384 : rows > 128 && rows <= 192; }
 
 // A work item: the rows [row0, row0 + rows) of a unit against n_tiles key tiles.  n_tiles = 0: no more items.
 struct LseItem {
@@ -305,7 +309,8 @@ __device__ __forceinline__ void lse_merge(const float2 (&state)[2][LSE_MB][2][12
 }
 
 // NH: 64-dim halves of the head dimension (head_dim = 64 NH); a K tile is NH x [128 keys][64 bf16].
-template <int NPOLY, int NH, bool WIN>
+// REGS: what the epilogue carries of all blocks of an item stays in registers (lse_moves).
+template <int NPOLY, int NH, bool WIN, bool REGS>
 __global__ void __launch_bounds__(LSE_THREADS, 1)
 score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap qmap, const TcArgs ta,
                     const Exp2Cubic cubic) {
@@ -619,9 +624,9 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
       const int n_jobs = n_tiles * n_mb, b_short = twice ? n_mb - 1 : -1;
       float2* st0 = &bars->state[sp][grp][0][half][rib];
       int key0 = (x->t_begin + (n_mb == 1 ? grp : 0)) * TK + half * 64;
-      // Two blocks that change places, and three: the next job is of the block before this one, cyclically, and of the same tile only
-      // from the first of three to the last.  The (reference, sum) of all blocks stay in registers: ms is the next job's, m1 and m2 the
-      // ones after it (in shared memory 284 -> 276 us for 384 rows, 4 layers x 8 heads, 4 x 16000 keys, at the power cap; 192 rows 179 -> 174).
+      // A group that stays with one row block keeps its (reference, sum) in registers and has little left to count per job.  Two blocks
+      // that change places, and three: the next job is of the block before this one, cyclically, and of the same tile only from the first
+      // of three to the last.  REGS: ms is the next job's (reference, sum), m1 and m2 those of the jobs after it.
       int b = n_mb == 1 ? 0 : grp;
       bool wide = b != b_short;
       int off = wide ? 0 : upper * 32;
@@ -634,17 +639,22 @@ score_tc_lse_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_const
         fpar ^= 1u;
         key0 += step;
         if (moves) {
+          if constexpr (!REGS) st0[b * (2 * 128)] = ms;
           if (b == 0 && n_mb == 3) key0 -= TK;
           b = (b == 0 ? n_mb : b) - 1;
           wide = b != b_short;
           off = wide ? 0 : upper * 32;
-          const float2 t = ms;
-          ms = m1;
-          if (n_mb == 3) { m1 = m2; m2 = t; } else m1 = t;
+          if constexpr (REGS) {
+            const float2 t = ms;
+            ms = m1;
+            if (n_mb == 3) { m1 = m2; m2 = t; } else m1 = t;
+          } else {
+            ms = st0[b * (2 * 128)];
+          }
         }
       }
-      if (moves || grp < n_jobs) st0[b * (2 * 128)] = ms;
-      if (moves) {
+      if (REGS ? moves || grp < n_jobs : !moves && grp < n_jobs) st0[b * (2 * 128)] = ms;
+      if (REGS && moves) {
         b = (b == 0 ? n_mb : b) - 1;
         st0[b * (2 * 128)] = m1;
         if (n_mb == 3) st0[(b == 0 ? 2 : b - 1) * (2 * 128)] = m2;
