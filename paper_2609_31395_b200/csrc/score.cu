@@ -112,7 +112,7 @@ static int score_impl(int mode, const actkv_pool_t* pool, const actkv_tables_t* 
     if (use_tc && (mode & 1))
       n_chunks = tc::lse_split((int64_t)nls * Hkv * R * tc::lse_row_groups(max_win * G), (max_tok + tc::TK - 1) / tc::TK,
                                  (double)sum_tok / ((double)R * max_tok), (double)sum_win / ((double)R * max_win),
-                                 tc::lse_item_overhead(max_win * G, D), lay.n_chunks_max);
+                                 tc::lse_item_overhead(max_win * G, D), tc::lse_tail(max_win * G), lay.n_chunks_max);
     int chunk = (max_tok + n_chunks - 1) / n_chunks;
     chunk = (chunk + 127) / 128 * 128;
     if (chunk < LSE_CHUNK) chunk = LSE_CHUNK;

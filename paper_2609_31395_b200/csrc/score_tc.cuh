@@ -79,6 +79,9 @@ inline double lse_item_overhead(int rows, int head_dim) {
   return rows <= 128 ? 3.0 : rows > 256 && rows <= 384 && head_dim == 128 ? 2.8 : 2.0;
 }
 
+// Share of a last item by which launches of unequal requests end late: half of one of two blocks, and as many jobs of one of three.
+inline double lse_tail(int rows) { return rows > 256 && rows <= 384 ? 0.75 : 0.5; }
+
 // Chunks per unit of the LSE pass, whose CTAs go on from item to item, for a launch over `units` units of `tiles` key tiles, an item costing
 // its tiles and `ovh` more.  Equal units run in rounds of 148 of which the last is partly empty; requests of different lengths or windows
 // (mean over longest: `len`, `win`) spread evenly but for the last items, half of one on average, once there are more items than SMs.
@@ -86,7 +89,7 @@ inline double lse_item_overhead(int rows, int head_dim) {
 // 8 layers x 8 heads, 4 requests of 6500-15000 keys, head_dim 64, 200-512 rows: 410 us with whole units, 341 with the three chunks this
 // gives (four 336, five 334, eight 344).  4 layers x 8 heads, 4 x 16000 keys, 192 rows: 148 us with whole units, 158 with eight chunks (half
 // a percent in the model decided for those before).
-inline int lse_split(int64_t units, int tiles, double len, double win, double ovh, int n_max) {
+inline int lse_split(int64_t units, int tiles, double len, double win, double ovh, double tail, int n_max) {
   const bool equal = len > 0.999 && win > 0.999;
   int best = 1;
   double best_t = 1e300;
@@ -97,7 +100,7 @@ inline int lse_split(int64_t units, int tiles, double len, double win, double ov
     double t;
     if (equal) t = (double)((items + 147) / 148) * (tpc + ovh);
     else if (items <= 148) t = tpc + ovh;
-    else t = ((double)units * tiles * len * win + (double)items * len * ovh) / 148.0 + 0.5 * (tpc + ovh);
+    else t = ((double)units * tiles * len * win + (double)items * len * ovh) / 148.0 + tail * (tpc + ovh);
     if (t < best_t * (equal ? 0.99 : 0.995)) { best_t = t; best = n; }
   }
   return best;
